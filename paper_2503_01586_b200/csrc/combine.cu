@@ -6,17 +6,25 @@
 //   o[b,h,:] = o_lat . W_uv[:, h*d_h:(h+1)*d_h]        (B^v folded outwards, Section 5;
 //                                                      V = c W_uv of Section 3.2)
 //
-// Fast kernel (d_h = 128, d_c % 128 == 0): grid (n_h, d_c/128).  A block owns one head and one
-// 128-wide slice of the latent axis: it stages W_uv's [128 x 128] sub-block in shared memory
-// once, then for every group of 16 sequences merges the items' partial outputs of its slice
-// (16-byte loads, weights 2^(m_s-M)/L) and multiplies.  The d_c/128 slice results of a head are
-// written to scratch; the block that finishes last for that (head, sequence group) adds them in
-// a fixed order and writes bf16, so the result does not depend on scheduling.
+// Fast kernel (d_h = 128, d_c % 128 == 0): grid (n_h, d_c/128, groups of 16 rows; a row is a
+// sequence, or a query row of one).  A block stages W_uv's [128 x 128] sub-block of its head and
+// latent slice in shared memory, merges the items' partial outputs of its slice (16-byte loads,
+// weights 2^(m_s-M)/L) and multiplies.  The d_c/128 slice results of a head are written to
+// scratch; the block that finishes last for that (head, group) adds them in a fixed order and
+// writes bf16, so the result does not depend on scheduling.
+//
+// Bound: the latency of its dependent trips to L2 (a few MB to tens of MB move in ~10 us).  So
+// groups are blocks of their own and not a loop (a [128 x 128] weight block read again from L2
+// costs less than another round of trips), a warp takes its two rows from the statistics to the
+// merged result without a block barrier, and the first partial results are requested together
+// with the statistics.  Time from the end of the split-K kernel to the end of this one, against the
+// form that looped over groups with a barrier per step: 7B 75 % B16 17 -> 11 us, ragged B64 61 -> 30,
+// 13B B32 44 -> 26, 50 % B32 50 -> 35, 87.5 % B32 33 -> 12, four rows x B16 36 -> 27.
 //
 // Generic kernel: any even d_h <= 512, any d_c; block per (head, 8 sequences).
 //
-// With several query rows per sequence the kernels see rows x heads "heads" (n_h below); entry
-// i * heads + h multiplies with head h's columns of W_uv (n_phys = heads).
+// With several query rows per sequence the partial results are [item][row][head]; every row uses
+// its head's columns of W_uv.
 //
 // With separated latents (S-LRD) the partial outputs span the value latent only; `d_c` below is
 // then d_cv and W_uv is B^v_S.
@@ -33,176 +41,178 @@ __device__ __forceinline__ void mma_bf16_16816(float* c, const uint32_t* a, uint
 }
 
 // ------------------------------------------------------------------ fast path
-constexpr int kFB = 16;          // sequences per group
+constexpr int kFB = 16;          // rows (sequence, query row) per block
 constexpr int kFK = 128;         // latent slice
 constexpr int kFD = 128;         // head dim
 constexpr int kFThreads = 256;
-constexpr int kFI = 16;          // items per sequence whose merge weights are staged in shared memory
-constexpr int kFStage = 448;     // items per sequence group whose (m, l) are staged in shared memory
+constexpr int kFPitch = kFD + 8; // shared-memory row pitch in bf16: 16 bytes of padding keep ldmatrix free of bank conflicts
+constexpr int kFAhead = 4;       // partial results per row in flight beside the statistics
 
-__global__ void __launch_bounds__(kFThreads)
+__device__ __forceinline__ void ldmatrix_x4(uint32_t* r, const bf16* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, const bf16* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+__global__ void __launch_bounds__(kFThreads, 4)
 combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by the split-K kernel while this
                                                                    // kernel may already be resident: read
                                                                    // with plain L2 loads, never ld.global.nc
                     const int32_t* seq_first, const bf16* __restrict__ Wuv,
-                    float* __restrict__ slice_out /* [n_slices][B][n_h][128] */,
-                    int32_t* __restrict__ counters /* [n_h][n_groups], zeroed by the plan kernel */,
-                    bf16* __restrict__ out, int B, int n_h /* query rows x heads */, int n_phys /* heads */,
-                    int d_c) {
-  __shared__ __align__(16) bf16 s_w[kFK][kFD + 8];      // W_uv slice; rows padded by 16 bytes so that the
-                                                        // fragment loads of the product spread over the banks
-  __shared__ __align__(16) float s_x[kFB][kFK + 8];     // merged latent outputs (padded rows: bank spread)
-  __shared__ float s_M[kFB], s_invL[kFB];
-  __shared__ float s_wt[kFB][kFI];
-  __shared__ float2 s_ml[kFStage];
-  __shared__ int s_first[kFB + 1];
+                    float* __restrict__ slice_out /* [n_slices][B * rows][n_h][128] */,
+                    int32_t* __restrict__ counters /* [n_h][groups], zeroed by the plan kernel */,
+                    bf16* __restrict__ out, int B, int rows, int n_h, int d_c) {
+  __shared__ __align__(16) bf16 s_w[kFK][kFPitch];        // W_uv slice
+  __shared__ __align__(16) bf16 s_hi[kFB][kFPitch];       // merged latent outputs: bf16 head ...
+  __shared__ __align__(16) bf16 s_lo[kFB][kFPitch];       // ... and remainder
   __shared__ int s_last;
-  const int h = blockIdx.x, slice = blockIdx.y, n_slices = gridDim.y;
+  const int h = blockIdx.x, slice = blockIdx.y, n_slices = gridDim.y, g = blockIdx.z;
   const int k0 = slice * kFK;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n_rows = B * rows, r0 = g * kFB, nb = min(kFB, n_rows - r0);
 
-  // W_uv[k0 + k][h*128 + d] -> shared, 16-byte asynchronous copies that land while the softmax
-  // statistics of the first group are worked out
+  // W_uv[k0 + k][h*128 + d] -> shared, 16-byte asynchronous copies that land while the split-K
+  // kernel drains and the partial results are merged
   for (int e = tid; e < kFK * (kFD / 8); e += kFThreads) {
     const int k = e / (kFD / 8), v = e % (kFD / 8);
-    cp_async16(&s_w[k][v * 8], Wuv + (size_t)(k0 + k) * n_phys * kFD + (size_t)(h % n_phys) * kFD + v * 8);
+    cp_async16(&s_w[k][v * 8], Wuv + (size_t)(k0 + k) * n_h * kFD + (size_t)h * kFD + v * 8);
   }
   cp_async_commit();
-  const int n_groups = (B + kFB - 1) / kFB;
-  // The plan (seq_first) was written before the split-K kernel started computing (that kernel
-  // waited for it before it let this one be launched), so the first group's item ranges are
-  // fetched while the split-K kernel is still running.
-  if (tid <= min(kFB, B)) s_first[tid] = __ldcg(seq_first + tid);
+  // Row r = (sequence r / rows, query row r % rows).  Warp w merges rows 2w and 2w + 1; half a warp
+  // holds a row's softmax statistics, lane j of the half those of its j-th item.  The plan was
+  // written before the split-K kernel started computing (that kernel waited for it before it let
+  // this one be launched), so the item ranges are fetched while the split-K kernel still runs.
+  const int half = lane >> 4, j = lane & 15;
+  int i0[2], ni[2];
+  size_t src0[2];                // first partial result of the row on this slice, in floats
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int rr = 2 * warp + e;
+    i0[e] = ni[e] = 0;
+    src0[e] = 0;
+    if (rr < nb) {
+      const int b = (r0 + rr) / rows, q = (r0 + rr) % rows;
+      i0[e] = __ldcg(seq_first + b);
+      ni[e] = __ldcg(seq_first + b + 1) - i0[e];
+      src0[e] = (((size_t)i0[e] * rows + q) * n_h + h) * d_c + k0 + lane * 4;
+    }
+  }
+  const size_t stride = (size_t)rows * n_h * d_c;                // from one item to the next
+  const int my_i0 = half ? i0[1] : i0[0], my_ni = half ? ni[1] : ni[0];
+  const int my_q = (r0 + 2 * warp + half) % rows;
+  auto item_ml = [&](int k) -> float2 {
+    return __ldcg((const float2*)part_ml + ((size_t)(my_i0 + k) * rows + my_q) * n_h + h);
+  };
   ekv_pdl_wait();         // everything below reads the split-K kernel's output
+  ekv_pdl_trigger();
 
-  for (int g = 0; g < n_groups; ++g) {
-    const int b0 = g * kFB, nb = min(kFB, B - b0);
-    __syncthreads();
-    if (g > 0 && tid <= nb) s_first[tid] = __ldcg(seq_first + b0 + tid);
-    __syncthreads();
-    // (m, l) of the group's items for this head: one trip to global memory, then shared
-    const int gi0 = s_first[0], gin = s_first[nb] - gi0;
-    for (int e = tid; e < min(gin, kFStage); e += kFThreads)
-      s_ml[e] = __ldcg((const float2*)(part_ml + ((size_t)(gi0 + e) * n_h + h) * 2));
-    __syncthreads();
-    auto item_ml = [&](int i) -> float2 {
-      return i - gi0 < kFStage ? s_ml[i - gi0] : __ldcg((const float2*)(part_ml + ((size_t)i * n_h + h) * 2));
-    };
-    // softmax statistics per sequence: one warp each
-    for (int bb = warp; bb < nb; bb += kFThreads / 32) {
-      const int i0 = s_first[bb], i1 = s_first[bb + 1];
-      float M = -INFINITY;
-      for (int i = i0 + lane; i < i1; i += 32) M = fmaxf(M, item_ml(i).x);
-      M = warp_max(M);
-      float Ls = 0.f;
-      for (int i = i0 + lane; i < i1; i += 32) {
-        const float2 ml = item_ml(i);
-        Ls += ml.y * exp2f(ml.x - M);
-      }
-      Ls = warp_sum(Ls);
-      if (lane == 0) {
-        s_M[bb] = M;
-        s_invL[bb] = (i1 > i0 && Ls > 0.f) ? 1.f / Ls : 0.f;
-      }
+  // statistics and the first partial results of both rows are requested together
+  float2 ml = make_float2(-INFINITY, 0.f);
+  if (j < my_ni) ml = item_ml(j);
+  float4 p[2][kFAhead];
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+#pragma unroll
+    for (int k = 0; k < kFAhead; ++k)
+      p[e][k] = k < ni[e] ? __ldcg((const float4*)(part_acc + src0[e] + k * stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float M = ml.x;
+  for (int k = j + 16; k < my_ni; k += 16) M = fmaxf(M, item_ml(k).x);       // rare: more than 16 items
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  float L = j < my_ni ? ml.y * exp2f(ml.x - M) : 0.f;
+  for (int k = j + 16; k < my_ni; k += 16) {
+    const float2 x = item_ml(k);
+    L += x.y * exp2f(x.x - M);
+  }
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+  const float invL = my_ni > 0 && L > 0.f ? 1.f / L : 0.f;
+  float wt = j < my_ni ? exp2f(ml.x - M) * invL : 0.f;                      // normalised weight of item j
+  float4 acc[2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [](float4& x, float w, const float4& y) {
+    x.x = fmaf(w, y.x, x.x); x.y = fmaf(w, y.y, x.y); x.z = fmaf(w, y.z, x.z); x.w = fmaf(w, y.w, x.w);
+  };
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+#pragma unroll
+    for (int k = 0; k < kFAhead; ++k) add(acc[e], __shfl_sync(0xffffffffu, wt, 16 * e + k), p[e][k]);
+  const int n_most = max(ni[0], ni[1]);
+  for (int k0b = kFAhead; k0b < n_most; k0b += kFAhead) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+      for (int k = 0; k < kFAhead; ++k)
+        p[e][k] = k0b + k < ni[e] ? __ldcg((const float4*)(part_acc + src0[e] + (size_t)(k0b + k) * stride))
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+    if ((k0b & 15) == 0) wt = k0b + j < my_ni ? exp2f(item_ml(k0b + j).x - M) * invL : 0.f;
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+      for (int k = 0; k < kFAhead; ++k) add(acc[e], __shfl_sync(0xffffffffu, wt, 16 * e + ((k0b + k) & 15)), p[e][k]);
+  }
+  // the fp32 rows are fed to the product as a bf16 head plus a bf16 remainder, so nothing but the
+  // last ~2^-17 of them is lost; W_uv is bf16 as stored
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const bf162 h0 = __floats2bfloat162_rn(acc[e].x, acc[e].y), h1 = __floats2bfloat162_rn(acc[e].z, acc[e].w);
+    const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+    const bf162 l0 = __floats2bfloat162_rn(acc[e].x - f0.x, acc[e].y - f0.y);
+    const bf162 l1 = __floats2bfloat162_rn(acc[e].z - f1.x, acc[e].w - f1.y);
+    *(uint2*)&s_hi[2 * warp + e][lane * 4] = make_uint2(*(const uint32_t*)&h0, *(const uint32_t*)&h1);
+    *(uint2*)&s_lo[2 * warp + e][lane * 4] = make_uint2(*(const uint32_t*)&l0, *(const uint32_t*)&l1);
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  // [16 x 128] . [128 x 128] on mma.sync (m16n8k16, bf16 in, fp32 accumulate): one warp per 16 output dims
+  {
+    const int n0 = warp * 16;
+    float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+    for (int kk = 0; kk < kFK; kk += 16) {
+      uint32_t ahi[4], alo[4], w[4];
+      ldmatrix_x4(ahi, &s_hi[lane & 15][kk + (lane >> 4) * 8]);
+      ldmatrix_x4(alo, &s_lo[lane & 15][kk + (lane >> 4) * 8]);
+      ldmatrix_x4_trans(w, &s_w[kk + (lane & 15)][n0 + (lane >> 4) * 8]);
+      mma_bf16_16816(c[0], ahi, w[0], w[1]);
+      mma_bf16_16816(c[1], ahi, w[2], w[3]);
+      mma_bf16_16816(c[0], alo, w[0], w[1]);
+      mma_bf16_16816(c[1], alo, w[2], w[3]);
     }
-    __syncthreads();
-    // normalised merge weights 2^(m_s - M) / L of the first kFI items of every sequence
-    for (int e = tid; e < kFB * kFI; e += kFThreads) {
-      const int bb = e / kFI, j = e % kFI;
-      float wv = 0.f;
-      if (bb < nb) {
-        const int i = s_first[bb] + j;
-        if (i < s_first[bb + 1]) wv = exp2f(item_ml(i).x - s_M[bb]) * s_invL[bb];
-      }
-      s_wt[bb][j] = wv;
+    const int gr = lane >> 2, t = lane & 3;
+    float* dst = slice_out + (((size_t)slice * n_rows + r0) * n_h + h) * kFD + n0 + 2 * t;
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      if (gr < nb) __stcg((float2*)(dst + (size_t)gr * n_h * kFD + nt * 8), make_float2(c[nt][0], c[nt][1]));
+      if (gr + 8 < nb) __stcg((float2*)(dst + (size_t)(gr + 8) * n_h * kFD + nt * 8), make_float2(c[nt][2], c[nt][3]));
     }
-    __syncthreads();
-    // merge the items of each sequence on this latent slice (independent 16-byte loads)
-    for (int e = tid; e < kFB * (kFK / 4); e += kFThreads) {
-      const int bb = e / (kFK / 4), v = e % (kFK / 4);
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (bb < nb) {
-        const int i0 = s_first[bb], ni = s_first[bb + 1] - i0;
-        const float* src = part_acc + ((size_t)i0 * n_h + h) * d_c + k0 + v * 4;
-        const size_t stride = (size_t)n_h * d_c;
-        const int nfast = min(ni, kFI);
-        // eight independent 16-byte loads in flight per thread
-        for (int j0 = 0; j0 < nfast; j0 += 8) {
-          float4 p[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            p[j] = j0 + j < nfast ? __ldcg((const float4*)(src + (size_t)(j0 + j) * stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float w = j0 + j < nfast ? s_wt[bb][j0 + j] : 0.f;
-            acc.x = fmaf(w, p[j].x, acc.x); acc.y = fmaf(w, p[j].y, acc.y);
-            acc.z = fmaf(w, p[j].z, acc.z); acc.w = fmaf(w, p[j].w, acc.w);
-          }
-        }
-        for (int j = kFI; j < ni; ++j) {     // rare: a sequence cut into more than kFI items
-          const float w = exp2f(item_ml(i0 + j).x - s_M[bb]) * s_invL[bb];
-          const float4 p = __ldcg((const float4*)(src + (size_t)j * stride));
-          acc.x = fmaf(w, p.x, acc.x); acc.y = fmaf(w, p.y, acc.y);
-          acc.z = fmaf(w, p.z, acc.z); acc.w = fmaf(w, p.w, acc.w);
-        }
-      }
-      *(float4*)&s_x[bb][v * 4] = acc;
-    }
-    cp_async_wait<0>();      // the W_uv slice (first group only; later a no-op)
-    __syncthreads();
-    // [16 x 128] . [128 x 128] on mma.sync (m16n8k16, bf16 in, fp32 accumulate): one warp per 16
-    // output dims.  The fp32 rows of x are fed as a bf16 head plus a bf16 remainder (two MMAs),
-    // so nothing but the last ~2^-17 of x is lost; W_uv is bf16 as stored.
-    {
-      const int g = lane >> 2, t = lane & 3, n0 = warp * 16;
-      float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll 2
-      for (int kk = 0; kk < kFK; kk += 16) {
-        uint32_t ahi[4], alo[4];
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          const float2 x = *(const float2*)&s_x[g + (f & 1) * 8][kk + 2 * t + (f >> 1) * 8];
-          const bf162 hi = __floats2bfloat162_rn(x.x, x.y);
-          const float2 hf = __bfloat1622float2(hi);
-          const bf162 lo = __floats2bfloat162_rn(x.x - hf.x, x.y - hf.y);
-          ahi[f] = *(const uint32_t*)&hi;
-          alo[f] = *(const uint32_t*)&lo;
-        }
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-          const unsigned short* wp = (const unsigned short*)&s_w[kk + 2 * t][n0 + nt * 8 + g];
-          const uint32_t b0r = (uint32_t)wp[0] | ((uint32_t)wp[kFD + 8] << 16);
-          const uint32_t b1r = (uint32_t)wp[8 * (kFD + 8)] | ((uint32_t)wp[9 * (kFD + 8)] << 16);
-          mma_bf16_16816(acc[nt], ahi, b0r, b1r);
-          mma_bf16_16816(acc[nt], alo, b0r, b1r);
-        }
-      }
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const int d = n0 + nt * 8 + 2 * t;
-        if (g < nb)
-          *(float2*)(slice_out + (((size_t)slice * B + b0 + g) * n_h + h) * kFD + d) = make_float2(acc[nt][0], acc[nt][1]);
-        if (g + 8 < nb)
-          *(float2*)(slice_out + (((size_t)slice * B + b0 + g + 8) * n_h + h) * kFD + d) = make_float2(acc[nt][2], acc[nt][3]);
-      }
-    }
-    // last block of this (head, group) adds the slices in order
+  }
+  // the block of a (head, group) that arrives last adds the slices in order
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&counters[h * gridDim.z + g], 1) == n_slices - 1;
+  __syncthreads();
+  if (s_last) {
     __threadfence();
-    __syncthreads();
-    if (tid == 0) s_last = atomicAdd(&counters[h * n_groups + g], 1) == n_slices - 1;
-    __syncthreads();
-    if (s_last) {
-      __threadfence();
-      for (int e = tid; e < nb * (kFD / 2); e += kFThreads) {
-        const int bb = e / (kFD / 2), p2 = e % (kFD / 2);
-        float2 v = make_float2(0.f, 0.f);
-        for (int s = 0; s < n_slices; ++s) {
-          const float2 t = __ldcg((const float2*)(slice_out + (((size_t)s * B + b0 + bb) * n_h + h) * kFD + 2 * p2));
-          v.x += t.x;
-          v.y += t.y;
-        }
-        *(bf162*)(out + ((size_t)(b0 + bb) * n_h + h) * kFD + 2 * p2) = __floats2bfloat162_rn(v.x, v.y);
+    for (int e = tid; e < nb * (kFD / 4); e += kFThreads) {
+      const int rr = e / (kFD / 4), d = (e % (kFD / 4)) * 4;
+      const float* src = slice_out + ((size_t)(r0 + rr) * n_h + h) * kFD + d;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int s = 0; s < n_slices; ++s) {
+        const float4 y = __ldcg((const float4*)(src + (size_t)s * n_rows * n_h * kFD));
+        v.x += y.x; v.y += y.y; v.z += y.z; v.w += y.w;
       }
+      const bf162 o0 = __floats2bfloat162_rn(v.x, v.y), o1 = __floats2bfloat162_rn(v.z, v.w);
+      bf162* dst = (bf162*)(out + ((size_t)(r0 + rr) * n_h + h) * kFD + d);      // the caller's `out` is 4-byte aligned
+      dst[0] = o0;
+      dst[1] = o1;
     }
   }
 }
@@ -323,10 +333,11 @@ int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, v
   // and of the output; it uses head h's slice of W_uv
   const int nv = (ws.rows > 0 ? ws.rows : 1) * L->n_h;
   if (ekv_combine_fast_ok(L)) {
-    dim3 grid(nv, L->vw / kFK);
+    const int rows = ws.rows > 0 ? ws.rows : 1;
+    dim3 grid(L->n_h, L->vw / kFK, (B * rows + kFB - 1) / kFB);
     EKV_CUDA_OK(ekv_launch_pdl(combine_fast_kernel, grid, dim3(kFThreads), 0, st, (const float*)ws.part_acc,
                                (const float*)ws.part_ml, (const int32_t*)ws.seq_first, (const bf16*)L->d_Wuv,
-                               ws.slice_out, ws.counters, (bf16*)out, B, nv, L->n_h, L->vw));
+                               ws.slice_out, ws.counters, (bf16*)out, B, rows, L->n_h, L->vw));
     EKV_CUDA_OK(cudaGetLastError());
     return ELITEKV_OK;
   }
