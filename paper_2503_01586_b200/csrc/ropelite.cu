@@ -12,163 +12,285 @@
 // so with D_i = a_i (cos(phi) - 1) - b_i sin(phi) the difference between the fully rotated score
 // and the trial score is  R - D_j,  R = sum of D_i over the chunks not in e.  One pass over the
 // pairs therefore yields the distances of ALL candidates of a round:  dist[j] = sum |R - D_j|.
-// This is FP32 arithmetic on CUDA cores (there is no contraction deeper than 2 here).
+// With both vectors rotated by HALF their angle, q' = q e^{i m theta/2}, k' = k e^{i n theta/2},
+//     D_i = -2 sin((m - n) theta_i / 2) (q'_y k'_x - q'_x k'_y),
+// three FP32 operations instead of six, and just as exact at small angles (the sine is a factor,
+// nothing cancels).  The common sign is dropped: D_i = s_i t_i, s = 2 sin(.), t = q'_y k'_x - q'_x k'_y.
 //
-// distance kernel: grid (row tiles of 16 query positions, heads), 128 threads.  Warp w owns query
-// rows m0 + 4 w .. m0 + 4 w + 3, its lanes own keys; key tiles of 64 are staged in shared memory as fp32 pairs
-// [chunk][key] together with the slice of the (cos - 1, sin) table the tile's relative positions
-// need, [chunk][m - n].  A thread keeps the 64 D_i of its pair and 64 running sums in registers.
-// Block results go to a [head][row tile][chunk] array; the select kernel adds them in a fixed
-// order (the result does not depend on scheduling), masks the chunks already chosen and takes
-// the first minimum.
+// Bound: FP32 issue (the contraction is 2 deep).  A thread owns 16 query rows x 4 keys, sums R over
+// the free chunks (t: multiply, FMA; R: FMA), then goes over the chunks once more for |R - D_j|
+// (FMA, add with |.|): 7 operations per pair and chunk, D_i is never stored, and the 64 pairs of a
+// thread share their operands, 15 16-byte shared-memory loads per chunk and pass.  32 heads x 2048
+// tokens x d_h 128: 1.58 ms a round (19 T FP32 lane operations/s, 0.51 of 148 SMs x 128 lanes x
+// 1.965 GHz; issue slots 66 % busy, shared-memory pipe 44 %).  The form that held the 64 D_i of one
+// pair in registers took 3.04 ms: 9 operations and three loads per pair and chunk, shared-memory
+// bound.  128 threads (one warp per scheduler): 1.87 ms; with the next chunk's operands fetched
+// ahead in registers: 2.09 ms.
+//
+// distance kernel: grid (items, heads), 256 threads; an item is 128 query rows x up to `span` key
+// tiles of 128.  Per key tile the rotated keys (x plane, y plane, [chunk][key]) and the slice of
+// the sine table that the tile's relative positions need are staged in shared memory; the table is
+// zero at negative relative positions, which is the causal mask.  Item results go to a
+// [head][item][chunk] array; the select kernel adds them in a fixed order (the result does not
+// depend on scheduling), masks the chunks already chosen and takes the first minimum.
 #include "common.cuh"
 
 namespace {
 
-constexpr int kRlRows = 16;       // query rows per block (four per warp)
-constexpr int kRlWarps = 4;
-constexpr int kRlRowsPerWarp = kRlRows / kRlWarps;
-constexpr int kRlKeys = 64;       // keys per stage
-constexpr int kRlThreads = 128;
-constexpr int kRlSpan = kRlKeys + kRlRows - 1;     // relative positions a stage can meet
-constexpr int kRlSpanPad = kRlSpan + 1;
+constexpr int kRlRows = 128;      // query rows per block
+constexpr int kRlTR = 16;         // ... per warp (and thread)
+constexpr int kRlKeys = 128;      // keys per stage
+constexpr int kRlTK = 4;          // ... per thread
+constexpr int kRlThreads = 256;
+constexpr int kRlAcc = 8;         // lanes of a warp that keep running distances
+constexpr int kRlSpan = kRlKeys + kRlRows;         // sine table entries of a stage (relative positions, reversed)
+constexpr int kRlPad = 256;       // zeros behind the sine table: negative relative positions
+static_assert(kRlRows == kRlThreads / 32 * kRlTR && kRlKeys == 32 * kRlTK, "thread tiles cover the block's tile");
 
-// (cos(d theta_i) - 1, sin(d theta_i)) for d in [0, n), laid out [chunk][d]; double precision,
-// rounded once
-__global__ void ropelite_table_kernel(float2* __restrict__ tab, int n, int half, int d_h, double base) {
+// entries of a chunk's reversed sine table: entry x holds 2 sin((n_up - x) theta / 2), zero past n_up
+__host__ __device__ inline int rl_n_up(int n) { return (n + kRlRows - 1) / kRlRows * kRlRows; }
+__host__ __device__ inline int rl_sin_len(int n) { return rl_n_up(n) + kRlPad; }
+
+// (cos, sin)(pos theta_i / 2) laid out [pos][chunk], and the reversed sine table [chunk][...];
+// double precision, rounded once
+__global__ void ropelite_table_kernel(float2* __restrict__ cs, float* __restrict__ sn, int n, int half, int d_h,
+                                      double base) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)n * half) return;
-  const int i = (int)(e / n), d = (int)(e % n);
-  const double theta = pow(base, -2.0 * (double)i / (double)d_h);
-  const double ang = (double)d * theta;
-  tab[e] = make_float2((float)(cos(ang) - 1.0), (float)sin(ang));
+  const int n_up = rl_n_up(n), len = rl_sin_len(n);
+  if (e >= (long long)len * half) return;
+  const int i = (int)(e % half), x = (int)(e / half);
+  const int pos = n_up - x;
+  float s2 = 0.f;
+  if (pos > 0) {
+    const double theta = pow(base, -2.0 * (double)i / (double)d_h);
+    double s, c;
+    sincos(0.5 * (double)pos * theta, &s, &c);
+    s2 = (float)(2.0 * s);
+    if (pos < n) cs[(size_t)pos * half + i] = make_float2((float)c, (float)s);
+  } else if (pos == 0) {
+    cs[i] = make_float2(1.f, 0.f);
+  }
+  sn[(size_t)i * len + x] = s2;
+}
+
+// four chunks (16 bytes) of a query or key row, rotated by half their angle
+__device__ __forceinline__ void rl_rotate4(const bf16* row, const float2* cs, float2* out) {
+  const uint4 raw = *(const uint4*)row;
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+  const float4 c01 = __ldg((const float4*)cs), c23 = __ldg((const float4*)cs + 1);
+  const float2 c[4] = {{c01.x, c01.y}, {c01.z, c01.w}, {c23.x, c23.y}, {c23.z, c23.w}};
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const float x = __uint_as_float(w[u] << 16), y = __uint_as_float(w[u] & 0xffff0000u);
+    out[u] = make_float2(x * c[u].x - y * c[u].y, x * c[u].y + y * c[u].x);
+  }
+}
+
+template <int HALF>
+struct RlSmem {
+  float kx[HALF][kRlKeys], ky[HALF][kRlKeys];
+  float sn[HALF][kRlSpan];
+  float2 q[HALF][kRlRows];
+  float acc[HALF][kRlThreads / 32 * kRlAcc];     // running distances
+  int list[HALF];                    // chunks not chosen yet
+};
+
+// operands of a thread's 64 pairs for one chunk
+struct RlOps {
+  float kx[kRlTK], ky[kRlTK], s[kRlTR + kRlTK];
+  float2 q[kRlTR];
+};
+template <int HALF>
+__device__ __forceinline__ void rl_load(RlOps& o, const RlSmem<HALF>& sm, int i, int warp, int lane) {
+  *(float4*)o.kx = *(const float4*)&sm.kx[i][lane * kRlTK];
+  *(float4*)o.ky = *(const float4*)&sm.ky[i][lane * kRlTK];
+  // entry u of the stage's slice: relative position (m0 - n0) + 128 - u; this thread's pairs need
+  // u = 4 lane + j - (16 warp + r) + 128, from 4 lane - 16 warp + 113 on
+  const float* sp = &sm.sn[i][kRlTK * lane - kRlTR * warp + kRlRows - kRlTR];
+#pragma unroll
+  for (int u = 0; u < (kRlTR + kRlTK) / 4; ++u) *(float4*)&o.s[4 * u] = *(const float4*)(sp + 4 * u);
+  const float4* qp = (const float4*)&sm.q[i][kRlTR * warp];
+#pragma unroll
+  for (int u = 0; u < kRlTR / 2; ++u) *(float4*)&o.q[2 * u] = qp[u];
 }
 
 template <int HALF>
 __global__ void __launch_bounds__(kRlThreads)
 ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, int n,
-                         const float2* __restrict__ tab, const unsigned long long* __restrict__ masks,
-                         float* __restrict__ partial /* [heads][row tiles][HALF] */) {
+                         const float2* __restrict__ cs, const float* __restrict__ sn,
+                         const unsigned long long* __restrict__ masks, int span,
+                         float* __restrict__ partial /* [heads][items][HALF] */) {
   constexpr int d_h = 2 * HALF;
-  extern __shared__ __align__(16) float2 smem_rl[];
-  // keys stay packed as they come (a bf16 pair per chunk: one 4-byte load per pair and chunk, widened in registers)
-  float2 (*s_t)[kRlSpanPad] = (float2 (*)[kRlSpanPad])smem_rl;                        // [HALF][relative position]
-  float2 (*s_q)[HALF] = (float2 (*)[HALF])(smem_rl + HALF * kRlSpanPad);             // [rows][HALF]
-  float (*s_red)[HALF] = (float (*)[HALF])(smem_rl + HALF * (kRlSpanPad + kRlRows)); // [warps][HALF]
-  uint32_t (*s_k)[kRlKeys] = (uint32_t (*)[kRlKeys])(&s_red[kRlWarps][0]);           // [HALF][keys]
-  const int n_tiles = gridDim.x;
-  const int mt = n_tiles - 1 - (int)blockIdx.x;          // long rows first
-  const int head = blockIdx.y;
+  extern __shared__ __align__(16) unsigned char smem_rl[];
+  RlSmem<HALF>& sm = *(RlSmem<HALF>*)smem_rl;
+  const int head = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // item -> (row tile, group of key tiles), long rows first
+  int mt = (n + kRlRows - 1) / kRlRows - 1, kg = blockIdx.x;
+  for (;; --mt) {
+    const int groups = ((mt + 1) * kRlRows + kRlKeys * span - 1) / (kRlKeys * span);
+    if (kg < groups) break;
+    kg -= groups;
+  }
   const int m0 = mt * kRlRows;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n_lo = kg * span * kRlKeys, n_hi = min(n_lo + span * kRlKeys, m0 + kRlRows);
   const unsigned long long mask = masks ? masks[head] : 0ull;
+  const int n_free = HALF - __popcll(HALF == 64 ? mask : mask & ((1ull << (HALF & 63)) - 1));
+  float* out = partial + ((size_t)head * gridDim.x + blockIdx.x) * HALF;
+  if (n_free <= 1) {                 // a single free chunk: R = D_j for every pair
+    for (int j = threadIdx.x; j < HALF; j += kRlThreads) out[j] = 0.f;
+    return;
+  }
+  if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
+    sm.list[threadIdx.x - __popcll(mask & ((1ull << threadIdx.x) - 1))] = threadIdx.x;
   const bf16* Qh = Q + (size_t)head * n * d_h;
   const bf16* Kh = K + (size_t)head * n * d_h;
-
-  for (int e = threadIdx.x; e < kRlRows * HALF; e += kRlThreads) {
-    const int rr = e / HALF, i = e % HALF;
-    float2 v = make_float2(0.f, 0.f);
-    if (m0 + rr < n) v = __bfloat1622float2(*(const bf162*)(Qh + (size_t)(m0 + rr) * d_h + 2 * i));
-    s_q[rr][i] = v;
-  }
-  float acc[HALF];
+  // (consecutive threads take consecutive rows: the transposed stores hit different banks)
+  for (int e = threadIdx.x; e < kRlRows * (HALF / 4); e += kRlThreads) {
+    const int rr = e % kRlRows, g4 = e / kRlRows;
+    float2 v[4] = {};
+    if (m0 + rr < n) rl_rotate4(Qh + (size_t)(m0 + rr) * d_h + g4 * 8, cs + (size_t)(m0 + rr) * HALF + g4 * 4, v);
 #pragma unroll
-  for (int j = 0; j < HALF; ++j) acc[j] = 0.f;
+    for (int u = 0; u < 4; ++u) sm.q[g4 * 4 + u][rr] = v[u];
+  }
+  for (int e = threadIdx.x; e < HALF * (kRlThreads / 32) * kRlAcc; e += kRlThreads) (&sm.acc[0][0])[e] = 0.f;
+  const int n_up = rl_n_up(n), sn_len = rl_sin_len(n);
 
-  const int m_last = min(m0 + kRlRows - 1, n - 1);
-  for (int n0 = 0; n0 <= m_last; n0 += kRlKeys) {
+  for (int n0 = n_lo; n0 < n_hi; n0 += kRlKeys) {
     __syncthreads();
-    // keys of the stage: consecutive threads take consecutive keys (conflict-free stores)
+    // entry u holds relative position (m0 - n0) + 128 - u (table entry n_up - that), so that the
+    // slice starts on a 16-byte boundary
+    const int x0 = n_up - (m0 - n0) - kRlRows;
+    for (int e = threadIdx.x; e < HALF * (kRlSpan / 4); e += kRlThreads) {
+      const int i = e / (kRlSpan / 4), u = (e % (kRlSpan / 4)) * 4;
+      cp_async16(&sm.sn[i][u], sn + (size_t)i * sn_len + x0 + u);
+    }
+    cp_async_commit();
+#pragma unroll
     for (int e = threadIdx.x; e < kRlKeys * (HALF / 4); e += kRlThreads) {
       const int nn = e % kRlKeys, g4 = e / kRlKeys;         // 4 chunks = 8 elements = 16 bytes
-      uint4 raw = make_uint4(0, 0, 0, 0);
-      if (n0 + nn < n) raw = *(const uint4*)(Kh + (size_t)(n0 + nn) * d_h + g4 * 8);
-      s_k[g4 * 4 + 0][nn] = raw.x; s_k[g4 * 4 + 1][nn] = raw.y;
-      s_k[g4 * 4 + 2][nn] = raw.z; s_k[g4 * 4 + 3][nn] = raw.w;
-    }
-    // table slice: relative positions d_min .. d_min + span - 1 (negative ones belong to masked pairs)
-    const int d_min = m0 - n0 - (kRlKeys - 1);
-    for (int e = threadIdx.x; e < HALF * kRlSpan; e += kRlThreads) {
-      const int i = e / kRlSpan, dd = e % kRlSpan;
-      const int d = d_min + dd;
-      s_t[i][dd] = (d >= 0 && d < n) ? tab[(size_t)i * n + d] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int e = 0; e < kRlRowsPerWarp * (kRlKeys / 32); ++e) {
-      const int rr = warp * kRlRowsPerWarp + e / (kRlKeys / 32);     // row inside the block
-      const int m = m0 + rr;
-      const int nn = lane + 32 * (e % (kRlKeys / 32));
-      const int key = n0 + nn;
-      if (!(key <= m && m < n)) continue;                  // causal pairs only
-      const int dd = rr + (kRlKeys - 1) - nn;              // (m - key) - d_min
-      float d[HALF];
-      float R = 0.f;
+      float2 v[4] = {};
+      if (n0 + nn < n) rl_rotate4(Kh + (size_t)(n0 + nn) * d_h + g4 * 8, cs + (size_t)(n0 + nn) * HALF + g4 * 4, v);
 #pragma unroll
-      for (int i = 0; i < HALF; ++i) {
-        const float2 q = s_q[rr][i], t = s_t[i][dd];
-        const uint32_t kp = s_k[i][nn];
-        const float2 k = make_float2(__uint_as_float(kp << 16), __uint_as_float(kp & 0xffff0000u));   // bf16 pair -> fp32
-        const float a = fmaf(q.x, k.x, q.y * k.y);
-        const float b = fmaf(q.y, k.x, -(q.x * k.y));
-        d[i] = fmaf(a, t.x, -(b * t.y));
-        if (!((mask >> i) & 1ull)) R += d[i];
+      for (int u = 0; u < 4; ++u) {
+        sm.kx[g4 * 4 + u][nn] = v[u].x;
+        sm.ky[g4 * 4 + u][nn] = v[u].y;
       }
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    if (n0 > m0 + kRlTR * warp + kRlTR - 1) continue;       // every pair of this warp lies above the diagonal
+    float R[kRlTR][kRlTK];
 #pragma unroll
-      for (int j = 0; j < HALF; ++j) acc[j] += fabsf(R - d[j]);
+    for (int r = 0; r < kRlTR; ++r)
+#pragma unroll
+      for (int j = 0; j < kRlTK; ++j) R[r][j] = 0.f;
+#pragma unroll 2
+    for (int c = 0; c < n_free; ++c) {
+      RlOps o;
+      rl_load(o, sm, sm.list[c], warp, lane);
+#pragma unroll
+      for (int r = 0; r < kRlTR; ++r)
+#pragma unroll
+        for (int j = 0; j < kRlTK; ++j) {
+          const float t = fmaf(o.q[r].y, o.kx[j], -(o.q[r].x * o.ky[j]));
+          R[r][j] = fmaf(o.s[j - r + kRlTR], t, R[r][j]);
+        }
+    }
+#pragma unroll 2
+    for (int c = 0; c < n_free; ++c) {
+      RlOps o;
+      const int i = sm.list[c];
+      rl_load(o, sm, i, warp, lane);
+      float v[kRlTK] = {};
+#pragma unroll
+      for (int r = 0; r < kRlTR; ++r)
+#pragma unroll
+        for (int j = 0; j < kRlTK; ++j) {
+          const float t = fmaf(o.q[r].y, o.kx[j], -(o.q[r].x * o.ky[j]));
+          v[j] += fabsf(fmaf(-o.s[j - r + kRlTR], t, R[r][j]));
+        }
+      float d = (v[0] + v[1]) + (v[2] + v[3]);
+      d += __shfl_xor_sync(0xffffffffu, d, 16);
+      d += __shfl_xor_sync(0xffffffffu, d, 8);
+      if (lane < kRlAcc) sm.acc[i][warp * kRlAcc + lane] += d;
     }
   }
-  // block result: lanes, then warps, in a fixed order
-#pragma unroll
-  for (int j = 0; j < HALF; ++j) {
-    const float v = warp_sum(acc[j]);
-    if (lane == 0) s_red[warp][j] = v;
-  }
+  // block result: threads in a fixed order
   __syncthreads();
-  for (int j = threadIdx.x; j < HALF; j += kRlThreads) {
+  for (int j = warp; j < HALF; j += kRlThreads / 32) {
     float v = 0.f;
 #pragma unroll
-    for (int w = 0; w < kRlWarps; ++w) v += s_red[w][j];
-    partial[((size_t)head * n_tiles + mt) * HALF + j] = v;
+    for (int w = 0; w < kRlThreads / 32 * kRlAcc; w += 32) v += sm.acc[j][w + lane];
+    v = warp_sum(v);
+    if (lane == 0) out[j] = v;
   }
 }
 
-// One block per head: adds the row tiles' results in order, writes the round's distances
+// One block per head: adds the items' results in a fixed order, writes the round's distances
 // (+inf for chunks already chosen) and, when `elite_idx` is given, appends the first minimum to
 // the head's list and to its mask.
-__global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_tiles, int half,
+constexpr int kRlSelect = 8;      // threads per chunk
+__global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_items, int half,
                                        unsigned long long* __restrict__ masks, float* __restrict__ dist_out,
                                        int32_t* __restrict__ elite_idx, int r, int round) {
-  __shared__ float s_d[64];
-  const int head = blockIdx.x, j = threadIdx.x;
+  __shared__ float s_d[kRlSelect][64];
+  const int head = blockIdx.x, j = threadIdx.x & 63, part = threadIdx.x >> 6;
   const unsigned long long mask = masks ? masks[head] : 0ull;
-  float v = INFINITY;
-  if (j < half && !((mask >> j) & 1ull)) {
-    v = 0.f;
-    for (int t = 0; t < n_tiles; ++t) v += partial[((size_t)head * n_tiles + t) * half + j];
+  float v = 0.f;
+  if (j < half) {
+    const float* src = partial + (size_t)head * n_items * half + j;
+#pragma unroll 4
+    for (int t = part; t < n_items; t += kRlSelect) v += src[(size_t)t * half];
   }
-  if (j < half && dist_out) dist_out[(size_t)head * half + j] = v;
-  s_d[j] = j < half ? v : INFINITY;
+  s_d[part][j] = v;
   __syncthreads();
-  if (j == 0 && elite_idx) {
+  if (threadIdx.x < 64) {
+    v = INFINITY;
+    if (j < half && !((mask >> j) & 1ull)) {
+      v = 0.f;
+#pragma unroll
+      for (int p = 0; p < kRlSelect; ++p) v += s_d[p][j];
+    }
+    if (j < half && dist_out) dist_out[(size_t)head * half + j] = v;
+    s_d[0][j] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && elite_idx) {
     int best = 0;
     for (int c = 1; c < half; ++c)
-      if (s_d[c] < s_d[best]) best = c;
+      if (s_d[0][c] < s_d[0][best]) best = c;
     elite_idx[(size_t)head * r + round] = best;
     masks[head] = mask | (1ull << best);
   }
 }
 
 struct RlCarve {
-  size_t off_tab, off_partial, off_masks, total;
+  size_t off_cs, off_sin, off_partial, off_masks, total;
+  int span, items;              // key tiles per item, items per head
 };
 inline size_t rl_align(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Key tiles per item: whole rows cut into at most 16 items, at least 4 tiles long (the rotated
+// queries of an item are prepared anew); single tiles where that would leave most of the
+// device without work (fewer blocks than four for each of 148 SMs).
+void rl_items(int heads, int n, RlCarve* c) {
+  const int tiles = (n + kRlKeys - 1) / kRlKeys;
+  auto count = [&](int span) {
+    long long k = 0;
+    for (int m = kRlRows; m < n + kRlRows; m += kRlRows) k += (m + kRlKeys * span - 1) / (kRlKeys * span);
+    return k;
+  };
+  c->span = tiles > 64 ? (tiles + 15) / 16 : 4;
+  if (heads * count(c->span) < 4 * 148) c->span = 1;
+  c->items = (int)count(c->span);
+}
 RlCarve rl_carve(int heads, int n, int half) {
   RlCarve c;
+  rl_items(heads, n, &c);
   size_t o = 0;
-  const int n_tiles = (n + kRlRows - 1) / kRlRows;
-  c.off_tab = o;     o = rl_align(o + sizeof(float2) * (size_t)half * n);
-  c.off_partial = o; o = rl_align(o + sizeof(float) * (size_t)heads * n_tiles * half);
+  c.off_cs = o;      o = rl_align(o + sizeof(float2) * (size_t)half * n);
+  c.off_sin = o;     o = rl_align(o + sizeof(float) * (size_t)half * rl_sin_len(n));
+  c.off_partial = o; o = rl_align(o + sizeof(float) * (size_t)heads * c.items * half);
   c.off_masks = o;   o = rl_align(o + sizeof(unsigned long long) * (size_t)heads);
   c.total = o;
   return c;
@@ -181,26 +303,27 @@ int rl_check(int heads, int n, int d_h) {
   return ELITEKV_OK;
 }
 
-int rl_launch_distance(const void* Q, const void* K, int heads, int n, int d_h, const float2* tab,
-                       const unsigned long long* masks, float* partial, cudaStream_t st) {
-  dim3 grid((unsigned)((n + kRlRows - 1) / kRlRows), (unsigned)heads);
-  const int half = d_h / 2;
-  const int smem = half * (kRlSpanPad + kRlRows) * (int)sizeof(float2) + kRlWarps * half * (int)sizeof(float) +
-                   half * kRlKeys * (int)sizeof(uint32_t);
-  if (d_h == 128) {
-    EKV_CUDA_OK(cudaFuncSetAttribute(ropelite_distance_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ropelite_distance_kernel<64><<<grid, kRlThreads, smem, st>>>((const bf16*)Q, (const bf16*)K, n, tab, masks, partial);
-  } else {
-    EKV_CUDA_OK(cudaFuncSetAttribute(ropelite_distance_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ropelite_distance_kernel<32><<<grid, kRlThreads, smem, st>>>((const bf16*)Q, (const bf16*)K, n, tab, masks, partial);
-  }
+template <int HALF>
+int rl_launch_half(const void* Q, const void* K, int heads, int n, const RlCarve& c, unsigned char* base,
+                   const unsigned long long* masks, cudaStream_t st) {
+  const int smem = (int)sizeof(RlSmem<HALF>);
+  EKV_CUDA_OK(cudaFuncSetAttribute(ropelite_distance_kernel<HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  ropelite_distance_kernel<HALF><<<dim3((unsigned)c.items, (unsigned)heads), kRlThreads, smem, st>>>(
+      (const bf16*)Q, (const bf16*)K, n, (const float2*)(base + c.off_cs), (const float*)(base + c.off_sin), masks,
+      c.span, (float*)(base + c.off_partial));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }
+int rl_launch_distance(const void* Q, const void* K, int heads, int n, int d_h, const RlCarve& c, unsigned char* base,
+                       const unsigned long long* masks, cudaStream_t st) {
+  return d_h == 128 ? rl_launch_half<64>(Q, K, heads, n, c, base, masks, st)
+                    : rl_launch_half<32>(Q, K, heads, n, c, base, masks, st);
+}
 
-int rl_launch_table(float2* tab, int n, int d_h, float base, cudaStream_t st) {
-  const long long total = (long long)n * (d_h / 2);
-  ropelite_table_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(tab, n, d_h / 2, d_h, (double)base);
+int rl_launch_table(const RlCarve& c, unsigned char* base_ptr, int n, int d_h, float base, cudaStream_t st) {
+  const long long total = (long long)rl_sin_len(n) * (d_h / 2);
+  ropelite_table_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
+      (float2*)(base_ptr + c.off_cs), (float*)(base_ptr + c.off_sin), n, d_h / 2, d_h, (double)base);
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }
@@ -226,14 +349,13 @@ extern "C" int elitekv_ropelite_distances(const void* Q, const void* K, int32_t 
   const RlCarve c = rl_carve(n_heads, n, half);
   if (((uintptr_t)workspace & 255) || workspace_bytes < c.total) return ELITEKV_ERR_WORKSPACE_TOO_SMALL;
   unsigned char* base = (unsigned char*)workspace;
-  float2* tab = (float2*)(base + c.off_tab);
   float* partial = (float*)(base + c.off_partial);
   cudaStream_t st = (cudaStream_t)stream;
-  rc = rl_launch_table(tab, n, d_h, rope_base, st);
+  rc = rl_launch_table(c, base, n, d_h, rope_base, st);
   if (rc != ELITEKV_OK) return rc;
-  rc = rl_launch_distance(Q, K, n_heads, n, d_h, tab, (const unsigned long long*)elite_mask, partial, st);
+  rc = rl_launch_distance(Q, K, n_heads, n, d_h, c, base, (const unsigned long long*)elite_mask, st);
   if (rc != ELITEKV_OK) return rc;
-  ropelite_select_kernel<<<n_heads, 64, 0, st>>>(partial, (n + kRlRows - 1) / kRlRows, half,
+  ropelite_select_kernel<<<n_heads, 64 * kRlSelect, 0, st>>>(partial, c.items, half,
                                                  (unsigned long long*)elite_mask, dist, nullptr, 0, 0);
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
@@ -251,18 +373,16 @@ extern "C" int elitekv_ropelite_search(const void* Q, const void* K, int32_t n_h
   const RlCarve c = rl_carve(n_heads, n, half);
   if (((uintptr_t)workspace & 255) || workspace_bytes < c.total) return ELITEKV_ERR_WORKSPACE_TOO_SMALL;
   unsigned char* base = (unsigned char*)workspace;
-  float2* tab = (float2*)(base + c.off_tab);
   float* partial = (float*)(base + c.off_partial);
   unsigned long long* masks = (unsigned long long*)(base + c.off_masks);
   cudaStream_t st = (cudaStream_t)stream;
-  rc = rl_launch_table(tab, n, d_h, rope_base, st);
+  rc = rl_launch_table(c, base, n, d_h, rope_base, st);
   if (rc != ELITEKV_OK) return rc;
   EKV_CUDA_OK(cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)n_heads, st));
-  const int n_tiles = (n + kRlRows - 1) / kRlRows;
   for (int round = 0; round < r; ++round) {
-    rc = rl_launch_distance(Q, K, n_heads, n, d_h, tab, masks, partial, st);
+    rc = rl_launch_distance(Q, K, n_heads, n, d_h, c, base, masks, st);
     if (rc != ELITEKV_OK) return rc;
-    ropelite_select_kernel<<<n_heads, 64, 0, st>>>(partial, n_tiles, half, masks,
+    ropelite_select_kernel<<<n_heads, 64 * kRlSelect, 0, st>>>(partial, c.items, half, masks,
                                                    dist_trace ? dist_trace + (size_t)round * n_heads * half : nullptr,
                                                    elite_idx, r, round);
     EKV_CUDA_OK(cudaGetLastError());

@@ -32,3 +32,35 @@ def test_combine_items_per_sequence(ek, n_items):
     _, first, _ = ek.elitekv_plan_workers(st.lens_dev, tile, n_workers, max_items, overhead)
     assert first.tolist() == [0, n_items, n_items + 1]
     H.check_parity(st, H.run_decode(st), H.sample_units(st, 24, seed=n_items))
+
+
+# ------------------------------------------------------------------ RoPElite search
+@pytest.mark.parametrize("heads,n,d_h", [(2, 127, 64), (2, 128, 128), (2, 129, 128), (2, 257, 64), (2, 520, 128),
+                                         (300, 257, 64)])
+def test_ropelite_distances_tile_edges(ek, heads, n, d_h):
+    """Rows and keys around the 128 x 128 tile, key tiles in items of their own and (many heads) several
+    per item, no mask / some chunks / all but one chosen.  fp32 sums of up to n (n + 1) / 2 terms of
+    relative rounding 2^-24 each, added through chains of at most ~200 terms: 1e-5 is ample."""
+    from oracle import ropelite_oracle as R
+    g = torch.Generator().manual_seed(heads + n)
+    Q, K = (torch.randn((heads, n, d_h), generator=g).to(torch.bfloat16) for _ in range(2))
+    half = d_h // 2
+    full = (1 << half) - 1
+    masks = [0, 5 | (1 << (half - 1))] + [full & ~2] * (heads - 2)
+    dev = torch.from_numpy(np.array(masks, dtype=np.uint64).view(np.int64)).cuda()
+    got = ek.elitekv_ropelite_distances(Q.cuda(), K.cuda(), elite_mask=dev).cpu().double().numpy()
+    for h in (0, 1, heads - 1):
+        elite = [i for i in range(half) if (masks[h] >> i) & 1]
+        want = R.distances(Q[h].double().numpy(), K[h].double().numpy(), elite, d_h)
+        fin = np.isfinite(want)
+        assert np.array_equal(np.isinf(got[h]), ~fin)
+        assert np.allclose(got[h][fin], want[fin], rtol=1e-5, atol=1e-6)
+
+
+def test_ropelite_search_down_to_the_last_chunk(ek):
+    """All d_h / 2 rounds: every chunk is chosen once and the last free one costs nothing."""
+    g = torch.Generator().manual_seed(3)
+    Q, K = (torch.randn((2, 140, 64), generator=g).to(torch.bfloat16).cuda() for _ in range(2))
+    idx, trace = ek.elitekv_ropelite_search(Q, K, 32, trace=True)
+    assert sorted(idx[0].tolist()) == list(range(32)) and sorted(idx[1].tolist()) == list(range(32))
+    assert trace[31][torch.isfinite(trace[31])].abs().max().item() == 0.0
