@@ -176,11 +176,9 @@ int elitekv_decode(const elitekv_layer* layer, const elitekv_cache* cache, const
  * prepared at that same position (elitekv_absorb_query with q_pos = pos) into the caller's
  * q_rope / q_abs buffers, and elitekv_decode runs over seq_lens (the lengths INCLUDING the new
  * tokens).  Arguments, shapes, alignment and errors are those of the three calls; the result
- * is bit-identical to calling them in order.  The append and the work plan depend only on the
- * new tokens and the lengths, so they run on a stream the layer owns, beside the query
- * preparation on `stream`, and are joined before the attention kernel; to the caller the call
- * behaves like work enqueued on `stream` alone (it may be captured in a CUDA graph).  Two
- * threads must not run steps of the same layer object at the same time. */
+ * is bit-identical to calling them in order.  The append, the work plan and the query
+ * preparation depend only on the step's inputs, so one kernel does all three; the attention and
+ * the combine follow on `stream` (the call may be captured in a CUDA graph). */
 int elitekv_decode_step(const elitekv_layer* layer, const elitekv_cache* cache, const void* k_e,
                         const void* c, const int32_t* seq_id, const int32_t* pos, const void* q,
                         const int32_t* seq_lens, int32_t B, void* q_rope, void* q_abs,

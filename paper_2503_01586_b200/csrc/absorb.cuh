@@ -1,0 +1,181 @@
+// Query preparation (absorb.cu has the description): shared by the stand-alone kernel and by the
+// kernel that prepares a whole decode step.
+#pragma once
+
+#include "tc_ptx.cuh"
+
+constexpr int kAbsorbThreads = 256;    // 8 warps x 16 coordinates
+constexpr int kAbsorbCoords = 128;
+constexpr int kAbsorbPitch = kAbsorbCoords + 8;   // slab row pitch: 16 bytes of padding keep ldmatrix free of bank conflicts
+constexpr int kAbsorbMaxTiles = 4;     // 16-row query tiles per block
+
+struct AbsorbArgs {
+  const bf16* q;
+  const int32_t* q_pos;
+  int B;
+  const bf16* WukT;
+  const int32_t* qdims;
+  const int32_t* idx;
+  const float2* cs;
+  bf16* q_rope;
+  bf16* q_abs;
+  int n_h, d_h, r, kw, max_pos;      // kw: width of the latent the scores read
+  int32_t* status;
+};
+
+__device__ __forceinline__ void absorb_mma(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Query RoPE of one head (every sequence).
+__device__ __forceinline__ void absorb_rope(const AbsorbArgs& a, int h) {
+  const int32_t* dims = a.qdims + (size_t)h * a.d_h;
+  ekv_pdl_wait();
+  for (int e = threadIdx.x; e < a.B * a.r; e += blockDim.x) {
+    const int b = e / a.r, j = e % a.r;
+    int p = a.q_pos[b];
+    if (p < 0 || p >= a.max_pos) {
+      ekv_record(a.status, ELITEKV_ERR_BAD_POSITION, b, p);
+      p = 0;
+    }
+    const float2 w = a.cs[(size_t)p * (a.d_h / 2) + a.idx[h * a.r + j]];
+    const bf16* qq = a.q + ((size_t)b * a.n_h + h) * a.d_h;
+    const float x0 = __bfloat162float(qq[dims[2 * j]]), x1 = __bfloat162float(qq[dims[2 * j + 1]]);
+    const float y0 = __fsub_rn(__fmul_rn(x0, w.x), __fmul_rn(x1, w.y));
+    const float y1 = __fadd_rn(__fmul_rn(x0, w.y), __fmul_rn(x1, w.x));
+    bf162* dst = (bf162*)(a.q_rope + ((size_t)b * a.n_h + h) * 2 * a.r + 2 * j);
+    *dst = __floats2bfloat162_rn(y0, y1);
+  }
+}
+
+// Absorbed queries of one head, 128 latent coordinates from k0 on, sequences [b0, b0 + 16 MT).  The
+// product runs over all d_h query dims in their own order: the weight row of a dim goes to the
+// shared-memory row of that dim, and the rows of the rotated (elite) dims are zeros, so the queries
+// are used as they come.  (A non-finite elite dim makes the row's rope scores non-finite as well.)
+template <int MT>
+__device__ __forceinline__ void absorb_block(const AbsorbArgs& a, int h, int k0, int b0, unsigned char* smem_b) {
+  const int dn = a.d_h - 2 * a.r;
+  const int kpad = (a.d_h + 15) & ~15;               // K of the product, zero-padded to 16
+  const int qpitch = kpad + 8;                       // row pitch of the query tile (bank spread)
+  bf16* s_w = (bf16*)smem_b;                         // [kpad][128 + 8] weight slab
+  bf16* s_q = s_w + (size_t)kpad * kAbsorbPitch;     // [16 MT][qpitch] queries; then [16 MT][128 + 8] results
+  __shared__ __align__(8) uint64_t w_bar;
+  __shared__ int s_abort;
+  const int32_t* dims = a.qdims + (size_t)h * a.d_h;
+  const int kw = min(kAbsorbCoords, a.kw - k0);      // coordinates of this slab (a multiple of 8)
+  const int nb = min(16 * MT, a.B - b0);
+  if (threadIdx.x == 0) {
+    mbar_init(smem_u32(&w_bar), 1);
+    s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_proxy_async();
+  }
+  __syncthreads();
+  // weights and tables belong to the layer: fetched while earlier kernels of the stream still run
+  if (threadIdx.x < 32) {
+    if (dn > 0) {
+      if (threadIdx.x == 0) mbar_expect_tx(smem_u32(&w_bar), (uint32_t)(dn * kw * 2));
+      __syncwarp();
+      const bf16* src = a.WukT + (size_t)h * dn * a.kw + k0;
+      for (int i = threadIdx.x; i < dn; i += 32)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(smem_u32(s_w + (size_t)__ldg(dims + 2 * a.r + i) * kAbsorbPitch)), "l"(src + (size_t)i * a.kw),
+                       "r"(kw * 2), "r"(smem_u32(&w_bar)) : "memory");
+    }
+  } else {
+    // the elite dims' rows of the slab, and the rows past d_h (K padding)
+    const int n_zero = 2 * a.r + kpad - a.d_h;
+    for (int e = threadIdx.x - 32; e < n_zero * (kAbsorbCoords / 8); e += kAbsorbThreads - 32) {
+      const int i = e / (kAbsorbCoords / 8);
+      const int row = i < 2 * a.r ? __ldg(dims + i) : a.d_h + i - 2 * a.r;
+      *(uint4*)(s_w + (size_t)row * kAbsorbPitch + (e % (kAbsorbCoords / 8)) * 8) = make_uint4(0, 0, 0, 0);
+    }
+  }
+  ekv_pdl_wait();
+  // the queries, 16 bytes a load where rows are whole 16-byte units; padding and missing rows are zeros
+  if ((a.d_h & 7) == 0) {
+    const int v8 = kpad / 8;
+#pragma unroll MT
+    for (int e = threadIdx.x; e < 16 * MT * v8; e += kAbsorbThreads) {
+      const int bb = e / v8, v = e - bb * v8;
+      uint4 raw = make_uint4(0, 0, 0, 0);
+      if (bb < nb && v * 8 < a.d_h) raw = *((const uint4*)(a.q + ((size_t)(b0 + bb) * a.n_h + h) * a.d_h) + v);
+      *(uint4*)(s_q + bb * qpitch + v * 8) = raw;
+    }
+  } else {
+    for (int e = threadIdx.x; e < 16 * MT * kpad; e += kAbsorbThreads) {
+      const int bb = e / kpad, i = e - bb * kpad;
+      s_q[bb * qpitch + i] = bb < nb && i < a.d_h ? a.q[((size_t)(b0 + bb) * a.n_h + h) * a.d_h + i] : __float2bfloat16_rn(0.f);
+    }
+  }
+  __syncthreads();
+  if (dn > 0) {
+    // the weight slab has landed (bounded wait; a timeout is recorded and the block leaves)
+    volatile int* abort_flag = &s_abort;
+    if (!mbar_wait(smem_u32(&w_bar), 0, abort_flag, 1) && threadIdx.x == 0) ekv_record(a.status, ELITEKV_ERR_TIMEOUT, h, k0);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n0 = warp * 16;                          // first coordinate (inside the slab) of this warp
+  float acc[MT][2][4] = {};
+  if (n0 < kw) {
+    for (int kk = 0; kk < kpad; kk += 16) {
+      uint32_t w[4];
+      ldmatrix_x4_trans(w, s_w + (size_t)(kk + (lane & 15)) * kAbsorbPitch + n0 + (lane >> 4) * 8);
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        uint32_t x[4];
+        ldmatrix_x4(x, s_q + (16 * mt + (lane & 15)) * qpitch + kk + (lane >> 4) * 8);
+        absorb_mma(acc[mt][0], x, w[0], w[1]);
+        absorb_mma(acc[mt][1], x, w[2], w[3]);
+      }
+    }
+  }
+  if (__syncthreads_or(s_abort != 0)) {
+    drain_after_abort();
+    return;
+  }
+  // through shared memory, so that whole rows of 256 bytes are written
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      bf16* dst = s_q + (16 * mt + g) * kAbsorbPitch + n0 + nt * 8 + 2 * t;
+      *(bf162*)dst = __floats2bfloat162_rn(acc[mt][nt][0], acc[mt][nt][1]);
+      *(bf162*)(dst + 8 * kAbsorbPitch) = __floats2bfloat162_rn(acc[mt][nt][2], acc[mt][nt][3]);
+    }
+  __syncthreads();
+#pragma unroll MT
+  for (int e = threadIdx.x; e < 16 * MT * (kAbsorbCoords / 8); e += kAbsorbThreads) {
+    const int bb = e / (kAbsorbCoords / 8), v = e % (kAbsorbCoords / 8);
+    if (bb < nb && v * 8 < kw)
+      *(uint4*)(a.q_abs + ((size_t)(b0 + bb) * a.n_h + h) * a.kw + k0 + v * 8) = *(const uint4*)(s_q + bb * kAbsorbPitch + v * 8);
+  }
+}
+
+// 16-row tiles per block (1, 2 or 4), blocks along the latent and along the sequences, shared memory
+struct AbsorbShape {
+  int mt, slices, groups;
+  size_t smem;
+};
+inline AbsorbShape absorb_shape(const elitekv_layer* L, int B) {
+  AbsorbShape s;
+  s.mt = B <= 16 ? 1 : B <= 32 ? 2 : kAbsorbMaxTiles;
+  s.slices = (L->kw + kAbsorbCoords - 1) / kAbsorbCoords;
+  s.groups = (B + 16 * s.mt - 1) / (16 * s.mt);
+  const size_t kpad = (size_t)((L->d_h + 15) & ~15);
+  const size_t pitch = kpad + 8 > (size_t)kAbsorbPitch ? kpad + 8 : kAbsorbPitch;
+  s.smem = sizeof(bf16) * (kpad * kAbsorbPitch + 16 * s.mt * pitch) + 16;
+  return s;
+}
+inline bool absorb_ok(const elitekv_layer* L, const AbsorbShape& s) {
+  return (int)s.smem <= L->smem_optin && L->kw % 8 == 0;
+}
+inline AbsorbArgs absorb_args(const elitekv_layer* L, const void* q, const int32_t* q_pos, int B, void* q_rope, void* q_abs) {
+  return AbsorbArgs{(const bf16*)q, q_pos, B, L->d_WukT, L->d_qdims, L->d_idx, L->d_cs, (bf16*)q_rope, (bf16*)q_abs,
+                    L->n_h, L->d_h, L->r, L->kw, L->max_pos, L->d_status};
+}

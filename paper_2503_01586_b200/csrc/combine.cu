@@ -48,17 +48,6 @@ constexpr int kFThreads = 256;
 constexpr int kFPitch = kFD + 8; // shared-memory row pitch in bf16: 16 bytes of padding keep ldmatrix free of bank conflicts
 constexpr int kFAhead = 4;       // partial results per row in flight beside the statistics
 
-__device__ __forceinline__ void ldmatrix_x4(uint32_t* r, const bf16* p) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
-}
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, const bf16* p) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
-}
-
 __global__ void __launch_bounds__(kFThreads, 4)
 combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by the split-K kernel while this
                                                                    // kernel may already be resident: read

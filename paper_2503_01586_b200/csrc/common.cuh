@@ -39,8 +39,6 @@ struct elitekv_layer {
   int32_t* last_detail;            // host [3]: detail words + count read by the last check_status
   int d;                           // model width (0: no projection weights)
   bf16* d_WcatT;                   // [n_h*2r + d_c][d]: [W^k_e | A^kv] transposed (rows = output columns)
-  cudaStream_t side;               // second stream of elitekv_decode_step (append + plan beside the absorb)
-  cudaEvent_t ev_fork, ev_join;    // its fork from / join into the caller's stream
 };
 
 constexpr int kProfileSlots = 512;
@@ -85,6 +83,17 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
+}
+
+__device__ __forceinline__ void ldmatrix_x4(uint32_t* r, const bf16* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, const bf16* p) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
 }
 
 // Programmatic dependent launch: the kernels of one decode step are launched with the
@@ -152,16 +161,12 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
                               cudaStream_t st);
 int ekv_launch_absorb(const elitekv_layer* L, const void* q, const int32_t* q_pos, int B,
                       void* q_rope, void* q_abs, cudaStream_t st);
-// max_len: tokens one sequence can hold in the cache; longer (or negative) lengths are recorded
-// in `status` (may be null) as BAD_POSITION and clamped.
-int ekv_launch_plan(const int32_t* seq_lens, int B, int tile_tokens, int max_items, int32_t* items,
-                    int32_t* seq_first_item, int32_t* zero_ints, int n_zero, long long max_len,
-                    int32_t* status, cudaStream_t st);
-
-int ekv_launch_plan_balanced(const int32_t* seq_lens, int B, int tile_tokens, int n_workers,
-                             int max_items, int32_t* items, int32_t* seq_first_item,
-                             int32_t* worker_first, int32_t* zero_ints, int n_zero, long long max_len,
-                             int32_t* status, int overhead_tiles, cudaStream_t st);
+struct PlanArgs;      // plan.cuh
+int ekv_launch_plan(const PlanArgs& a, cudaStream_t st);
+// append + plan + query preparation of a decode step in one launch
+int ekv_launch_step_prep(const elitekv_layer* L, const elitekv_cache* cache, const CacheView& cv, const void* k_e,
+                         const void* c, const int32_t* seq_id, const int32_t* pos, const void* q, int B, void* q_rope,
+                         void* q_abs, const PlanArgs& plan, cudaStream_t st);
 
 struct DecodeScratch {
   int max_items;          // capacity of the plan

@@ -64,3 +64,53 @@ def test_ropelite_search_down_to_the_last_chunk(ek):
     idx, trace = ek.elitekv_ropelite_search(Q, K, 32, trace=True)
     assert sorted(idx[0].tolist()) == list(range(32)) and sorted(idx[1].tolist()) == list(range(32))
     assert trace[31][torch.isfinite(trace[31])].abs().max().item() == 0.0
+
+
+# ------------------------------------------------------------------ query preparation and the step's front end
+@pytest.mark.parametrize("B", [1, 16, 17, 32, 33, 64, 65])
+@pytest.mark.parametrize("shape", [dict(), dict(n_h=3, d_h=44, r=5, d_c=136, d=128), dict(n_h=4, d_h=64, r=32, d_c=128, d=256)],
+                         ids=["7b", "odd", "all-elite"])
+def test_absorb_row_tiles(ek, B, shape):
+    """1, 2 and 4 row tiles per block, several groups; a head dim that is no multiple of 8 and a latent
+    that ends inside a 128-wide slab; no un-rotated dim at all."""
+    w = replace(gen.LLAMA7B_75, B=B, seed=900 + B, **shape)
+    idx = gen.elite_index_sets(w)
+    W_uk, W_uv = gen.up_projections(w, "cuda")
+    layer = ek.Layer(w.n_h, w.d_h, w.r, w.d_c, idx, W_uk, W_uv, 300)
+    q = gen.queries(w, "cuda")
+    q_pos = (torch.arange(B, dtype=torch.int32) * 37 % 300).cuda()
+    q_rope, q_abs = ek.elitekv_absorb_query(layer, q, q_pos)
+    assert ek.elitekv_check_status(layer) == 0
+    for b in {0, B // 2, B - 1}:
+        want_rope, want_abs = O.absorb_query(H.f64(q[b]), int(q_pos[b]), idx.numpy().astype(np.int64), H.f64(W_uk), w.d_h, w.rope_base)
+        # bf16 results of exact products with fp32 sums: half a unit of 2^-8 relative to the row's largest entry
+        assert np.max(np.abs(H.f64(q_rope[b]) - want_rope)) <= 2.0 ** -8 * np.max(np.abs(want_rope))
+        assert np.max(np.abs(H.f64(q_abs[b]) - want_abs)) <= 2.0 ** -8 * np.max(np.abs(want_abs)) + 1e-30
+
+
+@pytest.mark.parametrize("B", [1, 33, 200])
+def test_step_front_end_equals_the_three_calls(ek, B):
+    """One launch for append, plan and query preparation: more tokens than append blocks (200), and
+    batches of one and of several row tiles, bit for bit as the separate calls."""
+    w = gen.shrink(gen.SWEEP_875, B=B, ctx=70)
+    lens = [1 + 17 * b % 70 for b in range(B)]
+    out = []
+    for single in (False, True):
+        st = H.setup(w, lens=lens, fill=False)
+        st.rope_plane.normal_(generator=torch.Generator(device="cuda").manual_seed(1))
+        st.latent_plane.normal_(generator=torch.Generator(device="cuda").manual_seed(2))
+        last = torch.from_numpy(st.starts[1:] - 1).cuda()
+        k_e, c, seq, pos = (x[last].contiguous() for x in (st.k_e, st.c, st.seq_id, st.pos))
+        q_rope = torch.zeros((B, w.n_h, 2 * w.r), dtype=torch.bfloat16, device="cuda")
+        q_abs = torch.zeros((B, w.n_h, w.d_c), dtype=torch.bfloat16, device="cuda")
+        o = torch.zeros((B, w.n_h, w.d_h), dtype=torch.bfloat16, device="cuda")
+        if single:
+            ek.elitekv_decode_step(st.layer, st.cache, k_e, c, seq, pos, st.q, st.lens_dev, q_rope, q_abs, st.workspace, o)
+        else:
+            ek.elitekv_append(st.layer, st.cache, k_e, c, seq, pos)
+            ek.elitekv_absorb_query(st.layer, st.q, pos, q_rope, q_abs)
+            ek.elitekv_decode(st.layer, st.cache, q_rope, q_abs, st.lens_dev, st.workspace, o)
+        assert ek.elitekv_check_status(st.layer) == 0
+        out.append((st.rope_plane, st.latent_plane, q_rope, q_abs, o))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
