@@ -77,8 +77,10 @@ typedef struct {
   int32_t decode_kernel;      /* 0 = choose by shape; 1 = generic CUDA-core kernel; 2 = tcgen05
                                  kernel that streams each 128-token tile twice (scores, then
                                  values); 3 = tcgen05 kernel that keeps a 64-token tile
-                                 resident in shared memory between the two products.  2 and 3
-                                 fail with UNSUPPORTED_SHAPE when the shape is not covered.    */
+                                 resident in shared memory between the two products (block
+                                 pairs); 4 = the same on clusters of 2, 4, 5 or 8 blocks.  2, 3
+                                 and 4 fail with UNSUPPORTED_SHAPE when the shape is not
+                                 covered.                                                      */
   /* Only for elitekv_project_append (all three 0 / NULL otherwise): the projections that make
    * the cache row of a token from its hidden state x (Section 3.2, Eq. 2). */
   int32_t d;                  /* model width                                                   */
@@ -273,7 +275,7 @@ int elitekv_plan_workers(const int32_t* seq_lens, int32_t B, int32_t tile_tokens
 
 /* Which split-K kernel and plan elitekv_decode uses for this layer, cache layout (may be NULL:
  * shape-only answer) and batch (the paper has no counterpart).  info is a HOST array:
- * info[0] = kernel (1, 2, 3 as in elitekv_params.decode_kernel), info[1] = tokens per plan tile,
+ * info[0] = kernel (1 to 4 as in elitekv_params.decode_kernel), info[1] = tokens per plan tile,
  * info[2] = persistent workers (0: the plain plan of elitekv_plan), info[3] = plan capacity,
  * info[4] = item_overhead_tiles of elitekv_plan_workers. */
 int elitekv_decode_plan_info(const elitekv_layer* layer, const elitekv_cache* cache, int32_t B,

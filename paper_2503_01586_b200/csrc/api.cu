@@ -7,21 +7,26 @@ namespace {
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Which split-K kernel serves a layer (and cache): 1 = generic CUDA-core kernel, 2 = two-pass
-// tcgen05 kernel, 3 = resident-tile tcgen05 kernel on block pairs, -1 = none.  `cache` may be
+// tcgen05 kernel, 3 = resident-tile tcgen05 kernel on block pairs, 4 = tcgen05 kernel on larger
+// clusters, -1 = none.  `cache` may be
 // null (shape-only question).
 int select_kernel(const elitekv_layer* L, const elitekv_cache* cache) {
   const bool tc = ekv_tc_supported(L, cache) != 0;
   const bool rt = ekv_rt_supported(L, cache) != 0;
+  const bool cl = L->cl_clusters > 0 && ekv_cl_supported(L, cache) != 0;
+  if (L->decode_kernel == 4) return cl ? 4 : -1;
   if (L->decode_kernel == 3) return rt ? 3 : -1;
   if (L->decode_kernel == 2) return tc ? 2 : -1;
   if (L->decode_kernel == 1) return ekv_generic_supported(L) ? 1 : -1;
-  // Choice by shape when both tensor-core kernels cover the layer (measured on B200): the
-  // resident-tile kernel has the lower fixed cost and wins on batches of up to a few hundred
-  // thousand cached tokens at d_c = 1536 (80 us against 90 us at 16 x 4096); its per-tile chain
-  // (exchange between the two blocks of a pair, softmax, value product) makes it the slower one
-  // on long streams (0.73 against 0.82 of the copy bandwidth on the 4.6 GB ragged batch) and
-  // at narrow latents (d_c = 768).  Lengths live on the device, so the capacity of the cache
-  // stands in for them.
+  // Choice by shape (measured on B200, whole decode steps in sustained loops, where the power cap sets
+  // the pace of the long ones).  The cluster kernel where it covers the layer: 7B 75 % 16 x 4096 82 us
+  // against 91 with the resident-tile kernel, ragged 64 x [1024, 32768] 981 against 1006 with the
+  // two-pass one, 13B 32 x 16384 652 / 863, 50 % 32 x 8192 531 / 613, 87.5 % 140 / 161, S-LRD 207 / 209.
+  if (cl) return 4;
+  // Elsewhere, of the other two tensor-core kernels, the resident-tile one has the lower fixed cost
+  // and wins on batches of up to a few hundred thousand cached tokens at d_c = 1536; its per-tile
+  // chain makes it the slower one on long streams and at narrow latents (d_c = 768).  Lengths live
+  // on the device, so the capacity of the cache stands in for them.
   if (rt && tc) {
     long long capacity = 0;
     if (cache) capacity = cache->page_table ? (long long)cache->num_pages * cache->page_size
@@ -35,6 +40,7 @@ int select_kernel(const elitekv_layer* L, const elitekv_cache* cache) {
 }
 
 int max_items_for(const elitekv_layer* L, int B, int kernel, int rows = 1) {
+  if (kernel == 4) return ekv_cl_max_items(L, B);
   if (kernel == 3) return ekv_rt_max_items(L, B);
   return kernel == 2 ? ekv_tc_max_items(L, B, rows) : ekv_generic_max_items(L, B);
 }
@@ -43,9 +49,9 @@ int max_items_for(const elitekv_layer* L, int B, int kernel, int rows = 1) {
 int plan_tile_for(int kernel) { return kernel == 2 ? 128 : ELITEKV_TILE_TOKENS; }
 // Tiles' worth of time that starting an item costs a worker (measured on B200: about one
 // 64-token tile for the resident-tile kernel).
-int item_overhead_for(int kernel) { return kernel == 3 ? 1 : 0; }
+int item_overhead_for(int kernel) { return kernel == 4 ? 2 : kernel == 3 ? 1 : 0; }
 int workers_for(const elitekv_layer* L, int kernel, int rows = 1) {
-  return kernel == 3 ? ekv_rt_workers(L) : kernel == 2 ? ekv_tc_workers(L, rows) : 0;
+  return kernel == 4 ? ekv_cl_workers(L) : kernel == 3 ? ekv_rt_workers(L) : kernel == 2 ? ekv_tc_workers(L, rows) : 0;
 }
 
 // The workspace is sized for whichever kernel may be picked once the cache layout is known.
@@ -59,6 +65,10 @@ int max_items_any(const elitekv_layer* L, int B) {
   }
   if (ekv_rt_supported(L, nullptr) && (want == 0 || want == 3)) {
     const int t = ekv_rt_max_items(L, B);
+    if (t > m) m = t;
+  }
+  if (L->cl_clusters > 0 && (want == 0 || want == 4)) {
+    const int t = ekv_cl_max_items(L, B);
     if (t > m) m = t;
   }
   return m;
@@ -190,7 +200,8 @@ int decode_impl(const elitekv_layer* L, const elitekv_cache* cache, const void* 
   if (rc != ELITEKV_OK) return rc;
   EkvProfile* prof = (L->prof && L->prof->enabled && L->prof->count < kProfileSlots) ? L->prof : nullptr;
   if (prof) EKV_CUDA_OK(cudaEventRecord(prof->ev[2 * prof->count], st));
-  rc = kernel == 3   ? ekv_launch_decode_rt(L, cache, cv, q_rope, q_abs, B, ws, st)
+  rc = kernel == 4   ? ekv_launch_decode_cl(L, cache, cv, q_rope, q_abs, B, ws, st)
+       : kernel == 3 ? ekv_launch_decode_rt(L, cache, cv, q_rope, q_abs, B, ws, st)
        : kernel == 2 ? ekv_launch_decode_tc(L, cache, cv, q_rope, q_abs, B, ws, st)
                      : ekv_launch_decode_generic(L, cache, cv, q_rope, q_abs, B, ws, st);
   if (rc != ELITEKV_OK) return rc;

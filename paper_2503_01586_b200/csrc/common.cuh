@@ -26,6 +26,7 @@ struct elitekv_layer {
   int decode_kernel;
   int device;
   int sm_count;
+  int cl_clusters;                 // clusters of the cluster-resident kernel that fit the device at once (0: shape not covered)
   int smem_optin;                  // max dynamic shared memory per block
   int32_t* d_idx;                  // [n_h][r] elite chunk ids
   int32_t* d_qdims;                // [n_h][d_h]: 2r dims of the elite chunks in cache order,
@@ -203,6 +204,13 @@ int ekv_rt_supported(const elitekv_layer* L, const elitekv_cache* cache);   // c
 int ekv_rt_workers(const elitekv_layer* L);
 int ekv_rt_max_items(const elitekv_layer* L, int B);
 int ekv_launch_decode_rt(const elitekv_layer* L, const elitekv_cache* cache, const CacheView& cv,
+                         const void* q_rope, const void* q_abs, int B, const DecodeScratch& ws,
+                         cudaStream_t st);
+int ekv_cl_supported(const elitekv_layer* L, const elitekv_cache* cache);   // cache may be null
+int ekv_cl_max_clusters(const elitekv_layer* L);              // device query, at layer creation
+int ekv_cl_workers(const elitekv_layer* L);
+int ekv_cl_max_items(const elitekv_layer* L, int B);
+int ekv_launch_decode_cl(const elitekv_layer* L, const elitekv_cache* cache, const CacheView& cv,
                          const void* q_rope, const void* q_abs, int B, const DecodeScratch& ws,
                          cudaStream_t st);
 int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, void* out,

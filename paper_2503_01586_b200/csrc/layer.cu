@@ -38,7 +38,7 @@ extern "C" int elitekv_layer_create(const elitekv_params* p, elitekv_layer** out
   if (!p->W_uv || (p->d_h - 2 * p->r > 0 && !p->W_uk)) return ELITEKV_ERR_INVALID_ARG;
   if (p->max_pos <= 0 || !(p->rope_base > 0.f)) return ELITEKV_ERR_INVALID_ARG;
   if (p->pair_mode != 0 && p->pair_mode != 1) return ELITEKV_ERR_INVALID_ARG;
-  if (p->decode_kernel < 0 || p->decode_kernel > 3) return ELITEKV_ERR_INVALID_ARG;
+  if (p->decode_kernel < 0 || p->decode_kernel > 4) return ELITEKV_ERR_INVALID_ARG;
   if (p->d_c % 8 != 0 || p->d_h > 512) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
   if (p->d_ck < 0 || p->d_ck >= p->d_c) return ELITEKV_ERR_INVALID_ARG;
   if (p->d_ck % 8 != 0) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
@@ -132,6 +132,7 @@ extern "C" int elitekv_layer_create(const elitekv_params* p, elitekv_layer** out
       regroup_wuk_kernel<<<grid2, block>>>((const bf16*)p->W_down, L->d_WcatT + (size_t)rope_w * p->d, p->d, p->d_c);
       if (cudaGetLastError() != cudaSuccess) break;
     }
+    L->cl_clusters = ekv_cl_supported(L, nullptr) ? ekv_cl_max_clusters(L) : 0;
     if (cudaDeviceSynchronize() != cudaSuccess) break;
     rc = ELITEKV_OK;
   } while (0);

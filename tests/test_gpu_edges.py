@@ -114,3 +114,66 @@ def test_step_front_end_equals_the_three_calls(ek, B):
         out.append((st.rope_plane, st.latent_plane, q_rope, q_abs, o))
     for a, b in zip(*out):
         assert torch.equal(a, b)
+
+
+# ------------------------------------------------------------------ cluster kernel (decode_kernel = 4)
+CLUSTER_SHAPES = {"c2": gen.SWEEP_875, "c4": gen.LLAMA7B_75, "c5": gen.LLAMA13B_75, "c8": gen.SWEEP_50,
+                  "c4-slrd": gen.SWEEP_75_SLRD}
+
+
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("shape", CLUSTER_SHAPES)
+def test_cluster_kernel_tile_edges(ek, shape, paged):
+    """One tile (one stream only), two and three tiles, the 16-token steps of a ragged last tile, an
+    empty sequence, and every cluster size."""
+    lens = [64, 1, 15, 17, 63, 65, 128, 129, 200, 0, 413]
+    w = gen.shrink(CLUSTER_SHAPES[shape], B=len(lens), ctx=413)
+    if paged:
+        w = replace(w, paged=True, page_size=64)
+    st = H.setup(w, lens=lens, decode_kernel=4)
+    assert ek.elitekv_decode_plan_info(st.layer, st.cache, len(lens))[0] == 4
+    out = H.run_decode(st)
+    assert not out[9].any()
+    H.check_parity(st, out, [u for u in H.sample_units(st, 120, seed=4) if u[0] != 9] + [(0, 0), (1, w.n_h - 1), (10, w.n_h // 2)])
+
+
+@pytest.mark.parametrize("shape", ["c4", "c5"])
+def test_cluster_kernel_many_items_per_worker(ek, shape):
+    """Workers walk many short items: queries replaced, accumulators merged and reused, statistics
+    slots coming round; and one sequence cut over all workers."""
+    w = gen.shrink(CLUSTER_SHAPES[shape], B=301, ctx=300)
+    lens = [1 + (37 * i) % 300 for i in range(301)]
+    st = H.setup(w, lens=lens, decode_kernel=4)
+    H.check_parity(st, H.run_decode(st), H.sample_units(st, 64))
+    st = H.setup(gen.shrink(CLUSTER_SHAPES[shape], B=1, ctx=15000), lens=[15000], decode_kernel=4)
+    H.check_parity(st, H.run_decode(st), H.sample_units(st, 3))
+
+
+@pytest.mark.parametrize("page_size", [64, 256])
+def test_cluster_kernel_pages_and_bad_page(ek, page_size):
+    """Several tiles per page, more than 32 tiles (rows are looked up 32 at a time), and a page id outside
+    the pool: recorded, and the other sequences' results untouched."""
+    w = replace(gen.shrink(gen.LLAMA7B_75, B=3, ctx=9000), paged=True, page_size=page_size)
+    st = H.setup(w, lens=[9000, 2500, 64], decode_kernel=4)
+    good = H.run_decode(st).clone()
+    H.check_parity(st, good, H.sample_units(st, 8))
+    st.page_table[1, 2] = st.cache.num_pages + 5
+    q_rope, q_abs = ek.elitekv_absorb_query(st.layer, st.q, st.q_pos)
+    out = ek.elitekv_decode(st.layer, st.cache, q_rope, q_abs, st.lens_dev, st.workspace)
+    assert ek.elitekv_check_status(st.layer) == ek.ERR_BAD_PAGE
+    assert ek.elitekv_last_status_detail(st.layer)[:2] == (1, st.cache.num_pages + 5)
+    assert torch.equal(out[0], good[0]) and torch.equal(out[2], good[2])
+
+
+@pytest.mark.parametrize("mode", ["scaled", "planted"])
+def test_cluster_kernel_peaked(ek, mode):
+    """The reference maximum moves inside items, in one stream and not in the other."""
+    from .test_gpu_peaked import _run
+    assert _run(ek, "7b", mode, 4) == 4
+
+
+def test_cluster_kernel_refuses_uncovered_shapes(ek):
+    w = replace(gen.LLAMA7B_75, B=2, ctx=64, n_h=24)          # 384 rope dims: clusters of three are not built
+    with pytest.raises(ek.ElitekvError) as e:
+        H.setup(w, lens=[5, 5], decode_kernel=4)
+    assert e.value.code == ek.ERR_UNSUPPORTED_SHAPE
