@@ -45,8 +45,11 @@ int max_items_for(const elitekv_layer* L, int B, int kernel, int rows = 1) {
   return kernel == 2 ? ekv_tc_max_items(L, B, rows) : ekv_generic_max_items(L, B);
 }
 
-// Tokens per plan tile and persistent workers (0: the plain plan) of each kernel.
-int plan_tile_for(int kernel) { return kernel == 2 ? 128 : ELITEKV_TILE_TOKENS; }
+// Tokens per plan tile and persistent workers (0: the plain plan) of each kernel.  The generic kernel
+// takes any cut: a short context is spread over the device in pieces of 16 tokens (four of its
+// 4-token batches; one sequence of 256 tokens, 4 heads: 20 us in pieces of 64, 7.3 us in pieces of 16),
+// a long one comes out in larger pieces anyway because the plan's capacity bounds their number.
+int plan_tile_for(int kernel) { return kernel == 2 ? 128 : kernel == 1 ? 16 : 64; }
 // Tiles' worth of time that starting an item costs a worker (measured on B200: about one
 // 64-token tile for the resident-tile kernel).
 int item_overhead_for(int kernel) { return kernel == 4 ? 2 : kernel == 3 ? 1 : 0; }

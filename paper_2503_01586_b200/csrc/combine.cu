@@ -212,8 +212,8 @@ constexpr int kCombThreads = 256;
 constexpr int kCombChunk = 128;
 
 __global__ void __launch_bounds__(kCombThreads)
-combine_upproj_kernel(const float* __restrict__ part_acc, const float* __restrict__ part_ml,
-                      const int32_t* __restrict__ seq_first, const bf16* __restrict__ Wuv,
+combine_upproj_kernel(const float* part_acc, const float* part_ml,      // (as above: never ld.global.nc)
+                      const int32_t* seq_first, const bf16* __restrict__ Wuv,
                       bf16* __restrict__ out, int B, int n_h /* query rows x heads */, int n_phys /* heads */,
                       int d_h, int d_c) {
   __shared__ float s_olat[kCombBatch][kCombChunk];
@@ -229,6 +229,8 @@ combine_upproj_kernel(const float* __restrict__ part_acc, const float* __restric
   const int kg = threadIdx.x / npair;
   const bool worker = kg < kgroups;
 
+  ekv_pdl_wait();
+  ekv_pdl_trigger();
   if (threadIdx.x <= nb) s_first[threadIdx.x] = seq_first[b0 + threadIdx.x];
   __syncthreads();
   {
@@ -263,6 +265,7 @@ combine_upproj_kernel(const float* __restrict__ part_acc, const float* __restric
       float v = 0.f;
       if (bb < nb && k < kc) {
         const float M = s_M[bb];
+#pragma unroll 4
         for (int i = s_first[bb]; i < s_first[bb + 1]; ++i) {
           const float w = exp2f(part_ml[((size_t)i * n_h + h) * 2] - M);
           v = fmaf(w, part_acc[((size_t)i * n_h + h) * d_c + k0 + k], v);
@@ -337,9 +340,9 @@ int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, v
   dim3 grid(nv, (B + kCombBatch - 1) / kCombBatch);
   EKV_CUDA_OK(cudaFuncSetAttribute(combine_upproj_kernel,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  combine_upproj_kernel<<<grid, kCombThreads, smem, st>>>(ws.part_acc, ws.part_ml, ws.seq_first,
-                                                          L->d_Wuv, (bf16*)out, B, nv, L->n_h, L->d_h,
-                                                          L->vw);
+  EKV_CUDA_OK(ekv_launch_pdl(combine_upproj_kernel, grid, dim3(kCombThreads), smem, st, (const float*)ws.part_acc,
+                             (const float*)ws.part_ml, (const int32_t*)ws.seq_first, (const bf16*)L->d_Wuv, (bf16*)out, B,
+                             nv, L->n_h, L->d_h, L->vw));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }

@@ -11,10 +11,6 @@
 typedef __nv_bfloat16 bf16;
 typedef __nv_bfloat162 bf162;
 
-// The work plan cuts sequences in units of this many tokens (also the page size the
-// tensor-core kernel expects).
-#define ELITEKV_TILE_TOKENS 64
-
 struct elitekv_layer {
   int n_h, d_h, r, d_c, dn;        // dn = d_h - 2r (un-rotated key dims per head); d_c = width of a latent row
   int kw, voff, vw;                // latent columns the scores read: [0, kw); the outputs: [voff, voff + vw).

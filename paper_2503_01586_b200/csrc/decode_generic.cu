@@ -39,6 +39,8 @@ template <int NCH>
 __global__ void __launch_bounds__(kThreads)
 decode_generic_kernel(const GenericArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  ekv_pdl_wait();         // the plan, the queries and the cache come from kernels earlier in the stream
+  ekv_pdl_trigger();
   const int item = blockIdx.x;
   const int seq = a.items[4 * item + 0];
   if (seq < 0) return;
@@ -102,7 +104,7 @@ decode_generic_kernel(const GenericArgs a) {
     __syncthreads();
     bf16* dl = s_lat + (size_t)buf * T * d_c;
     bf16* dr = s_rope + (size_t)buf * T * rope_w_pad;
-    for (int e = threadIdx.x; e < T * lat_vecs; e += kThreads) {
+    for (int e = threadIdx.x; e < nt * lat_vecs; e += kThreads) {
       const int tt = e / lat_vecs, v = e - tt * lat_vecs;
       const long long row = s_rows[buf][tt];
       bf16* dst = dl + (size_t)tt * d_c + v * 8;
@@ -111,7 +113,7 @@ decode_generic_kernel(const GenericArgs a) {
     }
     if (rope_vec) {
       const int rv = rope_w >> 3;
-      for (int e = threadIdx.x; e < T * rv; e += kThreads) {
+      for (int e = threadIdx.x; e < nt * rv; e += kThreads) {
         const int tt = e / rv, v = e - tt * rv;
         const long long row = s_rows[buf][tt];
         bf16* dst = dr + (size_t)tt * rope_w_pad + v * 8;
@@ -119,7 +121,7 @@ decode_generic_kernel(const GenericArgs a) {
         else *(uint4*)dst = make_uint4(0, 0, 0, 0);
       }
     } else {
-      for (int e = threadIdx.x; e < T * rope_w; e += kThreads) {
+      for (int e = threadIdx.x; e < nt * rope_w; e += kThreads) {
         const int tt = e / rope_w, v = e - tt * rope_w;
         const long long row = s_rows[buf][tt];
         dr[(size_t)tt * rope_w_pad + v] =
@@ -147,7 +149,7 @@ decode_generic_kernel(const GenericArgs a) {
         float s[kTokBatch];
 #pragma unroll
         for (int u = 0; u < kTokBatch; ++u) {
-          const int tt = tt0 + u;          // rows >= nt were zero-filled or are stale but finite? -> masked below
+          const int tt = tt0 + u;          // rows past nt are neither loaded nor read
           float sum = 0.f;
           if (tt < nt) {
 #pragma unroll
@@ -247,7 +249,7 @@ template <int NCH>
 int launch_nch(const elitekv_layer* L, const GenericArgs& a, dim3 grid, size_t smem, cudaStream_t st) {
   EKV_CUDA_OK(cudaFuncSetAttribute(decode_generic_kernel<NCH>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  decode_generic_kernel<NCH><<<grid, kThreads, smem, st>>>(a);
+  EKV_CUDA_OK(ekv_launch_pdl(decode_generic_kernel<NCH>, grid, dim3(kThreads), smem, st, a));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }

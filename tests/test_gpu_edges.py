@@ -177,3 +177,13 @@ def test_cluster_kernel_refuses_uncovered_shapes(ek):
     with pytest.raises(ek.ElitekvError) as e:
         H.setup(w, lens=[5, 5], decode_kernel=4)
     assert e.value.code == ek.ERR_UNSUPPORTED_SHAPE
+
+
+@pytest.mark.parametrize("lens", [[16], [17], [1000], [15, 16, 9000]])
+def test_generic_kernel_item_edges(ek, lens):
+    """Items of 16 tokens, a ragged last one, more items than a warp has lanes in the combine, and
+    contexts long enough for larger pieces."""
+    w = gen.shrink(gen.TINY, B=len(lens), ctx=max(lens))
+    st = H.setup(w, lens=lens)
+    assert ek.elitekv_decode_plan_info(st.layer, st.cache, len(lens))[:2] == (1, 16)
+    H.check_parity(st, H.run_decode(st), H.all_units(st))
