@@ -9,11 +9,11 @@
 // (cos, sin) of pos * theta_{idx[h][j]}, everything is rounded once to bf16 and written straight
 // to the token's cache row (contiguous or paged).  k_e and c never touch memory.
 //
-// One block computes a [128 tokens x 128 output columns] tile (prefill-sized calls: 256 x 256,
-// see further down): warp 0 streams the operand tiles
+// One block computes a [128 tokens x 128 output columns] tile (prefill-sized calls: 256 or 512
+// x 256 per block pair, see further down): warp 0 streams the operand tiles
 // ([128 x 64] of x and of the transposed weight, 128-byte swizzle) through a 4-stage ring, warp 1
 // issues tcgen05.mma (M = 128, N = 128, K = 16, bf16 in, fp32 in TMEM), warps 2-5 run the epilogue.
-// A tile lies either in the rope part or in the latent part (both are multiples of 128 wide).
+// A 128-wide tile lies either in the rope part or in the latent part (both are multiples of 128 wide).
 //
 // A batch of at most 128 tokens (a decode step) has one token tile, so the grid above would be
 // n_out / 128 blocks reading the 2 d n_out bytes of weights between them: 16 blocks for the 7B
@@ -241,38 +241,59 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
 }
 
-// ------------------------------------------------------------------ prefill form: 256 x 256 tiles
+// ------------------------------------------------------------------ prefill form: block pairs
 // A 128 x 128 tile asks L2 for 32 KB of operands per 256 tensor-core clocks; at prefill size all
 // SMs together ask for more than L2 delivers, and the tensor pipe idles more than half of the
-// time.  A block of the prefill form computes 256 tokens x 256 columns: the two halves of the
-// token rows are two accumulators (TMEM columns 0-255 and 256-511) that share every weight tile,
-// so a stage of 64 KB (256 rows of x and 256 rows of the weights, 64 of d each) feeds eight
-// M128 N256 K16 MMAs = 1024 clocks: half the operand bytes per flop.
-constexpr int kBM = 256, kBN = 256;
-constexpr int kBStages = 3;
-constexpr int kBStageBytes = (kBM + kBN) * kPK * 2;   // 64 KB
-constexpr int kBThreads = 224;    // warp 0 loads x, warp 6 the weights (one issuing warp draws ~50 GB/s, two
-                                  // about twice that), warp 1 issues the MMAs, warps 2-5 run the epilogue
+// time.  Here a cluster of two blocks computes 256 H tokens x 256 columns with paired instructions
+// (cta_group::2: M = 256 over both blocks, N = 256): a block keeps 128 H rows of x and HALF of the 256
+// weight rows per 64 of depth, the other half of the weights is read out of its peer's shared memory
+// by the tensor core.  H = 2: two accumulators (TMEM columns 0-255 and 256-511), 48 KB per 1024 clocks
+// and block, which L2 can deliver to the whole chip.  H = 1: 32 KB per 512 clocks, for calls whose
+// tiles of 512 tokens would leave half of the chip idle.
+// The ring holds 14 units of 128 rows (weights and 128 tokens each in turn), not whole stages: a unit
+// is refilled as soon as its own product has read it, and a load takes about 3000 clocks under this
+// traffic, three stages' time.  Every block loads its own units, but onto the first block's barriers:
+// its MMA warp issues for both.
+// The epilogue of a rope tile reads the tokens' whole (cos, sin) rows into idle ring units while the
+// last products run, rotates out of shared memory and writes 256-byte pieces of the cache rows.
+// 4096 tokens of the 7B shape (68.7 GFLOP): 54 us, 1.27 PFLOP/s (82 us with 256 x 256 tiles of one
+// block), 63 us back to back at the power cap; the main loop keeps the tensor cores busy (67.2 k of
+// 65.5 k clocks), 10 k clocks of epilogue follow.  2048 tokens: 32 us (46 us with 128 x 128 tiles).
+constexpr int kBN = 256;                 // columns per pair
+constexpr int kUnits = 14;
+constexpr int kUnitBytes = 128 * kPK * 2;                 // 16 KB
+constexpr int kBThreads = 320;           // warp 0 loads, warp 1 MMA (first block), warps 2-9 epilogue
 
-struct __align__(8) BigBarriers {
-  uint64_t full[kBStages], empty[kBStages], done;
+struct __align__(8) PairBarriers {
+  uint64_t full[kUnits], empty[kUnits], done;      // full: of the first block only, for both blocks' units
 };
 
+// Epilogue buffers lie in the operand ring, in the units read last.  Per warp of 32 tokens: the tokens'
+// rows of the (cos, sin) table in one unit (512 bytes a row, entry e at e ^ row: equal columns of 32
+// tokens are on different banks), which starts to fill as soon as that unit's last product is done;
+// and 128 finished columns of the 32 cache rows in half a unit (16-byte pieces XORed with the row).
+constexpr int kCsHalf = 64;              // table rows of up to 64 chunks
+static_assert(32 * kCsHalf * 8 == kUnitBytes && 2 * 32 * 256 == kUnitBytes && 8 + 4 <= kUnits, "epilogue buffers fit");
+
+template <int H>
 __global__ void __launch_bounds__(kBThreads, 1)
-project_append_big_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                          const ProjArgs a) {
+project_append_pair_kernel(const __grid_constant__ CUtensorMap map_t, const __grid_constant__ CUtensorMap map_w,
+                           const ProjArgs a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  BigBarriers* bars = (BigBarriers*)(base + kBStages * kBStageBytes);
+  PairBarriers* bars = (PairBarriers*)(base + kUnits * kUnitBytes);
   uint32_t* s_tmem = (uint32_t*)(bars + 1);
   volatile int* s_abort = (volatile int*)(s_tmem + 1);
+  static_assert(sizeof(PairBarriers) % 16 == 8, "s_idx on 16 bytes");
+  int* s_idx = (int*)(s_tmem + 2);                 // [128] chunk ids of the tile's rope columns
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * kBN;
-  const long long t0 = (long long)blockIdx.y * kBM;
+  const uint32_t rank = cluster_ctarank();
+  const int n0 = (blockIdx.x >> 1) * kBN;
+  const long long t0 = (long long)blockIdx.y * (256 * H) + rank * (128 * H);      // first token of this block
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kBStages; ++i) {
-      mbar_init(smem_u32(&bars->full[i]), 2);      // one arrival per loading warp
+    for (int i = 0; i < kUnits; ++i) {
+      mbar_init(smem_u32(&bars->full[i]), 1);
       mbar_init(smem_u32(&bars->empty[i]), 1);
     }
     mbar_init(smem_u32(&bars->done), 1);
@@ -280,80 +301,170 @@ project_append_big_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
-  constexpr uint32_t tmem_cols = 512;      // the whole tensor memory: one block per SM (192 KB of shared memory)
+  constexpr uint32_t tmem_cols = 512;      // the whole tensor memory: one block per SM (224 KB of shared memory)
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(tmem_cols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(tmem_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x >= 64 && threadIdx.x < 192) {
+    const int pr = (n0 >> 1) + (int)threadIdx.x - 64;
+    s_idx[threadIdx.x - 64] = 2 * pr < a.rope_w ? __ldg(a.idx + pr) : 0;
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();                      // both blocks' barriers and tensor memory exist
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
 
-  if (warp == 0 || warp == 6) {
-    // ---- warp 0: one 256-row box of x per stage (rows past the end: zeros); warp 6: one of the weights
-    const bool wload = warp == 6;
+  if (warp == 0) {
+    // ---- per 64 of depth: this block's 128 weight rows and its H units of 128 token rows (zeros past
+    //      the end).  (Prefetching later steps into L2 takes the same copy engine: 41 us instead of 33
+    //      for 2048 tokens.)
+    const int w0 = n0 + (int)rank * (kBN / 2);
     bool ok = true;
+    int slot = 0;
+    uint32_t turn = 1;                     // parity of `empty` before the first pass over the ring
     for (int k = 0; k < a.nk && ok; ++k) {
-      const int s = k % kBStages;
-      ok = warp_wait(smem_u32(&bars->empty[s]), ((k / kBStages) & 1) ^ 1, s_abort, wload ? 4 : 1);
-      if (!ok) break;
-      if (elect_one()) {
-        const uint32_t fb = smem_u32(&bars->full[s]);
-        mbar_expect_tx(fb, (uint32_t)(kBStageBytes / 2));
-        if (wload) tma_load_2d(smem_u32(base + s * kBStageBytes + kBM * kPK * 2), &map_w, k * kPK, n0, fb);
-        else tma_load_2d(smem_u32(base + s * kBStageBytes), &map_x, k * kPK, (int)t0, fb);
-      }
-      __syncwarp();
-    }
-  } else if (warp == 1) {
-    constexpr uint32_t idesc = make_idesc(128, kBN, 0, 0);
-    constexpr uint32_t hi_sw = desc_hi(1024, 2);
-    const uint32_t base16 = (smem_u32(base) >> 4) & 0x3FFFu;
-    bool ok = true;
-    for (int k = 0; k < a.nk && ok; ++k) {
-      const int s = k % kBStages;
-      ok = warp_wait(smem_u32(&bars->full[s]), (k / kBStages) & 1, s_abort, 2);
-      if (!ok) break;
-      const uint32_t la0 = (base16 + (uint32_t)s * (kBStageBytes >> 4)) | (1u << 16);   // token rows 0-127
-      const uint32_t la1 = la0 + ((128 * kPK * 2) >> 4);                                // token rows 128-255
-      const uint32_t lb = la0 + ((kBM * kPK * 2) >> 4);
-      if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {          // +32 bytes along d per step
-          tc_mma_w(tmem_base, la0 + 2 * ks, hi_sw, lb + 2 * ks, hi_sw, idesc, (k | ks) != 0);
-          tc_mma_w(tmem_base + kBN, la1 + 2 * ks, hi_sw, lb + 2 * ks, hi_sw, idesc, (k | ks) != 0);
+      for (int u = 0; u <= H; ++u) {
+        ok = warp_wait(smem_u32(&bars->empty[slot]), turn, s_abort, 1);
+        if (!ok) break;
+        if (elect_one()) {
+          const uint32_t fb = smem_u32(&bars->full[slot]);
+          if (rank == 0) mbar_expect_tx(fb, 2 * kUnitBytes);
+          tma_load_2d_pair(smem_u32(base + slot * kUnitBytes), u == 0 ? &map_w : &map_t, k * kPK,
+                           u == 0 ? w0 : (int)t0 + (u - 1) * 128, map_to_cta(fb, 0));
         }
-        tc_commit(smem_u32(&bars->empty[s]));
+        __syncwarp();
+        if (++slot == kUnits) { slot = 0; turn ^= 1; }
       }
-      __syncwarp();
     }
-    if (ok && elect_one()) tc_commit(smem_u32(&bars->done));
-    __syncwarp();
-  } else {
-    // ---- epilogue: a thread owns token rows trow and trow + 128 of the tile
-    const int quarter = warp & 3;
-    const int trow = quarter * 32 + lane;
-    long long row[2];
-    int p[2] = {0, 0};
+  } else if (warp == 1 && rank == 0) {
+    constexpr uint32_t idesc = make_idesc(256, kBN, 0, 0);
+    constexpr uint32_t hi_sw = desc_hi(1024, 2);
+    const uint32_t base16 = ((smem_u32(base) >> 4) & 0x3FFFu) | (1u << 16);
+    bool ok = true;
+    int slot = 0;
+    uint32_t turn = 0;
+    for (int k = 0; k < a.nk && ok; ++k) {
+      uint32_t lb = 0;
+      int slot_w = 0;
 #pragma unroll
-    for (int hf = 0; hf < 2; ++hf) {
-      const long long t = t0 + hf * 128 + trow;
-      row[hf] = t < a.T ? token_row(a, t, &p[hf]) : -1;
+      for (int u = 0; u <= H; ++u) {
+        ok = warp_wait(smem_u32(&bars->full[slot]), turn, s_abort, 2);
+        if (!ok) break;
+        const uint32_t lo = base16 + (uint32_t)slot * (kUnitBytes >> 4);
+        if (u == 0) {
+          lb = lo;
+          slot_w = slot;
+        } else {
+          tc_fence_after();
+          if (elect_one()) {
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)            // +32 bytes along d per step
+              tc_mma_pair(tmem_base + (u - 1) * kBN, lo + 2 * ks, hi_sw, lb + 2 * ks, hi_sw, idesc, (k | ks) != 0);
+            tc_commit_pair(smem_u32(&bars->empty[slot]));                // frees the unit in both blocks
+            if (u == H) tc_commit_pair(smem_u32(&bars->empty[slot_w]));
+          }
+          __syncwarp();
+        }
+        if (++slot == kUnits) { slot = 0; turn ^= 1; }
+      }
     }
-    const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->done), 0, s_abort, 3));
+    if (ok && elect_one()) tc_commit_pair(smem_u32(&bars->done));
+    __syncwarp();
+  } else if (warp >= 2) {
+    // ---- epilogue: warps 2-5 the first accumulator (H = 1: its first 128 columns), 6-9 the second
+    //      (its second 128 columns)
+    const int quarter = warp & 3, hf = (warp - 2) >> 2;
+    const int tok = H == 2 ? hf * 128 : 0, part0 = H == 2 ? 0 : hf, parts = H;      // tokens and columns of this warp
+    const long long t = t0 + tok + quarter * 32 + lane;
+    int p = 0;
+    const long long row = t < a.T ? token_row(a, t, &p) : -1;
+    if (row < 0) p = 0;
+    const int w8 = warp - 2, first = (H + 1) * a.nk - kUnits;     // the units of the ring's last turn
+    unsigned char* s_cs = base + (first + w8) % kUnits * kUnitBytes;
+    unsigned char* s_out = base + (first + 8 + (w8 >> 1)) % kUnits * kUnitBytes + (w8 & 1) * (kUnitBytes / 2);
+    const bool staged = a.half <= kCsHalf && (a.half & 1) == 0;
+    bool ok = true;
+    if (n0 + part0 * 128 < a.rope_w && staged) {
+      // the 32 tokens' table rows, a whole row per request: a look-up by every token on its own would
+      // touch 32 rows per request (33 k clocks for a tile of rope columns)
+      for (int f = 0; ok && f <= (first + w8) / kUnits; ++f)
+        ok = warp_wait(smem_u32(&bars->empty[(first + w8) % kUnits]), f & 1, s_abort, 4);
+      if (ok) {
+#pragma unroll 16
+        for (int k = 0; k < 32; ++k) {
+          const int pk = __shfl_sync(0xffffffffu, p, k);
+          if (2 * lane < a.half) {
+            const float4 w = __ldg((const float4*)(a.cs + (long long)pk * a.half) + lane);
+            float2* dst = (float2*)(s_cs + k * (kCsHalf * 8));
+            dst[(2 * lane) ^ k] = make_float2(w.x, w.y);
+            dst[(2 * lane + 1) ^ k] = make_float2(w.z, w.w);
+          }
+        }
+        __syncwarp();
+      }
+    }
+    ok = ok && __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->done), 0, s_abort, 3));
     tc_fence_after();
     if (ok) {
-#pragma unroll 1
-      for (int hf = 0; hf < 2; ++hf) {
-        for (int cc = 0; cc < kBN / 32; ++cc) {
+      const float2* cs_row = (const float2*)(s_cs + lane * (kCsHalf * 8));
+      for (int part = part0; part < part0 + parts; ++part) {        // 128 columns: all rope or all latent
+        const int g0 = n0 + part * 128;
+        const bool rope = g0 < a.rope_w;
+        bf16* const out = rope ? a.rope + g0 : a.latent + (g0 - a.rope_w);
+        const long long pitch = rope ? a.rope_w : a.d_c;
+#pragma unroll 2
+        for (int cc = 0; cc < 4; ++cc) {
           float v[32];
-          tc_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(hf * kBN + cc * 32), v);
-          tc_wait_ld();
-          if (row[hf] < 0) continue;
+          tc_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(tok * 2 + part * 128 + cc * 32), v);
+          float2 w[16];
+          if (rope) {
+            const int4* id4 = (const int4*)(s_idx + part * 64 + cc * 16);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) finish_columns(a, v + 8 * q, row[hf], p[hf], n0 + cc * 32 + 8 * q);
+            for (int k = 0; k < 4; ++k) {
+              const int4 id = id4[k];
+              if (staged) {
+                w[4 * k] = cs_row[id.x ^ lane]; w[4 * k + 1] = cs_row[id.y ^ lane];
+                w[4 * k + 2] = cs_row[id.z ^ lane]; w[4 * k + 3] = cs_row[id.w ^ lane];
+              } else {
+                const float2* src = a.cs + (long long)p * a.half;
+                w[4 * k] = __ldg(src + id.x); w[4 * k + 1] = __ldg(src + id.y);
+                w[4 * k + 2] = __ldg(src + id.z); w[4 * k + 3] = __ldg(src + id.w);
+              }
+            }
+          }
+          tc_wait_ld();
+          if (rope) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+              const float x0 = v[2 * k], x1 = v[2 * k + 1];
+              v[2 * k] = __fsub_rn(__fmul_rn(x0, w[k].x), __fmul_rn(x1, w[k].y));
+              v[2 * k + 1] = __fadd_rn(__fmul_rn(x0, w[k].y), __fmul_rn(x1, w[k].x));
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint32_t packed[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const bf162 y = __floats2bfloat162_rn(v[8 * q + 2 * k], v[8 * q + 2 * k + 1]);
+              packed[k] = *(const uint32_t*)&y;
+            }
+            *(uint4*)(s_out + lane * 256 + (((cc * 4 + q) ^ (lane & 15)) << 4)) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+          }
         }
+        __syncwarp();
+        // 256 bytes of two tokens' cache rows per request
+#pragma unroll 8
+        for (int k = 0; k < 16; ++k) {
+          const int tk = 2 * k + (lane >> 4);
+          const long long rk = __shfl_sync(0xffffffffu, row, tk);
+          const uint4 y = *(const uint4*)(s_out + tk * 256 + (((lane ^ tk) & 15) << 4));
+          if (rk >= 0) *(uint4*)(out + rk * pitch + (lane & 15) * 8) = y;
+        }
+        __syncwarp();
       }
     }
   }
@@ -362,9 +473,10 @@ project_append_big_kernel(const __grid_constant__ CUtensorMap map_x, const __gri
   __syncthreads();
   if (*s_abort) drain_after_abort();
   if (threadIdx.x == 0 && *s_abort) ekv_record(a.status, ELITEKV_ERR_TIMEOUT, (int)blockIdx.x | (*s_abort << 16), (int)blockIdx.y);
+  cluster_sync_all();                      // the tensor core reads both blocks' shared memory until the end
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
 }
 
@@ -377,34 +489,6 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
   const int n_out = rope_w + L->d_c;
   if (L->d % kPK != 0 || rope_w % kPN != 0 || L->d_c % kPN != 0) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
   if (T >= (1ll << 31)) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
-  // prefill-sized calls whose output width is whole 256-column tiles: the 256 x 256 form
-  if (T >= 1024 && n_out % kBN == 0) {
-    const int smem_big = kBStages * kBStageBytes + (int)sizeof(BigBarriers) + 64 + 1024;
-    if (smem_big <= L->smem_optin) {
-      CUtensorMap b_x, b_w;
-      int rcb = make_map(&b_x, x, (unsigned long long)T, (unsigned long long)L->d, kBM);
-      if (rcb == ELITEKV_OK) rcb = make_map(&b_w, L->d_WcatT, (unsigned long long)n_out, (unsigned long long)L->d, kBN);
-      if (rcb != ELITEKV_OK) return rcb;
-      ProjArgs b;
-      b.seq_id = seq_id; b.pos = pos; b.T = T;
-      b.rope = (bf16*)cache->rope; b.latent = (bf16*)cache->latent; b.cv = cv;
-      b.idx = L->d_idx; b.cs = L->d_cs; b.rope_w = rope_w; b.d_c = L->d_c;
-      b.half = L->d_h / 2; b.max_pos = L->max_pos; b.nk = L->d / kPK; b.status = L->d_status;
-      EKV_CUDA_OK(cudaFuncSetAttribute(project_append_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_big));
-      dim3 grid((unsigned)(n_out / kBN), (unsigned)((T + kBM - 1) / kBM));
-      project_append_big_kernel<<<grid, kBThreads, smem_big, st>>>(b_x, b_w, b);
-      EKV_CUDA_OK(cudaGetLastError());
-      return ELITEKV_OK;
-    }
-  }
-  // at most one token tile and enough depth for every block of a cluster: the split-depth form
-  const bool split = T <= kPM && L->d / kPK >= kSplit;
-  const int smem = kPStages * kPStageBytes + (split ? kRecvBytes : 0) + (int)sizeof(ProjBarriers) + 64 + 1024;
-  if (smem > L->smem_optin) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
-  CUtensorMap m_x, m_w;
-  int rc = make_map(&m_x, x, (unsigned long long)T, (unsigned long long)L->d, kPM);
-  if (rc == ELITEKV_OK) rc = make_map(&m_w, L->d_WcatT, (unsigned long long)n_out, (unsigned long long)L->d, kPN);
-  if (rc != ELITEKV_OK) return rc;
   ProjArgs a;
   a.seq_id = seq_id;
   a.pos = pos;
@@ -420,6 +504,52 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
   a.max_pos = L->max_pos;
   a.nk = L->d / kPK;
   a.status = L->d_status;
+  // More than one token tile and an output width of whole 256-column tiles: the form whose blocks need
+  // least time for the call.  All take whole waves over the chip; microseconds for 64 depth steps
+  // measured on 7B shapes at 256 to 16384 tokens (one tile per block 28, 46, 67, 85 for 1 to 4 waves,
+  // H = 1 33, 59, H = 2 50, 102, 152; other depths scale all three alike).
+  const int smem_pair = kUnits * kUnitBytes + (int)sizeof(PairBarriers) + 16 + 128 * 4 + 1024;
+  int form = 0;
+  if (T > kPM && n_out % kBN == 0 && 2 * a.nk >= kUnits && smem_pair <= L->smem_optin) {
+    const auto waves = [&](long long cols, long long rows, long long at_once) {
+      return (n_out / cols * ((T + rows - 1) / rows) + at_once - 1) / at_once;
+    };
+    const long long t0 = 7 + 20 * waves(kPN, kPM, L->sm_count);
+    const long long t1 = 4 + 29 * waves(kBN, 256, L->sm_count / 2);
+    const long long t2 = 2 + 50 * waves(kBN, 512, L->sm_count / 2);
+    form = t2 <= t1 && t2 <= t0 ? 2 : t1 <= t0 ? 1 : 0;
+  }
+  if (form != 0) {
+    CUtensorMap b_x, b_w;
+    int rcb = make_map(&b_x, x, (unsigned long long)T, (unsigned long long)L->d, 128);
+    if (rcb == ELITEKV_OK) rcb = make_map(&b_w, L->d_WcatT, (unsigned long long)n_out, (unsigned long long)L->d, kBN / 2);
+    if (rcb != ELITEKV_OK) return rcb;
+    const auto kern = form == 2 ? project_append_pair_kernel<2> : project_append_pair_kernel<1>;
+    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_pair));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * (n_out / kBN)), (unsigned)((T + 256 * form - 1) / (256 * form)));
+    cfg.blockDim = dim3(kBThreads);
+    cfg.dynamicSmemBytes = (size_t)smem_pair;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    EKV_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, b_x, b_w, a));
+    EKV_CUDA_OK(cudaGetLastError());
+    return ELITEKV_OK;
+  }
+  // at most one token tile and enough depth for every block of a cluster: the split-depth form
+  const bool split = T <= kPM && L->d / kPK >= kSplit;
+  const int smem = kPStages * kPStageBytes + (split ? kRecvBytes : 0) + (int)sizeof(ProjBarriers) + 64 + 1024;
+  if (smem > L->smem_optin) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
+  CUtensorMap m_x, m_w;
+  int rc = make_map(&m_x, x, (unsigned long long)T, (unsigned long long)L->d, kPM);
+  if (rc == ELITEKV_OK) rc = make_map(&m_w, L->d_WcatT, (unsigned long long)n_out, (unsigned long long)L->d, kPN);
+  if (rc != ELITEKV_OK) return rc;
   if (split) {
     EKV_CUDA_OK(cudaFuncSetAttribute(project_append_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg = {};

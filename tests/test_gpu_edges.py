@@ -187,3 +187,25 @@ def test_generic_kernel_item_edges(ek, lens):
     st = H.setup(w, lens=lens)
     assert ek.elitekv_decode_plan_info(st.layer, st.cache, len(lens))[:2] == (1, 16)
     H.check_parity(st, H.run_decode(st), H.all_units(st))
+
+
+# ------------------------------------------------------------------ projection, paired forms
+# one small layer per property: 256 columns of rope and latent side by side in a tile (128 + 128), table
+# rows as long as a buffer holds (half = 64) and longer (half = 96, read directly), the smallest depth
+PAIR_SHAPES = {
+    "7b": (gen.LLAMA7B_75, 4096),
+    "split-tile": (replace(gen.LLAMA7B_75, n_h=16, r=4, d_c=128), 448),
+    "wide-heads": (replace(gen.LLAMA7B_75, n_h=16, d_h=192, r=8, d_c=256), 512),
+}
+
+
+@pytest.mark.parametrize("shape,T", [("7b", 1153), ("7b", 2304), ("7b", 2305), ("split-tile", 9473), ("split-tile", 18945),
+                                     ("wide-heads", 4737), ("wide-heads", 9473)])
+@pytest.mark.parametrize("paged", [False, True])
+def test_project_append_paired_forms(ek, shape, T, paged):
+    """Calls on both sides of the lines between the forms (one tile of 128 x 128 per block; pairs of
+    blocks with 256 or 512 tokens x 256 columns), with ragged last token tiles."""
+    from .test_gpu_parity import _projection_case
+    w, d = PAIR_SHAPES[shape]
+    lens = [T - 200, 137, 63]
+    _projection_case(ek, gen.shrink(w, B=3, ctx=max(lens)), d, lens, paged, T)
