@@ -186,6 +186,11 @@ int elitekv_decode_step(const elitekv_layer* layer, const elitekv_cache* cache, 
                         const int32_t* seq_lens, int32_t B, void* q_rope, void* q_abs,
                         void* workspace, size_t workspace_bytes, void* out, elitekv_stream_t stream);
 
+/* Copies bytes between device memory and PINNED host memory (either way) with a kernel on `stream`:
+ * before and after elitekv_decode_step such copies overlap the launches of its kernels.  dst and src
+ * are 16-byte aligned; memory that the device cannot address is refused (ELITEKV_ERR_INVALID_ARG). */
+int elitekv_copy(void* dst, const void* src, int64_t bytes, elitekv_stream_t stream);
+
 /* Several query rows per sequence over the cache, with the causal rule (Section 3.1: the score
  * equation holds for any query position m and key position n): a chunk of a prefill, or the
  * draft tokens of speculative decoding.  The m new tokens of every sequence are in the cache

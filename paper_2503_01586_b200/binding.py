@@ -68,6 +68,7 @@ def lib() -> C.CDLL:
         L.elitekv_decode_workspace_size.argtypes = [vp, i32, C.POINTER(sz)]
         L.elitekv_decode.argtypes = [vp, C.POINTER(CacheDesc), vp, vp, vp, i32, vp, sz, vp, vp]
         L.elitekv_decode_step.argtypes = [vp, C.POINTER(CacheDesc), vp, vp, vp, vp, vp, vp, i32, vp, vp, vp, sz, vp, vp]
+        L.elitekv_copy.argtypes = [vp, vp, i64, vp]
         L.elitekv_attend_rows_workspace_size.argtypes = [vp, i32, i32, C.POINTER(sz)]
         L.elitekv_attend_rows.argtypes = [vp, C.POINTER(CacheDesc), vp, vp, vp, i32, i32, vp, sz, vp, vp]
         L.elitekv_ropelite_workspace_size.argtypes = [i32, i32, i32, C.POINTER(sz)]
@@ -92,7 +93,7 @@ def lib() -> C.CDLL:
                      "elitekv_profile_enable", "elitekv_profile_collect", "elitekv_decode_static",
                      "elitekv_mha_decode", "elitekv_plan_workers", "elitekv_decode_plan_info",
                      "elitekv_last_status_detail", "elitekv_selftest_bounded_wait",
-                     "elitekv_project_append", "elitekv_decode_step",
+                     "elitekv_project_append", "elitekv_decode_step", "elitekv_copy",
                      "elitekv_attend_rows_workspace_size", "elitekv_attend_rows",
                      "elitekv_ropelite_workspace_size", "elitekv_ropelite_distances", "elitekv_ropelite_search"):
             getattr(L, name).restype = C.c_int
@@ -298,14 +299,25 @@ def elitekv_ropelite_search(Q, K, r: int, rope_base: float = 10000.0, trace: boo
     return (idx, tr) if trace else idx
 
 
+def elitekv_copy(dst, src) -> None:
+    """Copy between a device tensor and a pinned host tensor of the same size, by a kernel."""
+    if dst.numel() * dst.element_size() != src.numel() * src.element_size():
+        raise ValueError("elitekv_copy: sizes differ")
+    if not (dst.is_contiguous() and src.is_contiguous()):
+        raise ValueError("elitekv_copy: tensors must be contiguous")
+    _check(lib().elitekv_copy(C.c_void_p(dst.data_ptr()), C.c_void_p(src.data_ptr()),
+                              dst.numel() * dst.element_size(), _stream()), "elitekv_copy")
+
+
 class DecodeStepRunner:
     """Host-to-host decode step of one layer at a fixed batch size B.  The step's six input
     arrays live in ONE pinned staging buffer (`host[...]`: k_e [B][n_h][2r], c [B][d_c],
     q [B][n_h][d_h], seq_id / pos / lens [B] int32) that crosses in one copy; the result comes
-    back into the pinned `out_host` [B][n_h][d_h].  With `graph=True` the copy in, the
-    elitekv_decode_step call and the copy out are captured in a CUDA graph on the second `run()`
-    and replayed from then on; otherwise `run()` enqueues the three eagerly.  Marshalling only: every byte of
-    arithmetic happens in the library's kernels."""
+    back into the pinned `out_host` [B][n_h][d_h].  Both copies are kernels, links of the step's
+    chain of launches.  With `graph=True` the copy in, the elitekv_decode_step call and the copy
+    out are captured in a CUDA graph on the second `run()` and replayed from then on; otherwise
+    `run()` enqueues the three eagerly.  Marshalling only: every byte of arithmetic happens in the
+    library's kernels."""
 
     ORDER = ("k_e", "c", "q", "seq_id", "pos", "lens")
 
@@ -342,10 +354,10 @@ class DecodeStepRunner:
 
     def _enqueue(self):
         d = self.dev
-        self.pack_dev.copy_(self.pack_host, non_blocking=True)
+        elitekv_copy(self.pack_dev, self.pack_host)
         elitekv_decode_step(self.layer, self.cache, d["k_e"], d["c"], d["seq_id"], d["pos"], d["q"], d["lens"],
                             self.q_rope, self.q_abs, self.workspace, self.out)
-        self.out_host.copy_(self.out, non_blocking=True)
+        elitekv_copy(self.out_host, self.out)
 
     def run(self, wait: bool = True):
         """One step from `host[...]` to `out_host`; with `wait`, returns once the result is there.

@@ -209,3 +209,24 @@ def test_project_append_paired_forms(ek, shape, T, paged):
     w, d = PAIR_SHAPES[shape]
     lens = [T - 200, 137, 63]
     _projection_case(ek, gen.shrink(w, B=3, ctx=max(lens)), d, lens, paged, T)
+
+
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 4096, 16 * 256 * 512 * 4 + 16 * 300 + 5])
+def test_copy_both_ways(ek, n):
+    """Bytes below, at and above one 16-byte request, and more than one round of the largest grid;
+    neighbouring bytes stay as they are."""
+    host = torch.randint(0, 256, (n,), dtype=torch.uint8).pin_memory()
+    dev = torch.full((n + 16,), 7, dtype=torch.uint8, device="cuda")
+    back = torch.full((n + 16,), 9, dtype=torch.uint8).pin_memory()
+    ek.elitekv_copy(dev[:n], host)
+    ek.elitekv_copy(back[:n], dev[:n])
+    torch.cuda.synchronize()
+    assert torch.equal(dev[:n].cpu(), host) and torch.equal(back[:n], host)
+    assert (dev[n:] == 7).all() and (back[n:] == 9).all()
+
+
+def test_copy_refuses_what_the_device_cannot_address(ek):
+    dev = torch.zeros(64, dtype=torch.uint8, device="cuda")
+    for dst, src in ((dev[:32], torch.zeros(32, dtype=torch.uint8)), (dev[1:33], dev[32:])):
+        with pytest.raises((ek.ElitekvError, ValueError)):
+            ek.elitekv_copy(dst, src)
