@@ -48,7 +48,8 @@ constexpr int kFThreads = 256;
 constexpr int kFPitch = kFD + 8; // shared-memory row pitch in bf16: 16 bytes of padding keep ldmatrix free of bank conflicts
 constexpr int kFAhead = 4;       // partial results per row in flight beside the statistics
 
-__global__ void __launch_bounds__(kFThreads, 4)
+template <bool kShare>
+__global__ void __launch_bounds__(kFThreads, kShare ? 3 : 4)
 combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by the split-K kernel while this
                                                                    // kernel may already be resident: read
                                                                    // with plain L2 loads, never ld.global.nc
@@ -57,8 +58,9 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
                     int32_t* __restrict__ counters /* [n_h][groups], zeroed by the plan kernel */,
                     bf16* __restrict__ out, int B, int rows, int n_h, int d_c) {
   __shared__ __align__(16) bf16 s_w[kFK][kFPitch];        // W_uv slice
-  __shared__ __align__(16) bf16 s_hi[kFB][kFPitch];       // merged latent outputs: bf16 head ...
-  __shared__ __align__(16) bf16 s_lo[kFB][kFPitch];       // ... and remainder
+  __shared__ __align__(16) bf16 s_o[2][kFB][kFPitch];     // merged latent outputs: bf16 head and remainder
+  bf16 (*const s_hi)[kFPitch] = s_o[0];
+  bf16 (*const s_lo)[kFPitch] = s_o[1];
   __shared__ int s_last;
   const int h = blockIdx.x, slice = blockIdx.y, n_slices = gridDim.y, g = blockIdx.z;
   const int k0 = slice * kFK;
@@ -72,16 +74,19 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
     cp_async16(&s_w[k][v * 8], Wuv + (size_t)(k0 + k) * n_h * kFD + (size_t)h * kFD + v * 8);
   }
   cp_async_commit();
-  // Row r = (sequence r / rows, query row r % rows).  Warp w merges rows 2w and 2w + 1; half a warp
-  // holds a row's softmax statistics, lane j of the half those of its j-th item.  The plan was
-  // written before the split-K kernel started computing (that kernel waited for it before it let
-  // this one be launched), so the item ranges are fetched while the split-K kernel still runs.
+  // Row r = (sequence r / rows, query row r % rows).  A warp merges two rows; half a warp holds a row's
+  // softmax statistics, lane j of the half those of its j-th item.  kShare: at most 8 rows, and 8 / 4 / 2
+  // warps take turns at the items of a pair.  The plan was written before the split-K kernel started
+  // computing (that kernel waited for it before it let this one be launched), so the item ranges are
+  // fetched while the split-K kernel still runs.
+  const int share = !kShare ? 1 : nb <= 2 ? 8 : nb <= 4 ? 4 : 2;
+  const int row_w = 2 * (warp / share), sub = warp % share;
   const int half = lane >> 4, j = lane & 15;
   int i0[2], ni[2];
   size_t src0[2];                // first partial result of the row on this slice, in floats
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
-    const int rr = 2 * warp + e;
+    const int rr = row_w + e;
     i0[e] = ni[e] = 0;
     src0[e] = 0;
     if (rr < nb) {
@@ -93,7 +98,7 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
   }
   const size_t stride = (size_t)rows * n_h * d_c;                // from one item to the next
   const int my_i0 = half ? i0[1] : i0[0], my_ni = half ? ni[1] : ni[0];
-  const int my_q = (r0 + 2 * warp + half) % rows;
+  const int my_q = (r0 + row_w + half) % rows;
   auto item_ml = [&](int k) -> float2 {
     return __ldcg((const float2*)part_ml + ((size_t)(my_i0 + k) * rows + my_q) * n_h + h);
   };
@@ -101,27 +106,34 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
   ekv_pdl_trigger();
 
   // statistics and the first partial results of both rows are requested together
-  float2 ml = make_float2(-INFINITY, 0.f);
+  float2 ml = make_float2(-INFINITY, 0.f), ml2 = ml;
   if (j < my_ni) ml = item_ml(j);
+  if (kShare && j + 16 < my_ni) ml2 = item_ml(j + 16);
+  const int first = kShare ? kFAhead * sub : 0;      // this warp's first item
   float4 p[2][kFAhead];
 #pragma unroll
   for (int e = 0; e < 2; ++e)
 #pragma unroll
     for (int k = 0; k < kFAhead; ++k)
-      p[e][k] = k < ni[e] ? __ldcg((const float4*)(part_acc + src0[e] + k * stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
-  float M = ml.x;
-  for (int k = j + 16; k < my_ni; k += 16) M = fmaxf(M, item_ml(k).x);       // rare: more than 16 items
+      p[e][k] = first + k < ni[e] ? __ldcg((const float4*)(part_acc + src0[e] + (first + k) * stride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  constexpr int kHeld = kShare ? 32 : 16;    // items whose statistics are in registers
+  float M = kShare ? fmaxf(ml.x, ml2.x) : ml.x;
+  for (int k = j + kHeld; k < my_ni; k += 16) M = fmaxf(M, item_ml(k).x);       // rare: more items
 #pragma unroll
   for (int o = 1; o < 16; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
   float L = j < my_ni ? ml.y * exp2f(ml.x - M) : 0.f;
-  for (int k = j + 16; k < my_ni; k += 16) {
+  if (kShare && j + 16 < my_ni) L = fmaf(ml2.y, exp2f(ml2.x - M), L);
+  for (int k = j + kHeld; k < my_ni; k += 16) {
     const float2 x = item_ml(k);
     L += x.y * exp2f(x.x - M);
   }
 #pragma unroll
   for (int o = 1; o < 16; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
   const float invL = my_ni > 0 && L > 0.f ? 1.f / L : 0.f;
-  float wt = j < my_ni ? exp2f(ml.x - M) * invL : 0.f;                      // normalised weight of item j
+  // normalised weight of item j (shared rows: of the warp's first group of items)
+  float wt = j < my_ni ? exp2f(ml.x - M) * invL : 0.f;
+  const float wt2 = kShare && j + 16 < my_ni ? exp2f(ml2.x - M) * invL : 0.f;
+  if (kShare && first >= 16) wt = wt2;
   float4 acc[2];
 #pragma unroll
   for (int e = 0; e < 2; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -131,16 +143,21 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
 #pragma unroll
   for (int e = 0; e < 2; ++e)
 #pragma unroll
-    for (int k = 0; k < kFAhead; ++k) add(acc[e], __shfl_sync(0xffffffffu, wt, 16 * e + k), p[e][k]);
+    for (int k = 0; k < kFAhead; ++k) add(acc[e], __shfl_sync(0xffffffffu, wt, 16 * e + ((first + k) & 15)), p[e][k]);
   const int n_most = max(ni[0], ni[1]);
-  for (int k0b = kFAhead; k0b < n_most; k0b += kFAhead) {
+  for (int k0b = first + kFAhead * share; k0b < n_most; k0b += kFAhead * share) {
 #pragma unroll
     for (int e = 0; e < 2; ++e)
 #pragma unroll
       for (int k = 0; k < kFAhead; ++k)
         p[e][k] = k0b + k < ni[e] ? __ldcg((const float4*)(part_acc + src0[e] + (size_t)(k0b + k) * stride))
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-    if ((k0b & 15) == 0) wt = k0b + j < my_ni ? exp2f(item_ml(k0b + j).x - M) * invL : 0.f;
+    if (kShare) {
+      const int kj = (k0b & ~15) + j;
+      wt = k0b < 16 ? (j < my_ni ? exp2f(ml.x - M) * invL : 0.f) : k0b < 32 ? wt2 : kj < my_ni ? exp2f(item_ml(kj).x - M) * invL : 0.f;
+    } else if ((k0b & 15) == 0) {
+      wt = k0b + j < my_ni ? exp2f(item_ml(k0b + j).x - M) * invL : 0.f;
+    }
 #pragma unroll
     for (int e = 0; e < 2; ++e)
 #pragma unroll
@@ -148,14 +165,31 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
   }
   // the fp32 rows are fed to the product as a bf16 head plus a bf16 remainder, so nothing but the
   // last ~2^-17 of them is lost; W_uv is bf16 as stored
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const bf162 h0 = __floats2bfloat162_rn(acc[e].x, acc[e].y), h1 = __floats2bfloat162_rn(acc[e].z, acc[e].w);
+  auto store_row = [&](int rr, const float4& x) {
+    const bf162 h0 = __floats2bfloat162_rn(x.x, x.y), h1 = __floats2bfloat162_rn(x.z, x.w);
     const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
-    const bf162 l0 = __floats2bfloat162_rn(acc[e].x - f0.x, acc[e].y - f0.y);
-    const bf162 l1 = __floats2bfloat162_rn(acc[e].z - f1.x, acc[e].w - f1.y);
-    *(uint2*)&s_hi[2 * warp + e][lane * 4] = make_uint2(*(const uint32_t*)&h0, *(const uint32_t*)&h1);
-    *(uint2*)&s_lo[2 * warp + e][lane * 4] = make_uint2(*(const uint32_t*)&l0, *(const uint32_t*)&l1);
+    const bf162 l0 = __floats2bfloat162_rn(x.x - f0.x, x.y - f0.y);
+    const bf162 l1 = __floats2bfloat162_rn(x.z - f1.x, x.w - f1.y);
+    *(uint2*)&s_hi[rr][lane * 4] = make_uint2(*(const uint32_t*)&h0, *(const uint32_t*)&h1);
+    *(uint2*)&s_lo[rr][lane * 4] = make_uint2(*(const uint32_t*)&l0, *(const uint32_t*)&l1);
+  };
+  if (!kShare) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) store_row(row_w + e, acc[e]);
+  } else {
+    // the sums of the warps that shared a pair, added in order by a warp per row; rows 8 to 15 hold
+    // nothing that is stored
+    static_assert(kFThreads / 32 * 2 * 32 * sizeof(float4) <= sizeof(s_o), "partial sums take the rows' place");
+    float4* const s_part = (float4*)s_o;                   // [warp][2][32]
+#pragma unroll
+    for (int e = 0; e < 2; ++e) s_part[(2 * warp + e) * 32 + lane] = acc[e];
+    __syncthreads();
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (warp < nb)
+      for (int s = 0; s < share; ++s) add(x, 1.f, s_part[(2 * (warp / 2 * share + s) + (warp & 1)) * 32 + lane]);
+    __syncthreads();
+    store_row(warp, x);
+    store_row(warp + 8, make_float4(0.f, 0.f, 0.f, 0.f));
   }
   cp_async_wait<0>();
   __syncthreads();
@@ -327,7 +361,9 @@ int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, v
   if (ekv_combine_fast_ok(L)) {
     const int rows = ws.rows > 0 ? ws.rows : 1;
     dim3 grid(L->n_h, L->vw / kFK, (B * rows + kFB - 1) / kFB);
-    EKV_CUDA_OK(ekv_launch_pdl(combine_fast_kernel, grid, dim3(kFThreads), 0, st, (const float*)ws.part_acc,
+    // at most 8 rows: idle warps share the rows' items (a 7B step of one sequence: 34.8 -> 32.4 us at 32
+    // items, 8 sequences 50.1 -> 49.4); from 9 rows on at least half of the warps have a pair of their own
+    EKV_CUDA_OK(ekv_launch_pdl(B * rows <= 8 ? combine_fast_kernel<true> : combine_fast_kernel<false>, grid, dim3(kFThreads), 0, st, (const float*)ws.part_acc,
                                (const float*)ws.part_ml, (const int32_t*)ws.seq_first, (const bf16*)L->d_Wuv,
                                ws.slice_out, ws.counters, (bf16*)out, B, rows, L->n_h, L->vw));
     EKV_CUDA_OK(cudaGetLastError());

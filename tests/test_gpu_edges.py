@@ -230,3 +230,14 @@ def test_copy_refuses_what_the_device_cannot_address(ek):
     for dst, src in ((dev[:32], torch.zeros(32, dtype=torch.uint8)), (dev[1:33], dev[32:])):
         with pytest.raises((ek.ElitekvError, ValueError)):
             ek.elitekv_copy(dst, src)
+
+
+@pytest.mark.parametrize("B", [1, 3, 4, 5, 8, 9])
+@pytest.mark.parametrize("n_items", [3, 33, 40])
+def test_combine_rows_sharing_warps(ek, B, n_items):
+    """Up to 8 rows, 8 / 4 / 2 warps take turns at the items of a pair of rows (4 items a turn, the
+    statistics of 32 in registers); from 9 rows on each pair has one warp.  One long sequence among
+    short ones, and an empty one."""
+    w = gen.shrink(gen.LLAMA7B_75, B=B, ctx=128 * n_items)
+    st = H.setup(w, lens=([128 * n_items] + [65, 0, 300, 1, 128, 129, 77, 64])[:B], decode_kernel=2)
+    H.check_parity(st, H.run_decode(st), H.sample_units(st, 24, seed=n_items))
