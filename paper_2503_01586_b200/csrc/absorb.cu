@@ -8,7 +8,7 @@
 // head and 128 latent coordinates: it computes the [16..64 x d_h] . [d_h x 128] product with mma.sync
 // (m16n8k16, bf16 in, fp32 accumulate; both operands are bf16 already, so the products are exact),
 // one warp per 16 coordinates.  The weights come regrouped as [n_h][dn][kw] (kw contiguous); the
-// block's slab is brought into shared memory by one bulk copy per weight row.  The blocks of the
+// block's slab is copied into shared memory asynchronously.  The blocks of the
 // last grid row do the query RoPE (dependent look-ups), off the path of the others.  kw is the
 // width of the latent the scores read: the whole latent row, or the key latent d_ck when keys and
 // values have latents of their own (S-LRD, Section 3.2).

@@ -14,8 +14,8 @@ namespace {
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const PlanArgs a) {
   ekv_pdl_wait();         // earlier kernels may still read the arrays written here
   ekv_pdl_trigger();
-  if (a.n_workers > 0) plan_balanced(a);
-  else plan_even(a);
+  __shared__ PlanShared sh;
+  plan_any(a, sh);
 }
 
 }  // namespace

@@ -7,6 +7,13 @@
 constexpr int kPlanThreads = 256;
 constexpr int kPlanStage = 4096;       // items whose worker ids are staged in shared memory
 
+struct __align__(16) PlanShared {        // the block's shared memory
+  long long total;
+  int warp_tot[kPlanThreads / 32];
+  int first[kPlanThreads], g0[kPlanThreads], len[kPlanThreads], tiles[kPlanThreads];
+  short w0[kPlanThreads], wk[kPlanStage];    // wk: worker of each item (n_workers < 32768)
+};
+
 // exclusive scan over the block (warp shuffles + one shared array of warp totals)
 __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -57,7 +64,94 @@ struct PlanArgs {
   int overhead;
 };
 
-__device__ __forceinline__ void plan_even(const PlanArgs& a) {
+// 32-bit division where the operands allow it (a 64-bit one is a subroutine of over 100 instructions)
+__device__ __forceinline__ long long plan_div(long long x, long long y) {
+  return ((unsigned long long)(x | y) >> 32) == 0 ? (long long)((unsigned)x / (unsigned)y) : x / y;
+}
+
+// Batches of at most a sequence per thread: both plans in one trip for the lengths, two scans and one
+// pass with a thread per ITEM.  (A thread per sequence that writes the sequence's items one after the
+// other, two 64-bit divisions each, took 9 us for one sequence in 33 items and 5 us for 16 sequences,
+// twice as long as the query preparation beside it; this form takes 2.3 and 3.6 us.)  The arithmetic is
+// that of plan_even and plan_balanced below.
+__device__ __forceinline__ bool plan_small_ok(const PlanArgs& a) {
+  return a.B <= kPlanThreads && a.n_workers + a.B <= kPlanStage;
+}
+__device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
+  int* const warp_tot = sh.warp_tot;
+  int *const s_first = sh.first, *const s_g0 = sh.g0, *const s_len = sh.len, *const s_tiles = sh.tiles;
+  short *const s_w0 = sh.w0, *const s_wk = sh.wk;
+  const int t = threadIdx.x, B = a.B;
+  const bool balanced = a.n_workers > 0;
+  const int overhead = balanced ? a.overhead : 0;      // empty tiles in front of every sequence
+  const int n = t < B ? checked_len(a.seq_lens, t, a.max_len, a.status, true) : 0;
+  for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
+  const int tiles = n > 0 ? (int)plan_div((long long)n + a.tile - 1, a.tile) + overhead : 0;
+  int sum;
+  const int g0 = block_exclusive_scan(tiles, warp_tot, &sum);
+  const long long total = sum > 0 ? sum : 1;
+  const long long nw = balanced ? (total < a.n_workers ? total : a.n_workers) : 1;
+  auto bound = [&](long long w) -> long long { return plan_div(w * total, nw); };
+  auto owner = [&](long long g) -> int { return (int)plan_div((g + 1) * nw - 1, total); };
+  int pieces = 0, w0 = 0;
+  if (tiles > 0) {
+    if (balanced) {
+      w0 = owner(g0 + overhead);
+      pieces = owner((long long)g0 + tiles - 1) - w0 + 1;
+    } else {
+      const long long budget = a.max_items - B > 0 ? a.max_items - B : 1;
+      const long long target = plan_div(total + budget - 1, budget);
+      pieces = (int)plan_div(tiles + target - 1, target);
+    }
+  }
+  int n_items;
+  const int first = block_exclusive_scan(pieces, warp_tot, &n_items);
+  if (t < B) {
+    a.seq_first[t] = first;
+    s_first[t] = first; s_g0[t] = g0; s_len[t] = n; s_tiles[t] = tiles; s_w0[t] = (short)w0;
+  }
+  if (t == 0) a.seq_first[B] = n_items;
+  __syncthreads();
+  for (int it = t; it < a.max_items; it += kPlanThreads) {
+    int4 item = make_int4(-1, 0, 0, 0);
+    if (it < n_items) {
+      int lo = 0, hi = B;                    // the last sequence whose first item is not past this one
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (s_first[mid] <= it) lo = mid; else hi = mid;
+      }
+      const int j = it - s_first[lo], len = s_len[lo], tl = s_tiles[lo];
+      int ta, tb, w = 0;                     // tiles of the sequence
+      if (balanced) {
+        const long long base = (long long)s_g0[lo] + overhead;
+        w = s_w0[lo] + j;
+        ta = (int)(max(base, bound(w)) - base);
+        tb = (int)(min((long long)s_g0[lo] + tl, bound(w + 1)) - base);
+        s_wk[it] = (short)w;
+      } else {
+        const int np = (lo + 1 < B ? s_first[lo + 1] : n_items) - s_first[lo];
+        ta = (int)plan_div((long long)tl * j, np);
+        tb = (int)plan_div((long long)tl * (j + 1), np);
+      }
+      const int tok0 = ta * a.tile;
+      item = make_int4(lo, tok0, min(tb * a.tile, len) - tok0, w);
+    }
+    *(int4*)(a.items + 4 * it) = item;
+  }
+  if (!balanced) return;
+  __syncthreads();
+  const int held = min(n_items, a.max_items);
+  for (int w = t; w <= a.n_workers; w += kPlanThreads) {
+    int lo = 0, hi = held;                   // first item whose worker is >= w
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (s_wk[mid] < w) lo = mid + 1; else hi = mid;
+    }
+    a.worker_first[w] = lo;
+  }
+}
+
+__device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
   const int32_t* __restrict__ seq_lens = a.seq_lens;
   const int B = a.B, tile = a.tile, max_items = a.max_items, n_zero = a.n_zero;
   int32_t* __restrict__ items = a.items;
@@ -65,8 +159,8 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a) {
   int32_t* __restrict__ zero_ints = a.zero_ints;
   const long long max_len = a.max_len;
   int32_t* status = a.status;
-  __shared__ int warp_tot[kPlanThreads / 32];
-  __shared__ long long s_total;
+  int* const warp_tot = sh.warp_tot;
+  long long& s_total = sh.total;
   const int t = threadIdx.x;
   for (int i = t; i < n_zero; i += blockDim.x) zero_ints[i] = 0;
   if (t == 0) s_total = 0;
@@ -121,7 +215,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a) {
 // result to write out), and a worker whose range contains the start of a sequence has one item
 // more than the others.  The tile list therefore carries `overhead` empty tiles in front of every
 // sequence: they take room in a worker's quota and hold no tokens.
-__device__ __forceinline__ void plan_balanced(const PlanArgs& a) {
+__device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh) {
   const int32_t* __restrict__ seq_lens = a.seq_lens;
   const int B = a.B, tile = a.tile, n_workers = a.n_workers, max_items = a.max_items, overhead = a.overhead, n_zero = a.n_zero;
   int32_t* __restrict__ items = a.items;
@@ -130,9 +224,9 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a) {
   int32_t* __restrict__ zero_ints = a.zero_ints;
   const long long max_len = a.max_len;
   int32_t* status = a.status;
-  __shared__ int warp_tot[kPlanThreads / 32];
-  __shared__ long long s_total;
-  __shared__ short s_wk[kPlanStage];       // worker of each item (n_workers < 32768)
+  int* const warp_tot = sh.warp_tot;
+  long long& s_total = sh.total;
+  short* const s_wk = sh.wk;
   const int t = threadIdx.x;
   for (int i = t; i < n_zero; i += blockDim.x) zero_ints[i] = 0;
   if (t == 0) s_total = 0;
@@ -214,4 +308,10 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a) {
       for (int w = n_workers - 1; w >= 0; --w)
         if (worker_first[w] > worker_first[w + 1]) worker_first[w] = worker_first[w + 1];
   }
+}
+
+__device__ __forceinline__ void plan_any(const PlanArgs& a, PlanShared& sh) {
+  if (plan_small_ok(a)) plan_small(a, sh);
+  else if (a.n_workers > 0) plan_balanced(a, sh);
+  else plan_even(a, sh);
 }

@@ -6,8 +6,10 @@
 // the chain of programmatic dependent launches.  Here they are blocks of one grid: block 0 the plan, then
 // the appended tokens, the query RoPE of a head each, and the (head, 128 coordinates, sequences)
 // blocks of the absorption, whose weight slabs are fetched before the dependency wait.
-// From the end of one step's combine to the start of the next step's attention: 7B 75 % B16 16 -> 7 us,
-// ragged B64 21 -> 13; a step of the smallest model (4 heads, host-bound) 51 -> 38 us.
+// From the release of the grid by the previous step's combine to its end: one sequence 2.5 us, 7B 75 % B16
+// 3.7, ragged B64 7.0, 13B B32 5.3, 50 % B32 9.5 (11 to 12 us for the last three while a single warp fetched
+// the weights and registers kept blocks waiting for a second wave; the 50 % shape's 833 blocks still do not
+// all fit).  As separate launches: 16 us at B16, 21 at ragged B64.
 #include "absorb.cuh"
 #include "append.cuh"
 #include "plan.cuh"
@@ -17,15 +19,14 @@ namespace {
 static_assert(kPlanThreads == kAbsorbThreads, "one block size for every part");
 
 template <int MT>
-__global__ void __launch_bounds__(kAbsorbThreads)
+__global__ void __launch_bounds__(kAbsorbThreads, MT == kAbsorbMaxTiles ? 4 : 5)     // what shared memory holds
 step_prep_kernel(const AbsorbArgs q, const AppendArgs t, const PlanArgs p, int n_append, int vec, int slices) {
   extern __shared__ __align__(16) unsigned char smem_b[];
   ekv_pdl_trigger();      // the attention kernel waits for this grid's completion itself
   int blk = blockIdx.x;
   if (blk == 0) {
     ekv_pdl_wait();
-    if (p.n_workers > 0) plan_balanced(p);
-    else plan_even(p);
+    plan_any(p, *(PlanShared*)smem_b);
     return;
   }
   blk -= 1;
@@ -56,9 +57,10 @@ int ekv_launch_step_prep(const elitekv_layer* L, const elitekv_cache* cache, con
   const AppendArgs t = append_args(L, cache, cv, k_e, c, seq_id, pos, B);
   const int n_append = B < L->sm_count ? B : L->sm_count;      // a block per token; more tokens go round
   const int grid = 1 + n_append + L->n_h * (1 + s.slices * s.groups);
+  const size_t smem = s.smem > sizeof(PlanShared) ? s.smem : sizeof(PlanShared);
   auto launch = [&](auto kern) -> int {
-    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
-    EKV_CUDA_OK(ekv_launch_pdl(kern, dim3((unsigned)grid), dim3(kAbsorbThreads), s.smem, st, a, t, plan, n_append,
+    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    EKV_CUDA_OK(ekv_launch_pdl(kern, dim3((unsigned)grid), dim3(kAbsorbThreads), smem, st, a, t, plan, n_append,
                                (int)append_vec_ok(L), s.slices));
     EKV_CUDA_OK(cudaGetLastError());
     return ELITEKV_OK;

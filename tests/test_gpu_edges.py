@@ -241,3 +241,15 @@ def test_combine_rows_sharing_warps(ek, B, n_items):
     w = gen.shrink(gen.LLAMA7B_75, B=B, ctx=128 * n_items)
     st = H.setup(w, lens=([128 * n_items] + [65, 0, 300, 1, 128, 129, 77, 64])[:B], decode_kernel=2)
     H.check_parity(st, H.run_decode(st), H.sample_units(st, 24, seed=n_items))
+
+
+# ------------------------------------------------------------------ work plans
+@pytest.mark.parametrize("B,n_workers", [(255, 148), (256, 1), (256, 3840), (256, 3841), (257, 148)])
+def test_plans_on_both_sides_of_a_sequence_per_thread(ek, B, n_workers):
+    """Up to 256 sequences (and 4096 items) the plan has a thread per sequence, then a thread per item;
+    beyond that a sequence's items are written one after the other.  Both against the rules the
+    plans promise, with empty sequences at both ends of a thread's neighbours."""
+    from . import test_gpu_parity as T
+    lens = [0 if b % 5 in (0, 4) else 1 + (7919 * b) % 9000 for b in range(B)]
+    T.test_worker_plan_structure(ek, lens, 64, n_workers, 2)
+    T.test_plan_partitions_every_sequence(ek, lens, B + 300)
