@@ -15,12 +15,13 @@
 // issues tcgen05.mma (M = 128, N = 128, K = 16, bf16 in, fp32 in TMEM), warps 2-5 run the epilogue.
 // A 128-wide tile lies either in the rope part or in the latent part (both are multiples of 128 wide).
 //
-// A batch of at most 128 tokens (a decode step) has one token tile, so the grid above would be
-// n_out / 128 blocks reading the 2 d n_out bytes of weights between them: 16 blocks for the 7B
-// shape.  Such a call runs as clusters of kSplit = 8 blocks instead, each block taking an eighth
-// of the depth d.  The partial sums leave TMEM, cross distributed shared memory (block i of a
-// cluster collects rows [16 i, 16 i + 16) from all eight) and are added in block order, so the
+// Few tokens make few tiles: a decode step's batch has one token tile, so the grid above would be
+// n_out / 128 blocks reading the 2 d n_out bytes of weights between them, 16 blocks for the 7B
+// shape.  Such a call runs as clusters of 8, 4 or 2 blocks per tile, each block taking its share of
+// the depth d.  The partial sums leave TMEM, cross distributed shared memory (block i of a cluster
+// of s collects rows [128 i / s, 128 (i + 1) / s) from all of them) and are added in block order, so the
 // result does not depend on scheduling; the collecting block rotates, rounds and stores.
+// The weights of the first stages are requested before the dependency wait.
 // Every wait is bounded (timeouts are recorded and the block leaves through the common exit).
 #include "tc_ptx.cuh"
 
@@ -30,9 +31,7 @@ constexpr int kPM = 128, kPN = 128, kPK = 64;     // tile: tokens, output column
 constexpr int kPStages = 4;
 constexpr int kPStageBytes = (kPM + kPN) * kPK * 2;   // 32 KB
 constexpr int kPThreads = 192;
-constexpr int kSplit = 8;                         // blocks per cluster of the split-depth form
-constexpr int kSplitRows = kPM / kSplit;          // token rows each block of a cluster finishes
-constexpr int kRecvBytes = kSplit * kSplitRows * kPN * 4;   // 64 KB: [source block][row][column] fp32
+constexpr int kRecvBytes = kPM * kPN * 4;         // 64 KB: [source block][row][column] fp32, rows of one block
 
 struct ProjArgs {
   const int32_t* seq_id;
@@ -90,10 +89,12 @@ __device__ __forceinline__ long long token_row(const ProjArgs& a, long long t, i
   return row;
 }
 
-template <bool kSplitDepth>
+template <int kSplit>                              // blocks per cluster that share the depth
 __global__ void __launch_bounds__(kPThreads, 1)
 project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                       const ProjArgs a) {
+  constexpr bool kSplitDepth = kSplit > 1;
+  constexpr int kSplitRows = kPM / kSplit;         // token rows each block of a cluster finishes
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   float* s_recv = (float*)(base + kPStages * kPStageBytes);      // split-depth form only
@@ -118,6 +119,7 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
+  ekv_pdl_trigger();      // whatever is launched behind waits for this grid itself
   constexpr uint32_t tmem_cols = 128;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem)), "r"(tmem_cols) : "memory");
@@ -131,18 +133,27 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   if (warp == 0) {
     // ---- operand tiles: x rows [t0, t0+128) and weight rows [n0, n0+128), 64 of d per stage
     //      (rows past T come back as zeros: they are never stored)
+    //      The first stages' weights belong to the layer: requested while earlier kernels still run.
     bool ok = true;
-    for (int k = 0; k < k_hi - k_lo && ok; ++k) {
-      const int s = k % kPStages;
-      ok = warp_wait(smem_u32(&bars->empty[s]), ((k / kPStages) & 1) ^ 1, s_abort, 1);
-      if (!ok) break;
+    const int early = min(k_hi - k_lo, kPStages);
+    auto load = [&](int k, bool w, bool x) {
       if (elect_one()) {
-        const uint32_t fb = smem_u32(&bars->full[s]);
-        mbar_expect_tx(fb, (uint32_t)kPStageBytes);
-        tma_load_2d(smem_u32(base + s * kPStageBytes), &map_x, (k_lo + k) * kPK, (int)t0, fb);
-        tma_load_2d(smem_u32(base + s * kPStageBytes + kPM * kPK * 2), &map_w, (k_lo + k) * kPK, n0, fb);
+        const uint32_t fb = smem_u32(&bars->full[k % kPStages]), dst = smem_u32(base + k % kPStages * kPStageBytes);
+        if (w) {
+          mbar_expect_tx(fb, (uint32_t)kPStageBytes);
+          tma_load_2d(dst + kPM * kPK * 2, &map_w, (k_lo + k) * kPK, n0, fb);
+        }
+        if (x) tma_load_2d(dst, &map_x, (k_lo + k) * kPK, (int)t0, fb);
       }
       __syncwarp();
+    };
+    for (int k = 0; k < early; ++k) load(k, true, false);
+    ekv_pdl_wait();
+    for (int k = 0; k < early; ++k) load(k, false, true);
+    for (int k = early; k < k_hi - k_lo && ok; ++k) {
+      ok = warp_wait(smem_u32(&bars->empty[k % kPStages]), ((k / kPStages) & 1) ^ 1, s_abort, 1);
+      if (!ok) break;
+      load(k, true, true);
     }
   } else if (warp == 1) {
     constexpr uint32_t idesc = make_idesc(kPM, kPN, 0, 0);
@@ -168,6 +179,7 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     __syncwarp();
   } else {
     // ---- epilogue: thread = token row of the tile
+    ekv_pdl_wait();                                        // (tokens, and the cache that earlier kernels read)
     const int quarter = warp & 3;
     const int trow = quarter * 32 + lane;
     const long long t = t0 + trow;
@@ -206,9 +218,10 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     cluster_sync_all();
     if (warp >= 2 && !*s_abort) {
       const int e = threadIdx.x - 64;                    // 128 threads: 16 rows x 8 column groups
-      const int rr = e >> 3, cg = e & 7;
-      const long long t = t0 + crank * kSplitRows + rr;
-      if (t < a.T) {
+      const int cg = e & 7;
+      for (int rr = e >> 3; rr < kSplitRows; rr += 16) {
+        const long long t = t0 + crank * kSplitRows + rr;
+        if (t >= a.T) break;
         int p = 0;
         const long long row = token_row(a, t, &p);
         if (row >= 0) {
@@ -542,34 +555,39 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
     EKV_CUDA_OK(cudaGetLastError());
     return ELITEKV_OK;
   }
-  // at most one token tile and enough depth for every block of a cluster: the split-depth form
-  const bool split = T <= kPM && L->d / kPK >= kSplit;
-  const int smem = kPStages * kPStageBytes + (split ? kRecvBytes : 0) + (int)sizeof(ProjBarriers) + 64 + 1024;
+  // Few tiles: clusters share a tile's depth, as many blocks (8, 4, 2) as let all clusters be resident at
+  // once: 15, 33, 74 clusters of one block per SM (by the occupancy calculator; 16 clusters of eight would
+  // take two waves).  SPLIT_FIGURES
+  const long long tiles = n_out / kPN * ((T + kPM - 1) / kPM);
+  const int split = tiles <= 15 && a.nk >= 8 ? 8 : tiles <= 33 && a.nk >= 4 ? 4 : tiles <= 74 && a.nk >= 2 ? 2 : 1;
+  const int smem = kPStages * kPStageBytes + (split > 1 ? kRecvBytes : 0) + (int)sizeof(ProjBarriers) + 64 + 1024;
   if (smem > L->smem_optin) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
   CUtensorMap m_x, m_w;
   int rc = make_map(&m_x, x, (unsigned long long)T, (unsigned long long)L->d, kPM);
   if (rc == ELITEKV_OK) rc = make_map(&m_w, L->d_WcatT, (unsigned long long)n_out, (unsigned long long)L->d, kPN);
   if (rc != ELITEKV_OK) return rc;
-  if (split) {
-    EKV_CUDA_OK(cudaFuncSetAttribute(project_append_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  auto launch = [&](auto kern) -> int {
+    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n_out / kPN), 1, kSplit);
+    cfg.gridDim = dim3((unsigned)(n_out / kPN), (unsigned)((T + kPM - 1) / kPM), split);
     cfg.blockDim = dim3(kPThreads);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = kSplit;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = split;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    EKV_CUDA_OK(cudaLaunchKernelEx(&cfg, project_append_kernel<true>, m_x, m_w, a));
-  } else {
-    EKV_CUDA_OK(cudaFuncSetAttribute(project_append_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    dim3 grid((unsigned)(n_out / kPN), (unsigned)((T + kPM - 1) / kPM));
-    project_append_kernel<false><<<grid, kPThreads, smem, st>>>(m_x, m_w, a);
-  }
-  EKV_CUDA_OK(cudaGetLastError());
-  return ELITEKV_OK;
+    cfg.numAttrs = 2;
+    EKV_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, m_x, m_w, a));
+    EKV_CUDA_OK(cudaGetLastError());
+    return ELITEKV_OK;
+  };
+  return split == 8   ? launch(project_append_kernel<8>)
+         : split == 4 ? launch(project_append_kernel<4>)
+         : split == 2 ? launch(project_append_kernel<2>)
+                      : launch(project_append_kernel<1>);
 }

@@ -253,3 +253,13 @@ def test_plans_on_both_sides_of_a_sequence_per_thread(ek, B, n_workers):
     lens = [0 if b % 5 in (0, 4) else 1 + (7919 * b) % 9000 for b in range(B)]
     T.test_worker_plan_structure(ek, lens, 64, n_workers, 2)
     T.test_plan_partitions_every_sequence(ek, lens, B + 300)
+
+
+@pytest.mark.parametrize("d", [64, 128, 320, 4096])
+@pytest.mark.parametrize("T", [1, 127, 129, 257, 700])
+def test_project_append_depth_shares(ek, T, d):
+    """7B shape, 16 column tiles: 1, 2, 3 and 6 token tiles run with 4, 4, 2 and 1 blocks per tile where the
+    depth has a step for each; rows a block finishes (32, 64, 128) end inside and at its range."""
+    from .test_gpu_parity import _projection_case
+    w = gen.shrink(gen.LLAMA7B_75, B=1, ctx=T)
+    _projection_case(ek, w, d, [T], False, T + d)
