@@ -10,9 +10,13 @@
 //
 // Prefill-sized calls (thousands of tokens) run the staged form instead: a block moves groups of
 // tokens through a three-stage shared-memory ring with bulk asynchronous copies, one per row
-// (un-rotated rope row and latent row in, cache rows out), so that two groups of loads are in
-// flight behind the group being rotated and stored and no row passes through registers except
+// (un-rotated rope row and latent row in, cache rows out), and no row passes through registers except
 // the rope pairs while they are rotated in place.  Same arithmetic, same bits.
+// Bound: memory, once enough blocks are in flight.  An iteration of a block is a chain (look-ups, loads
+// landing, rotation, stores reading the stage), so many small blocks beat few deep ones, and a stage is
+// filled again two iterations after its stores were issued and not right behind them.  131072 tokens of
+// the 7B shape (1.07 GB): 2 blocks per SM with 32 KB stages refilled at once 199 us, 4 blocks with 16 KB
+// stages 173 (170 before the power cap; 0.96 of the measured copy rate), 6 with 12 KB 235.
 #include "append.cuh"
 #include "tc_ptx.cuh"
 
@@ -26,7 +30,10 @@ append_kernel(const AppendArgs a) {
 
 // ------------------------------------------------------------------ staged form (prefill)
 constexpr int kStages = 3;
-constexpr int kStageBudget = 32 * 1024;   // bytes of token rows per stage
+constexpr int kLag = 1;                   // iterations between a group's loads and its stores
+constexpr int kStageBytes = 16 * 1024;    // token rows per stage (a longer row: one token)
+constexpr int kMaxRow = 32 * 1024;        // longest token row
+constexpr int kBlocksPerSm = 4;
 constexpr int kMaxGroup = 16;             // tokens per stage at most
 constexpr int kStagedThreads = 128;
 
@@ -44,9 +51,9 @@ __device__ __forceinline__ void bulk_store_row(void* dst, uint32_t src, uint32_t
 
 // Tokens per group G; group g of the call = tokens [g G, g G + G).  Block b takes groups b,
 // b + gridDim.x, ...  In iteration `it` lane l < G of warp 0 issues the loads of its token of the
-// block's it-th group, and the whole block rotates and stores the group loaded kStages - 1
-// iterations earlier.  A stage is loaded again one iteration after its stores were issued; the
-// issuing lane first waits until those stores have read the stage.
+// block's it-th group, and the whole block rotates and stores the group loaded kLag
+// iterations earlier.  A stage is loaded again kStages - kLag iterations after its stores were issued;
+// the issuing lane first waits until those stores have read the stage.
 __global__ void __launch_bounds__(kStagedThreads)
 append_staged_kernel(const AppendArgs a, int G) {
   extern __shared__ __align__(128) unsigned char smem_stage[];
@@ -69,11 +76,11 @@ append_staged_kernel(const AppendArgs a, int G) {
   __syncthreads();
   const long long n_groups = (a.T + G - 1) / G;
   const long long mine = blockIdx.x < n_groups ? (n_groups - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  for (long long it = 0; it < mine + kStages - 1; ++it) {
+  for (long long it = 0; it < mine + kLag; ++it) {
     // ---- loads of the block's it-th group (warp 0, one lane per token)
     if (warp == 0 && lane < G && it < mine && !*s_abort) {
       const int st = (int)(it % kStages);
-      bulk_wait_group_read<0>();        // this lane's stores out of the stage (previous iteration) have read it
+      bulk_wait_group_read<kStages - kLag - 1>();        // this lane's stores out of the stage have read it
       const long long t = (blockIdx.x + it * gridDim.x) * G + lane;
       long long row = -1;
       int p = 0;
@@ -100,8 +107,8 @@ append_staged_kernel(const AppendArgs a, int G) {
         mbar_arrive(fb);
       }
     }
-    // ---- the group loaded kStages - 1 iterations ago: rotate in place, store
-    const long long gp = it - (kStages - 1);
+    // ---- the group loaded kLag iterations ago: rotate in place, store
+    const long long gp = it - kLag;
     if (gp >= 0) {
       const int st = (int)(gp % kStages);
       const bool ok = mbar_wait(smem_u32(&bars.full[st]), (uint32_t)((gp / kStages) & 1), s_abort, 1);
@@ -173,12 +180,12 @@ int ekv_launch_append(const elitekv_layer* L, const elitekv_cache* cache, const 
   // prefill-sized calls: the staged form (rows are whole 16-byte units, and the buffers are
   // 16-byte aligned: checked at the entry point)
   const long long tok_bytes = (long long)L->n_h * L->r * 4 + (long long)L->d_c * 2;
-  if (T >= 2048 && (L->n_h * L->r) % 4 == 0 && tok_bytes <= kStageBudget) {
-    int G = (int)(kStageBudget / tok_bytes);
+  if (T >= 2048 && (L->n_h * L->r) % 4 == 0 && tok_bytes <= kMaxRow) {
+    int G = tok_bytes < kStageBytes ? (int)(kStageBytes / tok_bytes) : 1;
     if (G > kMaxGroup) G = kMaxGroup;
     const size_t smem = (size_t)kStages * G * tok_bytes;
     const long long n_groups = (T + G - 1) / G;
-    const long long want = (long long)L->sm_count * 2;       // two blocks of ~100 KB per SM
+    const long long want = (long long)L->sm_count * kBlocksPerSm;
     EKV_CUDA_OK(cudaFuncSetAttribute(append_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     append_staged_kernel<<<(unsigned)(n_groups < want ? n_groups : want), kStagedThreads, smem, st>>>(a, G);
     EKV_CUDA_OK(cudaGetLastError());

@@ -263,3 +263,24 @@ def test_project_append_depth_shares(ek, T, d):
     from .test_gpu_parity import _projection_case
     w = gen.shrink(gen.LLAMA7B_75, B=1, ctx=T)
     _projection_case(ek, w, d, [T], False, T + d)
+
+
+# ------------------------------------------------------------------ append, staged form
+@pytest.mark.parametrize("T", [2047, 2048, 2049, 4 * 148 * 4 * 2 + 3])
+@pytest.mark.parametrize("shape", [dict(), dict(n_h=4, r=2, d_c=64), dict(r=48, d_c=3072)])
+def test_append_staged_groups(ek, shape, T):
+    """The staged form starts at 2048 tokens; groups of 4 tokens (7B rows), of 16 (the most) and of one
+    (12 KB rows); a ragged last group, and more groups than one round of the grid.  Latent rows are
+    copied bit for bit; the rotation is the register form's, bit for bit."""
+    w = gen.shrink(replace(gen.LLAMA7B_75, **shape), B=1, ctx=T)
+    st = H.setup(w, lens=[T], fill=False)
+    perm = torch.randperm(T, generator=torch.Generator().manual_seed(T)).cuda()
+    args = [x[perm].contiguous() for x in (st.k_e, st.c, st.seq_id, st.pos)]
+    ek.elitekv_append(st.layer, st.cache, *args)
+    rope, latent = st.rope_plane.clone(), st.latent_plane.clone()
+    st.rope_plane.zero_()
+    for a in range(0, T, 1000):
+        ek.elitekv_append(st.layer, st.cache, *[x[a:a + 1000].contiguous() for x in args])
+    assert ek.elitekv_check_status(st.layer) == 0
+    assert torch.equal(rope, st.rope_plane)
+    assert torch.equal(latent[st.pos.long()].view(torch.int16), st.c.view(torch.int16).view(T, -1))
