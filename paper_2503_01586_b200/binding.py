@@ -122,7 +122,20 @@ def _dev(t: torch.Tensor, dtype) -> torch.Tensor:
     return t
 
 
+def _in(t: torch.Tensor, dtype) -> int:
+    """_ptr(_dev(t, dtype)) in one check."""
+    assert t.is_cuda and t.dtype == dtype and t.is_contiguous(), (t.device, t.dtype)
+    return t.data_ptr()
+
+
+# handle of the current stream: the raw look-up costs 0.4 us a call, a Stream object 3.3 us of the 16 us
+# that the host needs for a decode step
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
     return torch.cuda.current_stream().cuda_stream
 
 
@@ -235,12 +248,11 @@ def elitekv_decode_step(layer: Layer, cache: CacheDesc, k_e, c, seq_id, pos, q, 
     """Append + query preparation + decode attention of one step in one call (buffers are the
     caller's: nothing is allocated here)."""
     B = q.shape[0]
-    _check(lib().elitekv_decode_step(layer.handle, C.byref(cache), _ptr(k_e), _ptr(_dev(c, torch.bfloat16)),
-                                     _ptr(_dev(seq_id, torch.int32)), _ptr(_dev(pos, torch.int32)),
-                                     _ptr(_dev(q, torch.bfloat16)), _ptr(_dev(seq_lens, torch.int32)), B,
-                                     _ptr(q_rope), _ptr(_dev(q_abs, torch.bfloat16)), workspace.data_ptr(),
-                                     workspace.numel() * workspace.element_size(),
-                                     _ptr(_dev(out, torch.bfloat16)), _stream()), "elitekv_decode_step")
+    bf16, i32 = torch.bfloat16, torch.int32
+    _check(lib().elitekv_decode_step(layer.handle, C.byref(cache), _ptr(k_e), _in(c, bf16), _in(seq_id, i32), _in(pos, i32),
+                                     _in(q, bf16), _in(seq_lens, i32), B, _ptr(q_rope), _in(q_abs, bf16),
+                                     workspace.data_ptr(), workspace.numel() * workspace.element_size(), _in(out, bf16),
+                                     _stream()), "elitekv_decode_step")
     return out
 
 

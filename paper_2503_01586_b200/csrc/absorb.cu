@@ -45,7 +45,7 @@ int ekv_launch_absorb(const elitekv_layer* L, const void* q, const int32_t* q_po
   const AbsorbArgs a = absorb_args(L, q, q_pos, B, q_rope, q_abs);
   const dim3 grid(L->n_h, s.slices + 1, s.groups);
   auto launch = [&](auto kern) -> int {
-    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
+    EKV_CUDA_OK(ekv_allow_smem(kern, s.smem));
     EKV_CUDA_OK(ekv_launch_pdl(kern, grid, dim3(kAbsorbThreads), s.smem, st, a));
     EKV_CUDA_OK(cudaGetLastError());
     return ELITEKV_OK;

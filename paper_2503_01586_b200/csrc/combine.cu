@@ -374,8 +374,7 @@ int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, v
   const int kgroups = kCombThreads / npair > 0 ? kCombThreads / npair : 1;
   const size_t smem = sizeof(float) * (size_t)kgroups * kCombBatch * L->d_h;
   dim3 grid(nv, (B + kCombBatch - 1) / kCombBatch);
-  EKV_CUDA_OK(cudaFuncSetAttribute(combine_upproj_kernel,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EKV_CUDA_OK(ekv_allow_smem(combine_upproj_kernel, smem));
   EKV_CUDA_OK(ekv_launch_pdl(combine_upproj_kernel, grid, dim3(kCombThreads), smem, st, (const float*)ws.part_acc,
                              (const float*)ws.part_ml, (const int32_t*)ws.seq_first, (const bf16*)L->d_Wuv, (bf16*)out, B,
                              nv, L->n_h, L->d_h, L->vw));

@@ -101,6 +101,13 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, const bf16* p) {
 __device__ __forceinline__ void ekv_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void ekv_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Leave for more dynamic shared memory than every kernel has anyway (48 KB with its static part: asked
+// for from 32 KB on; the call costs the host about half a microsecond).
+template <typename... KArgs>
+inline cudaError_t ekv_allow_smem(void (*kern)(KArgs...), size_t bytes) {
+  return bytes > 32 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t ekv_launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                   Args... args) {

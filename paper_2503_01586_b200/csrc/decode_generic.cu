@@ -247,8 +247,7 @@ int pick_sub_tokens(const elitekv_layer* L) {
 
 template <int NCH>
 int launch_nch(const elitekv_layer* L, const GenericArgs& a, dim3 grid, size_t smem, cudaStream_t st) {
-  EKV_CUDA_OK(cudaFuncSetAttribute(decode_generic_kernel<NCH>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EKV_CUDA_OK(ekv_allow_smem(decode_generic_kernel<NCH>, smem));
   EKV_CUDA_OK(ekv_launch_pdl(decode_generic_kernel<NCH>, grid, dim3(kThreads), smem, st, a));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;

@@ -59,7 +59,7 @@ int ekv_launch_step_prep(const elitekv_layer* L, const elitekv_cache* cache, con
   const int grid = 1 + n_append + L->n_h * (1 + s.slices * s.groups);
   const size_t smem = s.smem > sizeof(PlanShared) ? s.smem : sizeof(PlanShared);
   auto launch = [&](auto kern) -> int {
-    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    EKV_CUDA_OK(ekv_allow_smem(kern, smem));
     EKV_CUDA_OK(ekv_launch_pdl(kern, dim3((unsigned)grid), dim3(kAbsorbThreads), smem, st, a, t, plan, n_append,
                                (int)append_vec_ok(L), s.slices));
     EKV_CUDA_OK(cudaGetLastError());
