@@ -3,7 +3,7 @@
 
 One step = one pass of the whole decode hot path for one layer over a batch of sequences:
     elitekv_append (1 new token per sequence) | elitekv_absorb_query -> elitekv_decode
-(the append and the query preparation are independent and run on two streams).
+(append, work plan and query preparation are blocks of one kernel).
 Metric: decode-attention tokens/s (= sequences advanced per second for one layer), plus the
 achieved cache-read bandwidth.  Workload at one GPU: LLaMA2-7B-shaped layer, 75 % KV reduction
 (r = 8 elite chunks/head, d_c = 1536), batch 16, context 4096, contiguous cache, bf16,
@@ -157,7 +157,7 @@ def config_of(w: gen.Workload, world: int):
          "batch_per_gpu": w.B, "context": w.ctx, "paged": w.paged,
          "l2": "256 MiB flush write before every timed step; cache larger than L2",
          "parallelism": f"replicas x{world} (independent sequences, no collective)",
-         "streams": "elitekv_decode_step: append + plan on the layer's second stream beside absorb_query; joined before the attention kernel"}
+         "streams": "one: elitekv_decode_step launches three kernels (append + plan + query preparation, attention, combine), each dependent on the one before"}
     return c
 
 
@@ -263,13 +263,13 @@ def build_workload(w: gen.Workload, ek, device, decode_kernel: int = 0):
 
 
 def step(ek, layer, cache, d, ws, bufs):
-    """One decode step through the library's single-call entry: the append and the work plan run
-    on the layer's second stream beside the query preparation, joined before the attention."""
+    """One decode step through the library's single-call entry: append, work plan and query
+    preparation in one kernel, then the attention and the combine."""
     ek.elitekv_decode_step(layer, cache, d["k_e"], d["c"], d["seq_id"], d["pos"], d["q"], d["lens"],
                            bufs["q_rope"], bufs["q_abs"], ws, bufs["out"])
 
 
-KERNELS_PER_STEP = 5   # append, absorb, plan, split-K attention, combine + up-projection
+KERNELS_PER_STEP = 3   # append + plan + query preparation, split-K attention, combine + up-projection
 
 SWEEP = ["7b-75pct-paged-b64-ragged", "13b-75pct-b32-ctx16384", "7b-50pct-b32-ctx8192",
          "7b-75pct-b32-ctx8192", "7b-87.5pct-b32-ctx8192", "7b-75pct-slrd512+1024-b32-ctx8192"]
