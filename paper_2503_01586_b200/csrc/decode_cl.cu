@@ -42,12 +42,13 @@
 // Every wait is bounded; on a timeout the block records ELITEKV_ERR_TIMEOUT, stops issuing work
 // and leaves through the common exit (its peers then run into their own limit).
 //
-// Measured (kernel time; cache bytes over it; before: the resident-tile or two-pass kernel): 7B 75 %
-// 16 x 4096 59 us, 4.6 TB/s (71 us); ragged 64 x [1024, 32768] 832 us, 5.6 TB/s (901); 13B 32 x 16384
-// 560 us, 4.8 TB/s on 130 of 148 SMs (769); 50 % 32 x 8192 480 us, 4.5 TB/s on 120 SMs (526);
-// 87.5 % 105 us, 5.1 TB/s (120); S-LRD 168 us, 6.4 TB/s (179).  Back to back the long ones run at
-// the board's power limit (clock 1.75-1.9 GHz), so bytes moved twice and products computed for
-// padding cost time even where they would fit beside the loads.
+// Measured (CUDA events around the kernel, L2 flushed before each step; in brackets the kernel that the
+// shape had before): 7B 75 % 16 x 4096 68 us, 3.9 TB/s (78 us, resident tiles on block pairs); ragged
+// 64 x [1024, 32768] 840 us, 5.5 TB/s (881, two passes); 13B 32 x 16384 566 us, 4.7 TB/s on 130 of 148
+// SMs (773); 50 % 32 x 8192 492 us, 4.4 TB/s on 120 SMs (529); 75 % 32 x 8192 212 us, 5.1 TB/s (237);
+// 87.5 % 107 us, 5.0 TB/s (130); S-LRD 184 us, 5.8 TB/s (199).  DRAM traffic 1.01 of the cache bytes.
+// Back to back the long ones run at the board's power limit (clock 1.75-1.9 GHz), so bytes moved
+// twice and products computed for padding cost time even where they would fit beside the loads.
 #include <map>
 #include <mutex>
 #include <tuple>
