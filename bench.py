@@ -750,7 +750,7 @@ def run_gpu(args, w: gen.Workload):
 # dram__bytes_read.sum + dram__bytes_write.sum of one split-K launch on the named workload, from an
 # ncu capture of the kernel that serves it (None where no capture of the current kernel exists).
 TRAFFIC_BYTES_PER_LAUNCH = {
-    "7b-75pct-b16-ctx4096": 270263040 + 4182528,     # resident-tile kernel, one launch
+    "7b-75pct-b16-ctx4096": 270101504 + 707584,     # cluster-resident kernel, one launch
 }
 
 
