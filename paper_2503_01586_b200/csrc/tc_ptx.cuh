@@ -143,11 +143,6 @@ __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
       ::"r"(dst), "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy) : "memory");
 }
-__device__ __forceinline__ uint64_t make_l2_policy_evict_normal() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
 __device__ __forceinline__ uint64_t make_l2_policy_evict_last() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
@@ -170,23 +165,11 @@ template <int kPending>
 __device__ __forceinline__ void bulk_wait_group_read() {
   asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kPending) : "memory");
 }
-// L2 prefetch of one tensor-map box: no shared memory, no barrier
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-               ::"l"((uint64_t)map), "r"(x), "r"(y) : "memory");
-}
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // Same with the descriptors given as 32-bit halves: the high words (stride offset, version,
 // swizzle mode) are constants and the low words (address, leading offset) advance by small
@@ -284,18 +267,8 @@ __device__ __forceinline__ void named_bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// Shared-memory matrix descriptor of tcgen05.mma: start address, leading / stride byte offsets
-// (each >> 4), descriptor version 1, swizzle mode in the top bits (2 = 128-byte, 0 = none).
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes, uint32_t layout) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFF) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)layout << 61;
-  return d;
-}
-// The two 32-bit halves of the same descriptor.
+// Shared-memory matrix descriptor of tcgen05.mma, as two 32-bit halves: start address, leading / stride
+// byte offsets (each >> 4), descriptor version 1, swizzle mode in the top bits (2 = 128-byte, 0 = none).
 __host__ __device__ constexpr uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
   return ((saddr >> 4) & 0x3FFF) | (((lbo_bytes >> 4) & 0x3FFF) << 16);
 }
@@ -387,19 +360,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   }
   if (*abort_flag == 0) *abort_flag = why;
   return false;
-}
-// mbar_wait_group for a barrier the peer block arrives on: same protocol, with the acquire of
-// every thread taken at cluster scope so that the peer's stores are visible afterwards.
-__device__ __forceinline__ bool mbar_wait_group_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                                        volatile int* verdict, unsigned& turn, bool leader, int id,
-                                                        int n, int why, unsigned limit = kSpinLimit) {
-  volatile int* word = verdict + (turn & 1u);
-  ++turn;
-  if (leader) *word = mbar_spin(bar, parity, abort_flag, why, limit) ? 1 : 0;
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-  const bool ok = *word != 0;
-  if (ok) (void)mbar_try_wait_cluster(bar, parity);
-  return ok;
 }
 
 // ---------------------------------------------------------------- host side
