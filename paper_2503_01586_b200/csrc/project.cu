@@ -277,8 +277,11 @@ constexpr int kUnits = 14;
 constexpr int kUnitBytes = 128 * kPK * 2;                 // 16 KB
 constexpr int kBThreads = 320;           // warp 0 loads, warp 1 MMA (first block), warps 2-9 epilogue
 
+constexpr int kCsUnits = 8;              // units that take table rows for the epilogue, one per epilogue warp
+
 struct __align__(8) PairBarriers {
   uint64_t full[kUnits], empty[kUnits], done;      // full: of the first block only, for both blocks' units
+  uint64_t last[kCsUnits];                         // the last product of such a unit is done: one phase only
 };
 
 // Epilogue buffers lie in the operand ring, in the units read last.  Per warp of 32 tokens: the tokens'
@@ -286,7 +289,7 @@ struct __align__(8) PairBarriers {
 // tokens are on different banks), which starts to fill as soon as that unit's last product is done;
 // and 128 finished columns of the 32 cache rows in half a unit (16-byte pieces XORed with the row).
 constexpr int kCsHalf = 64;              // table rows of up to 64 chunks
-static_assert(32 * kCsHalf * 8 == kUnitBytes && 2 * 32 * 256 == kUnitBytes && 8 + 4 <= kUnits, "epilogue buffers fit");
+static_assert(32 * kCsHalf * 8 == kUnitBytes && 2 * 32 * 256 == kUnitBytes && kCsUnits + 4 <= kUnits, "epilogue buffers fit");
 
 template <int H>
 __global__ void __launch_bounds__(kBThreads, 1)
@@ -310,6 +313,7 @@ project_append_pair_kernel(const __grid_constant__ CUtensorMap map_t, const __gr
       mbar_init(smem_u32(&bars->empty[i]), 1);
     }
     mbar_init(smem_u32(&bars->done), 1);
+    for (int i = 0; i < kCsUnits; ++i) mbar_init(smem_u32(&bars->last[i]), 1);
     *s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
@@ -359,6 +363,7 @@ project_append_pair_kernel(const __grid_constant__ CUtensorMap map_t, const __gr
     bool ok = true;
     int slot = 0;
     uint32_t turn = 0;
+    int left = (H + 1) * a.nk;             // units still to come, the current one included
     for (int k = 0; k < a.nk && ok; ++k) {
       uint32_t lb = 0;
       int slot_w = 0;
@@ -378,10 +383,16 @@ project_append_pair_kernel(const __grid_constant__ CUtensorMap map_t, const __gr
               tc_mma_pair(tmem_base + (u - 1) * kBN, lo + 2 * ks, hi_sw, lb + 2 * ks, hi_sw, idesc, (k | ks) != 0);
             tc_commit_pair(smem_u32(&bars->empty[slot]));                // frees the unit in both blocks
             if (u == H) tc_commit_pair(smem_u32(&bars->empty[slot_w]));
+            // the ring's last turn: the epilogue's units are told apart by barriers of their own (the
+            // epilogue warps do not hold the ring back, so a phase of `empty` could pass them by)
+            const int i = kUnits - left;
+            if (i >= 0 && i < kCsUnits) tc_commit_pair(smem_u32(&bars->last[i]));
+            if (u == H && i >= H && i - H < kCsUnits) tc_commit_pair(smem_u32(&bars->last[i - H]));
           }
           __syncwarp();
         }
         if (++slot == kUnits) { slot = 0; turn ^= 1; }
+        --left;
       }
     }
     if (ok && elect_one()) tc_commit_pair(smem_u32(&bars->done));
@@ -403,8 +414,7 @@ project_append_pair_kernel(const __grid_constant__ CUtensorMap map_t, const __gr
     if (n0 + part0 * 128 < a.rope_w && staged) {
       // the 32 tokens' table rows, a whole row per request: a look-up by every token on its own would
       // touch 32 rows per request (33 k clocks for a tile of rope columns)
-      for (int f = 0; ok && f <= (first + w8) / kUnits; ++f)
-        ok = warp_wait(smem_u32(&bars->empty[(first + w8) % kUnits]), f & 1, s_abort, 4);
+      ok = warp_wait(smem_u32(&bars->last[w8]), 0, s_abort, 4);
       if (ok) {
 #pragma unroll 16
         for (int k = 0; k < 32; ++k) {

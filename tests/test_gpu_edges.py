@@ -284,3 +284,34 @@ def test_append_staged_groups(ek, shape, T):
     assert ek.elitekv_check_status(st.layer) == 0
     assert torch.equal(rope, st.rope_plane)
     assert torch.equal(latent[st.pos.long()].view(torch.int16), st.c.view(torch.int16).view(T, -1))
+
+
+@pytest.mark.parametrize("T", [1153, 2305, 4096])
+def test_project_append_paired_forms_with_late_epilogue_warps(ek, T):
+    """40 of 41 tokens have a position outside the cache: every thread that meets one records it with
+    atomics on one word, so the epilogue warps of the paired forms come to their shared-memory units long
+    after the ring has gone round.  The faults are reported as such (no wait runs out), the other tokens'
+    rows are written and no other row is touched."""
+    d, w = 4096, gen.LLAMA7B_75
+    g = torch.Generator().manual_seed(T)
+    rope_w = w.n_h * 2 * w.r
+    W_ke, W_down = ((torch.randn(d, n, generator=g) / 64).to(torch.bfloat16).cuda() for n in (rope_w, w.d_c))
+    idx = gen.elite_index_sets(w)
+    layer = ek.Layer(w.n_h, w.d_h, w.r, w.d_c, idx, *gen.up_projections(w, "cuda"), T, W_ke=W_ke, W_down=W_down)
+    rope, latent = (torch.zeros((T, n), dtype=torch.bfloat16, device="cuda") for n in (rope_w, w.d_c))
+    cache = ek.make_cache(rope, latent, n_seqs=1, max_ctx=T)
+    x = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()
+    seq, pos = torch.zeros(T, dtype=torch.int32), torch.arange(T, dtype=torch.int32)
+    good = pos % 41 == 7
+    pos[~good] += T
+    ek.elitekv_project_append(layer, cache, x, seq.cuda(), pos.cuda())
+    assert ek.elitekv_check_status(layer) == ek.ERR_BAD_POSITION
+    assert ek.elitekv_check_status(layer) == 0
+    assert not rope[~good.cuda()].any() and not latent[~good.cuda()].any()
+    zeros = [np.zeros((T, n), dtype=np.uint16) for n in (rope_w, w.d_c)]
+    _, _, rows64, c64 = O.project_append_expected(*zeros, H.f64(x[good.cuda()]), H.f64(W_ke), H.f64(W_down), seq[good].numpy(),
+                                                  pos[good].numpy(), idx.numpy(), w.d_h, base=w.rope_base, max_ctx=T,
+                                                  page_table=None, page_size=w.page_size)
+    for got, want in ((rope, rows64), (latent, c64)):
+        # as for the other projections: one bf16 rounding plus fp32 accumulation over d terms
+        assert np.all(np.abs(H.f64(got[good.cuda()]) - want) <= np.abs(want) * 2.0 ** -8 + 2e-5 * d ** 0.5)
