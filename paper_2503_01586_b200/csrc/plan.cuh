@@ -9,26 +9,29 @@ constexpr int kPlanStage = 4096;       // items whose worker ids are staged in s
 
 struct __align__(16) PlanShared {        // the block's shared memory
   long long total;
-  int warp_tot[kPlanThreads / 32];
-  int first[kPlanThreads], g0[kPlanThreads], len[kPlanThreads], tiles[kPlanThreads];
+  long long warp_tot[kPlanThreads / 32];
+  long long g0[kPlanThreads];
+  int first[kPlanThreads], len[kPlanThreads], tiles[kPlanThreads];
   short w0[kPlanThreads], wk[kPlanStage];    // wk: worker of each item (n_workers < 32768)
 };
 
-// exclusive scan over the block (warp shuffles + one shared array of warp totals)
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* total) {
+// exclusive scan over the block (warp shuffles + one shared array of warp totals); tiles are summed in
+// 64 bits: lengths of up to 2^31 - 1 tokens in tiles of one pass 2^31 with two sequences
+template <class T>
+__device__ __forceinline__ T block_exclusive_scan(T v, long long* warp_tot, T* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = v;
+  T incl = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+    const T x = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += x;
   }
   if (lane == 31) warp_tot[warp] = incl;
   __syncthreads();
-  int before = 0, all = 0;
+  T before = 0, all = 0;
 #pragma unroll
   for (int w = 0; w < kPlanThreads / 32; ++w) {
-    const int t = warp_tot[w];
+    const T t = (T)warp_tot[w];
     if (w < warp) before += t;
     all += t;
   }
@@ -78,17 +81,18 @@ __device__ __forceinline__ bool plan_small_ok(const PlanArgs& a) {
   return a.B <= kPlanThreads && a.n_workers + a.B <= kPlanStage;
 }
 __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
-  int* const warp_tot = sh.warp_tot;
-  int *const s_first = sh.first, *const s_g0 = sh.g0, *const s_len = sh.len, *const s_tiles = sh.tiles;
+  long long *const warp_tot = sh.warp_tot, *const s_g0 = sh.g0;
+  int *const s_first = sh.first, *const s_len = sh.len, *const s_tiles = sh.tiles;
   short *const s_w0 = sh.w0, *const s_wk = sh.wk;
   const int t = threadIdx.x, B = a.B;
   const bool balanced = a.n_workers > 0;
   const int overhead = balanced ? a.overhead : 0;      // empty tiles in front of every sequence
   const int n = t < B ? checked_len(a.seq_lens, t, a.max_len, a.status, true) : 0;
   for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
-  const int tiles = n > 0 ? (int)plan_div((long long)n + a.tile - 1, a.tile) + overhead : 0;
-  int sum;
-  const int g0 = block_exclusive_scan(tiles, warp_tot, &sum);
+  const int real = n > 0 ? (int)plan_div((long long)n + a.tile - 1, a.tile) : 0;
+  const long long tiles = real > 0 ? (long long)real + overhead : 0;
+  long long sum;
+  const long long g0 = block_exclusive_scan(tiles, warp_tot, &sum);
   const long long total = sum > 0 ? sum : 1;
   const long long nw = balanced ? (total < a.n_workers ? total : a.n_workers) : 1;
   auto bound = [&](long long w) -> long long { return plan_div(w * total, nw); };
@@ -97,7 +101,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
   if (tiles > 0) {
     if (balanced) {
       w0 = owner(g0 + overhead);
-      pieces = owner((long long)g0 + tiles - 1) - w0 + 1;
+      pieces = owner(g0 + tiles - 1) - w0 + 1;
     } else {
       const long long budget = a.max_items - B > 0 ? a.max_items - B : 1;
       const long long target = plan_div(total + budget - 1, budget);
@@ -108,7 +112,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
   const int first = block_exclusive_scan(pieces, warp_tot, &n_items);
   if (t < B) {
     a.seq_first[t] = first;
-    s_first[t] = first; s_g0[t] = g0; s_len[t] = n; s_tiles[t] = tiles; s_w0[t] = (short)w0;
+    s_first[t] = first; s_g0[t] = g0; s_len[t] = n; s_tiles[t] = real; s_w0[t] = (short)w0;
   }
   if (t == 0) a.seq_first[B] = n_items;
   __syncthreads();
@@ -123,10 +127,10 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
       const int j = it - s_first[lo], len = s_len[lo], tl = s_tiles[lo];
       int ta, tb, w = 0;                     // tiles of the sequence
       if (balanced) {
-        const long long base = (long long)s_g0[lo] + overhead;
+        const long long base = s_g0[lo] + overhead;
         w = s_w0[lo] + j;
         ta = (int)(max(base, bound(w)) - base);
-        tb = (int)(min((long long)s_g0[lo] + tl, bound(w + 1)) - base);
+        tb = (int)(min(base + tl, bound(w + 1)) - base);
         s_wk[it] = (short)w;
       } else {
         const int np = (lo + 1 < B ? s_first[lo + 1] : n_items) - s_first[lo];
@@ -134,7 +138,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
         tb = (int)plan_div((long long)tl * (j + 1), np);
       }
       const int tok0 = ta * a.tile;
-      item = make_int4(lo, tok0, min(tb * a.tile, len) - tok0, w);
+      item = make_int4(lo, tok0, (int)min((long long)tb * a.tile, (long long)len) - tok0, w);
     }
     *(int4*)(a.items + 4 * it) = item;
   }
@@ -159,7 +163,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
   int32_t* __restrict__ zero_ints = a.zero_ints;
   const long long max_len = a.max_len;
   int32_t* status = a.status;
-  int* const warp_tot = sh.warp_tot;
+  long long* const warp_tot = sh.warp_tot;
   long long& s_total = sh.total;
   const int t = threadIdx.x;
   for (int i = t; i < n_zero; i += blockDim.x) zero_ints[i] = 0;
@@ -168,7 +172,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
   long long local = 0;
   for (int b = t; b < B; b += blockDim.x) {
     int n = checked_len(seq_lens, b, max_len, status, true);
-    local += n > 0 ? (n + tile - 1) / tile : 0;
+    local += n > 0 ? plan_div((long long)n + tile - 1, tile) : 0;
   }
   if (local) atomicAdd((unsigned long long*)&s_total, (unsigned long long)local);
   __syncthreads();
@@ -183,7 +187,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
     int n = 0, tiles = 0, pieces = 0;
     if (b < B) {
       n = checked_len(seq_lens, b, max_len, status, false);
-      tiles = n > 0 ? (n + tile - 1) / tile : 0;
+      tiles = n > 0 ? (int)plan_div((long long)n + tile - 1, tile) : 0;
       pieces = (int)((tiles + target - 1) / target);
     }
     int chunk_total;
@@ -194,7 +198,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
         const int ta = (int)((long long)tiles * j / pieces);
         const int tb = (int)((long long)tiles * (j + 1) / pieces);
         const int tok0 = ta * tile;
-        const int tok1 = min(tb * tile, n);
+        const int tok1 = (int)min((long long)tb * tile, (long long)n);
         const int it = first + j;
         if (it < max_items) *(int4*)(items + 4 * it) = make_int4(b, tok0, tok1 - tok0, 0);
       }
@@ -224,7 +228,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
   int32_t* __restrict__ zero_ints = a.zero_ints;
   const long long max_len = a.max_len;
   int32_t* status = a.status;
-  int* const warp_tot = sh.warp_tot;
+  long long* const warp_tot = sh.warp_tot;
   long long& s_total = sh.total;
   short* const s_wk = sh.wk;
   const int t = threadIdx.x;
@@ -234,7 +238,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
   long long local = 0;
   for (int b = t; b < B; b += blockDim.x) {
     int n = checked_len(seq_lens, b, max_len, status, true);
-    local += n > 0 ? (n + tile - 1) / tile + overhead : 0;
+    local += n > 0 ? plan_div((long long)n + tile - 1, tile) + overhead : 0;
   }
   if (local) atomicAdd((unsigned long long*)&s_total, (unsigned long long)local);
   __syncthreads();
@@ -244,17 +248,19 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
   const long long nw = total < n_workers ? total : n_workers;
   auto bound = [&](long long w) -> long long { return w * total / nw; };
   auto owner = [&](long long g) -> int { return (int)(((g + 1) * nw - 1) / total); };
-  int carry_tiles = 0, carry_items = 0;
+  long long carry_tiles = 0;
+  int carry_items = 0;
   {
     for (int b0 = 0; b0 < B; b0 += blockDim.x) {
       const int b = b0 + t;
-      int n = 0, tiles = 0;
+      int n = 0;
+      long long tiles = 0;
       if (b < B) {
         n = checked_len(seq_lens, b, max_len, status, false);
-        tiles = n > 0 ? (n + tile - 1) / tile + overhead : 0;     // with the empty tiles in front
+        tiles = n > 0 ? plan_div((long long)n + tile - 1, tile) + overhead : 0;     // with the empty tiles in front
       }
-      int chunk_tiles;
-      const int g0 = carry_tiles + block_exclusive_scan(tiles, warp_tot, &chunk_tiles);
+      long long chunk_tiles;
+      const long long g0 = carry_tiles + block_exclusive_scan(tiles, warp_tot, &chunk_tiles);
       int pieces = 0, w0 = 0;
       if (tiles > 0) {
         w0 = owner(g0 + overhead);                                // workers that hold real tiles
@@ -266,10 +272,10 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
       if (b < B) {
         seq_first[b] = first;
         for (int j = 0; j < pieces; ++j) {
-          const long long ga = max((long long)g0 + overhead, bound(w0 + j));
-          const long long gb = min((long long)g0 + tiles, bound(w0 + j + 1));
+          const long long ga = max(g0 + overhead, bound(w0 + j));
+          const long long gb = min(g0 + tiles, bound(w0 + j + 1));
           const int tok0 = (int)(ga - g0 - overhead) * tile;
-          const int tok1 = min((int)(gb - g0 - overhead) * tile, n);
+          const int tok1 = (int)min((gb - g0 - overhead) * tile, (long long)n);
           const int it = first + j;
           if (it < max_items) *(int4*)(items + 4 * it) = make_int4(b, tok0, tok1 - tok0, w0 + j);
           if (it < kPlanStage) s_wk[it] = (short)(w0 + j);

@@ -255,6 +255,44 @@ def test_plans_on_both_sides_of_a_sequence_per_thread(ek, B, n_workers):
     T.test_plan_partitions_every_sequence(ek, lens, B + 300)
 
 
+MOST = 2 ** 31 - 1
+
+
+@pytest.mark.parametrize("lens,tile", [([MOST] * 3, 1), ([MOST - 5, 0, 7, MOST], 1), ([MOST] * 256, 1), ([MOST] * 257, 3),
+                                       ([MOST, 5] * 150, 1), ([MOST] * 3, 64), ([MOST], 2)])
+def test_plans_of_more_tiles_than_31_bits_hold(ek, lens, tile):
+    """The lengths' tiles sum to more than 2^31 on both sides of the sequence-per-thread line; items
+    of both plans against the plans' rules in 64 bits (lengths alone: there is no cache)."""
+    B, n_workers, overhead = len(lens), 148, 2
+    t = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    lens = np.array(lens, dtype=np.int64)
+    tiles = -(-lens // tile)
+    for balanced in (False, True):
+        n_max = B + (n_workers if balanced else 300)
+        if balanced:
+            items, first, wfirst = ek.elitekv_plan_workers(t, tile, n_workers, n_max, overhead)
+        else:
+            items, first = ek.elitekv_plan(t, tile, n_max)
+        items, first = items.cpu().numpy().astype(np.int64), first.cpu().numpy()
+        assert first[0] == 0 and np.all(np.diff(first) >= (lens > 0)) and first[B] <= n_max
+        assert np.all(items[first[B]:, 0] == -1)
+        for b in range(B):
+            rows = items[first[b]:first[b + 1]]
+            assert np.all(rows[:, 0] == b) and np.all(rows[:, 2] > 0) and np.all(rows[:, 1] % tile == 0)
+            assert np.array_equal(np.cumsum(rows[:, 2]), np.append(rows[1:, 1], lens[b])[:len(rows)])
+        its = items[:first[B]]
+        if balanced:
+            slots = np.where(tiles > 0, tiles + overhead, 0)
+            g0, total = np.concatenate([[0], np.cumsum(slots)]), int(slots.sum())
+            bound = np.array([w * total // n_workers for w in range(n_workers + 1)])
+            ga = g0[its[:, 0]] + overhead + its[:, 1] // tile
+            assert np.all(bound[its[:, 3]] <= ga) and np.all(ga - its[:, 1] // tile + -(-(its[:, 1] + its[:, 2]) // tile) <= bound[its[:, 3] + 1])
+            assert np.array_equal(wfirst.cpu().numpy(), np.searchsorted(its[:, 3], np.arange(n_workers + 1)))
+        else:
+            target = -(-int(tiles.sum()) // (n_max - B))
+            assert np.all(its[:, 2] <= target * tile)
+
+
 @pytest.mark.parametrize("d", [64, 128, 320, 4096])
 @pytest.mark.parametrize("T", [1, 127, 129, 257, 700])
 def test_project_append_depth_shares(ek, T, d):
