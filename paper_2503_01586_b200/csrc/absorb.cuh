@@ -15,6 +15,7 @@ struct AbsorbArgs {
   int B;
   const bf16* WukT;
   const int32_t* qdims;
+  const uint16_t* qkeep;
   const int32_t* idx;
   const float2* cs;
   bf16* q_rope;
@@ -54,8 +55,8 @@ __device__ __forceinline__ void absorb_rope(const AbsorbArgs& a, int h) {
 
 // Absorbed queries of one head, 128 latent coordinates from k0 on, sequences [b0, b0 + 16 MT).  The
 // product runs over all d_h query dims in their own order: the weight row of a dim goes to the
-// shared-memory row of that dim, and the rows of the rotated (elite) dims are zeros, so the queries
-// are used as they come.  (A non-finite elite dim makes the row's rope scores non-finite as well.)
+// shared-memory row of that dim, and the rows of the rotated (elite) dims are zeros.  Those dims of the
+// queries are zeros too (a zero weight alone would turn an infinite one into NaN).
 template <int MT>
 __device__ __forceinline__ void absorb_block(const AbsorbArgs& a, int h, int k0, int b0, unsigned char* smem_b) {
   const int dn = a.d_h - 2 * a.r;
@@ -64,6 +65,7 @@ __device__ __forceinline__ void absorb_block(const AbsorbArgs& a, int h, int k0,
   bf16* s_w = (bf16*)smem_b;                         // [kpad][128 + 8] weight slab
   bf16* s_q = s_w + (size_t)kpad * kAbsorbPitch;     // [16 MT][qpitch] queries; then [16 MT][128 + 8] results
   const int32_t* dims = a.qdims + (size_t)h * a.d_h;
+  const uint16_t* keep = a.qkeep + (size_t)h * a.d_h;      // all ones at un-rotated dims
   const int kw = min(kAbsorbCoords, a.kw - k0);      // coordinates of this slab (a multiple of 8)
   const int nb = min(16 * MT, a.B - b0);
   // weights and tables belong to the layer: fetched while earlier kernels of the stream still run.
@@ -91,21 +93,31 @@ __device__ __forceinline__ void absorb_block(const AbsorbArgs& a, int h, int k0,
       *(uint4*)(s_w + (size_t)row * kAbsorbPitch + (e % (kAbsorbCoords / 8)) * 8) = make_uint4(0, 0, 0, 0);
     }
   }
+  // a thread's 16-byte units of the queries lie in one column of the rows: one mask for all of them
+  const int v8 = kpad / 8, bb0 = threadIdx.x / v8, v = threadIdx.x - bb0 * v8, step = kAbsorbThreads / v8;
+  const bool vec = (a.d_h & 7) == 0, in = vec && bb0 < step && v * 8 < a.d_h;
+  const uint4 mask = in ? __ldg((const uint4*)keep + v) : make_uint4(0, 0, 0, 0);
   ekv_pdl_wait();
   // the queries, 16 bytes a load where rows are whole 16-byte units; padding and missing rows are zeros
-  if ((a.d_h & 7) == 0) {
-    const int v8 = kpad / 8;
-#pragma unroll MT
-    for (int e = threadIdx.x; e < 16 * MT * v8; e += kAbsorbThreads) {
-      const int bb = e / v8, v = e - bb * v8;
-      uint4 raw = make_uint4(0, 0, 0, 0);
-      if (bb < nb && v * 8 < a.d_h) raw = *((const uint4*)(a.q + ((size_t)(b0 + bb) * a.n_h + h) * a.d_h) + v);
-      *(uint4*)(s_q + bb * qpitch + v * 8) = raw;
+  if (vec) {
+    const bf16* src = a.q + ((size_t)b0 * a.n_h + h) * a.d_h + v * 8;
+    for (int bb = bb0 < step ? bb0 : 16 * MT; bb < 16 * MT; bb += MT * step) {
+      uint4 raw[MT];
+#pragma unroll
+      for (int k = 0; k < MT; ++k)
+        raw[k] = in && bb + k * step < nb ? *(const uint4*)(src + (size_t)(bb + k * step) * a.n_h * a.d_h) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int k = 0; k < MT; ++k)
+        if (bb + k * step < 16 * MT)
+          *(uint4*)(s_q + (bb + k * step) * qpitch + v * 8) =
+              make_uint4(raw[k].x & mask.x, raw[k].y & mask.y, raw[k].z & mask.z, raw[k].w & mask.w);
     }
   } else {
     for (int e = threadIdx.x; e < 16 * MT * kpad; e += kAbsorbThreads) {
       const int bb = e / kpad, i = e - bb * kpad;
-      s_q[bb * qpitch + i] = bb < nb && i < a.d_h ? a.q[((size_t)(b0 + bb) * a.n_h + h) * a.d_h + i] : __float2bfloat16_rn(0.f);
+      const bool there = bb < nb && i < a.d_h;
+      const uint16_t x = there ? ((const uint16_t*)a.q)[((size_t)(b0 + bb) * a.n_h + h) * a.d_h + i] : (uint16_t)0;
+      ((uint16_t*)s_q)[bb * qpitch + i] = there ? (uint16_t)(x & __ldg(keep + i)) : (uint16_t)0;
     }
   }
   cp_async_wait<0>();
@@ -165,6 +177,6 @@ inline bool absorb_ok(const elitekv_layer* L, const AbsorbShape& s) {
   return (int)s.smem <= L->smem_optin && L->kw % 8 == 0;
 }
 inline AbsorbArgs absorb_args(const elitekv_layer* L, const void* q, const int32_t* q_pos, int B, void* q_rope, void* q_abs) {
-  return AbsorbArgs{(const bf16*)q, q_pos, B, L->d_WukT, L->d_qdims, L->d_idx, L->d_cs, (bf16*)q_rope, (bf16*)q_abs,
+  return AbsorbArgs{(const bf16*)q, q_pos, B, L->d_WukT, L->d_qdims, L->d_qkeep, L->d_idx, L->d_cs, (bf16*)q_rope, (bf16*)q_abs,
                     L->n_h, L->d_h, L->r, L->kw, L->max_pos, L->d_status};
 }

@@ -27,6 +27,7 @@ struct elitekv_layer {
   int32_t* d_idx;                  // [n_h][r] elite chunk ids
   int32_t* d_qdims;                // [n_h][d_h]: 2r dims of the elite chunks in cache order,
                                    // then the dn remaining dims ascending
+  uint16_t* d_qkeep;               // [n_h][d_h] mask of a query dim: all ones, zero at the dims of elite chunks
   const float2* d_cs;              // [max_pos][d_h/2] (cos, sin)
   float2* d_cs_owned;              // same pointer when the library built the table
   bf16* d_WukT;                    // [n_h][dn][kw]: W_uk regrouped per head, latent axis contiguous

@@ -48,6 +48,7 @@ extern "C" int elitekv_layer_create(const elitekv_params* p, elitekv_layer** out
 
   // index sets: in range, distinct per head; dims of the query each cache slot pairs with
   std::vector<int32_t> qdims((size_t)n_h * d_h);
+  std::vector<uint16_t> qkeep((size_t)n_h * d_h, 0);
   for (int h = 0; h < n_h; ++h) {
     std::vector<char> used(d_h, 0);
     for (int j = 0; j < r; ++j) {
@@ -62,7 +63,10 @@ extern "C" int elitekv_layer_create(const elitekv_params* p, elitekv_layer** out
     }
     int w = 2 * r;
     for (int d = 0; d < d_h; ++d)
-      if (!used[d]) qdims[(size_t)h * d_h + w++] = d;
+      if (!used[d]) {
+        qdims[(size_t)h * d_h + w++] = d;
+        qkeep[(size_t)h * d_h + d] = 0xffff;
+      }
   }
 
   elitekv_layer* L = (elitekv_layer*)calloc(1, sizeof(elitekv_layer));
@@ -86,6 +90,8 @@ extern "C" int elitekv_layer_create(const elitekv_params* p, elitekv_layer** out
     if (cudaMemset(L->d_status, 0, 4 * sizeof(int32_t)) != cudaSuccess) break;
     if (cudaMalloc(&L->d_qdims, qdims.size() * sizeof(int32_t)) != cudaSuccess) break;
     if (cudaMemcpy(L->d_qdims, qdims.data(), qdims.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) break;
+    if (cudaMalloc(&L->d_qkeep, qkeep.size() * sizeof(uint16_t)) != cudaSuccess) break;
+    if (cudaMemcpy(L->d_qkeep, qkeep.data(), qkeep.size() * sizeof(uint16_t), cudaMemcpyHostToDevice) != cudaSuccess) break;
     if (cudaMalloc(&L->d_idx, sizeof(int32_t) * (size_t)(n_h * r > 0 ? n_h * r : 1)) != cudaSuccess) break;
     if (r > 0 && cudaMemcpy(L->d_idx, p->elite_idx, sizeof(int32_t) * (size_t)n_h * r, cudaMemcpyHostToDevice) != cudaSuccess) break;
 
@@ -149,6 +155,7 @@ extern "C" int elitekv_layer_destroy(elitekv_layer* L) {
   if (!L) return ELITEKV_ERR_INVALID_ARG;
   cudaFree(L->d_status);
   cudaFree(L->d_qdims);
+  cudaFree(L->d_qkeep);
   cudaFree(L->d_idx);
   cudaFree(L->d_cs_owned);
   cudaFree(L->d_WukT);

@@ -88,6 +88,23 @@ def test_absorb_row_tiles(ek, B, shape):
         assert np.max(np.abs(H.f64(q_abs[b]) - want_abs)) <= 2.0 ** -8 * np.max(np.abs(want_abs)) + 1e-30
 
 
+@pytest.mark.parametrize("B,pair_mode,d_h", [(3, 0, 128), (40, 1, 128), (5, 1, 44)])
+def test_absorb_takes_nothing_from_elite_dims(ek, B, pair_mode, d_h):
+    """q_abs sums over the un-rotated dims only: infinities and NaN in the elite dims (pairs of neighbours
+    or half a head apart) leave it as it is with zeros there, bit for bit."""
+    w = replace(gen.LLAMA7B_75, B=B, n_h=3, d_h=d_h, r=5, seed=70 + B)
+    idx = gen.elite_index_sets(w)
+    layer = ek.Layer(w.n_h, d_h, w.r, w.d_c, idx, *gen.up_projections(w, "cuda"), 300, pair_mode=pair_mode)
+    q = gen.queries(w, "cuda")
+    q_pos = (torch.arange(B, dtype=torch.int32) % 300).cuda()
+    at = idx.long().cuda()
+    dims = torch.cat([2 * at, 2 * at + 1] if pair_mode == 0 else [at, at + d_h // 2], dim=1).expand(B, -1, -1)
+    got = []
+    for v in (0.0, float("inf"), float("-inf"), float("nan")):
+        got.append(ek.elitekv_absorb_query(layer, q.scatter(2, dims, v), q_pos)[1])
+    assert torch.isfinite(got[0]).all() and got[0].any()
+    assert all(torch.equal(got[0], x) for x in got[1:])
+
 @pytest.mark.parametrize("B", [1, 33, 200])
 def test_step_front_end_equals_the_three_calls(ek, B):
     """One launch for append, plan and query preparation: more tokens than append blocks (200), and
