@@ -61,6 +61,8 @@ constexpr int kT = 64;                 // tokens per tile
 constexpr int kUnit = 16384;           // 128 columns of a tile: [2 chunks][64 tokens][64 bf16]
 constexpr int kMaxRing = 12;           // units in the ring
 constexpr int kTileBars = 8;           // tiles whose loads can be under way at once (more than the ring holds)
+constexpr float kNoRef = -3.402823466e38f;   // reference maximum of a stream that has seen no finite score: any finite one moves
+                                       // it, and a tile of scores that are all -inf has zero probabilities (not NaN)
 constexpr int kFinSlots = 3;           // items whose softmax statistics can be under way at once
 
 struct ClArgs {
@@ -556,8 +558,8 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
         fac[v] = f0;
         fac[NH + v] = f1;
         if (rank == 0 && quarter == 0)
-          __stcg((float2*)(a.part_ml + ((size_t)c.item * NH + v) * 2),
-                 make_float2(M, (f0 != 0.f ? x0.y * f0 : 0.f) + (f1 != 0.f ? x1.y * f1 : 0.f)));
+          __stcg((float2*)(a.part_ml + ((size_t)c.item * NH + v) * 2),      // (no finite score in the whole item: weightless)
+                 make_float2(M > kNoRef ? M : -INFINITY, (f0 != 0.f ? x0.y * f0 : 0.f) + (f1 != 0.f ? x1.y * f1 : 0.f)));
       }
       __syncwarp();
       // a [128 columns x heads] block leaves TMEM with one thread per latent column: for a fixed
@@ -718,7 +720,7 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
       if (fresh) {
 #pragma unroll
         for (int h = 0; h < 4 * QW; ++h) {
-          m_ref[h] = -INFINITY;
+          m_ref[h] = kNoRef;
           l_sum[h] = 0.f;
         }
       }

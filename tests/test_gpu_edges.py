@@ -189,6 +189,49 @@ def test_cluster_kernel_peaked(ek, mode):
     assert _run(ek, "7b", mode, 4) == 4
 
 
+@pytest.mark.parametrize("shape", CLUSTER_SHAPES)
+def test_cluster_kernel_tiles_without_a_finite_score(ek, shape):
+    """Keys that give one head scores of -inf in whole 64-token tiles (finite bf16 rope dims whose fp32
+    products overflow) weigh nothing, wherever the tile lies in its item: the head's output is that of
+    the other tokens.  The plan makes items of one, two and three tiles."""
+    B, h = 220, 3
+    w = gen.shrink(CLUSTER_SHAPES[shape], B=B, ctx=192)
+    idx = gen.elite_index_sets(w)
+    tab = torch.zeros((194, w.d_h // 2, 2), device="cuda")
+    tab[..., 0] = 1.0                                      # no rotation: signs below are those of the scores
+    dead = [(), (0,), (1,), (2,), (0, 1), (1, 2)]          # tiles without a finite score, by sequence
+
+    def edit(st):
+        q = st.q[:, h].float()
+        at = idx[h].long().cuda()
+        qe = torch.stack([q[:, 2 * at], q[:, 2 * at + 1]], dim=2)              # [B][r][2]
+        qe = torch.where(qe < 0, -2.0, 2.0)
+        st.q[:, h, 2 * at], st.q[:, h, 2 * at + 1] = qe[..., 0].to(torch.bfloat16), qe[..., 1].to(torch.bfloat16)
+        for b in range(B):
+            for t in dead[b % len(dead)]:
+                lo = int(st.starts[b]) + 64 * t
+                st.k_e[lo:lo + 64, h] = (-3e38 * torch.sign(qe[b])).to(torch.bfloat16)
+
+    st = H.setup(w, lens=[192] * B, decode_kernel=4, cos_sin=tab, edit_tokens=edit)
+    out = H.run_decode(st)
+    _, tile, n_workers, max_items, overhead = ek.elitekv_decode_plan_info(st.layer, st.cache, B)
+    first = ek.elitekv_plan_workers(st.lens_dev, tile, n_workers, max_items, overhead)[1]
+    assert first.diff().min().item() == 1                  # some sequences are one item of three tiles
+    assert torch.isfinite(out).all()
+    W_uk, W_uv, dn = H.f64(st.W_uk), H.f64(st.W_uv), w.d_h - 2 * w.r
+    at = idx[h].numpy().astype(np.int64)
+    el = np.stack([2 * at, 2 * at + 1], axis=1).reshape(-1)
+    rest = np.setdiff1d(np.arange(w.d_h), el)
+    for b in range(0, 24):
+        lo = int(st.starts[b])
+        keep = np.concatenate([np.arange(64 * t, 64 * t + 64) for t in range(3) if t not in dead[b % len(dead)]])
+        q, c, k = H.f64(st.q[b, h]), H.f64(st.c[lo:lo + 192])[keep], H.f64(st.k_e[lo:lo + 192, h])[keep].reshape(len(keep), -1)
+        ck, cv = (c[:, :st.d_ck], c[:, st.d_ck:]) if st.d_ck else (c, c)
+        s = (k @ q[el] + ck @ (W_uk[:, h * dn:(h + 1) * dn] @ q[rest])) / w.d_h ** 0.5
+        p = np.exp(s - s.max())
+        want = (p / p.sum()) @ cv @ W_uv[:, h * w.d_h:(h + 1) * w.d_h]
+        assert np.linalg.norm(H.f64(out[b, h]) - want) <= H.REL_L2_TOL * np.linalg.norm(want)
+
 def test_cluster_kernel_refuses_uncovered_shapes(ek):
     w = replace(gen.LLAMA7B_75, B=2, ctx=64, n_h=24)          # 384 rope dims: clusters of three are not built
     with pytest.raises(ek.ElitekvError) as e:
