@@ -409,7 +409,8 @@ project_append_pair_kernel(const __grid_constant__ CUtensorMap map_t, const __gr
     const int w8 = warp - 2, first = (H + 1) * a.nk - kUnits;     // the units of the ring's last turn
     unsigned char* s_cs = base + (first + w8) % kUnits * kUnitBytes;
     unsigned char* s_out = base + (first + 8 + (w8 >> 1)) % kUnits * kUnitBytes + (w8 & 1) * (kUnitBytes / 2);
-    const bool staged = a.half <= kCsHalf && (a.half & 1) == 0;
+    // (16-byte reads of the table: a caller's own table may start on any 8 bytes)
+    const bool staged = a.half <= kCsHalf && (a.half & 1) == 0 && ((uintptr_t)a.cs & 15) == 0;
     bool ok = true;
     if (n0 + part0 * 128 < a.rope_w && staged) {
       // the 32 tokens' table rows, a whole row per request: a look-up by every token on its own would

@@ -413,3 +413,28 @@ def test_project_append_paired_forms_with_late_epilogue_warps(ek, T):
     for got, want in ((rope, rows64), (latent, c64)):
         # as for the other projections: one bf16 rounding plus fp32 accumulation over d terms
         assert np.all(np.abs(H.f64(got[good.cuda()]) - want) <= np.abs(want) * 2.0 ** -8 + 2e-5 * d ** 0.5)
+
+
+@pytest.mark.parametrize("T", [100, 1153, 4096])
+def test_project_append_table_on_any_8_bytes(ek, T):
+    """A caller's (cos, sin) table that starts 8 bytes past a 16-byte boundary gives the bits of the same
+    table on one, in the split-depth form and in both paired forms."""
+    d, w = 1024, replace(gen.LLAMA7B_75, seed=T)
+    g = torch.Generator().manual_seed(T)
+    rope_w = w.n_h * 2 * w.r
+    W_ke, W_down = ((torch.randn(d, n, generator=g) / 32).to(torch.bfloat16).cuda() for n in (rope_w, w.d_c))
+    x = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()
+    tab = torch.from_numpy(O.rope_table_f32(T, w.d_h, w.rope_base)).cuda()
+    room = torch.zeros(tab.numel() + 2, device="cuda")
+    shifted = room[2:].view(tab.shape).copy_(tab)
+    assert shifted.data_ptr() % 16 == 8 and tab.data_ptr() % 16 == 0
+    seq, pos = torch.zeros(T, dtype=torch.int32, device="cuda"), torch.arange(T, dtype=torch.int32, device="cuda")
+    rows = []
+    for cs in (tab, shifted):
+        layer = ek.Layer(w.n_h, w.d_h, w.r, w.d_c, gen.elite_index_sets(w), *gen.up_projections(w, "cuda"), T, cos_sin=cs,
+                         W_ke=W_ke, W_down=W_down)
+        rope, latent = (torch.zeros((T, n), dtype=torch.bfloat16, device="cuda") for n in (rope_w, w.d_c))
+        ek.elitekv_project_append(layer, ek.make_cache(rope, latent, n_seqs=1, max_ctx=T), x, seq, pos)
+        assert ek.elitekv_check_status(layer) == 0
+        rows.append((rope, latent))
+    assert all(torch.equal(a, b) for a, b in zip(*rows))
