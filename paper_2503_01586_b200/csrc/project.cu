@@ -101,6 +101,7 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   ProjBarriers* bars = (ProjBarriers*)(base + kPStages * kPStageBytes + (kSplitDepth ? kRecvBytes : 0));
   uint32_t* s_tmem = (uint32_t*)(bars + 1);
   volatile int* s_abort = (volatile int*)(s_tmem + 1);
+  volatile int* s_lost = s_abort + 1;              // a block of the cluster gave up: no sum here is complete
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * kPN;                 // first output column of the tile
   const long long t0 = (long long)blockIdx.y * kPM; // first token of the tile
@@ -116,6 +117,7 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     }
     mbar_init(smem_u32(&bars->done), 1);
     *s_abort = 0;
+    *s_lost = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
@@ -128,6 +130,9 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // a block's shared memory is written by its peers once they know that it has started: every warp waits
+  // for that before its first remote store, behind the loads and products
+  if (kSplitDepth) cluster_arrive();
   const uint32_t tmem_base = *s_tmem;
 
   if (warp == 0) {
@@ -189,6 +194,7 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
     // one outcome per warp: the TMEM loads below want all 32 lanes
     const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->done), 0, s_abort, 3));
     tc_fence_after();
+    if (kSplitDepth) cluster_wait();
     if (ok) {
       // split depth: this row's partial sums go to the block that finishes the row
       const uint32_t dst = kSplitDepth
@@ -213,10 +219,14 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
   }
 
   if (kSplitDepth) {
-    // every block of the cluster has delivered (or given up): the barrier orders the remote
+    __syncwarp();
+    if (warp < 2) cluster_wait();
+    if (*s_abort && lane < kSplit) st_cluster_u32(map_to_cta(smem_u32((const void*)s_lost), (uint32_t)lane), 1u);
+    __syncwarp();
+    // every block of the cluster has delivered (or given up, and said so): the barrier orders the remote
     // stores above before the sums below, and nobody is written to after it
     cluster_sync_all();
-    if (warp >= 2 && !*s_abort) {
+    if (warp >= 2 && !*s_lost) {
       const int e = threadIdx.x - 64;                    // 128 threads: 16 rows x 8 column groups
       const int cg = e & 7;
       for (int rr = e >> 3; rr < kSplitRows; rr += 16) {
