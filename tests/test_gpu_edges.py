@@ -384,7 +384,7 @@ def test_append_staged_groups(ek, shape, T):
     assert torch.equal(latent[st.pos.long()].view(torch.int16), st.c.view(torch.int16).view(T, -1))
 
 
-@pytest.mark.parametrize("T", [1153, 2305, 4096])
+@pytest.mark.parametrize("T", [1153, 1500, 2305, 4096])
 def test_project_append_paired_forms_with_late_epilogue_warps(ek, T):
     """40 of 41 tokens have a position outside the cache: every thread that meets one records it with
     atomics on one word, so the epilogue warps of the paired forms come to their shared-memory units long
