@@ -24,31 +24,41 @@
 // with packed operations (all but the add with |.|): 43 % fewer instructions at the same number of
 // fp32 operations; pairs of neighbouring table entries are formed in registers.  32 heads x 2048 tokens
 // x d_h 128: 1.48 ms a round (1.58 with scalar operations, 1.53 with the chunk loops unrolled twice
-// and not eight times; 0.54 of 148 SMs x 128 lanes x 1.965 GHz).  The form that held the 64 D_i of one
+// and not eight times; 0.54 of 148 SMs x 128 lanes x 1.965 GHz).  The form that holds the 64 D_i of one
 // pair in registers took 3.04 ms: 9 operations and three loads per pair and chunk, shared-memory bound.
+// Short calibrations cannot fill the device with 128 x 128 tiles: there a thread owns 8 or 4 rows, and up
+// to 128 tokens the register form is the faster one (rl_form; one head of 64 tokens, four rounds: 235 us on
+// one such tile, 72 us).
 //
-// distance kernel: grid (items, heads), 256 threads; an item is 128 query rows x up to `span` key
+// distance kernel: grid (items, heads), 256 threads; an item is 128 (64, 32) query rows x up to `span` key
 // tiles of 128.  Per key tile the rotated keys (x plane, y plane, [chunk][key]) and the slice of
 // the sine table that the tile's relative positions need are staged in shared memory; the table is
 // zero at negative relative positions, which is the causal mask.  Item results go to a
 // [head][item][chunk] array; the select kernel adds them in a fixed order (the result does not
 // depend on scheduling), masks the chunks already chosen and takes the first minimum.
+#include <initializer_list>
+
 #include "common.cuh"
 
 namespace {
 
-constexpr int kRlRows = 128;      // query rows per block
-constexpr int kRlTR = 16;         // ... per warp (and thread)
 constexpr int kRlKeys = 128;      // keys per stage
 constexpr int kRlTK = 4;          // ... per thread
-constexpr int kRlThreads = 256;
 constexpr int kRlAcc = 8;         // lanes of a warp that keep running distances
-constexpr int kRlSpan = kRlKeys + kRlRows;         // sine table entries of a stage (relative positions)
 constexpr int kRlPad = 256;       // zeros in front of the sine table: negative relative positions
-static_assert(kRlRows == kRlThreads / 32 * kRlTR && kRlKeys == 32 * kRlTK, "thread tiles cover the block's tile");
+static_assert(kRlKeys == 32 * kRlTK, "thread tiles cover the block's keys");
+
+// blocks of 8 warps with TR query rows per warp (and thread): 16, or 8 or 4 where that fills the device better
+template <int TR_>
+struct Rl {
+  static constexpr int TR = TR_, NW = 8, THREADS = 32 * NW;
+  static constexpr int ROWS = NW * TR;                   // query rows per block
+  static constexpr int SPAN = kRlKeys + ROWS;            // sine table entries of a stage (relative positions)
+  static_assert(ROWS <= 128 && SPAN <= kRlPad, "a stage's slice lies inside the table");
+};
 
 // entries of a chunk's sine table: entry x holds 2 sin((x - kRlPad) theta / 2), zero up to kRlPad
-__host__ __device__ inline int rl_sin_len(int n) { return (n + kRlRows - 1) / kRlRows * kRlRows + kRlPad; }
+__host__ __device__ inline int rl_sin_len(int n) { return (n + 127) / 128 * 128 + kRlPad; }
 
 // (cos, sin)(pos theta_i / 2) laid out [pos][chunk], and the sine table [chunk][...];
 // double precision, rounded once
@@ -85,12 +95,12 @@ __device__ __forceinline__ void rl_rotate4(const bf16* row, const float2* cs, fl
   }
 }
 
-template <int HALF>
+template <int HALF, class F>
 struct RlSmem {
   float kx[HALF][kRlKeys], ky[HALF][kRlKeys];
-  float sn[HALF][kRlSpan];
-  float qx[HALF][kRlRows], qy[HALF][kRlRows];
-  float acc[HALF][kRlThreads / 32 * kRlAcc];     // running distances
+  float sn[HALF][F::SPAN];
+  float qx[HALF][F::ROWS], qy[HALF][F::ROWS];
+  float acc[HALF][F::NW * kRlAcc];     // running distances
   int list[HALF];                    // chunks not chosen yet
 };
 
@@ -117,14 +127,16 @@ __device__ __forceinline__ rl2 rl_fma(rl2 a, rl2 b, rl2 c) {
   return d;
 }
 
-// operands of a thread's 64 pairs for one chunk; kNeg: t with its sign turned
+// operands of a thread's 4 TR pairs for one chunk; kNeg: t with its sign turned
+template <int TR>
 struct RlOps {
   rl2 a[kRlTK], b[kRlTK];            // keys: t = q_y a + q_x b
-  rl2 qx[kRlTR / 2], qy[kRlTR / 2];
-  rl2 s[(kRlTR + kRlTK) / 2][2];     // [v][0]: table entries 2 v, 2 v + 1; [v][1]: 2 v + 1, 2 v + 2
+  rl2 qx[TR / 2], qy[TR / 2];
+  rl2 s[(TR + kRlTK) / 2][2];        // [v][0]: table entries 2 v, 2 v + 1; [v][1]: 2 v + 1, 2 v + 2
 };
-template <int HALF, bool kNeg>
-__device__ __forceinline__ void rl_load(RlOps& o, const RlSmem<HALF>& sm, int i, int warp, int lane) {
+template <int HALF, class F, bool kNeg>
+__device__ __forceinline__ void rl_load(RlOps<F::TR>& o, const RlSmem<HALF, F>& sm, int i, int warp, int lane) {
+  constexpr int TR = F::TR;
   const float4 kx = *(const float4*)&sm.kx[i][lane * kRlTK], ky = *(const float4*)&sm.ky[i][lane * kRlTK];
   const float x[kRlTK] = {kx.x, kx.y, kx.z, kx.w}, y[kRlTK] = {ky.x, ky.y, ky.z, ky.w};
 #pragma unroll
@@ -134,52 +146,53 @@ __device__ __forceinline__ void rl_load(RlOps& o, const RlSmem<HALF>& sm, int i,
     o.b[j] = rl_pack(b, b);
   }
   // entry u of the stage's slice: relative position (m0 - n0) - 128 + u; this thread's pairs need
-  // u = 16 warp + r - (4 lane + j) + 128, from 16 warp - 4 lane + 124 on
-  const float4* sp = (const float4*)&sm.sn[i][kRlTR * warp - kRlTK * lane + kRlRows - kRlTK];
-  float e[kRlTR + kRlTK];
+  // u = TR warp + r - (4 lane + j) + 128, from TR warp - 4 lane + 124 on
+  const float4* sp = (const float4*)&sm.sn[i][TR * warp - kRlTK * lane + kRlKeys - kRlTK];
+  float e[TR + kRlTK];
 #pragma unroll
-  for (int u = 0; u < (kRlTR + kRlTK) / 4; ++u) *(float4*)&e[4 * u] = sp[u];
+  for (int u = 0; u < (TR + kRlTK) / 4; ++u) *(float4*)&e[4 * u] = sp[u];
 #pragma unroll
-  for (int v = 0; v < (kRlTR + kRlTK) / 2; ++v) {
+  for (int v = 0; v < (TR + kRlTK) / 2; ++v) {
     o.s[v][0] = rl_pack(e[2 * v], e[2 * v + 1]);
-    if (2 * v + 2 < kRlTR + kRlTK) o.s[v][1] = rl_pack(e[2 * v + 1], e[2 * v + 2]);
+    if (2 * v + 2 < TR + kRlTK) o.s[v][1] = rl_pack(e[2 * v + 1], e[2 * v + 2]);
   }
-  const ulonglong2* qx = (const ulonglong2*)&sm.qx[i][kRlTR * warp];
-  const ulonglong2* qy = (const ulonglong2*)&sm.qy[i][kRlTR * warp];
+  const ulonglong2* qx = (const ulonglong2*)&sm.qx[i][TR * warp];
+  const ulonglong2* qy = (const ulonglong2*)&sm.qy[i][TR * warp];
 #pragma unroll
-  for (int u = 0; u < kRlTR / 4; ++u) {
+  for (int u = 0; u < TR / 4; ++u) {
     const ulonglong2 vx = qx[u], vy = qy[u];
     o.qx[2 * u] = vx.x; o.qx[2 * u + 1] = vx.y;
     o.qy[2 * u] = vy.x; o.qy[2 * u + 1] = vy.y;
   }
 }
 // table pair of rows 2 r, 2 r + 1 and key j: entries 2 r - j + 4 and the next
-__device__ __forceinline__ rl2 rl_sin(const RlOps& o, int r, int j) { return o.s[(2 * r - j + kRlTK) / 2][(2 * r - j + kRlTK) & 1]; }
+template <int TR>
+__device__ __forceinline__ rl2 rl_sin(const RlOps<TR>& o, int r, int j) { return o.s[(2 * r - j + kRlTK) / 2][(2 * r - j + kRlTK) & 1]; }
 
-template <int HALF>
-__global__ void __launch_bounds__(kRlThreads)
+template <int HALF, class F>
+__global__ void __launch_bounds__(F::THREADS)
 ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, int n,
                          const float2* __restrict__ cs, const float* __restrict__ sn,
                          const unsigned long long* __restrict__ masks, int span,
                          float* __restrict__ partial /* [heads][items][HALF] */) {
-  constexpr int d_h = 2 * HALF;
+  constexpr int d_h = 2 * HALF, TR = F::TR, NW = F::NW, THREADS = F::THREADS, ROWS = F::ROWS, SPAN = F::SPAN;
   extern __shared__ __align__(16) unsigned char smem_rl[];
-  RlSmem<HALF>& sm = *(RlSmem<HALF>*)smem_rl;
+  RlSmem<HALF, F>& sm = *(RlSmem<HALF, F>*)smem_rl;
   const int head = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // item -> (row tile, group of key tiles), long rows first
-  int mt = (n + kRlRows - 1) / kRlRows - 1, kg = blockIdx.x;
+  int mt = (n + ROWS - 1) / ROWS - 1, kg = blockIdx.x;
   for (;; --mt) {
-    const int groups = ((mt + 1) * kRlRows + kRlKeys * span - 1) / (kRlKeys * span);
+    const int groups = ((mt + 1) * ROWS + kRlKeys * span - 1) / (kRlKeys * span);
     if (kg < groups) break;
     kg -= groups;
   }
-  const int m0 = mt * kRlRows;
-  const int n_lo = kg * span * kRlKeys, n_hi = min(n_lo + span * kRlKeys, m0 + kRlRows);
+  const int m0 = mt * ROWS;
+  const int n_lo = kg * span * kRlKeys, n_hi = min(n_lo + span * kRlKeys, m0 + ROWS);
   const unsigned long long mask = masks ? masks[head] : 0ull;
   const int n_free = HALF - __popcll(HALF == 64 ? mask : mask & ((1ull << (HALF & 63)) - 1));
   float* out = partial + ((size_t)head * gridDim.x + blockIdx.x) * HALF;
   if (n_free <= 1) {                 // a single free chunk: R = D_j for every pair
-    for (int j = threadIdx.x; j < HALF; j += kRlThreads) out[j] = 0.f;
+    for (int j = threadIdx.x; j < HALF; j += THREADS) out[j] = 0.f;
     return;
   }
   if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
@@ -187,8 +200,8 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
   const bf16* Qh = Q + (size_t)head * n * d_h;
   const bf16* Kh = K + (size_t)head * n * d_h;
   // (consecutive threads take consecutive rows: the transposed stores hit different banks)
-  for (int e = threadIdx.x; e < kRlRows * (HALF / 4); e += kRlThreads) {
-    const int rr = e % kRlRows, g4 = e / kRlRows;
+  for (int e = threadIdx.x; e < ROWS * (HALF / 4); e += THREADS) {
+    const int rr = e % ROWS, g4 = e / ROWS;
     float2 v[4] = {};
     if (m0 + rr < n) rl_rotate4(Qh + (size_t)(m0 + rr) * d_h + g4 * 8, cs + (size_t)(m0 + rr) * HALF + g4 * 4, v);
 #pragma unroll
@@ -197,20 +210,20 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
       sm.qy[g4 * 4 + u][rr] = v[u].y;
     }
   }
-  for (int e = threadIdx.x; e < HALF * (kRlThreads / 32) * kRlAcc; e += kRlThreads) (&sm.acc[0][0])[e] = 0.f;
+  for (int e = threadIdx.x; e < HALF * NW * kRlAcc; e += THREADS) (&sm.acc[0][0])[e] = 0.f;
   const int sn_len = rl_sin_len(n);
 
   for (int n0 = n_lo; n0 < n_hi; n0 += kRlKeys) {
     __syncthreads();
     // entry u holds relative position (m0 - n0) - 128 + u
-    const int x0 = m0 - n0 - kRlRows + kRlPad;
-    for (int e = threadIdx.x; e < HALF * (kRlSpan / 4); e += kRlThreads) {
-      const int i = e / (kRlSpan / 4), u = (e % (kRlSpan / 4)) * 4;
+    const int x0 = m0 - n0 - kRlKeys + kRlPad;
+    for (int e = threadIdx.x; e < HALF * (SPAN / 4); e += THREADS) {
+      const int i = e / (SPAN / 4), u = (e % (SPAN / 4)) * 4;
       cp_async16(&sm.sn[i][u], sn + (size_t)i * sn_len + x0 + u);
     }
     cp_async_commit();
 #pragma unroll
-    for (int e = threadIdx.x; e < kRlKeys * (HALF / 4); e += kRlThreads) {
+    for (int e = threadIdx.x; e < kRlKeys * (HALF / 4); e += THREADS) {
       const int nn = e % kRlKeys, g4 = e / kRlKeys;         // 4 chunks = 8 elements = 16 bytes
       float2 v[4] = {};
       if (n0 + nn < n) rl_rotate4(Kh + (size_t)(n0 + nn) * d_h + g4 * 8, cs + (size_t)(n0 + nn) * HALF + g4 * 4, v);
@@ -222,18 +235,19 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
     }
     cp_async_wait<0>();
     __syncthreads();
-    if (n0 > m0 + kRlTR * warp + kRlTR - 1) continue;       // every pair of this warp lies above the diagonal
-    rl2 R[kRlTR / 2][kRlTK];
+    // every pair of this warp lies above the diagonal, or its rows past the last token
+    if (n0 > m0 + TR * warp + TR - 1 || m0 + TR * warp >= n) continue;
+    rl2 R[TR / 2][kRlTK];
 #pragma unroll
-    for (int r = 0; r < kRlTR / 2; ++r)
+    for (int r = 0; r < TR / 2; ++r)
 #pragma unroll
       for (int j = 0; j < kRlTK; ++j) R[r][j] = 0ull;
 #pragma unroll 8
     for (int c = 0; c < n_free; ++c) {
-      RlOps o;
-      rl_load<HALF, false>(o, sm, sm.list[c], warp, lane);
+      RlOps<TR> o;
+      rl_load<HALF, F, false>(o, sm, sm.list[c], warp, lane);
 #pragma unroll
-      for (int r = 0; r < kRlTR / 2; ++r)
+      for (int r = 0; r < TR / 2; ++r)
 #pragma unroll
         for (int j = 0; j < kRlTK; ++j) {
           const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
@@ -242,12 +256,12 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
     }
 #pragma unroll 8
     for (int c = 0; c < n_free; ++c) {
-      RlOps o;
+      RlOps<TR> o;
       const int i = sm.list[c];
-      rl_load<HALF, true>(o, sm, i, warp, lane);
+      rl_load<HALF, F, true>(o, sm, i, warp, lane);
       float v[kRlTK] = {};
 #pragma unroll
-      for (int r = 0; r < kRlTR / 2; ++r)
+      for (int r = 0; r < TR / 2; ++r)
 #pragma unroll
         for (int j = 0; j < kRlTK; ++j) {
           const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
@@ -263,12 +277,95 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
   }
   // block result: threads in a fixed order
   __syncthreads();
-  for (int j = warp; j < HALF; j += kRlThreads / 32) {
+  for (int j = warp; j < HALF; j += NW) {
     float v = 0.f;
 #pragma unroll
-    for (int w = 0; w < kRlThreads / 32 * kRlAcc; w += 32) v += sm.acc[j][w + lane];
+    for (int w = 0; w < NW * kRlAcc; w += 32) v += sm.acc[j][w + lane];
     v = warp_sum(v);
     if (lane == 0) out[j] = v;
+  }
+}
+
+// Small calls (rl_form): a block is 16 query rows and all their keys, 64 at a time; a thread takes one pair
+// at a time and holds its D_i in registers.  9 loads and operations per pair and chunk instead of 7 packed
+// ones, but no pair is computed that the causal rule leaves out, and a block's chain is short.
+constexpr int kRsRows = 16, kRsKeys = 64, kRsWarps = 4;
+template <int HALF>
+struct RsSmem {
+  float2 k[HALF][kRsKeys], q[kRsRows][HALF];
+  float sn[HALF][kRsKeys + kRsRows];
+  float red[kRsWarps][HALF];
+};
+template <int HALF>
+__global__ void __launch_bounds__(32 * kRsWarps)
+ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, int n,
+                               const float2* __restrict__ cs, const float* __restrict__ sn,
+                               const unsigned long long* __restrict__ masks,
+                               float* __restrict__ partial /* [heads][row tiles][HALF] */) {
+  constexpr int d_h = 2 * HALF, THREADS = 32 * kRsWarps;
+  extern __shared__ __align__(16) unsigned char smem_rl[];
+  RsSmem<HALF>& sm = *(RsSmem<HALF>*)smem_rl;
+  const int head = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = blockIdx.x * kRsRows, m_last = min(m0 + kRsRows, n) - 1;
+  const unsigned long long mask = masks ? masks[head] : 0ull;
+  const bf16* Qh = Q + (size_t)head * n * d_h;
+  const bf16* Kh = K + (size_t)head * n * d_h;
+  for (int e = threadIdx.x; e < kRsRows * (HALF / 4); e += THREADS) {
+    const int rr = e / (HALF / 4), g4 = e % (HALF / 4);
+    float2 v[4] = {};
+    if (m0 + rr < n) rl_rotate4(Qh + (size_t)(m0 + rr) * d_h + g4 * 8, cs + (size_t)(m0 + rr) * HALF + g4 * 4, v);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sm.q[rr][g4 * 4 + u] = v[u];
+  }
+  float acc[HALF];
+#pragma unroll
+  for (int j = 0; j < HALF; ++j) acc[j] = 0.f;
+  const int sn_len = rl_sin_len(n);
+  for (int n0 = 0; n0 <= m_last; n0 += kRsKeys) {
+    __syncthreads();
+    const int x0 = m0 - n0 - kRsKeys + kRlPad;              // entry u: relative position (m0 - n0) - 64 + u
+    for (int e = threadIdx.x; e < HALF * ((kRsKeys + kRsRows) / 4); e += THREADS) {
+      const int i = e / ((kRsKeys + kRsRows) / 4), u = e % ((kRsKeys + kRsRows) / 4) * 4;
+      cp_async16(&sm.sn[i][u], sn + (size_t)i * sn_len + x0 + u);
+    }
+    cp_async_commit();
+    for (int e = threadIdx.x; e < kRsKeys * (HALF / 4); e += THREADS) {
+      const int nn = e % kRsKeys, g4 = e / kRsKeys;
+      if (n0 + nn > m_last) continue;
+      float2 v[4];
+      rl_rotate4(Kh + (size_t)(n0 + nn) * d_h + g4 * 8, cs + (size_t)(n0 + nn) * HALF + g4 * 4, v);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sm.k[g4 * 4 + u][nn] = v[u];
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+#pragma unroll 1
+    for (int e = 0; e < kRsRows / kRsWarps * (kRsKeys / 32); ++e) {
+      const int rr = warp + e / (kRsKeys / 32) * kRsWarps, nn = lane + e % (kRsKeys / 32) * 32;
+      if (n0 + nn > m0 + rr || m0 + rr >= n) continue;      // causal pairs only
+      const int u = rr - nn + kRsKeys;
+      float d[HALF], R = 0.f;
+#pragma unroll
+      for (int i = 0; i < HALF; ++i) {
+        const float2 q = sm.q[rr][i], k = sm.k[i][nn];
+        d[i] = __fmul_rn(sm.sn[i][u], fmaf(q.y, k.x, -(q.x * k.y)));      // rounded: the last free chunk's R - D_j is 0
+        if (!((mask >> i) & 1ull)) R = __fadd_rn(R, d[i]);
+      }
+#pragma unroll
+      for (int j = 0; j < HALF; ++j) acc[j] += fabsf(R - d[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < HALF; ++j) {
+    const float v = warp_sum(acc[j]);
+    if (lane == 0) sm.red[warp][j] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < HALF) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < kRsWarps; ++w) v += sm.red[w][threadIdx.x];
+    partial[((size_t)head * gridDim.x + blockIdx.x) * HALF + threadIdx.x] = v;
   }
 }
 
@@ -312,27 +409,50 @@ __global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_
 
 struct RlCarve {
   size_t off_cs, off_sin, off_partial, off_masks, total;
-  int span, items;              // key tiles per item, items per head
+  int tr, span, items;          // rows per thread (1: the small form), key tiles per item, items per head
 };
 inline size_t rl_align(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Key tiles per item: whole rows cut into at most 16 items, at least 4 tiles long (the rotated
 // queries of an item are prepared anew); single tiles where that would leave most of the
 // device without work (fewer blocks than four for each of 148 SMs).
-void rl_items(int heads, int n, RlCarve* c) {
-  const int tiles = (n + kRlKeys - 1) / kRlKeys;
-  auto count = [&](int span) {
-    long long k = 0;
-    for (int m = kRlRows; m < n + kRlRows; m += kRlRows) k += (m + kRlKeys * span - 1) / (kRlKeys * span);
-    return k;
-  };
-  c->span = tiles > 64 ? (tiles + 15) / 16 : 4;
-  if (heads * count(c->span) < 4 * 148) c->span = 1;
-  c->items = (int)count(c->span);
+long long rl_count(int n, int rows, int span) {
+  long long k = 0;
+  for (int m = rows; m < n + rows; m += rows) k += (m + kRlKeys * span - 1) / (kRlKeys * span);
+  return k;
+}
+// Which form, for a device of 148 SMs.  A search of few tokens is a chain of small launches: its time is
+// that of one block.  Up to 64 tokens the small form is the faster one while a few of its blocks share an
+// SM, up to 128 tokens while each has its own.  Four rounds, d_h 128, us (small / 4 / 8 / 16 rows per
+// thread): 4 heads x 64 tokens 72 / 129 / 163 / 173, 4 x 128 105 / 133 / 171 / 246, 32 x 128 - / 132 / 172 / 250,
+// 32 x 300 - / 427 / 308 / 391, 16 x 512 - / 522 / 440 / 460, 16 x 1024 - / 1606 / 1111 / 894.  Beyond it the
+// form whose blocks take least time in all, in whole rounds over the device: a key tile of a block takes
+// 24, 33 and 52 us at d_h 128, and in the same proportions at d_h 64.
+void rl_form(int heads, int n, int half, RlCarve* c) {
+  constexpr int kSms = 148;
+  const long long small = (long long)heads * ((n + kRsRows - 1) / kRsRows);
+  c->span = 1;
+  if (n <= 2 * kRsKeys && small <= (n > kRsKeys ? 1 : half == 64 ? 2 : 4) * kSms) {
+    c->tr = 1;
+    c->items = (n + kRsRows - 1) / kRsRows;
+    return;
+  }
+  long long best = 0;
+  for (const int tr : {16, 8, 4}) {
+    const int cost = tr == 16 ? 52 : tr == 8 ? 33 : 24;
+    const long long t = (heads * rl_count(n, 8 * tr, 1) + kSms - 1) / kSms * cost;
+    if (tr == 16 || t < best) {
+      best = t;
+      c->tr = tr;
+    }
+  }
+  const int tiles = (n + kRlKeys - 1) / kRlKeys, span = tiles > 64 ? (tiles + 15) / 16 : 4;
+  if (heads * rl_count(n, 8 * c->tr, span) >= 4 * kSms) c->span = span;
+  c->items = (int)rl_count(n, 8 * c->tr, c->span);
 }
 RlCarve rl_carve(int heads, int n, int half) {
   RlCarve c;
-  rl_items(heads, n, &c);
+  rl_form(heads, n, half, &c);
   size_t o = 0;
   c.off_cs = o;      o = rl_align(o + sizeof(float2) * (size_t)half * n);
   c.off_sin = o;     o = rl_align(o + sizeof(float) * (size_t)half * rl_sin_len(n));
@@ -352,11 +472,25 @@ int rl_check(int heads, int n, int d_h) {
 template <int HALF>
 int rl_launch_half(const void* Q, const void* K, int heads, int n, const RlCarve& c, unsigned char* base,
                    const unsigned long long* masks, cudaStream_t st) {
-  const int smem = (int)sizeof(RlSmem<HALF>);
-  EKV_CUDA_OK(cudaFuncSetAttribute(ropelite_distance_kernel<HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  ropelite_distance_kernel<HALF><<<dim3((unsigned)c.items, (unsigned)heads), kRlThreads, smem, st>>>(
-      (const bf16*)Q, (const bf16*)K, n, (const float2*)(base + c.off_cs), (const float*)(base + c.off_sin), masks,
-      c.span, (float*)(base + c.off_partial));
+  const float2* cs = (const float2*)(base + c.off_cs);
+  const float* sn = (const float*)(base + c.off_sin);
+  float* partial = (float*)(base + c.off_partial);
+  const dim3 grid((unsigned)c.items, (unsigned)heads);
+  if (c.tr == 1) {
+    const auto kern = ropelite_distance_small_kernel<HALF>;
+    EKV_CUDA_OK(ekv_allow_smem(kern, sizeof(RsSmem<HALF>)));
+    kern<<<grid, 32 * kRsWarps, sizeof(RsSmem<HALF>), st>>>((const bf16*)Q, (const bf16*)K, n, cs, sn, masks, partial);
+  } else {
+    const auto launch = [&](auto form) -> int {
+      using F = decltype(form);
+      const auto kern = ropelite_distance_kernel<HALF, F>;
+      EKV_CUDA_OK(ekv_allow_smem(kern, sizeof(RlSmem<HALF, F>)));
+      kern<<<grid, F::THREADS, sizeof(RlSmem<HALF, F>), st>>>((const bf16*)Q, (const bf16*)K, n, cs, sn, masks, c.span, partial);
+      return ELITEKV_OK;
+    };
+    const int rc = c.tr == 16 ? launch(Rl<16>()) : c.tr == 8 ? launch(Rl<8>()) : launch(Rl<4>());
+    if (rc != ELITEKV_OK) return rc;
+  }
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }

@@ -57,6 +57,27 @@ def test_ropelite_distances_tile_edges(ek, heads, n, d_h):
         assert np.allclose(got[h][fin], want[fin], rtol=1e-5, atol=1e-6)
 
 
+@pytest.mark.parametrize("heads,n,d_h", [(1, 1, 64), (2, 16, 128), (3, 17, 64), (37, 64, 128), (75, 64, 64), (2, 65, 128), (18, 128, 128),
+                                         (19, 128, 64), (75, 63, 128), (6, 152, 64), (5, 161, 128), (40, 152, 128), (48, 193, 64),
+                                         (33, 300, 128), (64, 128, 64)])
+def test_ropelite_distances_of_every_form(ek, heads, n, d_h):
+    """The form for small calls (16 rows a block, 64 keys at a time) up to its lines at 64 and 128 tokens,
+    and 4 and 8 rows per thread with ragged row tiles and key tiles; every chunk free, some chosen,
+    two left.  Tolerance as above."""
+    from oracle import ropelite_oracle as R
+    g = torch.Generator().manual_seed(heads + n)
+    Q, K = (torch.randn((heads, n, d_h), generator=g).to(torch.bfloat16) for _ in range(2))
+    half = d_h // 2
+    full = (1 << half) - 1
+    masks = [(0, 9 | (1 << (half - 2)), full & ~(2 | (1 << (half - 1))))[h % 3] for h in range(heads)]
+    dev = torch.from_numpy(np.array(masks, dtype=np.uint64).view(np.int64)).cuda()
+    got = ek.elitekv_ropelite_distances(Q.cuda(), K.cuda(), elite_mask=dev).cpu().double().numpy()
+    for h in {0, heads // 2, heads - 1}:
+        want = R.distances(Q[h].double().numpy(), K[h].double().numpy(), [i for i in range(half) if (masks[h] >> i) & 1], d_h)
+        fin = np.isfinite(want)
+        assert np.array_equal(np.isinf(got[h]), ~fin)
+        assert np.allclose(got[h][fin], want[fin], rtol=1e-5, atol=1e-6)
+
 def test_ropelite_search_down_to_the_last_chunk(ek):
     """All d_h / 2 rounds: every chunk is chosen once and the last free one costs nothing."""
     g = torch.Generator().manual_seed(3)
