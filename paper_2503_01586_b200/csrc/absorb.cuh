@@ -21,6 +21,7 @@ struct AbsorbArgs {
   bf16* q_rope;
   bf16* q_abs;
   int n_h, d_h, r, kw, max_pos;      // kw: width of the latent the scores read
+  int row0;                          // the first row's index in the call, for reports
   int32_t* status;
 };
 
@@ -40,7 +41,7 @@ __device__ __forceinline__ void absorb_rope(const AbsorbArgs& a, int h) {
     const int b = e / a.r, j = e % a.r;
     int p = a.q_pos[b];
     if (p < 0 || p >= a.max_pos) {
-      ekv_record(a.status, ELITEKV_ERR_BAD_POSITION, b, p);
+      ekv_record(a.status, ELITEKV_ERR_BAD_POSITION, a.row0 + b, p);
       p = 0;
     }
     const float2 w = a.cs[(size_t)p * (a.d_h / 2) + a.idx[h * a.r + j]];
@@ -176,7 +177,9 @@ inline AbsorbShape absorb_shape(const elitekv_layer* L, int B) {
 inline bool absorb_ok(const elitekv_layer* L, const AbsorbShape& s) {
   return (int)s.smem <= L->smem_optin && L->kw % 8 == 0;
 }
-inline AbsorbArgs absorb_args(const elitekv_layer* L, const void* q, const int32_t* q_pos, int B, void* q_rope, void* q_abs) {
-  return AbsorbArgs{(const bf16*)q, q_pos, B, L->d_WukT, L->d_qdims, L->d_qkeep, L->d_idx, L->d_cs, (bf16*)q_rope, (bf16*)q_abs,
-                    L->n_h, L->d_h, L->r, L->kw, L->max_pos, L->d_status};
+// rows [b0, b0 + B) of the call's arrays
+inline AbsorbArgs absorb_args(const elitekv_layer* L, const void* q, const int32_t* q_pos, int b0, int B, void* q_rope, void* q_abs) {
+  const size_t at = (size_t)b0 * L->n_h;
+  return AbsorbArgs{(const bf16*)q + at * L->d_h, q_pos + b0, B, L->d_WukT, L->d_qdims, L->d_qkeep, L->d_idx, L->d_cs,
+                    (bf16*)q_rope + at * 2 * L->r, (bf16*)q_abs + at * L->kw, L->n_h, L->d_h, L->r, L->kw, L->max_pos, b0, L->d_status};
 }

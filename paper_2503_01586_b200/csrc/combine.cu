@@ -56,13 +56,13 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
                     const int32_t* seq_first, const bf16* __restrict__ Wuv,
                     float* __restrict__ slice_out /* [n_slices][B * rows][n_h][128] */,
                     int32_t* __restrict__ counters /* [n_h][groups], zeroed by the plan kernel */,
-                    bf16* __restrict__ out, int B, int rows, int n_h, int d_c) {
+                    bf16* __restrict__ out, int B, int rows, int n_h, int d_c, int g0, int n_groups) {
   __shared__ __align__(16) bf16 s_w[kFK][kFPitch];        // W_uv slice
   __shared__ __align__(16) bf16 s_o[2][kFB][kFPitch];     // merged latent outputs: bf16 head and remainder
   bf16 (*const s_hi)[kFPitch] = s_o[0];
   bf16 (*const s_lo)[kFPitch] = s_o[1];
   __shared__ int s_last;
-  const int h = blockIdx.x, slice = blockIdx.y, n_slices = gridDim.y, g = blockIdx.z;
+  const int h = blockIdx.x, slice = blockIdx.y, n_slices = gridDim.y, g = g0 + blockIdx.z;
   const int k0 = slice * kFK;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_rows = B * rows, r0 = g * kFB, nb = min(kFB, n_rows - r0);
@@ -219,7 +219,7 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
   // the block of a (head, group) that arrives last adds the slices in order
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&counters[h * gridDim.z + g], 1) == n_slices - 1;
+  if (tid == 0) s_last = atomicAdd(&counters[h * n_groups + g], 1) == n_slices - 1;
   __syncthreads();
   if (s_last) {
     __threadfence();
@@ -360,12 +360,16 @@ int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, v
   const int nv = (ws.rows > 0 ? ws.rows : 1) * L->n_h;
   if (ekv_combine_fast_ok(L)) {
     const int rows = ws.rows > 0 ? ws.rows : 1;
-    dim3 grid(L->n_h, L->vw / kFK, (B * rows + kFB - 1) / kFB);
+    const int n_groups = (B * rows + kFB - 1) / kFB;
     // at most 8 rows: idle warps share the rows' items (a 7B step of one sequence: 34.8 -> 32.4 us at 32
     // items, 8 sequences 50.1 -> 49.4); from 9 rows on at least half of the warps have a pair of their own
-    EKV_CUDA_OK(ekv_launch_pdl(B * rows <= 8 ? combine_fast_kernel<true> : combine_fast_kernel<false>, grid, dim3(kFThreads), 0, st, (const float*)ws.part_acc,
-                               (const float*)ws.part_ml, (const int32_t*)ws.seq_first, (const bf16*)L->d_Wuv,
-                               ws.slice_out, ws.counters, (bf16*)out, B, rows, L->n_h, L->vw));
+    const auto kern = B * rows <= 8 ? combine_fast_kernel<true> : combine_fast_kernel<false>;
+    for (int g0 = 0; g0 < n_groups; g0 += kGridZ) {      // one launch up to a million rows
+      const dim3 grid(L->n_h, L->vw / kFK, n_groups - g0 < kGridZ ? n_groups - g0 : kGridZ);
+      EKV_CUDA_OK(ekv_launch_pdl(kern, grid, dim3(kFThreads), 0, st, (const float*)ws.part_acc, (const float*)ws.part_ml,
+                                 (const int32_t*)ws.seq_first, (const bf16*)L->d_Wuv, ws.slice_out, ws.counters, (bf16*)out,
+                                 B, rows, L->n_h, L->vw, g0, n_groups));
+    }
     EKV_CUDA_OK(cudaGetLastError());
     return ELITEKV_OK;
   }

@@ -102,6 +102,8 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t* r, const bf16* p) {
 __device__ __forceinline__ void ekv_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void ekv_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+constexpr int kGridZ = 65535;        // largest third dimension of a grid
+
 // Leave for more dynamic shared memory than every kernel has anyway (48 KB with its static part: asked
 // for from 32 KB on; the call costs the host about half a microsecond).
 template <typename... KArgs>

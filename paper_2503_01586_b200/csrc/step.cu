@@ -53,7 +53,7 @@ int ekv_launch_step_prep(const elitekv_layer* L, const elitekv_cache* cache, con
                          void* q_abs, const PlanArgs& plan, cudaStream_t st) {
   const AbsorbShape s = absorb_shape(L, B);
   if (!absorb_ok(L, s)) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
-  const AbsorbArgs a = absorb_args(L, q, pos, B, q_rope, q_abs);
+  const AbsorbArgs a = absorb_args(L, q, pos, 0, B, q_rope, q_abs);
   const AppendArgs t = append_args(L, cache, cv, k_e, c, seq_id, pos, B);
   const int n_append = B < L->sm_count ? B : L->sm_count;      // a block per token; more tokens go round
   const int grid = 1 + n_append + L->n_h * (1 + s.slices * s.groups);

@@ -459,3 +459,33 @@ def test_project_append_table_on_any_8_bytes(ek, T):
         assert ek.elitekv_check_status(layer) == 0
         rows.append((rope, latent))
     assert all(torch.equal(a, b) for a, b in zip(*rows))
+
+
+def test_more_rows_than_a_grid_dimension(ek):
+    """Blocks of 16 rows (combine) and of 64 (query preparation) past the 65535 that a grid's third dimension
+    holds: sequences of one token, whose output is the up-projected latent, and absorbed queries whose
+    last rows are those of a small call."""
+    B = 16 * 65535 + 17
+    w = replace(gen.LLAMA7B_75, n_h=1, r=2, d_c=128, B=B, ctx=1)
+    layer = ek.Layer(1, w.d_h, w.r, w.d_c, gen.elite_index_sets(w), *(W := gen.up_projections(w, "cuda")), 2)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    latent = torch.randn((B, w.d_c), generator=g, device="cuda").to(torch.bfloat16)
+    rope = torch.zeros((B, 2 * w.r), dtype=torch.bfloat16, device="cuda")
+    q_rope, q_abs = torch.zeros((B, 1, 2 * w.r), dtype=torch.bfloat16, device="cuda"), torch.zeros((B, 1, w.d_c), dtype=torch.bfloat16, device="cuda")
+    lens = torch.ones(B, dtype=torch.int32, device="cuda")
+    ws = torch.empty(ek.elitekv_decode_workspace_size(layer, B), dtype=torch.uint8, device="cuda")
+    out = ek.elitekv_decode(layer, ek.make_cache(rope, latent, n_seqs=B, max_ctx=1), q_rope, q_abs, lens, ws)
+    assert ek.elitekv_check_status(layer) == 0
+    for at in (slice(0, 40), slice(B - 60, B)):
+        want = H.f64(latent[at]) @ H.f64(W[1])
+        assert np.linalg.norm(H.f64(out[at, 0]) - want) <= H.REL_L2_TOL * np.linalg.norm(want)
+    del latent, rope, q_rope, q_abs, ws, out
+    B = 64 * 65535 + 70
+    w = replace(w, d_h=16, d_c=8, B=B)
+    layer = ek.Layer(1, w.d_h, w.r, w.d_c, gen.elite_index_sets(w), *gen.up_projections(w, "cuda"), 2)
+    q = torch.randn((B, 1, w.d_h), generator=g, device="cuda").to(torch.bfloat16)
+    got = ek.elitekv_absorb_query(layer, q, lens.new_zeros(B))
+    assert ek.elitekv_check_status(layer) == 0
+    for at in (slice(0, 100), slice(B - 200, B)):
+        want = ek.elitekv_absorb_query(layer, q[at].contiguous(), lens.new_zeros(q[at].shape[0]))
+        assert all(torch.equal(a[at], b) for a, b in zip(got, want))
