@@ -522,6 +522,16 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
   const int n_out = rope_w + L->d_c;
   if (L->d % kPK != 0 || rope_w % kPN != 0 || L->d_c % kPN != 0) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
   if (T >= (1ll << 31)) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
+  // a grid's second dimension holds 65535 token tiles: more tokens than that in the smallest are several launches
+  constexpr long long kMost = 65535ll * kPM;
+  if (T > kMost) {
+    for (long long t = 0; t < T; t += kMost) {
+      const int rc = ekv_launch_project_append(L, cache, cv, (const bf16*)x + t * L->d, seq_id + t, pos + t,
+                                               T - t < kMost ? T - t : kMost, st);
+      if (rc != ELITEKV_OK) return rc;
+    }
+    return ELITEKV_OK;
+  }
   ProjArgs a;
   a.seq_id = seq_id;
   a.pos = pos;

@@ -489,3 +489,29 @@ def test_more_rows_than_a_grid_dimension(ek):
     for at in (slice(0, 100), slice(B - 200, B)):
         want = ek.elitekv_absorb_query(layer, q[at].contiguous(), lens.new_zeros(q[at].shape[0]))
         assert all(torch.equal(a[at], b) for a, b in zip(got, want))
+
+
+def test_project_append_more_tokens_than_a_grid_dimension(ek):
+    """More 128-token tiles than the 65535 of a grid's second dimension, at a depth that the paired forms
+    leave to them: the rows around the end are those of small calls."""
+    d, T, ctx = 64, 65535 * 128 + 200, 1000
+    w = replace(gen.LLAMA7B_75, n_h=16, r=4, d_c=128)
+    B, rope_w = -(-T // ctx), 128
+    g = torch.Generator(device="cuda").manual_seed(9)
+    W_ke, W_down = ((torch.randn((d, 128), generator=g, device="cuda") / 8).to(torch.bfloat16) for _ in range(2))
+    layer = ek.Layer(w.n_h, w.d_h, w.r, w.d_c, gen.elite_index_sets(w), *gen.up_projections(w, "cuda"), ctx, W_ke=W_ke, W_down=W_down)
+    x = torch.empty((T, d), dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    t = torch.arange(T, device="cuda")
+    seq, pos = (t // ctx).to(torch.int32), (t % ctx).to(torch.int32)
+    planes = [torch.zeros((B * ctx, n), dtype=torch.bfloat16, device="cuda") for n in (rope_w, w.d_c)]
+    cache = ek.make_cache(*planes, n_seqs=B, max_ctx=ctx)
+    ek.elitekv_project_append(layer, cache, x, seq, pos)
+    assert ek.elitekv_check_status(layer) == 0
+    for at in (slice(0, 300), slice(T - 400, T - 200), slice(T - 200, T)):
+        want = [p[at].clone() for p in planes]
+        assert all(p[at].any(dim=1).all() for p in planes)
+        for p in planes:
+            p[at] = 0
+        ek.elitekv_project_append(layer, cache, x[at].contiguous(), seq[at].contiguous(), pos[at].contiguous())
+        # the same fp32 sums in another order may round to the next bf16: one unit of 2^-7 at most
+        assert all(torch.allclose(p[at].float(), y.float(), rtol=2.0 ** -7, atol=1e-5) for p, y in zip(planes, want))
