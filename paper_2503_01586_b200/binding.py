@@ -312,7 +312,8 @@ def elitekv_ropelite_search(Q, K, r: int, rope_base: float = 10000.0, trace: boo
 
 
 def elitekv_copy(dst, src) -> None:
-    """Copy between a device tensor and a pinned host tensor of the same size, by a kernel."""
+    """Copy between a device tensor and a pinned host tensor of the same size, by a kernel.  Keep the
+    pinned tensor until the copy is through: its allocator does not see the kernel."""
     if dst.numel() * dst.element_size() != src.numel() * src.element_size():
         raise ValueError("elitekv_copy: sizes differ")
     if not (dst.is_contiguous() and src.is_contiguous()):
@@ -363,6 +364,16 @@ class DecodeStepRunner:
         self.d2h_bytes = self.out_host.numel() * self.out_host.element_size()
         self.graph = None
         self._want_graph, self._warm = graph, False
+        self._done, self._running = torch.cuda.Event(), False
+
+    def __del__(self):
+        # the copies are kernels that the allocator of pinned memory does not know of: the staging buffers
+        # go back to it (and to its next user) when the last step is through with them
+        if getattr(self, "_running", False):
+            try:
+                self._done.synchronize()
+            except Exception:
+                pass
 
     def _enqueue(self):
         d = self.dev
@@ -388,6 +399,9 @@ class DecodeStepRunner:
             self._warm = True
         if wait:
             torch.cuda.current_stream().synchronize()
+        else:
+            self._done.record()
+        self._running = not wait
         return self.out_host
 
 

@@ -306,6 +306,24 @@ def test_copy_both_ways(ek, n):
     assert (dev[n:] == 7).all() and (back[n:] == 9).all()
 
 
+@pytest.mark.parametrize("graph", [False, True])
+def test_step_runner_keeps_its_pinned_buffers_until_the_step_is_through(ek, graph):
+    """A runner that goes away with a step under way (behind 50 ms of other work) gives its pinned buffers
+    back when the step has read and written them, not before."""
+    w = gen.shrink(gen.TINY, B=2, ctx=20)
+    st = H.setup(w, lens=[20, 7])
+    run = ek.DecodeStepRunner(st.layer, st.cache, 2, "cuda", graph=graph)
+    for k, v in (("q", st.q), ("seq_id", torch.arange(2, dtype=torch.int32)), ("pos", st.lens - 1), ("lens", st.lens)):
+        run.host[k].copy_(v.cpu().view(run.host[k].shape))
+    for _ in range(3):
+        run.run()
+    torch.cuda._sleep(100_000_000)
+    run.run(wait=False)
+    stream = torch.cuda.current_stream()
+    assert not stream.query()
+    del run
+    assert stream.query()
+
 def test_copy_refuses_what_the_device_cannot_address(ek):
     dev = torch.zeros(64, dtype=torch.uint8, device="cuda")
     for dst, src in ((dev[:32], torch.zeros(32, dtype=torch.uint8)), (dev[1:33], dev[32:])):
