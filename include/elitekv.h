@@ -188,8 +188,8 @@ int elitekv_decode_step(const elitekv_layer* layer, const elitekv_cache* cache, 
 
 /* Copies bytes between device memory and PINNED host memory (either way) with a kernel on `stream`:
  * before and after elitekv_decode_step such copies overlap the launches of its kernels.  dst and src
- * are 16-byte aligned; memory that the device cannot address is refused (ELITEKV_ERR_INVALID_ARG).
- * Both stay valid until the stream has passed the copy. */
+ * are 16-byte aligned; memory that the device cannot address, another device's included, is refused
+ * (ELITEKV_ERR_INVALID_ARG).  Both stay valid until the stream has passed the copy. */
 int elitekv_copy(void* dst, const void* src, int64_t bytes, elitekv_stream_t stream);
 
 /* Several query rows per sequence over the cache, with the causal rule (Section 3.1: the score

@@ -6,6 +6,7 @@
 // A 7B step from host arrays to a host result: B1 58 -> 49 us, B16 92 -> 73, B64 (0.8 MB in, 0.5 MB
 // out) 245 -> 189.
 #include "common.cuh"
+#include "copy.cuh"
 
 namespace {
 
@@ -30,20 +31,22 @@ copy_kernel(unsigned char* dst, const unsigned char* src, long long bytes) {
   if (t < (bytes & 15)) dst[(n << 4) + t] = __ldcv(src + (n << 4) + t);
 }
 
-bool device_reads(const void* p) {
+bool device_reads(const void* p, int device) {
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return at.type != cudaMemoryTypeUnregistered && at.devicePointer == p;
+  return ekv_addressable(at, p, device);
 }
 
 }  // namespace
 
 extern "C" int elitekv_copy(void* dst, const void* src, int64_t bytes, elitekv_stream_t stream) {
   if (!dst || !src || bytes < 0 || (((uintptr_t)dst | (uintptr_t)src) & 15)) return ELITEKV_ERR_INVALID_ARG;
-  if (!device_reads(dst) || !device_reads(src)) return ELITEKV_ERR_INVALID_ARG;
+  int device = 0;
+  EKV_CUDA_OK(cudaGetDevice(&device));
+  if (!device_reads(dst, device) || !device_reads(src, device)) return ELITEKV_ERR_INVALID_ARG;
   if (bytes == 0) return ELITEKV_OK;
   const long long per_block = 16ll * kCopyThreads;
   long long blocks = (bytes + per_block - 1) / per_block;

@@ -61,3 +61,29 @@ def test_struct_layouts_match_the_header(tmp_path):
     want = [ctypes.sizeof(binding.Params)] + [getattr(binding.Params, f).offset for f in fields_p]
     want += [ctypes.sizeof(binding.CacheDesc)] + [getattr(binding.CacheDesc, f).offset for f in fields_c]
     assert got == want
+
+
+def test_copy_takes_no_memory_of_another_device(tmp_path):
+    """The rule of elitekv_copy on the attributes that the runtime reports of a pointer."""
+    import subprocess
+    src = tmp_path / "rule.cpp"
+    src.write_text('''#include "copy.cuh"
+#include <cstdio>
+#include <initializer_list>
+int main() {
+  char x, y;
+  const cudaMemoryType kinds[] = {cudaMemoryTypeUnregistered, cudaMemoryTypeHost, cudaMemoryTypeDevice, cudaMemoryTypeManaged};
+  for (cudaMemoryType k : kinds)
+    for (int device = 0; device < 2; ++device)
+      for (void* p : {(void*)&x, (void*)&y}) {
+        cudaPointerAttributes at = {};
+        at.type = k; at.device = device; at.devicePointer = p;
+        std::printf("%d", (int)ekv_addressable(at, &x, 0));
+      }
+}''')
+    exe = tmp_path / "rule"
+    subprocess.run(["g++", "-std=c++17", "-I/usr/local/cuda/include", "-I", os.path.join(ROOT, "paper_2503_01586_b200", "csrc"),
+                    str(src), "-o", str(exe)], check=True)
+    got = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout
+    # same address or another, on this device and on another one: unregistered, pinned, device, managed
+    assert got == "0000" + "1010" + "1000" + "1010"
