@@ -11,17 +11,18 @@
 
 namespace {
 
+template <class T>
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const PlanArgs a) {
   ekv_pdl_wait();         // earlier kernels may still read the arrays written here
   ekv_pdl_trigger();
-  __shared__ PlanShared sh;
+  __shared__ PlanShared<T> sh;
   plan_any(a, sh);
 }
 
 }  // namespace
 
 int ekv_launch_plan(const PlanArgs& a, cudaStream_t st) {
-  EKV_CUDA_OK(ekv_launch_pdl(plan_kernel, dim3(1), dim3(kPlanThreads), 0, st, a));
+  EKV_CUDA_OK(ekv_launch_pdl(plan_narrow(a) ? plan_kernel<int> : plan_kernel<long long>, dim3(1), dim3(kPlanThreads), 0, st, a));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }

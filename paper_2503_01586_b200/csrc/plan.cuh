@@ -7,31 +7,33 @@
 constexpr int kPlanThreads = 256;
 constexpr int kPlanStage = 4096;       // items whose worker ids are staged in shared memory
 
+// T: what tiles are summed in.  Lengths of up to 2^31 - 1 tokens in tiles of one pass 2^31 with two sequences;
+// what a device's memory holds is far below it (plan_narrow), and 64-bit sums there cost a step of one
+// sequence 0.6 us of 39.
+template <class T>
 struct __align__(16) PlanShared {        // the block's shared memory
   long long total;
-  long long warp_tot[kPlanThreads / 32];
-  long long g0[kPlanThreads];
-  int first[kPlanThreads], len[kPlanThreads], tiles[kPlanThreads];
+  T warp_tot[kPlanThreads / 32], g0[kPlanThreads], tiles[kPlanThreads];
+  int first[kPlanThreads], len[kPlanThreads];
   short w0[kPlanThreads], wk[kPlanStage];    // wk: worker of each item (n_workers < 32768)
 };
 
-// exclusive scan over the block (warp shuffles + one shared array of warp totals); tiles are summed in
-// 64 bits: lengths of up to 2^31 - 1 tokens in tiles of one pass 2^31 with two sequences
-template <class T>
-__device__ __forceinline__ T block_exclusive_scan(T v, long long* warp_tot, T* total) {
+// exclusive scan over the block (warp shuffles + one shared array of warp totals)
+template <class V, class T>
+__device__ __forceinline__ V block_exclusive_scan(V v, T* warp_tot, V* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T incl = v;
+  V incl = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const T x = __shfl_up_sync(0xffffffffu, incl, o);
+    const V x = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += x;
   }
   if (lane == 31) warp_tot[warp] = incl;
   __syncthreads();
-  T before = 0, all = 0;
+  V before = 0, all = 0;
 #pragma unroll
   for (int w = 0; w < kPlanThreads / 32; ++w) {
-    const T t = (T)warp_tot[w];
+    const V t = (V)warp_tot[w];
     if (w < warp) before += t;
     all += t;
   }
@@ -66,10 +68,19 @@ struct PlanArgs {
   int32_t* status;
   int overhead;
 };
+// B lengths of up to max_len tokens make less than 2^31 tiles, and the tile that holds the last token ends below 2^31
+inline bool plan_narrow(int B, int tile, long long max_len, int overhead) {
+  return max_len + tile <= 0x7fffffffLL && (max_len / tile + 1 + overhead) * B <= 0x7fffffffLL;
+}
+inline bool plan_narrow(const PlanArgs& a) { return plan_narrow(a.B, a.tile, a.max_len, a.overhead); }
 
 // 32-bit division where the operands allow it (a 64-bit one is a subroutine of over 100 instructions)
 __device__ __forceinline__ long long plan_div(long long x, long long y) {
   return ((unsigned long long)(x | y) >> 32) == 0 ? (long long)((unsigned)x / (unsigned)y) : x / y;
+}
+template <class T>
+__device__ __forceinline__ T plan_tiles(int n, int tile) {
+  return sizeof(T) == 8 ? (T)plan_div((long long)n + tile - 1, tile) : ((T)n + tile - 1) / tile;
 }
 
 // Batches of at most a sequence per thread: both plans in one trip for the lengths, two scans and one
@@ -80,19 +91,19 @@ __device__ __forceinline__ long long plan_div(long long x, long long y) {
 __device__ __forceinline__ bool plan_small_ok(const PlanArgs& a) {
   return a.B <= kPlanThreads && a.n_workers + a.B <= kPlanStage;
 }
-__device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
-  long long *const warp_tot = sh.warp_tot, *const s_g0 = sh.g0;
-  int *const s_first = sh.first, *const s_len = sh.len, *const s_tiles = sh.tiles;
+template <class T>
+__device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh) {
+  T *const warp_tot = sh.warp_tot, *const s_g0 = sh.g0, *const s_tiles = sh.tiles;
+  int *const s_first = sh.first, *const s_len = sh.len;
   short *const s_w0 = sh.w0, *const s_wk = sh.wk;
   const int t = threadIdx.x, B = a.B;
   const bool balanced = a.n_workers > 0;
   const int overhead = balanced ? a.overhead : 0;      // empty tiles in front of every sequence
   const int n = t < B ? checked_len(a.seq_lens, t, a.max_len, a.status, true) : 0;
   for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
-  const int real = n > 0 ? (int)plan_div((long long)n + a.tile - 1, a.tile) : 0;
-  const long long tiles = real > 0 ? (long long)real + overhead : 0;
-  long long sum;
-  const long long g0 = block_exclusive_scan(tiles, warp_tot, &sum);
+  const T tiles = n > 0 ? (T)plan_div((long long)n + a.tile - 1, a.tile) + overhead : 0;
+  T sum;
+  const T g0 = block_exclusive_scan(tiles, warp_tot, &sum);
   const long long total = sum > 0 ? sum : 1;
   const long long nw = balanced ? (total < a.n_workers ? total : a.n_workers) : 1;
   auto bound = [&](long long w) -> long long { return plan_div(w * total, nw); };
@@ -101,7 +112,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
   if (tiles > 0) {
     if (balanced) {
       w0 = owner(g0 + overhead);
-      pieces = owner(g0 + tiles - 1) - w0 + 1;
+      pieces = owner((long long)g0 + tiles - 1) - w0 + 1;
     } else {
       const long long budget = a.max_items - B > 0 ? a.max_items - B : 1;
       const long long target = plan_div(total + budget - 1, budget);
@@ -112,7 +123,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
   const int first = block_exclusive_scan(pieces, warp_tot, &n_items);
   if (t < B) {
     a.seq_first[t] = first;
-    s_first[t] = first; s_g0[t] = g0; s_len[t] = n; s_tiles[t] = real; s_w0[t] = (short)w0;
+    s_first[t] = first; s_g0[t] = g0; s_len[t] = n; s_tiles[t] = tiles; s_w0[t] = (short)w0;
   }
   if (t == 0) a.seq_first[B] = n_items;
   __syncthreads();
@@ -124,13 +135,14 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
         const int mid = (lo + hi) >> 1;
         if (s_first[mid] <= it) lo = mid; else hi = mid;
       }
-      const int j = it - s_first[lo], len = s_len[lo], tl = s_tiles[lo];
+      const int j = it - s_first[lo], len = s_len[lo];
+      const T tl = s_tiles[lo];
       int ta, tb, w = 0;                     // tiles of the sequence
       if (balanced) {
-        const long long base = s_g0[lo] + overhead;
+        const long long base = (long long)s_g0[lo] + overhead;
         w = s_w0[lo] + j;
         ta = (int)(max(base, bound(w)) - base);
-        tb = (int)(min(base + tl, bound(w + 1)) - base);
+        tb = (int)(min((long long)s_g0[lo] + tl, bound(w + 1)) - base);
         s_wk[it] = (short)w;
       } else {
         const int np = (lo + 1 < B ? s_first[lo + 1] : n_items) - s_first[lo];
@@ -138,7 +150,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
         tb = (int)plan_div((long long)tl * (j + 1), np);
       }
       const int tok0 = ta * a.tile;
-      item = make_int4(lo, tok0, (int)min((long long)tb * a.tile, (long long)len) - tok0, w);
+      item = make_int4(lo, tok0, (int)min((T)tb * a.tile, (T)len) - tok0, w);
     }
     *(int4*)(a.items + 4 * it) = item;
   }
@@ -155,7 +167,8 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared& sh) {
   }
 }
 
-__device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
+template <class T>
+__device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared<T>& sh) {
   const int32_t* __restrict__ seq_lens = a.seq_lens;
   const int B = a.B, tile = a.tile, max_items = a.max_items, n_zero = a.n_zero;
   int32_t* __restrict__ items = a.items;
@@ -163,7 +176,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
   int32_t* __restrict__ zero_ints = a.zero_ints;
   const long long max_len = a.max_len;
   int32_t* status = a.status;
-  long long* const warp_tot = sh.warp_tot;
+  T* const warp_tot = sh.warp_tot;
   long long& s_total = sh.total;
   const int t = threadIdx.x;
   for (int i = t; i < n_zero; i += blockDim.x) zero_ints[i] = 0;
@@ -172,7 +185,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
   long long local = 0;
   for (int b = t; b < B; b += blockDim.x) {
     int n = checked_len(seq_lens, b, max_len, status, true);
-    local += n > 0 ? plan_div((long long)n + tile - 1, tile) : 0;
+    local += n > 0 ? plan_tiles<T>(n, tile) : 0;
   }
   if (local) atomicAdd((unsigned long long*)&s_total, (unsigned long long)local);
   __syncthreads();
@@ -187,7 +200,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
     int n = 0, tiles = 0, pieces = 0;
     if (b < B) {
       n = checked_len(seq_lens, b, max_len, status, false);
-      tiles = n > 0 ? (int)plan_div((long long)n + tile - 1, tile) : 0;
+      tiles = n > 0 ? (int)plan_tiles<T>(n, tile) : 0;
       pieces = (int)((tiles + target - 1) / target);
     }
     int chunk_total;
@@ -198,7 +211,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
         const int ta = (int)((long long)tiles * j / pieces);
         const int tb = (int)((long long)tiles * (j + 1) / pieces);
         const int tok0 = ta * tile;
-        const int tok1 = (int)min((long long)tb * tile, (long long)n);
+        const int tok1 = (int)min((T)tb * tile, (T)n);
         const int it = first + j;
         if (it < max_items) *(int4*)(items + 4 * it) = make_int4(b, tok0, tok1 - tok0, 0);
       }
@@ -219,7 +232,8 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared& sh) {
 // result to write out), and a worker whose range contains the start of a sequence has one item
 // more than the others.  The tile list therefore carries `overhead` empty tiles in front of every
 // sequence: they take room in a worker's quota and hold no tokens.
-__device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh) {
+template <class T>
+__device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& sh) {
   const int32_t* __restrict__ seq_lens = a.seq_lens;
   const int B = a.B, tile = a.tile, n_workers = a.n_workers, max_items = a.max_items, overhead = a.overhead, n_zero = a.n_zero;
   int32_t* __restrict__ items = a.items;
@@ -228,7 +242,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
   int32_t* __restrict__ zero_ints = a.zero_ints;
   const long long max_len = a.max_len;
   int32_t* status = a.status;
-  long long* const warp_tot = sh.warp_tot;
+  T* const warp_tot = sh.warp_tot;
   long long& s_total = sh.total;
   short* const s_wk = sh.wk;
   const int t = threadIdx.x;
@@ -238,7 +252,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
   long long local = 0;
   for (int b = t; b < B; b += blockDim.x) {
     int n = checked_len(seq_lens, b, max_len, status, true);
-    local += n > 0 ? plan_div((long long)n + tile - 1, tile) + overhead : 0;
+    local += n > 0 ? plan_tiles<T>(n, tile) + overhead : 0;
   }
   if (local) atomicAdd((unsigned long long*)&s_total, (unsigned long long)local);
   __syncthreads();
@@ -248,19 +262,19 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
   const long long nw = total < n_workers ? total : n_workers;
   auto bound = [&](long long w) -> long long { return w * total / nw; };
   auto owner = [&](long long g) -> int { return (int)(((g + 1) * nw - 1) / total); };
-  long long carry_tiles = 0;
+  T carry_tiles = 0;
   int carry_items = 0;
   {
     for (int b0 = 0; b0 < B; b0 += blockDim.x) {
       const int b = b0 + t;
       int n = 0;
-      long long tiles = 0;
+      T tiles = 0;
       if (b < B) {
         n = checked_len(seq_lens, b, max_len, status, false);
-        tiles = n > 0 ? plan_div((long long)n + tile - 1, tile) + overhead : 0;     // with the empty tiles in front
+        tiles = n > 0 ? plan_tiles<T>(n, tile) + overhead : 0;     // with the empty tiles in front
       }
-      long long chunk_tiles;
-      const long long g0 = carry_tiles + block_exclusive_scan(tiles, warp_tot, &chunk_tiles);
+      T chunk_tiles;
+      const T g0 = carry_tiles + block_exclusive_scan(tiles, warp_tot, &chunk_tiles);
       int pieces = 0, w0 = 0;
       if (tiles > 0) {
         w0 = owner(g0 + overhead);                                // workers that hold real tiles
@@ -272,10 +286,10 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
       if (b < B) {
         seq_first[b] = first;
         for (int j = 0; j < pieces; ++j) {
-          const long long ga = max(g0 + overhead, bound(w0 + j));
-          const long long gb = min(g0 + tiles, bound(w0 + j + 1));
+          const long long ga = max((long long)g0 + overhead, bound(w0 + j));
+          const long long gb = min((long long)g0 + tiles, bound(w0 + j + 1));
           const int tok0 = (int)(ga - g0 - overhead) * tile;
-          const int tok1 = (int)min((gb - g0 - overhead) * tile, (long long)n);
+          const int tok1 = (int)min((T)(gb - g0 - overhead) * tile, (T)n);
           const int it = first + j;
           if (it < max_items) *(int4*)(items + 4 * it) = make_int4(b, tok0, tok1 - tok0, w0 + j);
           if (it < kPlanStage) s_wk[it] = (short)(w0 + j);
@@ -316,7 +330,8 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared& sh)
   }
 }
 
-__device__ __forceinline__ void plan_any(const PlanArgs& a, PlanShared& sh) {
+template <class T>
+__device__ __forceinline__ void plan_any(const PlanArgs& a, PlanShared<T>& sh) {
   if (plan_small_ok(a)) plan_small(a, sh);
   else if (a.n_workers > 0) plan_balanced(a, sh);
   else plan_even(a, sh);

@@ -26,7 +26,7 @@ step_prep_kernel(const AbsorbArgs q, const AppendArgs t, const PlanArgs p, int n
   int blk = blockIdx.x;
   if (blk == 0) {
     ekv_pdl_wait();
-    plan_any(p, *(PlanShared*)smem_b);
+    plan_any(p, *(PlanShared<int>*)smem_b);
     return;
   }
   blk -= 1;
@@ -53,11 +53,16 @@ int ekv_launch_step_prep(const elitekv_layer* L, const elitekv_cache* cache, con
                          void* q_abs, const PlanArgs& plan, cudaStream_t st) {
   const AbsorbShape s = absorb_shape(L, B);
   if (!absorb_ok(L, s)) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
+  if (!plan_narrow(plan)) {      // (lengths that only pages shared by many sequences can have)
+    int rc = ekv_launch_append(L, cache, cv, k_e, c, seq_id, pos, B, st);
+    if (rc == ELITEKV_OK) rc = ekv_launch_absorb(L, q, pos, B, q_rope, q_abs, st);
+    return rc == ELITEKV_OK ? ekv_launch_plan(plan, st) : rc;
+  }
   const AbsorbArgs a = absorb_args(L, q, pos, 0, B, q_rope, q_abs);
   const AppendArgs t = append_args(L, cache, cv, k_e, c, seq_id, pos, B);
   const int n_append = B < L->sm_count ? B : L->sm_count;      // a block per token; more tokens go round
   const int grid = 1 + n_append + L->n_h * (1 + s.slices * s.groups);
-  const size_t smem = s.smem > sizeof(PlanShared) ? s.smem : sizeof(PlanShared);
+  const size_t smem = s.smem > sizeof(PlanShared<int>) ? s.smem : sizeof(PlanShared<int>);
   auto launch = [&](auto kern) -> int {
     EKV_CUDA_OK(ekv_allow_smem(kern, smem));
     EKV_CUDA_OK(ekv_launch_pdl(kern, dim3((unsigned)grid), dim3(kAbsorbThreads), smem, st, a, t, plan, n_append,
