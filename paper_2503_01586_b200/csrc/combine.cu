@@ -48,7 +48,8 @@ constexpr int kFThreads = 256;
 constexpr int kFPitch = kFD + 8; // shared-memory row pitch in bf16: 16 bytes of padding keep ldmatrix free of bank conflicts
 constexpr int kFAhead = 4;       // partial results per row in flight beside the statistics
 
-template <bool kShare>
+// kMore: blocks start at group g0 of n_groups (calls of more rows than one grid holds)
+template <bool kShare, bool kMore>
 __global__ void __launch_bounds__(kFThreads, kShare ? 3 : 4)
 combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by the split-K kernel while this
                                                                    // kernel may already be resident: read
@@ -62,7 +63,7 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
   bf16 (*const s_hi)[kFPitch] = s_o[0];
   bf16 (*const s_lo)[kFPitch] = s_o[1];
   __shared__ int s_last;
-  const int h = blockIdx.x, slice = blockIdx.y, n_slices = gridDim.y, g = g0 + blockIdx.z;
+  const int h = blockIdx.x, slice = blockIdx.y, n_slices = gridDim.y, g = kMore ? g0 + blockIdx.z : blockIdx.z;
   const int k0 = slice * kFK;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_rows = B * rows, r0 = g * kFB, nb = min(kFB, n_rows - r0);
@@ -219,7 +220,7 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
   // the block of a (head, group) that arrives last adds the slices in order
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&counters[h * n_groups + g], 1) == n_slices - 1;
+  if (tid == 0) s_last = atomicAdd(&counters[h * (kMore ? n_groups : gridDim.z) + g], 1) == n_slices - 1;
   __syncthreads();
   if (s_last) {
     __threadfence();
@@ -363,7 +364,9 @@ int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, v
     const int n_groups = (B * rows + kFB - 1) / kFB;
     // at most 8 rows: idle warps share the rows' items (a 7B step of one sequence: 34.8 -> 32.4 us at 32
     // items, 8 sequences 50.1 -> 49.4); from 9 rows on at least half of the warps have a pair of their own
-    const auto kern = B * rows <= 8 ? combine_fast_kernel<true> : combine_fast_kernel<false>;
+    const auto kern = n_groups > kGridZ ? combine_fast_kernel<false, true>
+                      : B * rows <= 8   ? combine_fast_kernel<true, false>
+                                        : combine_fast_kernel<false, false>;
     for (int g0 = 0; g0 < n_groups; g0 += kGridZ) {      // one launch up to a million rows
       const dim3 grid(L->n_h, L->vw / kFK, n_groups - g0 < kGridZ ? n_groups - g0 : kGridZ);
       EKV_CUDA_OK(ekv_launch_pdl(kern, grid, dim3(kFThreads), 0, st, (const float*)ws.part_acc, (const float*)ws.part_ml,
