@@ -186,7 +186,7 @@ int ekv_launch_append(const elitekv_layer* L, const elitekv_cache* cache, const 
     const size_t smem = (size_t)kStages * G * tok_bytes;
     const long long n_groups = (T + G - 1) / G;
     const long long want = (long long)L->sm_count * kBlocksPerSm;
-    EKV_CUDA_OK(cudaFuncSetAttribute(append_staged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    EKV_CUDA_OK(ekv_allow_smem(append_staged_kernel, smem));
     append_staged_kernel<<<(unsigned)(n_groups < want ? n_groups : want), kStagedThreads, smem, st>>>(a, G);
     EKV_CUDA_OK(cudaGetLastError());
     return ELITEKV_OK;

@@ -105,10 +105,13 @@ __device__ __forceinline__ void ekv_pdl_trigger() { asm volatile("griddepcontrol
 constexpr int kGridZ = 65535;        // largest third dimension of a grid
 
 // Leave for more dynamic shared memory than every kernel has anyway (48 KB with its static part: asked
-// for from 32 KB on; the call costs the host about half a microsecond).
+// for from 32 KB on; the call costs the host about half a microsecond).  The leave belongs to the kernel, which
+// layers of several shapes share: it never shrinks, so that a thread that steps a smaller layer does not take it
+// from a launch that another thread is about to make.
+cudaError_t ekv_raise_smem(const void* kern, int bytes);
 template <typename... KArgs>
 inline cudaError_t ekv_allow_smem(void (*kern)(KArgs...), size_t bytes) {
-  return bytes > 32 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
+  return bytes > 32 * 1024 ? ekv_raise_smem((const void*)kern, (int)bytes) : cudaSuccess;
 }
 
 template <typename... KArgs, typename... Args>

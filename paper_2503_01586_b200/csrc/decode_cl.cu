@@ -917,7 +917,7 @@ int ekv_cl_max_clusters(const elitekv_layer* L) {
     const auto key = std::make_tuple(L->device, K::C, smem);
     const auto it = known.find(key);
     if (it != known.end()) return it->second;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 0;
+    if (ekv_allow_smem(kern, smem) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(K::C);
     cfg.blockDim = dim3(K::THREADS);
@@ -974,7 +974,7 @@ int ekv_launch_decode_cl(const elitekv_layer* L, const elitekv_cache* cache, con
     a.max_pages_per_seq = cv.max_pages_per_seq;
     a.vw = L->vw;
     a.scale_log2e = L->scale * 1.4426950408889634f;
-    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    EKV_CUDA_OK(ekv_allow_smem(kern, smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ws.n_workers * K::C));
     cfg.blockDim = dim3(K::THREADS);

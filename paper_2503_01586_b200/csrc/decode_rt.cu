@@ -702,7 +702,7 @@ cudaLaunchAttribute rt_cluster_attr() {
 template <int R2>
 int rt_launch(const CUtensorMap& m_lat, const CUtensorMap& m_q, const RtArgs& a,
               int n_workers, int smem, cudaStream_t st) {
-  EKV_CUDA_OK(cudaFuncSetAttribute(decode_rt_kernel<R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  EKV_CUDA_OK(ekv_allow_smem(decode_rt_kernel<R2>, smem));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * n_workers);
   cfg.blockDim = dim3(kRtThreads);
@@ -723,7 +723,7 @@ int rt_launch(const CUtensorMap& m_lat, const CUtensorMap& m_q, const RtArgs& a,
 // free SMs of one GPC).
 template <int R2>
 int rt_max_clusters(int smem) {
-  if (cudaFuncSetAttribute(decode_rt_kernel<R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+  if (ekv_allow_smem(decode_rt_kernel<R2>, smem) != cudaSuccess)
     return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2);

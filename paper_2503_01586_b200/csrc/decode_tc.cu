@@ -678,7 +678,7 @@ int ekv_launch_decode_tc(const elitekv_layer* L, const elitekv_cache* cache, con
   a.scale_log2e = L->scale * 1.4426950408889634f;
   const int smem = N == 32 ? Smem<32>::total(L->d_c) : Smem<16>::total(L->d_c);
   auto launch = [&](auto kern) -> int {
-    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    EKV_CUDA_OK(ekv_allow_smem(kern, smem));
     const dim3 grid(ws.n_workers * a.n_groups);
     // Blocks that share tiles (head groups, output shares, query rows) have to sit on neighbouring SMs,
     // as blocks of a grid that starts on an empty device do.  A dependent launch places them wherever an

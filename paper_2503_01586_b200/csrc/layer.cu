@@ -3,6 +3,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <mutex>
 #include <vector>
 
 #include <stdio.h>
@@ -241,6 +242,30 @@ extern "C" int elitekv_profile_collect(elitekv_layer* L, float* total_ms, int32_
   *launches = p->count;
   p->count = 0;
   return ELITEKV_OK;
+}
+
+cudaError_t ekv_raise_smem(const void* kern, int bytes) {
+  struct Leave {
+    const void* kern;
+    int device, bytes;
+  };
+  constexpr int kMost = 512;             // kernels x devices: a few dozen kernels on up to eight devices
+  static std::mutex mutex;
+  static Leave known[kMost];
+  static int n = 0;
+  int device = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mutex);             // held over the call: two sizes are set in order
+  int i = 0;
+  while (i < n && (known[i].kern != kern || known[i].device != device)) ++i;
+  if (i < n && known[i].bytes > bytes) bytes = known[i].bytes;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && i < kMost) {
+    known[i] = Leave{kern, device, bytes};
+    if (i == n) ++n;
+  }
+  return e;
 }
 
 int ekv_make_view(const elitekv_cache* c, CacheView* v) {

@@ -568,7 +568,7 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
     if (rcb == ELITEKV_OK) rcb = make_map(&b_w, L->d_WcatT, (unsigned long long)n_out, (unsigned long long)L->d, kBN / 2);
     if (rcb != ELITEKV_OK) return rcb;
     const auto kern = form == 2 ? project_append_pair_kernel<2> : project_append_pair_kernel<1>;
-    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_pair));
+    EKV_CUDA_OK(ekv_allow_smem(kern, smem_pair));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * (n_out / kBN)), (unsigned)((T + 256 * form - 1) / (256 * form)));
     cfg.blockDim = dim3(kBThreads);
@@ -597,7 +597,7 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
   if (rc == ELITEKV_OK) rc = make_map(&m_w, L->d_WcatT, (unsigned long long)n_out, (unsigned long long)L->d, kPN);
   if (rc != ELITEKV_OK) return rc;
   auto launch = [&](auto kern) -> int {
-    EKV_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    EKV_CUDA_OK(ekv_allow_smem(kern, smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(n_out / kPN), (unsigned)((T + kPM - 1) / kPM), split);
     cfg.blockDim = dim3(kPThreads);

@@ -533,3 +533,43 @@ def test_project_append_more_tokens_than_a_grid_dimension(ek):
         ek.elitekv_project_append(layer, cache, x[at].contiguous(), seq[at].contiguous(), pos[at].contiguous())
         # the same fp32 sums in another order may round to the next bf16: one unit of 2^-7 at most
         assert all(torch.allclose(p[at].float(), y.float(), rtol=2.0 ** -7, atol=1e-5) for p, y in zip(planes, want))
+
+
+def test_layers_of_several_shapes_step_in_several_threads(ek):
+    """Threads that step layers whose kernels are the same and want more or less shared memory each: no
+    launch is refused, and the outputs are those of a thread alone."""
+    import functools
+    import threading
+    shapes = [gen.LLAMA7B_75, gen.SWEEP_75_SLRD, replace(gen.LLAMA7B_75, d_c=1024), gen.SWEEP_75_SLRD]
+    steps = []
+    for w in shapes:
+        st = H.setup(gen.shrink(w, B=2, ctx=100), lens=[100, 70])
+        last = torch.from_numpy(st.starts[1:] - 1).cuda()
+        k_e, c, seq, pos = (x[last].contiguous() for x in (st.k_e, st.c, st.seq_id, st.pos))
+        q_rope, q_abs, out = (torch.empty((2, w.n_h, n), dtype=torch.bfloat16, device="cuda") for n in (2 * w.r, st.layer.kw, w.d_h))
+        steps.append((st, functools.partial(ek.elitekv_decode_step, st.layer, st.cache, k_e, c, seq, pos, st.q, st.lens_dev,
+                                            q_rope, q_abs, st.workspace, out)))
+    alone = []
+    for st, step in steps:
+        alone.append(step().clone())
+    torch.cuda.synchronize()
+    failed = []
+
+    def loop(step):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(2000):
+                    step()
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=loop, args=(step,)) for _, step in steps]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed[:2]
+    for (st, step), want in zip(steps, alone):
+        assert ek.elitekv_check_status(st.layer) == 0
+        assert torch.equal(step(), want)
