@@ -573,3 +573,26 @@ def test_layers_of_several_shapes_step_in_several_threads(ek):
     for (st, step), want in zip(steps, alone):
         assert ek.elitekv_check_status(st.layer) == 0
         assert torch.equal(step(), want)
+
+
+def test_step_of_a_cache_that_declares_more_tiles_than_31_bits_hold(ek):
+    """A page table of 2048 entries for pages of 2^20 tokens: the plan's sums are 64 bits wide and the step's
+    front end is the separate launches, with the same bits as the three calls."""
+    w = replace(gen.TINY, B=2)
+    layer = ek.Layer(w.n_h, w.d_h, w.r, w.d_c, gen.elite_index_sets(w), *gen.up_projections(w, "cuda"), 300)
+    table = torch.full((2, 2048), -1, dtype=torch.int32, device="cuda")
+    table[:, 0] = torch.tensor([1, 0], dtype=torch.int32, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(3)
+    rand = lambda *shape: torch.empty(shape, dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    lens = torch.tensor([270, 31], dtype=torch.int32, device="cuda")
+    seq, pos = torch.arange(2, dtype=torch.int32, device="cuda"), lens - 1
+    k_e, c, q = rand(2, w.n_h, w.r, 2), rand(2, w.d_c), rand(2, w.n_h, w.d_h)
+    rope, latent = rand(2 << 20, w.n_h * 2 * w.r), rand(2 << 20, w.d_c)
+    cache = ek.make_cache(rope, latent, n_seqs=2, page_table=table, page_size=1 << 20)
+    ws = torch.empty(ek.elitekv_decode_workspace_size(layer, 2), dtype=torch.uint8, device="cuda")
+    q_rope, q_abs, out = (torch.empty((2, w.n_h, n), dtype=torch.bfloat16, device="cuda") for n in (2 * w.r, layer.kw, w.d_h))
+    ek.elitekv_decode_step(layer, cache, k_e, c, seq, pos, q, lens, q_rope, q_abs, ws, out)
+    assert ek.elitekv_check_status(layer) == 0
+    assert torch.equal(latent[(table[:, 0].long() << 20) + pos.long()], c)
+    want = ek.elitekv_decode(layer, cache, *ek.elitekv_absorb_query(layer, q, pos), lens, ws)
+    assert torch.isfinite(out).all() and out.any() and torch.equal(out, want)
