@@ -25,14 +25,6 @@ struct AbsorbArgs {
   int32_t* status;
 };
 
-__device__ __forceinline__ void absorb_mma(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-      "{%0, %1, %2, %3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // Query RoPE of one head (every sequence).
 __device__ __forceinline__ void absorb_rope(const AbsorbArgs& a, int h) {
   const int32_t* dims = a.qdims + (size_t)h * a.d_h;
@@ -134,8 +126,8 @@ __device__ __forceinline__ void absorb_block(const AbsorbArgs& a, int h, int k0,
       for (int mt = 0; mt < MT; ++mt) {
         uint32_t x[4];
         ldmatrix_x4(x, s_q + (16 * mt + (lane & 15)) * qpitch + kk + (lane >> 4) * 8);
-        absorb_mma(acc[mt][0], x, w[0], w[1]);
-        absorb_mma(acc[mt][1], x, w[2], w[3]);
+        mma_bf16_16816(acc[mt][0], x, w[0], w[1]);
+        mma_bf16_16816(acc[mt][1], x, w[2], w[3]);
       }
     }
   }
