@@ -8,8 +8,7 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Which split-K kernel serves a layer (and cache): 1 = generic CUDA-core kernel, 2 = two-pass
 // tcgen05 kernel, 3 = resident-tile tcgen05 kernel on block pairs, 4 = tcgen05 kernel on larger
-// clusters, -1 = none.  `cache` may be
-// null (shape-only question).
+// clusters, -1 = none.  `cache` may be null (shape-only question).
 int select_kernel(const elitekv_layer* L, const elitekv_cache* cache) {
   const bool tc = ekv_tc_supported(L, cache) != 0;
   const bool rt = ekv_rt_supported(L, cache) != 0;
@@ -19,9 +18,10 @@ int select_kernel(const elitekv_layer* L, const elitekv_cache* cache) {
   if (L->decode_kernel == 2) return tc ? 2 : -1;
   if (L->decode_kernel == 1) return ekv_generic_supported(L) ? 1 : -1;
   // Choice by shape (measured on B200, whole decode steps in sustained loops, where the power cap sets
-  // the pace of the long ones).  The cluster kernel where it covers the layer: 7B 75 % 16 x 4096 82 us
-  // against 91 with the resident-tile kernel, ragged 64 x [1024, 32768] 981 against 1006 with the
-  // two-pass one, 13B 32 x 16384 652 / 863, 50 % 32 x 8192 531 / 613, 87.5 % 140 / 161, S-LRD 207 / 209.
+  // the pace of the long ones; the same front end and combine on both sides).  The cluster kernel where it
+  // covers the layer (us a step, cluster / resident-tile / two-pass kernel): 7B 75 % 16 x 4096 74 / 86 / 99,
+  // ragged 64 x [1024, 32768] 928 / 1027 / 976, 87.5 % 32 x 8192 from hidden states 126 / 196 / 149, 13B
+  // 32 x 16384 619 / - / 849, 50 % 32 x 8192 515 / - / 600, S-LRD 190 / - / 192.
   if (cl) return 4;
   // Elsewhere, of the other two tensor-core kernels, the resident-tile one has the lower fixed cost
   // and wins on batches of up to a few hundred thousand cached tokens at d_c = 1536; its per-tile

@@ -985,8 +985,8 @@ int ekv_launch_decode_cl(const elitekv_layer* L, const elitekv_cache* cache, con
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     // Clusters of an odd number of blocks only all fit when they are placed on an empty device: launched
-    // while the kernel before drains, one of the 26 clusters of 13B waited for another to end (1000 us
-    // a step instead of 655).  The others start as dependents (7B B16 84 us a step, 86.5 without).
+    // while the kernel before drains, one of the 26 clusters of 13B waited for another to end (875 us
+    // a step instead of 618).  The others start as dependents (7B B16 74.7 us a step, 76.7 without).
     cfg.numAttrs = K::C % 2 ? 1 : 2;
     EKV_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, m_lat, m_q, a));
     EKV_CUDA_OK(cudaGetLastError());

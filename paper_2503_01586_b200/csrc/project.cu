@@ -279,9 +279,9 @@ project_append_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_co
 // its MMA warp issues for both.
 // The epilogue of a rope tile reads the tokens' whole (cos, sin) rows into idle ring units while the
 // last products run, rotates out of shared memory and writes 256-byte pieces of the cache rows.
-// 4096 tokens of the 7B shape (68.7 GFLOP): 54 us, 1.27 PFLOP/s (82 us with 256 x 256 tiles of one
-// block), 63 us back to back at the power cap; the main loop keeps the tensor cores busy (67.2 k of
-// 65.5 k clocks), 10 k clocks of epilogue follow.  2048 tokens: 32 us (46 us with 128 x 128 tiles).
+// 4096 tokens of the 7B shape (68.7 GFLOP): 51 us, 1.34 PFLOP/s (82 us with 256 x 256 tiles of one
+// block), 63 us back to back at the power cap; the main loop keeps the tensor cores busy (65.5 k
+// clocks of products take 67.2 k), 10 k clocks of epilogue follow.  2048 tokens: 29 us (46 us with 128 x 128 tiles).
 constexpr int kBN = 256;                 // columns per pair
 constexpr int kUnits = 14;
 constexpr int kUnitBytes = 128 * kPK * 2;                 // 16 KB
@@ -586,8 +586,10 @@ int ekv_launch_project_append(const elitekv_layer* L, const elitekv_cache* cache
     return ELITEKV_OK;
   }
   // Few tiles: clusters share a tile's depth, as many blocks (8, 4, 2) as let all clusters be resident at
-  // once: 15, 33, 74 clusters of one block per SM (by the occupancy calculator; 16 clusters of eight would
-  // take two waves).  SPLIT_FIGURES
+  // once: 15, 33, 74 clusters of one block per SM (by the occupancy calculator; more take two waves).  us, cold,
+  // with 8 / 4 / 2 / 1 blocks per tile, depth 4096: 8 tiles 16.4 / 18.4 / 20.5 / 32.8, 16 tiles 22.5 / 20.5 /
+  // 22.5 / 32.8, 32 tiles 30.7 / 22.5 / 24.6 / 32.8, 64 tiles 53.2 / 34.8 / 28.7 / 36.9; 40 tiles of depth 5120
+  // 38.9 / 30.8 / 29.4 / 40.9.
   const long long tiles = n_out / kPN * ((T + kPM - 1) / kPM);
   const int split = tiles <= 15 && a.nk >= 8 ? 8 : tiles <= 33 && a.nk >= 4 ? 4 : tiles <= 74 && a.nk >= 2 ? 2 : 1;
   const int smem = kPStages * kPStageBytes + (split > 1 ? kRecvBytes : 0) + (int)sizeof(ProjBarriers) + 64 + 1024;

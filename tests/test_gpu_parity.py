@@ -216,9 +216,9 @@ def test_project_append_split_depth_uneven_shares(ek):
 
 @pytest.mark.parametrize("paged", [False, True])
 def test_project_append_prefill_sized_call(ek, paged):
-    """1000+ tokens with an output width of whole 256-column tiles take the 256 x 256 form (two
-    accumulators sharing every weight tile).  7B shape: 1400 tokens = 5 full token tiles and a
-    ragged sixth, shuffled order."""
+    """A prompt whose output width is whole 256-column tiles takes a paired form (blocks in pairs,
+    256 or 512 tokens x 256 columns).  7B shape: 1400 tokens, the last token tile ragged, shuffled
+    order."""
     _projection_case(ek, gen.shrink(gen.LLAMA7B_75, B=3, ctx=1000), 4096, [1000, 337, 63], paged, 101 + paged)
 
 
@@ -484,7 +484,7 @@ def _step_state(ek, paged):
 
 @pytest.mark.parametrize("paged", [False, True])
 def test_single_call_step_equals_the_three_calls(ek, paged):
-    """elitekv_decode_step (append and plan on the layer's second stream, joined before the
+    """elitekv_decode_step (append, plan and query preparation in one launch in front of the
     attention kernel) against append -> absorb -> decode on one stream: same cache rows, same
     output bits, several steps queued back to back without a synchronisation, and parity with the
     oracle from the raw inputs."""
@@ -508,8 +508,7 @@ def test_single_call_step_equals_the_three_calls(ek, paged):
 
 
 def test_single_call_step_replays_from_a_cuda_graph(ek):
-    """The fork to the layer's second stream and the join are event edges, so the whole step
-    can be captured from the caller's stream alone."""
+    """The step is launches on the caller's stream alone and can be captured from it."""
     w, st, new = _step_state(ek, False)
     q_live = st.q.clone()
     q_rope = torch.empty((4, w.n_h, 2 * w.r), dtype=torch.bfloat16, device="cuda")

@@ -36,7 +36,7 @@ def _acts(H, n, d_h, seed, graded=False):
 
 @pytest.mark.parametrize("d_h,n", [(128, 150), (64, 203), (128, 1), (128, 4), (64, 65)])
 def test_distances(ek, d_h, n):
-    """Rows that end inside a 4-row block, key tiles with a ragged end, one token (all zero)."""
+    """Rows that end inside a thread's rows, key tiles with a ragged end, one token (all zero)."""
     H = 3
     Q, K = _acts(H, n, d_h, 100 + n)
     half = d_h // 2
