@@ -169,12 +169,29 @@ __device__ __forceinline__ void rl_load(RlOps<F::TR>& o, const RlSmem<HALF, F>& 
 template <int TR>
 __device__ __forceinline__ rl2 rl_sin(const RlOps<TR>& o, int r, int j) { return o.s[(2 * r - j + kRlTK) / 2][(2 * r - j + kRlTK) & 1]; }
 
+// What a search keeps of a head from one round to the next, beside its sums R.
+struct RlState {
+  float norm;       // largest distance of the round that last summed R afresh
+  int last;         // chunk chosen in the round before
+  int fresh;        // the next round sums R afresh
+};
+
+// Tiles of 128 keys in a head's row tiles below mt (a row tile ends at the diagonal).
+template <class F>
+__host__ __device__ inline long long rl_tiles_below(int mt) {
+  constexpr int q = kRlKeys / F::ROWS;
+  const long long a = mt / q, b = mt % q;
+  return q * (a * (a + 1) / 2) + b * (a + 1);
+}
+
 template <int HALF, class F>
 __global__ void __launch_bounds__(F::THREADS)
 ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, int n,
                          const float2* __restrict__ cs, const float* __restrict__ sn,
                          const unsigned long long* __restrict__ masks, int span,
-                         float* __restrict__ partial /* [heads][items][HALF] */) {
+                         float* __restrict__ partial /* [heads][items][HALF] */,
+                         ulonglong2* __restrict__ kept /* [heads][tiles][TR][THREADS], null: R is not kept */,
+                         const RlState* __restrict__ state, int first_round, int last_round) {
   constexpr int d_h = 2 * HALF, TR = F::TR, NW = F::NW, THREADS = F::THREADS, ROWS = F::ROWS, SPAN = F::SPAN;
   extern __shared__ __align__(16) unsigned char smem_rl[];
   RlSmem<HALF, F>& sm = *(RlSmem<HALF, F>*)smem_rl;
@@ -197,6 +214,10 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
   }
   if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
     sm.list[threadIdx.x - __popcll(mask & ((1ull << threadIdx.x) - 1))] = threadIdx.x;
+  const bool fresh = kept == nullptr || first_round || state[head].fresh;
+  const int chosen = fresh ? 0 : state[head].last;
+  if (kept)
+    kept += (head * rl_tiles_below<F>((n + ROWS - 1) / ROWS) + rl_tiles_below<F>(mt)) * (TR * THREADS) + threadIdx.x;
   const bf16* Qh = Q + (size_t)head * n * d_h;
   const bf16* Kh = K + (size_t)head * n * d_h;
   // (consecutive threads take consecutive rows: the transposed stores hit different banks)
@@ -214,6 +235,18 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
   const int sn_len = rl_sin_len(n);
 
   for (int n0 = n_lo; n0 < n_hi; n0 += kRlKeys) {
+    // pairs of this warp that are not all above the diagonal, nor its rows past the last token
+    const bool live = n0 <= m0 + TR * warp + TR - 1 && m0 + TR * warp < n;
+    rl2 R[TR / 2][kRlTK];
+    ulonglong2* const keep_at = kept + (size_t)(n0 / kRlKeys) * (TR * THREADS);
+    if (!fresh && live) {                        // lands while the tile is staged
+#pragma unroll
+      for (int u = 0; u < TR; ++u) {
+        const ulonglong2 v = __ldcs(keep_at + u * THREADS);
+        R[u / 2][u % 2 * 2] = v.x;
+        R[u / 2][u % 2 * 2 + 1] = v.y;
+      }
+    }
     __syncthreads();
     // entry u holds relative position (m0 - n0) - 128 + u
     const int x0 = m0 - n0 - kRlKeys + kRlPad;
@@ -235,17 +268,27 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
     }
     cp_async_wait<0>();
     __syncthreads();
-    // every pair of this warp lies above the diagonal, or its rows past the last token
-    if (n0 > m0 + TR * warp + TR - 1 || m0 + TR * warp >= n) continue;
-    rl2 R[TR / 2][kRlTK];
+    if (!live) continue;
+    if (fresh) {
 #pragma unroll
-    for (int r = 0; r < TR / 2; ++r)
+      for (int r = 0; r < TR / 2; ++r)
 #pragma unroll
-      for (int j = 0; j < kRlTK; ++j) R[r][j] = 0ull;
+        for (int j = 0; j < kRlTK; ++j) R[r][j] = 0ull;
 #pragma unroll 8
-    for (int c = 0; c < n_free; ++c) {
+      for (int c = 0; c < n_free; ++c) {
+        RlOps<TR> o;
+        rl_load<HALF, F, false>(o, sm, sm.list[c], warp, lane);
+#pragma unroll
+        for (int r = 0; r < TR / 2; ++r)
+#pragma unroll
+          for (int j = 0; j < kRlTK; ++j) {
+            const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
+            R[r][j] = rl_fma(rl_sin(o, r, j), t, R[r][j]);
+          }
+      }
+    } else {                                     // R loses the chunk chosen in the round before
       RlOps<TR> o;
-      rl_load<HALF, F, false>(o, sm, sm.list[c], warp, lane);
+      rl_load<HALF, F, true>(o, sm, chosen, warp, lane);
 #pragma unroll
       for (int r = 0; r < TR / 2; ++r)
 #pragma unroll
@@ -253,6 +296,10 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
           const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
           R[r][j] = rl_fma(rl_sin(o, r, j), t, R[r][j]);
         }
+    }
+    if (kept && !last_round) {
+#pragma unroll
+      for (int u = 0; u < TR; ++u) __stcs(keep_at + u * THREADS, make_ulonglong2(R[u / 2][u % 2 * 2], R[u / 2][u % 2 * 2 + 1]));
     }
 #pragma unroll 8
     for (int c = 0; c < n_free; ++c) {
@@ -375,7 +422,8 @@ ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restric
 constexpr int kRlSelect = 8;      // threads per chunk
 __global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_items, int half,
                                        unsigned long long* __restrict__ masks, float* __restrict__ dist_out,
-                                       int32_t* __restrict__ elite_idx, int r, int round) {
+                                       int32_t* __restrict__ elite_idx, int r, int round,
+                                       RlState* __restrict__ state) {
   __shared__ float s_d[kRlSelect][64];
   const int head = blockIdx.x, j = threadIdx.x & 63, part = threadIdx.x >> 6;
   const unsigned long long mask = masks ? masks[head] : 0ull;
@@ -404,12 +452,28 @@ __global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_
       if (s_d[0][c] < s_d[0][best]) best = c;
     elite_idx[(size_t)head * r + round] = best;
     masks[head] = mask | (1ull << best);
+    if (state) {
+      // The winner's distance is the L1 norm of the next round's R.  Taking chunks out of a kept R adds
+      // rounding errors of the size of the R that was summed; below a quarter of it, or where anything
+      // is not finite, R is summed afresh, so that the errors stay of the size of those of a sum.
+      float norm = state[head].norm;
+      if (round == 0 || state[head].fresh) {
+        norm = 0.f;
+        for (int c = 0; c < half; ++c)
+          if (!((mask >> c) & 1ull)) norm = fmaxf(norm, s_d[0][c]);
+      }
+      state[head].norm = norm;
+      state[head].last = best;
+      state[head].fresh = !(4.f * s_d[0][best] >= norm && norm < INFINITY);
+    }
   }
 }
 
 struct RlCarve {
-  size_t off_cs, off_sin, off_partial, off_masks, total;
+  size_t off_cs, off_sin, off_partial, off_masks, off_state, total;
+  size_t off_kept, total_kept;  // the sums R of kept_heads heads behind the rest
   int tr, span, items;          // rows per thread (1: the small form), key tiles per item, items per head
+  int kept_heads;               // heads that a search takes through its rounds together (0: R is not kept)
 };
 inline size_t rl_align(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -450,6 +514,17 @@ void rl_form(int heads, int n, int half, RlCarve* c) {
   if (heads * rl_count(n, 8 * c->tr, span) >= 4 * kSms) c->span = span;
   c->items = (int)rl_count(n, 8 * c->tr, c->span);
 }
+// The sums R of a head, four bytes for each pair of its tiles (9 MB at 2048 tokens, 137 MB at 8192).  Heads are
+// independent, so a search whose heads need more than kRlKeptMost takes them through its rounds in groups;
+// one head of over 22000 tokens alone needs more, and its R is summed in every round.
+constexpr size_t kRlKeptMost = (size_t)1 << 30;
+template <class F>
+size_t rl_kept_bytes_of(int n) {
+  return (size_t)rl_tiles_below<F>((n + F::ROWS - 1) / F::ROWS) * F::TR * F::THREADS * sizeof(ulonglong2);
+}
+size_t rl_kept_bytes(int tr, int n) {
+  return tr == 16 ? rl_kept_bytes_of<Rl<16>>(n) : tr == 8 ? rl_kept_bytes_of<Rl<8>>(n) : rl_kept_bytes_of<Rl<4>>(n);
+}
 RlCarve rl_carve(int heads, int n, int half) {
   RlCarve c;
   rl_form(heads, n, half, &c);
@@ -458,7 +533,12 @@ RlCarve rl_carve(int heads, int n, int half) {
   c.off_sin = o;     o = rl_align(o + sizeof(float) * (size_t)half * rl_sin_len(n));
   c.off_partial = o; o = rl_align(o + sizeof(float) * (size_t)heads * c.items * half);
   c.off_masks = o;   o = rl_align(o + sizeof(unsigned long long) * (size_t)heads);
+  c.off_state = o;   o = rl_align(o + sizeof(RlState) * (size_t)heads);
   c.total = o;
+  c.off_kept = o;
+  const size_t per_head = rl_kept_bytes(c.tr, n);
+  c.kept_heads = c.tr == 1 || per_head > kRlKeptMost ? 0 : (int)(kRlKeptMost / per_head < (size_t)heads ? kRlKeptMost / per_head : (size_t)heads);
+  c.total_kept = o + (size_t)c.kept_heads * per_head;
   return c;
 }
 
@@ -469,9 +549,14 @@ int rl_check(int heads, int n, int d_h) {
   return ELITEKV_OK;
 }
 
+struct RlKeep {
+  ulonglong2* kept;             // null: R is summed in every round
+  const RlState* state;
+  int first_round, last_round;
+};
 template <int HALF>
 int rl_launch_half(const void* Q, const void* K, int heads, int n, const RlCarve& c, unsigned char* base,
-                   const unsigned long long* masks, cudaStream_t st) {
+                   const unsigned long long* masks, const RlKeep& k, cudaStream_t st) {
   const float2* cs = (const float2*)(base + c.off_cs);
   const float* sn = (const float*)(base + c.off_sin);
   float* partial = (float*)(base + c.off_partial);
@@ -485,7 +570,8 @@ int rl_launch_half(const void* Q, const void* K, int heads, int n, const RlCarve
       using F = decltype(form);
       const auto kern = ropelite_distance_kernel<HALF, F>;
       EKV_CUDA_OK(ekv_allow_smem(kern, sizeof(RlSmem<HALF, F>)));
-      kern<<<grid, F::THREADS, sizeof(RlSmem<HALF, F>), st>>>((const bf16*)Q, (const bf16*)K, n, cs, sn, masks, c.span, partial);
+      kern<<<grid, F::THREADS, sizeof(RlSmem<HALF, F>), st>>>((const bf16*)Q, (const bf16*)K, n, cs, sn, masks, c.span, partial,
+                                                              k.kept, k.state, k.first_round, k.last_round);
       return ELITEKV_OK;
     };
     const int rc = c.tr == 16 ? launch(Rl<16>()) : c.tr == 8 ? launch(Rl<8>()) : launch(Rl<4>());
@@ -495,9 +581,9 @@ int rl_launch_half(const void* Q, const void* K, int heads, int n, const RlCarve
   return ELITEKV_OK;
 }
 int rl_launch_distance(const void* Q, const void* K, int heads, int n, int d_h, const RlCarve& c, unsigned char* base,
-                       const unsigned long long* masks, cudaStream_t st) {
-  return d_h == 128 ? rl_launch_half<64>(Q, K, heads, n, c, base, masks, st)
-                    : rl_launch_half<32>(Q, K, heads, n, c, base, masks, st);
+                       const unsigned long long* masks, const RlKeep& k, cudaStream_t st) {
+  return d_h == 128 ? rl_launch_half<64>(Q, K, heads, n, c, base, masks, k, st)
+                    : rl_launch_half<32>(Q, K, heads, n, c, base, masks, k, st);
 }
 
 int rl_launch_table(const RlCarve& c, unsigned char* base_ptr, int n, int d_h, float base, cudaStream_t st) {
@@ -514,7 +600,7 @@ extern "C" int elitekv_ropelite_workspace_size(int32_t n_heads, int32_t n, int32
   if (!bytes) return ELITEKV_ERR_INVALID_ARG;
   const int rc = rl_check(n_heads, n, d_h);
   if (rc != ELITEKV_OK) return rc;
-  *bytes = rl_carve(n_heads, n, d_h / 2).total;
+  *bytes = rl_carve(n_heads, n, d_h / 2).total_kept;
   return ELITEKV_OK;
 }
 
@@ -533,10 +619,10 @@ extern "C" int elitekv_ropelite_distances(const void* Q, const void* K, int32_t 
   cudaStream_t st = (cudaStream_t)stream;
   rc = rl_launch_table(c, base, n, d_h, rope_base, st);
   if (rc != ELITEKV_OK) return rc;
-  rc = rl_launch_distance(Q, K, n_heads, n, d_h, c, base, (const unsigned long long*)elite_mask, st);
+  rc = rl_launch_distance(Q, K, n_heads, n, d_h, c, base, (const unsigned long long*)elite_mask, RlKeep{nullptr, nullptr, 1, 1}, st);
   if (rc != ELITEKV_OK) return rc;
   ropelite_select_kernel<<<n_heads, 64 * kRlSelect, 0, st>>>(partial, c.items, half,
-                                                 (unsigned long long*)elite_mask, dist, nullptr, 0, 0);
+                                                 (unsigned long long*)elite_mask, dist, nullptr, 0, 0, nullptr);
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }
@@ -555,17 +641,26 @@ extern "C" int elitekv_ropelite_search(const void* Q, const void* K, int32_t n_h
   unsigned char* base = (unsigned char*)workspace;
   float* partial = (float*)(base + c.off_partial);
   unsigned long long* masks = (unsigned long long*)(base + c.off_masks);
+  RlState* state = (RlState*)(base + c.off_state);
   cudaStream_t st = (cudaStream_t)stream;
   rc = rl_launch_table(c, base, n, d_h, rope_base, st);
   if (rc != ELITEKV_OK) return rc;
   EKV_CUDA_OK(cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)n_heads, st));
-  for (int round = 0; round < r; ++round) {
-    rc = rl_launch_distance(Q, K, n_heads, n, d_h, c, base, masks, st);
-    if (rc != ELITEKV_OK) return rc;
-    ropelite_select_kernel<<<n_heads, 64 * kRlSelect, 0, st>>>(partial, c.items, half, masks,
-                                                   dist_trace ? dist_trace + (size_t)round * n_heads * half : nullptr,
-                                                   elite_idx, r, round);
-    EKV_CUDA_OK(cudaGetLastError());
+  // a smaller workspace than the one asked for serves the form that keeps nothing
+  const bool keep = c.kept_heads > 0 && r > 1 && workspace_bytes >= c.total_kept;
+  const int group = keep ? c.kept_heads : n_heads;
+  for (int h0 = 0; h0 < n_heads; h0 += group) {
+    const int heads = n_heads - h0 < group ? n_heads - h0 : group;
+    const bf16 *Qg = (const bf16*)Q + (size_t)h0 * n * d_h, *Kg = (const bf16*)K + (size_t)h0 * n * d_h;
+    for (int round = 0; round < r; ++round) {
+      rc = rl_launch_distance(Qg, Kg, heads, n, d_h, c, base, masks + h0,
+                              RlKeep{keep ? (ulonglong2*)(base + c.off_kept) : nullptr, state + h0, round == 0, round == r - 1}, st);
+      if (rc != ELITEKV_OK) return rc;
+      ropelite_select_kernel<<<heads, 64 * kRlSelect, 0, st>>>(partial, c.items, half, masks + h0,
+                                                     dist_trace ? dist_trace + ((size_t)round * n_heads + h0) * half : nullptr,
+                                                     elite_idx + (size_t)h0 * r, r, round, keep ? state + h0 : nullptr);
+      EKV_CUDA_OK(cudaGetLastError());
+    }
   }
   return ELITEKV_OK;
 }
