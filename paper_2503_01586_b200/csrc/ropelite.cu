@@ -17,45 +17,51 @@
 // three FP32 operations instead of six, and just as exact at small angles (the sine is a factor,
 // nothing cancels).  The common sign is dropped: D_i = s_i t_i, s = 2 sin(.), t = q'_y k'_x - q'_x k'_y.
 //
-// Bound: FP32 pipe and issue (the contraction is 2 deep).  A thread owns 16 query rows x 4 keys, sums R
-// over the free chunks (t: multiply, FMA; R: FMA), then goes over the chunks once more for |R - D_j|
-// (FMA, add with |.|): 7 operations per pair and chunk, D_i is never stored, and the 64 pairs of a
-// thread share their operands, 15 16-byte shared-memory loads per chunk and pass.  Two rows at a time
-// with packed operations (all but the add with |.|): 43 % fewer instructions at the same number of
-// fp32 operations; pairs of neighbouring table entries are formed in registers.  32 heads x 2048 tokens
-// x d_h 128: 1.48 ms a round (1.58 with scalar operations, 1.53 with the chunk loops unrolled twice
-// and not eight times; 0.54 of 148 SMs x 128 lanes x 1.965 GHz).  The form that holds the 64 D_i of one
-// pair in registers took 3.04 ms: 9 operations and three loads per pair and chunk, shared-memory bound.
-// Short calibrations cannot fill the device with 128 x 128 tiles: there a thread owns 8 or 4 rows, and up
-// to 128 tokens the register form is the faster one (rl_form; one head of 64 tokens, four rounds: 235 us on
-// one such tile, 72 us).
+// Bound: FP32 pipe, issue and shared-memory reads (the contraction is 2 deep).  R is kept between rounds (four bytes a
+// pair in the workspace) and loses the chunk that was chosen: a round costs |R - D_j| for every free chunk and one
+// D_i, 4 operations per pair and chunk (multiply, two FMA, add with |.|) where summing R afresh takes 7; it is summed
+// afresh in the first round and where its norm has fallen so far that the rounding errors of what was
+// taken out would show (ropelite_select_kernel).  A thread owns 8 query rows x 8 keys, two rows at a
+// time in packed operations (all but the add with |.|): a chunk costs it 12 16-byte shared-memory reads for
+// 64 pairs, a byte of which takes as long for a broadcast as for 32 different words, so that the square tile beats
+// the 16 x 4 one (15 reads).  Rows and keys are rotated once per search and copied to shared memory by
+// the copy engine, three copies per chunk, four chunks a stage (six small copies per chunk kept warps
+// waiting: 9.4 ms instead of 8.4); three blocks of four warps share an SM and drift apart, so that one's start and waits lie
+// under the others' operations.  32 heads x 2048 tokens x d_h 128, 8 rounds: 8.4 ms; 11.9 with R summed
+// in every round, 9.1 with kept R on 16 x 4 tiles of one block per SM.  A round takes 0.97 ms, 0.52 of 148 SMs x 128 lanes x
+// 1.965 GHz.
+// Short calibrations cannot fill the device with such tiles: there a thread owns 4 x 4 pairs, and up to 128
+// tokens a form with the 64 D_i of one pair in registers is the faster one (rl_form).
 //
-// distance kernel: grid (items, heads), 256 threads; an item is 128 (64, 32) query rows x up to `span` key
-// tiles of 128.  Per key tile the rotated keys (x plane, y plane, [chunk][key]) and the slice of
-// the sine table that the tile's relative positions need are staged in shared memory; the table is
+// distance kernel: grid (items, heads); an item is 64 (32) query rows x up to `span` key tiles of 128.  The slice of
+// the sine table that a tile's relative positions need comes with its keys; the table is
 // zero at negative relative positions, which is the causal mask.  Item results go to a
 // [head][item][chunk] array; the select kernel adds them in a fixed order (the result does not
 // depend on scheduling), masks the chunks already chosen and takes the first minimum.
-#include <initializer_list>
-
-#include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace {
 
 constexpr int kRlKeys = 128;      // keys per stage
-constexpr int kRlTK = 4;          // ... per thread
 constexpr int kRlAcc = 8;         // lanes of a warp that keep running distances
 constexpr int kRlPad = 256;       // zeros in front of the sine table: negative relative positions
-static_assert(kRlKeys == 32 * kRlTK, "thread tiles cover the block's keys");
 
-// blocks of 8 warps with TR query rows per warp (and thread): 16, or 8 or 4 where that fills the device better
-template <int TR_>
+// TR query rows and TK keys per thread: 8 x 8 in blocks of 4 warps, or 4 x 4 in blocks of 8 where there are few pairs
+template <int TR_, int TK_>
 struct Rl {
-  static constexpr int TR = TR_, NW = 8, THREADS = 32 * NW;
-  static constexpr int ROWS = NW * TR;                   // query rows per block
+  static constexpr int TR = TR_, TK = TK_, NW = TK == 8 ? 4 : 8, THREADS = 32 * NW;
+  static constexpr int LANES = kRlKeys / TK;             // lanes that share a thread tile's rows
+  static constexpr int WROWS = TR * (32 / LANES);        // query rows per warp
+  static constexpr int ROWS = NW * WROWS;                // ... per block
   static constexpr int SPAN = kRlKeys + ROWS;            // sine table entries of a stage (relative positions)
-  static_assert(ROWS <= 128 && SPAN <= kRlPad, "a stage's slice lies inside the table");
+  static constexpr int VALUES = TR * TK / 4;             // 16-byte pieces of a thread's sums R
+  // chunks per stage, stages, and steps between a stage's load and its use (the other warps may be behind the
+  // first one, which loads, by the stages that are left)
+  static constexpr int PART = TK == 8 ? 4 : 8, STAGES = TK == 8 ? 6 : 5, AHEAD = TK == 8 ? 3 : 4;
+  static_assert(ROWS <= kRlKeys && kRlKeys % ROWS == 0 && SPAN <= kRlPad, "a stage's slice lies inside the table");
 };
+typedef Rl<8, 8> RlLarge;
+typedef Rl<4, 4> RlFew;
 
 // entries of a chunk's sine table: entry x holds 2 sin((x - kRlPad) theta / 2), zero up to kRlPad
 __host__ __device__ inline int rl_sin_len(int n) { return (n + 127) / 128 * 128 + kRlPad; }
@@ -63,9 +69,13 @@ __host__ __device__ inline int rl_sin_len(int n) { return (n + 127) / 128 * 128 
 // (cos, sin)(pos theta_i / 2) laid out [pos][chunk], and the sine table [chunk][...];
 // double precision, rounded once
 __global__ void ropelite_table_kernel(float2* __restrict__ cs, float* __restrict__ sn, int n, int half, int d_h,
-                                      double base) {
+                                      double base, unsigned long long* __restrict__ masks, int heads) {
+  ekv_pdl_wait();         // (here and below: the kernels of a search are a chain, each launched while the one before drains)
+  ekv_pdl_trigger();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int len = rl_sin_len(n);
+  if (masks)                // a search begins with no chunk chosen
+    for (long long h = e; h < heads; h += (long long)gridDim.x * blockDim.x) masks[h] = 0;
   if (e >= (long long)len * half) return;
   const int i = (int)(e % half), x = (int)(e / half);
   const int pos = x - kRlPad;
@@ -95,13 +105,42 @@ __device__ __forceinline__ void rl_rotate4(const bf16* row, const float2* cs, fl
   }
 }
 
+// Rows of Q and K rotated by half their angle, zeros past the last token, laid out as the distance kernel
+// copies them, per head Q [row tile][chunk][x, y][tile rows], K [tile of 128 keys][chunk][x, y][keys]; the first four of every
+// eight keys of a tile come before the others where a thread takes eight.  Every row tile, key tile and round reads them.
+// Grid (rows / 64, heads, Q or K), 256 threads.
+__global__ void ropelite_rotate_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, const float2* __restrict__ cs,
+                                       float* __restrict__ rot, int n, int n_pad, int half, int q_rows, int split) {
+  ekv_pdl_wait();
+  ekv_pdl_trigger();
+  const int row = blockIdx.x * 64 + threadIdx.x % 64, head = blockIdx.y, k = blockIdx.z;
+  const bf16* src = (k ? K : Q) + ((size_t)head * n + row) * 2 * half;
+  const int tile = k ? kRlKeys : q_rows, in = row % tile;
+  float* x = rot + ((size_t)head * 2 + k) * 2 * half * n_pad + (size_t)(row - in) * 2 * half +
+             (k && split ? (in >> 2 & 1) * 64 + (in >> 3) * 4 + (in & 3) : in);
+  for (int i = threadIdx.x / 64 * 4; i < half; i += 16) {
+    float2 v[4] = {};
+    if (row < n) rl_rotate4(src + 2 * i, cs + (size_t)row * half + i, v);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      x[(size_t)(i + u) * 2 * tile] = v[u].x;
+      x[(size_t)(i + u) * 2 * tile + tile] = v[u].y;
+    }
+  }
+}
+
+// one chunk of a stage
+template <class F>
+struct __align__(16) RlChunk {
+  float kx[kRlKeys], ky[kRlKeys], qx[F::ROWS], qy[F::ROWS], sn[F::SPAN];
+};
 template <int HALF, class F>
 struct RlSmem {
-  float kx[HALF][kRlKeys], ky[HALF][kRlKeys];
-  float sn[HALF][F::SPAN];
-  float qx[HALF][F::ROWS], qy[HALF][F::ROWS];
+  RlChunk<F> ring[F::STAGES][F::PART];
   float acc[HALF][F::NW * kRlAcc];     // running distances
-  int list[HALF];                    // chunks not chosen yet
+  uint64_t full[F::STAGES], empty[F::STAGES];
+  int list[HALF];                      // chunks in the order in which a tile needs them
+  int failed;
 };
 
 // Two rows (r, r + 1) at a time: packed fp32 operations, each element rounded as by itself
@@ -127,37 +166,41 @@ __device__ __forceinline__ rl2 rl_fma(rl2 a, rl2 b, rl2 c) {
   return d;
 }
 
-// operands of a thread's 4 TR pairs for one chunk; kNeg: t with its sign turned
-template <int TR>
+// operands of a thread's pairs for one chunk; kNeg: t with its sign turned
+template <class F>
 struct RlOps {
-  rl2 a[kRlTK], b[kRlTK];            // keys: t = q_y a + q_x b
-  rl2 qx[TR / 2], qy[TR / 2];
-  rl2 s[(TR + kRlTK) / 2][2];        // [v][0]: table entries 2 v, 2 v + 1; [v][1]: 2 v + 1, 2 v + 2
+  rl2 a[F::TK], b[F::TK];            // keys: t = q_y a + q_x b
+  rl2 qx[F::TR / 2], qy[F::TR / 2];
+  rl2 s[(F::TR + F::TK) / 2][2];     // [v][0]: table entries 2 v, 2 v + 1; [v][1]: 2 v + 1, 2 v + 2
 };
-template <int HALF, class F, bool kNeg>
-__device__ __forceinline__ void rl_load(RlOps<F::TR>& o, const RlSmem<HALF, F>& sm, int i, int warp, int lane) {
-  constexpr int TR = F::TR;
-  const float4 kx = *(const float4*)&sm.kx[i][lane * kRlTK], ky = *(const float4*)&sm.ky[i][lane * kRlTK];
-  const float x[kRlTK] = {kx.x, kx.y, kx.z, kx.w}, y[kRlTK] = {ky.x, ky.y, ky.z, ky.w};
+// rg: the thread's group of TR rows in the block; lk: its group of TK keys
+template <class F, bool kNeg>
+__device__ __forceinline__ void rl_load(RlOps<F>& o, const RlChunk<F>& ch, int rg, int lk) {
+  constexpr int TR = F::TR, TK = F::TK;
 #pragma unroll
-  for (int j = 0; j < kRlTK; ++j) {
-    const float a = kNeg ? -x[j] : x[j], b = kNeg ? y[j] : -y[j];
-    o.a[j] = rl_pack(a, a);
-    o.b[j] = rl_pack(b, b);
+  for (int h = 0; h < TK / 4; ++h) {       // (the keys' first fours come before their second ones: lanes read consecutive 16 bytes)
+    const float4 kx = *(const float4*)&ch.kx[kRlKeys / 2 * h + 4 * lk], ky = *(const float4*)&ch.ky[kRlKeys / 2 * h + 4 * lk];
+    const float x[4] = {kx.x, kx.y, kx.z, kx.w}, y[4] = {ky.x, ky.y, ky.z, ky.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float a = kNeg ? -x[j] : x[j], b = kNeg ? y[j] : -y[j];
+      o.a[4 * h + j] = rl_pack(a, a);
+      o.b[4 * h + j] = rl_pack(b, b);
+    }
   }
   // entry u of the stage's slice: relative position (m0 - n0) - 128 + u; this thread's pairs need
-  // u = TR warp + r - (4 lane + j) + 128, from TR warp - 4 lane + 124 on
-  const float4* sp = (const float4*)&sm.sn[i][TR * warp - kRlTK * lane + kRlKeys - kRlTK];
-  float e[TR + kRlTK];
+  // u = TR rg + r - (TK lk + j) + 128, from TR rg - TK lk + 128 - TK on
+  const float4* sp = (const float4*)&ch.sn[TR * rg - TK * lk + kRlKeys - TK];
+  float e[TR + TK];
 #pragma unroll
-  for (int u = 0; u < (TR + kRlTK) / 4; ++u) *(float4*)&e[4 * u] = sp[u];
+  for (int u = 0; u < (TR + TK) / 4; ++u) *(float4*)&e[4 * u] = sp[u];
 #pragma unroll
-  for (int v = 0; v < (TR + kRlTK) / 2; ++v) {
+  for (int v = 0; v < (TR + TK) / 2; ++v) {
     o.s[v][0] = rl_pack(e[2 * v], e[2 * v + 1]);
-    if (2 * v + 2 < TR + kRlTK) o.s[v][1] = rl_pack(e[2 * v + 1], e[2 * v + 2]);
+    if (2 * v + 2 < TR + TK) o.s[v][1] = rl_pack(e[2 * v + 1], e[2 * v + 2]);
   }
-  const ulonglong2* qx = (const ulonglong2*)&sm.qx[i][TR * warp];
-  const ulonglong2* qy = (const ulonglong2*)&sm.qy[i][TR * warp];
+  const ulonglong2* qx = (const ulonglong2*)&ch.qx[TR * rg];
+  const ulonglong2* qy = (const ulonglong2*)&ch.qy[TR * rg];
 #pragma unroll
   for (int u = 0; u < TR / 4; ++u) {
     const ulonglong2 vx = qx[u], vy = qy[u];
@@ -165,9 +208,28 @@ __device__ __forceinline__ void rl_load(RlOps<F::TR>& o, const RlSmem<HALF, F>& 
     o.qy[2 * u] = vy.x; o.qy[2 * u + 1] = vy.y;
   }
 }
-// table pair of rows 2 r, 2 r + 1 and key j: entries 2 r - j + 4 and the next
-template <int TR>
-__device__ __forceinline__ rl2 rl_sin(const RlOps<TR>& o, int r, int j) { return o.s[(2 * r - j + kRlTK) / 2][(2 * r - j + kRlTK) & 1]; }
+// table pair of rows 2 r, 2 r + 1 and key j: entries 2 r - j + TK and the next
+template <class F>
+__device__ __forceinline__ rl2 rl_sin(const RlOps<F>& o, int r, int j) { return o.s[(2 * r - j + F::TK) / 2][(2 * r - j + F::TK) & 1]; }
+
+// R += D of a chunk (kNeg: R -= D)
+template <class F, bool kNeg>
+__device__ __forceinline__ void rl_add(rl2 (&R)[F::TR / 2][F::TK], const RlChunk<F>& ch, int rg, int lk) {
+  RlOps<F> o;
+  rl_load<F, kNeg>(o, ch, rg, lk);
+#pragma unroll
+  for (int r = 0; r < F::TR / 2; ++r)
+#pragma unroll
+    for (int j = 0; j < F::TK; ++j) {
+      const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
+      R[r][j] = rl_fma(rl_sin(o, r, j), t, R[r][j]);
+    }
+}
+__device__ __forceinline__ void rl_bulk(void* dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+               "l"((uint64_t)src), "r"(bytes), "r"(bar)
+               : "memory");
+}
 
 // What a search keeps of a head from one round to the next, beside its sums R.
 struct RlState {
@@ -185,15 +247,14 @@ __host__ __device__ inline long long rl_tiles_below(int mt) {
 }
 
 template <int HALF, class F>
-__global__ void __launch_bounds__(F::THREADS)
-ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, int n,
-                         const float2* __restrict__ cs, const float* __restrict__ sn,
-                         const unsigned long long* __restrict__ masks, int span,
+__global__ void __launch_bounds__(F::THREADS, F::TR == 8 ? 3 : 2)
+ropelite_distance_kernel(const float* __restrict__ rot /* [heads]: Q, K (ropelite_rotate_kernel) */, int n, int n_pad,
+                         const float* __restrict__ sn, const unsigned long long* __restrict__ masks, int span,
                          float* __restrict__ partial /* [heads][items][HALF] */,
-                         ulonglong2* __restrict__ kept /* [heads][tiles][TR][THREADS], null: R is not kept */,
+                         ulonglong2* __restrict__ kept /* [heads][tiles][VALUES][THREADS], null: R is not kept */,
                          const RlState* __restrict__ state, int first_round, int last_round) {
-  constexpr int d_h = 2 * HALF, TR = F::TR, NW = F::NW, THREADS = F::THREADS, ROWS = F::ROWS, SPAN = F::SPAN;
-  extern __shared__ __align__(16) unsigned char smem_rl[];
+  constexpr int TR = F::TR, TK = F::TK, NW = F::NW, THREADS = F::THREADS, ROWS = F::ROWS;
+  extern __shared__ __align__(128) unsigned char smem_rl[];
   RlSmem<HALF, F>& sm = *(RlSmem<HALF, F>*)smem_rl;
   const int head = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // item -> (row tile, group of key tiles), long rows first
@@ -203,6 +264,8 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
     if (kg < groups) break;
     kg -= groups;
   }
+  ekv_pdl_wait();
+  ekv_pdl_trigger();
   const int m0 = mt * ROWS;
   const int n_lo = kg * span * kRlKeys, n_hi = min(n_lo + span * kRlKeys, m0 + ROWS);
   const unsigned long long mask = masks ? masks[head] : 0ull;
@@ -212,124 +275,149 @@ ropelite_distance_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K,
     for (int j = threadIdx.x; j < HALF; j += THREADS) out[j] = 0.f;
     return;
   }
-  if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
-    sm.list[threadIdx.x - __popcll(mask & ((1ull << threadIdx.x) - 1))] = threadIdx.x;
   const bool fresh = kept == nullptr || first_round || state[head].fresh;
-  const int chosen = fresh ? 0 : state[head].last;
-  if (kept)
-    kept += (head * rl_tiles_below<F>((n + ROWS - 1) / ROWS) + rl_tiles_below<F>(mt)) * (TR * THREADS) + threadIdx.x;
-  const bf16* Qh = Q + (size_t)head * n * d_h;
-  const bf16* Kh = K + (size_t)head * n * d_h;
-  // (consecutive threads take consecutive rows: the transposed stores hit different banks)
-  for (int e = threadIdx.x; e < ROWS * (HALF / 4); e += THREADS) {
-    const int rr = e % ROWS, g4 = e / ROWS;
-    float2 v[4] = {};
-    if (m0 + rr < n) rl_rotate4(Qh + (size_t)(m0 + rr) * d_h + g4 * 8, cs + (size_t)(m0 + rr) * HALF + g4 * 4, v);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      sm.qx[g4 * 4 + u][rr] = v[u].x;
-      sm.qy[g4 * 4 + u][rr] = v[u].y;
+  // one that R has to lose, then the free ones
+  const int n_old = fresh ? 0 : 1, n_list = n_old + n_free, parts = (n_list + F::PART - 1) / F::PART;
+  if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
+    sm.list[n_old + threadIdx.x - __popcll(mask & ((1ull << threadIdx.x) - 1))] = threadIdx.x;
+  if (threadIdx.x == 0) {
+    if (!fresh) sm.list[0] = state[head].last;
+    sm.failed = 0;
+    for (int i = 0; i < F::STAGES; ++i) {
+      mbar_init(smem_u32(&sm.full[i]), 1);
+      mbar_init(smem_u32(&sm.empty[i]), NW);
     }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_proxy_async();
   }
-  for (int e = threadIdx.x; e < HALF * NW * kRlAcc; e += THREADS) (&sm.acc[0][0])[e] = 0.f;
+  if (kept)
+    kept += (head * rl_tiles_below<F>((n + ROWS - 1) / ROWS) + rl_tiles_below<F>(mt)) * (F::VALUES * THREADS) + threadIdx.x;
+  const float* rot_h = rot + (size_t)head * 4 * HALF * n_pad;
   const int sn_len = rl_sin_len(n);
+  for (int e = threadIdx.x; e < HALF * NW * kRlAcc; e += THREADS) (&sm.acc[0][0])[e] = 0.f;
+  __syncthreads();
 
+  // Steps of the block: for each key tile the parts of its list, twice where R is summed afresh.  The first
+  // warp loads them.
+  const int tile_steps = fresh ? 2 * parts : parts;
+  auto wait = [&](uint64_t* b, uint32_t parity) {
+    unsigned tries = 0;
+    while (!mbar_try_wait(smem_u32(b), parity))
+      if (++tries > kWaitLimit) { sm.failed = 1; break; }
+  };
+  int load_n0 = n_lo, load_step = 0, load_slot = 0;
+  uint32_t load_parity = 1;
+  auto load = [&] {
+    if (load_n0 < n_hi) {
+      wait(&sm.empty[load_slot], load_parity);
+      const int c0 = load_step % parts * F::PART, cn = min(F::PART, n_list - c0);
+      const uint32_t bar = smem_u32(&sm.full[load_slot]);
+      if (lane == 0) mbar_expect_tx(bar, (uint32_t)(cn * sizeof(RlChunk<F>)));
+      __syncwarp();
+      for (int e = lane; e < 3 * cn; e += 32) {
+        const int c = e / 3, what = e - 3 * c;
+        const int i = sm.list[c0 + c];
+        RlChunk<F>& ch = sm.ring[load_slot][c];
+        const float* k = rot_h + (size_t)2 * HALF * (n_pad + load_n0) + (size_t)i * 2 * kRlKeys;
+        if (what == 0) rl_bulk(ch.kx, k, 2 * sizeof(ch.kx), bar);
+        else if (what == 1) rl_bulk(ch.qx, rot_h + (size_t)2 * HALF * m0 + (size_t)i * 2 * ROWS, 2 * sizeof(ch.qx), bar);
+        else rl_bulk(ch.sn, sn + (size_t)i * sn_len + m0 - load_n0 - kRlKeys + kRlPad, sizeof(ch.sn), bar);
+      }
+      if (++load_step == tile_steps) { load_step = 0; load_n0 += kRlKeys; }
+    }
+    if (++load_slot == F::STAGES) { load_slot = 0; load_parity ^= 1; }
+  };
+  if (warp == 0)
+    for (int i = 0; i < F::AHEAD; ++i) load();
+
+  const int rg = warp * (32 / F::LANES) + lane / F::LANES, lk = lane % F::LANES;
+  int slot = 0;
+  uint32_t parity = 0;
   for (int n0 = n_lo; n0 < n_hi; n0 += kRlKeys) {
     // pairs of this warp that are not all above the diagonal, nor its rows past the last token
-    const bool live = n0 <= m0 + TR * warp + TR - 1 && m0 + TR * warp < n;
-    rl2 R[TR / 2][kRlTK];
-    ulonglong2* const keep_at = kept + (size_t)(n0 / kRlKeys) * (TR * THREADS);
-    if (!fresh && live) {                        // lands while the tile is staged
-#pragma unroll
-      for (int u = 0; u < TR; ++u) {
-        const ulonglong2 v = __ldcs(keep_at + u * THREADS);
-        R[u / 2][u % 2 * 2] = v.x;
-        R[u / 2][u % 2 * 2 + 1] = v.y;
-      }
-    }
-    __syncthreads();
-    // entry u holds relative position (m0 - n0) - 128 + u
-    const int x0 = m0 - n0 - kRlKeys + kRlPad;
-    for (int e = threadIdx.x; e < HALF * (SPAN / 4); e += THREADS) {
-      const int i = e / (SPAN / 4), u = (e % (SPAN / 4)) * 4;
-      cp_async16(&sm.sn[i][u], sn + (size_t)i * sn_len + x0 + u);
-    }
-    cp_async_commit();
-#pragma unroll
-    for (int e = threadIdx.x; e < kRlKeys * (HALF / 4); e += THREADS) {
-      const int nn = e % kRlKeys, g4 = e / kRlKeys;         // 4 chunks = 8 elements = 16 bytes
-      float2 v[4] = {};
-      if (n0 + nn < n) rl_rotate4(Kh + (size_t)(n0 + nn) * d_h + g4 * 8, cs + (size_t)(n0 + nn) * HALF + g4 * 4, v);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        sm.kx[g4 * 4 + u][nn] = v[u].x;
-        sm.ky[g4 * 4 + u][nn] = v[u].y;
-      }
-    }
-    cp_async_wait<0>();
-    __syncthreads();
-    if (!live) continue;
+    const bool live = n0 < m0 + F::WROWS * (warp + 1) && m0 + F::WROWS * warp < n;
+    rl2 R[TR / 2][TK];
+    ulonglong2* const keep_at = kept + (size_t)(n0 / kRlKeys) * (F::VALUES * THREADS);
     if (fresh) {
 #pragma unroll
       for (int r = 0; r < TR / 2; ++r)
 #pragma unroll
-        for (int j = 0; j < kRlTK; ++j) R[r][j] = 0ull;
-#pragma unroll 8
-      for (int c = 0; c < n_free; ++c) {
-        RlOps<TR> o;
-        rl_load<HALF, F, false>(o, sm, sm.list[c], warp, lane);
+        for (int j = 0; j < TK; ++j) R[r][j] = 0ull;
+    } else {
+      if (live) {
 #pragma unroll
-        for (int r = 0; r < TR / 2; ++r)
-#pragma unroll
-          for (int j = 0; j < kRlTK; ++j) {
-            const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
-            R[r][j] = rl_fma(rl_sin(o, r, j), t, R[r][j]);
-          }
+        for (int u = 0; u < F::VALUES; ++u) {
+          const ulonglong2 v = __ldcs(keep_at + u * THREADS);
+          R[u / (TK / 2)][u % (TK / 2) * 2] = v.x;
+          R[u / (TK / 2)][u % (TK / 2) * 2 + 1] = v.y;
+        }
       }
-    } else {                                     // R loses the chunk chosen in the round before
-      RlOps<TR> o;
-      rl_load<HALF, F, true>(o, sm, chosen, warp, lane);
+      if (n0 + kRlKeys < n_hi && (threadIdx.x & 7) == 0) {      // the next tile's come into L2 meanwhile
 #pragma unroll
-      for (int r = 0; r < TR / 2; ++r)
-#pragma unroll
-        for (int j = 0; j < kRlTK; ++j) {
-          const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
-          R[r][j] = rl_fma(rl_sin(o, r, j), t, R[r][j]);
-        }
+        for (int u = 0; u < F::VALUES; ++u)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(keep_at + (F::VALUES + u) * THREADS));
+      }
     }
-    if (kept && !last_round) {
+#pragma unroll 1
+    for (int step = 0; step < tile_steps; ++step) {
+      if (warp == 0) load();
+      wait(&sm.full[slot], parity);
+      if (live) {
+        const bool sum = fresh && step < parts;
+        int c = 0;
+        const int part = sum || !fresh ? step : step - parts, cn = min(F::PART, n_list - part * F::PART);
+        const RlChunk<F>* ring = sm.ring[slot];
+        if (sum) {
+#pragma unroll 4
+          for (; c < cn; ++c) rl_add<F, false>(R, ring[c], rg, lk);
+        } else {
+          if (part == 0) {
+            if (!fresh) {                        // R loses the chunk chosen in the round before
+              rl_add<F, true>(R, ring[0], rg, lk);
+              c = 1;
+            }
+            if (kept && !last_round) {
 #pragma unroll
-      for (int u = 0; u < TR; ++u) __stcs(keep_at + u * THREADS, make_ulonglong2(R[u / 2][u % 2 * 2], R[u / 2][u % 2 * 2 + 1]));
-    }
-#pragma unroll 8
-    for (int c = 0; c < n_free; ++c) {
-      RlOps<TR> o;
-      const int i = sm.list[c];
-      rl_load<HALF, F, true>(o, sm, i, warp, lane);
-      float v[kRlTK] = {};
+              for (int u = 0; u < F::VALUES; ++u) __stcs(keep_at + u * THREADS, make_ulonglong2(R[u / (TK / 2)][u % (TK / 2) * 2], R[u / (TK / 2)][u % (TK / 2) * 2 + 1]));
+            }
+          }
+#pragma unroll 4
+          for (; c < cn; ++c) {
+            RlOps<F> o;
+            rl_load<F, true>(o, ring[c], rg, lk);
+            float v[TK] = {};
 #pragma unroll
-      for (int r = 0; r < TR / 2; ++r)
+            for (int r = 0; r < TR / 2; ++r)
 #pragma unroll
-        for (int j = 0; j < kRlTK; ++j) {
-          const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
-          const float2 x = rl_unpack(rl_fma(rl_sin(o, r, j), t, R[r][j]));
-          v[j] += fabsf(x.x);
-          v[j] += fabsf(x.y);
+              for (int j = 0; j < TK; ++j) {
+                const rl2 t = rl_fma(o.qx[r], o.b[j], rl_mul(o.qy[r], o.a[j]));
+                const float2 x = rl_unpack(rl_fma(rl_sin(o, r, j), t, R[r][j]));
+                v[j] += fabsf(x.x);
+                v[j] += fabsf(x.y);
+              }
+            float d = (v[0] + v[1]) + (v[2] + v[3]);
+            if constexpr (TK == 8) d += (v[4] + v[5]) + (v[6] + v[7]);
+            d += __shfl_xor_sync(0xffffffffu, d, 16);
+            d += __shfl_xor_sync(0xffffffffu, d, 8);
+            if (lane < kRlAcc) sm.acc[part * F::PART + c][warp * kRlAcc + lane] += d;
+          }
         }
-      float d = (v[0] + v[1]) + (v[2] + v[3]);
-      d += __shfl_xor_sync(0xffffffffu, d, 16);
-      d += __shfl_xor_sync(0xffffffffu, d, 8);
-      if (lane < kRlAcc) sm.acc[i][warp * kRlAcc + lane] += d;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sm.empty[slot]));
+      if (++slot == F::STAGES) { slot = 0; parity ^= 1; }
     }
   }
-  // block result: threads in a fixed order
   __syncthreads();
-  for (int j = warp; j < HALF; j += NW) {
+  if (sm.failed) drain_after_abort();
+  // block result: threads in a fixed order
+  const float bad = sm.failed ? NAN : 0.f;
+  for (int c = n_old + warp; c < n_list; c += NW) {
     float v = 0.f;
 #pragma unroll
-    for (int w = 0; w < NW * kRlAcc; w += 32) v += sm.acc[j][w + lane];
+    for (int w = 0; w < NW * kRlAcc; w += 32) v += sm.acc[c][w + lane];
     v = warp_sum(v);
-    if (lane == 0) out[j] = v;
+    if (lane == 0) out[sm.list[c]] = v + bad;
   }
 }
 
@@ -350,9 +438,11 @@ ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restric
                                const unsigned long long* __restrict__ masks,
                                float* __restrict__ partial /* [heads][row tiles][HALF] */) {
   constexpr int d_h = 2 * HALF, THREADS = 32 * kRsWarps;
-  extern __shared__ __align__(16) unsigned char smem_rl[];
+  extern __shared__ __align__(128) unsigned char smem_rl[];
   RsSmem<HALF>& sm = *(RsSmem<HALF>*)smem_rl;
   const int head = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  ekv_pdl_wait();
+  ekv_pdl_trigger();
   const int m0 = blockIdx.x * kRsRows, m_last = min(m0 + kRsRows, n) - 1;
   const unsigned long long mask = masks ? masks[head] : 0ull;
   const bf16* Qh = Q + (size_t)head * n * d_h;
@@ -425,6 +515,8 @@ __global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_
                                        int32_t* __restrict__ elite_idx, int r, int round,
                                        RlState* __restrict__ state) {
   __shared__ float s_d[kRlSelect][64];
+  ekv_pdl_wait();
+  ekv_pdl_trigger();
   const int head = blockIdx.x, j = threadIdx.x & 63, part = threadIdx.x >> 6;
   const unsigned long long mask = masks ? masks[head] : 0ull;
   float v = 0.f;
@@ -470,10 +562,10 @@ __global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_
 }
 
 struct RlCarve {
-  size_t off_cs, off_sin, off_partial, off_masks, off_state, total;
-  size_t off_kept, total_kept;  // the sums R of kept_heads heads behind the rest
+  size_t off_cs, off_sin, off_partial, off_masks, off_state, off_rot, off_kept, total;
   int tr, span, items;          // rows per thread (1: the small form), key tiles per item, items per head
-  int kept_heads;               // heads that a search takes through its rounds together (0: R is not kept)
+  int group;                    // heads that go through their rounds together
+  bool keep;                    // their sums R are kept between rounds
 };
 inline size_t rl_align(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -487,11 +579,11 @@ long long rl_count(int n, int rows, int span) {
 }
 // Which form, for a device of 148 SMs.  A search of few tokens is a chain of small launches: its time is
 // that of one block.  Up to 64 tokens the small form is the faster one while a few of its blocks share an
-// SM, up to 128 tokens while each has its own.  Four rounds, d_h 128, us (small / 4 / 8 / 16 rows per
-// thread): 4 heads x 64 tokens 72 / 129 / 163 / 173, 4 x 128 105 / 133 / 171 / 246, 32 x 128 - / 132 / 172 / 250,
-// 32 x 300 - / 427 / 308 / 391, 16 x 512 - / 522 / 440 / 460, 16 x 1024 - / 1606 / 1111 / 894.  Beyond it the
-// form whose blocks take least time in all, in whole rounds over the device: a key tile of a block takes
-// 24, 33 and 52 us at d_h 128, and in the same proportions at d_h 64.
+// SM, up to 128 tokens while each has its own.  Beyond it the form whose blocks take least time in all, in whole
+// rounds over the device: a key tile takes about 57 us with three blocks of 64 rows (8 x 8) on every SM
+// and 40 us with two of 32 (4 x 4), at d_h 128 and in the same proportion at d_h 64.  Four rounds, d_h 128, us
+// (4 x 4 / 8 x 8 pairs per thread): 32 heads x 128 tokens 144 / 204, 8 x 200 144 / 198, 32 x 300 285 / 246, 4 x 512
+// 166 / 205, 16 x 512 377 / 294, 16 x 1024 1165 / 689; eight rounds at d_h 64: 16 x 200 177 / 212, 32 x 512 616 / 460.
 void rl_form(int heads, int n, int half, RlCarve* c) {
   constexpr int kSms = 148;
   const long long small = (long long)heads * ((n + kRsRows - 1) / kRsRows);
@@ -501,44 +593,45 @@ void rl_form(int heads, int n, int half, RlCarve* c) {
     c->items = (n + kRsRows - 1) / kRsRows;
     return;
   }
-  long long best = 0;
-  for (const int tr : {16, 8, 4}) {
-    const int cost = tr == 16 ? 52 : tr == 8 ? 33 : 24;
-    const long long t = (heads * rl_count(n, 8 * tr, 1) + kSms - 1) / kSms * cost;
-    if (tr == 16 || t < best) {
-      best = t;
-      c->tr = tr;
-    }
-  }
+  // 8 x 8: three blocks of 64 rows share an SM; 4 x 4: two of 32
+  const long long large = (heads * rl_count(n, 64, 1) + 3 * kSms - 1) / (3 * kSms) * 57;
+  const long long few = (heads * rl_count(n, 32, 1) + 2 * kSms - 1) / (2 * kSms) * 40;
+  c->tr = few < large ? 4 : 8;
   const int tiles = (n + kRlKeys - 1) / kRlKeys, span = tiles > 64 ? (tiles + 15) / 16 : 4;
   if (heads * rl_count(n, 8 * c->tr, span) >= 4 * kSms) c->span = span;
   c->items = (int)rl_count(n, 8 * c->tr, c->span);
 }
-// The sums R of a head, four bytes for each pair of its tiles (9 MB at 2048 tokens, 137 MB at 8192).  Heads are
-// independent, so a search whose heads need more than kRlKeptMost takes them through its rounds in groups;
-// one head of over 22000 tokens alone needs more, and its R is summed in every round.
-constexpr size_t kRlKeptMost = (size_t)1 << 30;
+inline int rl_pad_n(int n) { return (n + kRlKeys - 1) / kRlKeys * kRlKeys; }
 template <class F>
 size_t rl_kept_bytes_of(int n) {
-  return (size_t)rl_tiles_below<F>((n + F::ROWS - 1) / F::ROWS) * F::TR * F::THREADS * sizeof(ulonglong2);
+  return (size_t)rl_tiles_below<F>((n + F::ROWS - 1) / F::ROWS) * F::VALUES * F::THREADS * sizeof(ulonglong2);
 }
 size_t rl_kept_bytes(int tr, int n) {
-  return tr == 16 ? rl_kept_bytes_of<Rl<16>>(n) : tr == 8 ? rl_kept_bytes_of<Rl<8>>(n) : rl_kept_bytes_of<Rl<4>>(n);
+  return tr == 8 ? rl_kept_bytes_of<RlLarge>(n) : rl_kept_bytes_of<RlFew>(n);
 }
+// Scratch of a head: its rotated rows (2 MB at 2048 tokens of d_h 128) and its sums R, four bytes for each pair of
+// its tiles (9 MB; 137 MB at 8192 tokens).  Heads are independent, so a call whose heads need more than
+// kRlScratch takes them through its rounds in groups.  A head of over 22000 tokens needs more by itself:
+// its R is summed in every round.
+constexpr size_t kRlScratch = (size_t)1 << 30;
 RlCarve rl_carve(int heads, int n, int half) {
   RlCarve c;
   rl_form(heads, n, half, &c);
+  const size_t rot = c.tr == 1 ? 0 : sizeof(float) * 4 * (size_t)half * rl_pad_n(n);
+  const size_t kept = c.tr == 1 ? 0 : rl_kept_bytes(c.tr, n);
+  c.keep = c.tr != 1 && rot + kept <= kRlScratch;
+  const size_t per_head = rot + (c.keep ? kept : 0);
+  c.group = heads;
+  if (per_head * heads > kRlScratch) c.group = per_head < kRlScratch ? (int)(kRlScratch / per_head) : 1;
   size_t o = 0;
   c.off_cs = o;      o = rl_align(o + sizeof(float2) * (size_t)half * n);
   c.off_sin = o;     o = rl_align(o + sizeof(float) * (size_t)half * rl_sin_len(n));
-  c.off_partial = o; o = rl_align(o + sizeof(float) * (size_t)heads * c.items * half);
+  c.off_partial = o; o = rl_align(o + sizeof(float) * (size_t)c.group * c.items * half);
   c.off_masks = o;   o = rl_align(o + sizeof(unsigned long long) * (size_t)heads);
   c.off_state = o;   o = rl_align(o + sizeof(RlState) * (size_t)heads);
+  c.off_rot = o;     o = rl_align(o + (size_t)c.group * rot);
+  c.off_kept = o;    o = rl_align(o + (c.keep ? (size_t)c.group * kept : 0));
   c.total = o;
-  c.off_kept = o;
-  const size_t per_head = rl_kept_bytes(c.tr, n);
-  c.kept_heads = c.tr == 1 || per_head > kRlKeptMost ? 0 : (int)(kRlKeptMost / per_head < (size_t)heads ? kRlKeptMost / per_head : (size_t)heads);
-  c.total_kept = o + (size_t)c.kept_heads * per_head;
   return c;
 }
 
@@ -549,14 +642,15 @@ int rl_check(int heads, int n, int d_h) {
   return ELITEKV_OK;
 }
 
-struct RlKeep {
-  ulonglong2* kept;             // null: R is summed in every round
-  const RlState* state;
-  int first_round, last_round;
+// One round of the group's heads.  Q, K (the small form's), masks and state are the group's first.
+struct RlRound {
+  const bf16 *Q, *K;
+  const unsigned long long* masks;
+  const RlState* state;         // null: R is not kept
+  int first, last;              // round of the search
 };
 template <int HALF>
-int rl_launch_half(const void* Q, const void* K, int heads, int n, const RlCarve& c, unsigned char* base,
-                   const unsigned long long* masks, const RlKeep& k, cudaStream_t st) {
+int rl_launch_half(const RlRound& d, int heads, int n, const RlCarve& c, unsigned char* base, cudaStream_t st) {
   const float2* cs = (const float2*)(base + c.off_cs);
   const float* sn = (const float*)(base + c.off_sin);
   float* partial = (float*)(base + c.off_partial);
@@ -564,32 +658,40 @@ int rl_launch_half(const void* Q, const void* K, int heads, int n, const RlCarve
   if (c.tr == 1) {
     const auto kern = ropelite_distance_small_kernel<HALF>;
     EKV_CUDA_OK(ekv_allow_smem(kern, sizeof(RsSmem<HALF>)));
-    kern<<<grid, 32 * kRsWarps, sizeof(RsSmem<HALF>), st>>>((const bf16*)Q, (const bf16*)K, n, cs, sn, masks, partial);
+    EKV_CUDA_OK(ekv_launch_pdl(kern, grid, dim3(32 * kRsWarps), sizeof(RsSmem<HALF>), st, d.Q, d.K, n, cs, sn, d.masks, partial));
   } else {
     const auto launch = [&](auto form) -> int {
       using F = decltype(form);
       const auto kern = ropelite_distance_kernel<HALF, F>;
       EKV_CUDA_OK(ekv_allow_smem(kern, sizeof(RlSmem<HALF, F>)));
-      kern<<<grid, F::THREADS, sizeof(RlSmem<HALF, F>), st>>>((const bf16*)Q, (const bf16*)K, n, cs, sn, masks, c.span, partial,
-                                                              k.kept, k.state, k.first_round, k.last_round);
+      EKV_CUDA_OK(ekv_launch_pdl(kern, grid, dim3(F::THREADS), sizeof(RlSmem<HALF, F>), st, (const float*)(base + c.off_rot), n,
+                                 rl_pad_n(n), sn, d.masks, c.span, partial,
+                                 d.state ? (ulonglong2*)(base + c.off_kept) : nullptr, d.state, d.first, d.last));
       return ELITEKV_OK;
     };
-    const int rc = c.tr == 16 ? launch(Rl<16>()) : c.tr == 8 ? launch(Rl<8>()) : launch(Rl<4>());
+    const int rc = c.tr == 8 ? launch(RlLarge()) : launch(RlFew());
     if (rc != ELITEKV_OK) return rc;
   }
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }
-int rl_launch_distance(const void* Q, const void* K, int heads, int n, int d_h, const RlCarve& c, unsigned char* base,
-                       const unsigned long long* masks, const RlKeep& k, cudaStream_t st) {
-  return d_h == 128 ? rl_launch_half<64>(Q, K, heads, n, c, base, masks, k, st)
-                    : rl_launch_half<32>(Q, K, heads, n, c, base, masks, k, st);
+int rl_launch_distance(const RlRound& d, int heads, int n, int d_h, const RlCarve& c, unsigned char* base, cudaStream_t st) {
+  return d_h == 128 ? rl_launch_half<64>(d, heads, n, c, base, st) : rl_launch_half<32>(d, heads, n, c, base, st);
+}
+int rl_launch_rotate(const bf16* Q, const bf16* K, int heads, int n, int d_h, const RlCarve& c, unsigned char* base, cudaStream_t st) {
+  if (c.tr == 1) return ELITEKV_OK;
+  EKV_CUDA_OK(ekv_launch_pdl(ropelite_rotate_kernel, dim3((unsigned)rl_pad_n(n) / 64, (unsigned)heads, 2), dim3(256), 0, st, Q, K,
+                             (const float2*)(base + c.off_cs), (float*)(base + c.off_rot), n, rl_pad_n(n), d_h / 2,
+                             c.tr == 8 ? RlLarge::ROWS : RlFew::ROWS, (int)(c.tr == 8)));
+  EKV_CUDA_OK(cudaGetLastError());
+  return ELITEKV_OK;
 }
 
-int rl_launch_table(const RlCarve& c, unsigned char* base_ptr, int n, int d_h, float base, cudaStream_t st) {
+int rl_launch_table(const RlCarve& c, unsigned char* base_ptr, int n, int d_h, float base, unsigned long long* masks, int heads,
+                    cudaStream_t st) {
   const long long total = (long long)rl_sin_len(n) * (d_h / 2);
-  ropelite_table_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
-      (float2*)(base_ptr + c.off_cs), (float*)(base_ptr + c.off_sin), n, d_h / 2, d_h, (double)base);
+  EKV_CUDA_OK(ekv_launch_pdl(ropelite_table_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st,
+                             (float2*)(base_ptr + c.off_cs), (float*)(base_ptr + c.off_sin), n, d_h / 2, d_h, (double)base, masks, heads));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }
@@ -600,7 +702,7 @@ extern "C" int elitekv_ropelite_workspace_size(int32_t n_heads, int32_t n, int32
   if (!bytes) return ELITEKV_ERR_INVALID_ARG;
   const int rc = rl_check(n_heads, n, d_h);
   if (rc != ELITEKV_OK) return rc;
-  *bytes = rl_carve(n_heads, n, d_h / 2).total_kept;
+  *bytes = rl_carve(n_heads, n, d_h / 2).total;
   return ELITEKV_OK;
 }
 
@@ -617,13 +719,20 @@ extern "C" int elitekv_ropelite_distances(const void* Q, const void* K, int32_t 
   unsigned char* base = (unsigned char*)workspace;
   float* partial = (float*)(base + c.off_partial);
   cudaStream_t st = (cudaStream_t)stream;
-  rc = rl_launch_table(c, base, n, d_h, rope_base, st);
+  rc = rl_launch_table(c, base, n, d_h, rope_base, nullptr, 0, st);
   if (rc != ELITEKV_OK) return rc;
-  rc = rl_launch_distance(Q, K, n_heads, n, d_h, c, base, (const unsigned long long*)elite_mask, RlKeep{nullptr, nullptr, 1, 1}, st);
-  if (rc != ELITEKV_OK) return rc;
-  ropelite_select_kernel<<<n_heads, 64 * kRlSelect, 0, st>>>(partial, c.items, half,
-                                                 (unsigned long long*)elite_mask, dist, nullptr, 0, 0, nullptr);
-  EKV_CUDA_OK(cudaGetLastError());
+  unsigned long long* masks = (unsigned long long*)elite_mask;
+  for (int h0 = 0; h0 < n_heads; h0 += c.group) {
+    const int heads = n_heads - h0 < c.group ? n_heads - h0 : c.group;
+    const size_t at = (size_t)h0 * n * d_h;
+    const RlRound d{(const bf16*)Q + at, (const bf16*)K + at, masks ? masks + h0 : nullptr, nullptr, 1, 1};
+    rc = rl_launch_rotate(d.Q, d.K, heads, n, d_h, c, base, st);
+    if (rc == ELITEKV_OK) rc = rl_launch_distance(d, heads, n, d_h, c, base, st);
+    if (rc != ELITEKV_OK) return rc;
+    EKV_CUDA_OK(ekv_launch_pdl(ropelite_select_kernel, dim3(heads), dim3(64 * kRlSelect), 0, st, partial, c.items, half,
+                               masks ? masks + h0 : nullptr, dist + (size_t)h0 * half, nullptr, 0, 0, nullptr));
+    EKV_CUDA_OK(cudaGetLastError());
+  }
   return ELITEKV_OK;
 }
 
@@ -643,22 +752,21 @@ extern "C" int elitekv_ropelite_search(const void* Q, const void* K, int32_t n_h
   unsigned long long* masks = (unsigned long long*)(base + c.off_masks);
   RlState* state = (RlState*)(base + c.off_state);
   cudaStream_t st = (cudaStream_t)stream;
-  rc = rl_launch_table(c, base, n, d_h, rope_base, st);
+  rc = rl_launch_table(c, base, n, d_h, rope_base, masks, n_heads, st);
   if (rc != ELITEKV_OK) return rc;
-  EKV_CUDA_OK(cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)n_heads, st));
-  // a smaller workspace than the one asked for serves the form that keeps nothing
-  const bool keep = c.kept_heads > 0 && r > 1 && workspace_bytes >= c.total_kept;
-  const int group = keep ? c.kept_heads : n_heads;
-  for (int h0 = 0; h0 < n_heads; h0 += group) {
-    const int heads = n_heads - h0 < group ? n_heads - h0 : group;
-    const bf16 *Qg = (const bf16*)Q + (size_t)h0 * n * d_h, *Kg = (const bf16*)K + (size_t)h0 * n * d_h;
+  for (int h0 = 0; h0 < n_heads; h0 += c.group) {
+    const int heads = n_heads - h0 < c.group ? n_heads - h0 : c.group;
+    const size_t at = (size_t)h0 * n * d_h;
+    RlState* kept = c.keep && r > 1 ? state + h0 : nullptr;
+    rc = r > 0 ? rl_launch_rotate((const bf16*)Q + at, (const bf16*)K + at, heads, n, d_h, c, base, st) : ELITEKV_OK;
+    if (rc != ELITEKV_OK) return rc;
     for (int round = 0; round < r; ++round) {
-      rc = rl_launch_distance(Qg, Kg, heads, n, d_h, c, base, masks + h0,
-                              RlKeep{keep ? (ulonglong2*)(base + c.off_kept) : nullptr, state + h0, round == 0, round == r - 1}, st);
+      rc = rl_launch_distance(RlRound{(const bf16*)Q + at, (const bf16*)K + at, masks + h0, kept, round == 0, round == r - 1},
+                              heads, n, d_h, c, base, st);
       if (rc != ELITEKV_OK) return rc;
-      ropelite_select_kernel<<<heads, 64 * kRlSelect, 0, st>>>(partial, c.items, half, masks + h0,
-                                                     dist_trace ? dist_trace + ((size_t)round * n_heads + h0) * half : nullptr,
-                                                     elite_idx + (size_t)h0 * r, r, round, keep ? state + h0 : nullptr);
+      EKV_CUDA_OK(ekv_launch_pdl(ropelite_select_kernel, dim3(heads), dim3(64 * kRlSelect), 0, st, partial, c.items, half, masks + h0,
+                                 dist_trace ? dist_trace + ((size_t)round * n_heads + h0) * half : nullptr,
+                                 elite_idx + (size_t)h0 * r, r, round, kept));
       EKV_CUDA_OK(cudaGetLastError());
     }
   }

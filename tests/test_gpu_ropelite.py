@@ -88,6 +88,52 @@ def test_search(ek, graded):
     assert torch.equal(idx2.cpu(), torch.from_numpy(idx)) and torch.equal(trace2.cpu().double(), torch.from_numpy(trace))
 
 
+@pytest.mark.parametrize("H,n,d_h,r,graded", [(2, 260, 128, 9, False), (2, 129, 64, 31, True), (40, 193, 64, 3, False)])
+def test_search_with_kept_sums(ek, H, n, d_h, r, graded):
+    """Calls beyond the small form keep R between rounds: tiles that end inside a block's rows and keys, both
+    thread tiles, graded energies, whose norm falls so fast that R is summed afresh every few rounds, and all
+    rounds but the last one.  Every round against the oracle on the GPU's own list so far."""
+    Q, K = _acts(H, n, d_h, 31 + n, graded)
+    idx, trace = ek.elitekv_ropelite_search(Q.cuda(), K.cuda(), r, trace=True)
+    torch.cuda.synchronize()
+    idx, trace = idx.cpu().numpy(), trace.cpu().double().numpy()
+    for h in {0, H - 1}:
+        q, k = Q[h].double().numpy(), K[h].double().numpy()
+        elite = []
+        for rnd in range(r):
+            want = R.distances(q, k, elite, d_h)
+            fin = np.isfinite(want)
+            assert np.array_equal(np.isinf(trace[rnd, h]), ~fin)
+            assert np.allclose(trace[rnd, h][fin], want[fin], rtol=TOL, atol=1e-6)
+            assert want[idx[h, rnd]] <= want[fin].min() * (1 + TOL) + 1e-6
+            elite.append(int(idx[h, rnd]))
+        assert len(set(elite)) == r
+
+
+def test_search_energy_in_one_chunk(ek):
+    """R is that chunk's D alone: it goes first, and what is left of R is nothing, not a rounding error."""
+    Q, K = _acts(1, 200, 128, 5)
+    Q[:, :, :14] = 0
+    Q[:, :, 16:] = 0
+    idx, trace = ek.elitekv_ropelite_search(Q.cuda(), K.cuda(), 4, trace=True)
+    assert idx[0].tolist() == [7, 0, 1, 2]
+    assert torch.all(trace[1:][torch.isfinite(trace[1:])] == 0)
+
+
+def test_search_in_groups_of_heads(ek):
+    """More heads than the scratch holds at a time: the heads on both sides of the seam and the last one as in
+    calls of their own (sums in another order where the call's form differs: fp32, 1e-6)."""
+    H, n, d_h, r = 100, 2048, 128, 2
+    g = torch.Generator(device="cuda").manual_seed(3)
+    Q, K = (torch.randn((H, n, d_h), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    idx, trace = ek.elitekv_ropelite_search(Q, K, r, trace=True)
+    dist = ek.elitekv_ropelite_distances(Q, K)
+    for h in (0, 91, 92, 93, 94, 95, 96, 99):
+        one, t = ek.elitekv_ropelite_search(Q[h:h + 1].contiguous(), K[h:h + 1].contiguous(), r, trace=True)
+        assert torch.equal(one[0], idx[h])
+        assert torch.allclose(t[:, 0], trace[:, h], rtol=1e-6) and torch.allclose(dist[h], trace[0, h], rtol=1e-6)
+
+
 def test_argument_checks(ek):
     Q, K = _acts(1, 8, 32, 1)
     with pytest.raises(ek.ElitekvError) as e:        # d_h = 32 is not covered
