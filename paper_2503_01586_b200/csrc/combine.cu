@@ -38,10 +38,11 @@ constexpr int kFK = 128;         // latent slice
 constexpr int kFD = 128;         // head dim
 constexpr int kFThreads = 256;
 constexpr int kFPitch = kFD + 8; // shared-memory row pitch in bf16: 16 bytes of padding keep ldmatrix free of bank conflicts
+constexpr int kFSum = 12;        // slice results in flight when they are added: 7B B16 2.4 us from the last arrival to the last store, 3.0 in fours
 constexpr int kFAhead = 4;       // partial results per row in flight beside the statistics
 
-// kMore: blocks start at group g0 of n_groups (calls of more rows than one grid holds)
-template <bool kShare, bool kMore>
+// kMore: blocks start at group g0 of n_groups (calls of more rows than one grid holds).  kOne: one query row per sequence
+template <bool kShare, bool kMore, bool kOne>
 __global__ void __launch_bounds__(kFThreads, kShare ? 3 : 4)
 combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by the split-K kernel while this
                                                                    // kernel may already be resident: read
@@ -49,7 +50,8 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
                     const int32_t* seq_first, const bf16* __restrict__ Wuv,
                     float* __restrict__ slice_out /* [n_slices][B * rows][n_h][128] */,
                     int32_t* __restrict__ counters /* [n_h][groups], zeroed by the plan kernel */,
-                    bf16* __restrict__ out, int B, int rows, int n_h, int d_c, int g0, int n_groups) {
+                    bf16* __restrict__ out, int B, int n_query, int n_h, int d_c, int g0, int n_groups) {
+  const int rows = kOne ? 1 : n_query;
   __shared__ __align__(16) bf16 s_w[kFK][kFPitch];        // W_uv slice
   __shared__ __align__(16) bf16 s_o[2][kFB][kFPitch];     // merged latent outputs: bf16 head and remainder
   bf16 (*const s_hi)[kFPitch] = s_o[0];
@@ -210,20 +212,26 @@ combine_fast_kernel(const float* part_acc, const float* part_ml,   // written by
     }
   }
   // the block of a (head, group) that arrives last adds the slices in order
-  __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&counters[h * (kMore ? n_groups : gridDim.z) + g], 1) == n_slices - 1;
+  if (tid == 0) {
+    int before;      // (the barrier in front orders the block's stores before the release, the one behind its loads after the acquire)
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;"
+                 : "=r"(before) : "l"(counters + h * (kMore ? n_groups : gridDim.z) + g) : "memory");
+    s_last = before == n_slices - 1;
+  }
   __syncthreads();
   if (s_last) {
-    __threadfence();
     for (int e = tid; e < nb * (kFD / 4); e += kFThreads) {
       const int rr = e / (kFD / 4), d = (e % (kFD / 4)) * 4;
       const float* src = slice_out + ((size_t)(r0 + rr) * n_h + h) * kFD + d;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-      for (int s = 0; s < n_slices; ++s) {
-        const float4 y = __ldcg((const float4*)(src + (size_t)s * n_rows * n_h * kFD));
-        v.x += y.x; v.y += y.y; v.z += y.z; v.w += y.w;
+      for (int s0 = 0; s0 < n_slices; s0 += kFSum) {
+        float4 y[kFSum];
+#pragma unroll
+        for (int s = 0; s < kFSum; ++s)
+          y[s] = s0 + s < n_slices ? __ldcg((const float4*)(src + (size_t)(s0 + s) * n_rows * n_h * kFD)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < kFSum; ++s) { v.x += y[s].x; v.y += y[s].y; v.z += y[s].z; v.w += y[s].w; }
       }
       const bf162 o0 = __floats2bfloat162_rn(v.x, v.y), o1 = __floats2bfloat162_rn(v.z, v.w);
       bf162* dst = (bf162*)(out + ((size_t)(r0 + rr) * n_h + h) * kFD + d);      // the caller's `out` is 4-byte aligned
@@ -356,9 +364,10 @@ int ekv_launch_combine(const elitekv_layer* L, int B, const DecodeScratch& ws, v
     const int n_groups = (B * rows + kFB - 1) / kFB;
     // at most 8 rows: idle warps share the rows' items (a 7B step of one sequence: 34.8 -> 32.4 us at 32
     // items, 8 sequences 50.1 -> 49.4); from 9 rows on at least half of the warps have a pair of their own
-    const auto kern = n_groups > kGridZ ? combine_fast_kernel<false, true>
-                      : B * rows <= 8   ? combine_fast_kernel<true, false>
-                                        : combine_fast_kernel<false, false>;
+    const auto kern = n_groups > kGridZ ? combine_fast_kernel<false, true, false>
+                      : rows > 1        ? (B * rows <= 8 ? combine_fast_kernel<true, false, false> : combine_fast_kernel<false, false, false>)
+                      : B <= 8          ? combine_fast_kernel<true, false, true>
+                                        : combine_fast_kernel<false, false, true>;
     for (int g0 = 0; g0 < n_groups; g0 += kGridZ) {      // one launch up to a million rows
       const dim3 grid(L->n_h, L->vw / kFK, n_groups - g0 < kGridZ ? n_groups - g0 : kGridZ);
       EKV_CUDA_OK(ekv_launch_pdl(kern, grid, dim3(kFThreads), 0, st, (const float*)ws.part_acc, (const float*)ws.part_ml,
