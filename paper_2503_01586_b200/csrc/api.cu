@@ -78,7 +78,7 @@ int max_items_any(const elitekv_layer* L, int B) {
 }
 
 struct Carve {
-  size_t off_items, off_first, off_ml, off_acc, off_slice, off_cnt, off_wfirst, total;
+  size_t off_items, off_first, off_ml, off_acc, off_slice, off_cnt, off_wfirst, off_wrec, total;
 };
 
 // `rows` query rows per sequence: the partial results, the combine's scratch and its counters
@@ -93,6 +93,7 @@ Carve carve(const elitekv_layer* L, int B, int max_items, int rows = 1) {
   c.off_slice = o; o = align256(o + ekv_combine_scratch_bytes(L, B) * rows);
   c.off_cnt = o;   o = align256(o + sizeof(int32_t) * (size_t)ekv_combine_counters(L, B) * rows);
   c.off_wfirst = o; o = align256(o + sizeof(int32_t) * ((size_t)L->sm_count + 2));
+  c.off_wrec = o; o = align256(o + 2 * sizeof(int4) * (size_t)L->sm_count);
   c.total = o;
   return c;
 }
@@ -195,11 +196,12 @@ int decode_impl(const elitekv_layer* L, const elitekv_cache* cache, const void* 
   ws.counters = (int32_t*)(base + cw.off_cnt);
   ws.n_counters = ekv_combine_counters(L, B) * rows;
   ws.worker_first = (int32_t*)(base + cw.off_wfirst);
+  ws.worker_rec = kernel == 4 ? (int4*)(base + cw.off_wrec) : nullptr;
   ws.n_workers = workers_for(L, kernel, rows);
   // tokens one sequence can hold: longer lengths are reported by the plan kernel and clamped
   const long long max_len = cv.page_table ? (long long)cv.max_pages_per_seq << cv.page_shift : cv.max_ctx;
   rc = front(PlanArgs{seq_lens, B, plan_tile_for(kernel), ws.n_workers, max_items, ws.items, ws.seq_first, ws.worker_first,
-                      ws.counters, ws.n_counters, max_len, L->d_status, item_overhead_for(kernel)}, cv);
+                      ws.counters, ws.n_counters, max_len, L->d_status, item_overhead_for(kernel), ws.worker_rec}, cv);
   if (rc != ELITEKV_OK) return rc;
   EkvProfile* prof = (L->prof && L->prof->enabled && L->prof->count < kProfileSlots) ? L->prof : nullptr;
   if (prof) EKV_CUDA_OK(cudaEventRecord(prof->ev[2 * prof->count], st));

@@ -197,6 +197,7 @@ struct DecodeScratch {
   int32_t* counters;      // combine: arrival counters, zeroed by the plan kernel
   int n_counters;
   int32_t* worker_first;  // balanced plan: [n_workers+1] first item of each worker
+  int4* worker_rec;       // ... and its first item (PlanArgs), where the kernel wants it
   int n_workers;
   int rows;               // query rows per sequence (1: decode).  With rows > 1 every "n_h" in the shapes
                           // above reads rows * n_h: row i, head h is entry i * n_h + h

@@ -67,7 +67,7 @@ constexpr int kFinSlots = 3;           // items whose softmax statistics can be 
 
 struct ClArgs {
   const int32_t* items;
-  const int32_t* worker_first;
+  const int4* worker_rec;   // a worker's items and the first of them (PlanArgs)
   const int32_t* page_table;
   float* part_acc;          // [items][n_h][vw]
   float* part_ml;           // [items][n_h][2]
@@ -239,7 +239,10 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
   // come from kernels earlier in the stream.
   ekv_pdl_wait();
   ekv_pdl_trigger();
-  const int item_lo = __ldcg(a.worker_first + worker), item_hi = __ldcg(a.worker_first + worker + 1);
+  // one trip to L2 (worker_first, then the item: 0.7 us more before the first load)
+  const int4 rec = __ldcg(a.worker_rec + 2 * worker), rec_n = __ldcg(a.worker_rec + 2 * worker + 1);
+  const int item_lo = rec.x, item_hi = rec.y;
+  const ClCursor c0{item_lo, 0, (rec_n.x + kT - 1) / kT, rec.z, rec.w, rec_n.x};      // the worker's first tile
 
   // first cache row of a tile (tiles start on multiples of 64 tokens and pages hold a multiple
   // of 64 tokens, so a tile never straddles pages)
@@ -263,8 +266,7 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
     const bool report = warp == 0 && rank == 0;
     unsigned slot = 0, par = 0, g = 0, n = warp == 3 ? 1 : 0;     // n even: this warp's unit
     int my_row = 0, first_row = -1;                        // rows of tiles [first_row, first_row + 32) of the item
-    ClCursor c{item_lo, 0, 0, 0, 0, 0};
-    cl_settle(a.items, item_hi, c);
+    ClCursor c = c0;
     bool ok = true;
     while (ok && c.item < item_hi) {
       if (c.t == 0 || c.t == first_row + 32) {
@@ -297,7 +299,7 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
   else if (warp == 2) {
     const uint64_t pol_keep = make_l2_policy_evict_last();
     for (int item = item_lo; item < item_hi; ++item) {
-      const int seq = __ldcg(a.items + 4 * item);
+      const int seq = item == item_lo ? rec.z : __ldcg(a.items + 4 * item);
       // the previous item's last score product has read the old ones
       if (item > item_lo && !cl_wait(smem_u32(&bars->q_free), (unsigned)(item - item_lo - 1) & 1, s_abort, 12)) break;
       if (elect_one()) {
@@ -320,9 +322,7 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
     auto lo16 = [&](const unsigned char* p) { return ((smem_u32(p) >> 4) & 0x3FFFu) | (1u << 16); };
     const uint32_t ring16 = (smem_u32(s_ring) >> 4) & 0x3FFFu, q16 = lo16(base + L.q);
     const uint32_t empty0 = smem_u32(&bars->empty[0]);
-    ClCursor cs{item_lo, 0, 0, 0, 0, 0}, cp;
-    cl_settle(a.items, item_hi, cs);
-    cp = cs;
+    ClCursor cs = c0, cp = c0;
     unsigned s_slot = 0;                             // ring position of the first unit of the next score product
     unsigned p_slot = a.joint ? 0 : ku;              // ... and of the next value product
     unsigned gs = 0, gp = 0;                         // tiles whose scores / values have been issued
@@ -479,8 +479,7 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
     for (int p = 0; p < C; ++p) rb[p] = map_to_cta(b0, p);
     const uint32_t off_bar0 = (uint32_t)((unsigned char*)&bars->recv_full[0][0] - base);
     const int t = 16 * quarter + (lane & 15);        // token of this lane's score row (M = 64: 16 rows per warp)
-    ClCursor c{item_lo, 0, 0, 0, 0, 0};
-    cl_settle(a.items, item_hi, c);
+    ClCursor c = c0;
     for (unsigned g = 0; c.item < item_hi; ++g, cl_advance(a.items, item_hi, c, 1)) {
       const unsigned s = g & 1;
       const uint32_t off_recv = (uint32_t)L.recv + (s * C + rank) * (K::SRC * 4) + t * 16;
@@ -514,8 +513,7 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
     const float2* s_fin = (const float2*)(base + L.fin);
     float* fac = (float*)(base + L.fac) + quarter * 2 * NH;
-    ClCursor c{item_lo, 0, 0, 0, 0, 0};
-    cl_settle(a.items, item_hi, c);
+    ClCursor c = c0;
     unsigned n_cmd = 0, g0 = 0;                      // commands taken; tiles before the item
     while (c.item < item_hi) {
       if (!cl_wait(smem_u32(&bars->cmd_full), n_cmd & 1, s_abort, 15)) break;
@@ -547,8 +545,6 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
       const int only = (int)(g0 & 1);                // a one-tile item went through one stream
       if (threadIdx.x == 256) mbar_expect_tx(smem_u32(&bars->fin_full[slot]), (uint32_t)((both ? 2 : 1) * NH * 8));
       if (!cl_wait(smem_u32(&bars->fin_full[slot]), (unsigned)(k / kFinSlots) & 1, s_abort, 16)) break;
-      if (!cl_wait(smem_u32(&bars->acc_full), (unsigned)k & 1, s_abort, 10)) break;
-      tc_fence_after();
       // merge factors of the two streams (every warp its own copy), and the item's statistics
       for (int v = lane; v < NH; v += 32) {
         const float2 x0 = s_fin[(slot * 2 + 0) * NH + v], x1 = s_fin[(slot * 2 + 1) * NH + v];
@@ -564,21 +560,33 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
       __syncwarp();
       // a [128 columns x heads] block leaves TMEM with one thread per latent column: for a fixed
       // head the lanes of a warp hold 32 consecutive columns, 128-byte stores from registers
+      // (The factors are read before the stores: behind one, each read of shared memory would wait for it.  From the
+      // last value product to the last store 2.1 us, 2.9 with a factor read per store.)
       float* dst = a.part_acc + (size_t)c.item * NH * a.vw + (size_t)rank * vu * 128 + quarter * 32 + lane;
-      for (int u = 0; u < vu; ++u) {
+      if (!cl_wait(smem_u32(&bars->acc_full), (unsigned)k & 1, s_abort, 10)) break;
+      tc_fence_after();
 #pragma unroll 1
-        for (int col = 0; col < NH; col += 8) {
+      for (int col = 0; col < NH; col += 8) {
+        float f0[8], f1[8];
+#pragma unroll
+        for (int j = 0; j < 8; j += 4) {
+          *(float4*)&f0[j] = *(const float4*)&fac[col + j];
+          *(float4*)&f1[j] = *(const float4*)&fac[NH + col + j];
+        }
+#pragma unroll 1
+        for (int u = 0; u < vu; ++u) {
           float v0[8], v1[8];
-          if (both || only == 0) tc_ld8(tmem_base + (uint32_t)(u * NP + col) + lane_base, v0);
-          if (both || only == 1) tc_ld8(tmem_base + (uint32_t)((vu + u) * NP + col) + lane_base, v1);
+          const uint32_t at = tmem_base + (uint32_t)(u * NP + col) + lane_base;
+          if (both || only == 0) tc_ld8(at, v0);
+          if (both || only == 1) tc_ld8(at + vu * NP, v1);
           tc_wait_ld();
+          float* out = dst + (size_t)col * a.vw + u * 128;
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const int v = col + j;
             float y = 0.f;
-            if (both || only == 0) y = v0[j] * fac[v];
-            if (both || only == 1) y = fmaf(v1[j], fac[NH + v], y);
-            __stcg(dst + (size_t)v * a.vw + u * 128, y);
+            if (both || only == 0) y = v0[j] * f0[j];
+            if (both || only == 1) y = fmaf(v1[j], f1[j], y);
+            __stcg(out + (size_t)j * a.vw, y);
           }
         }
       }
@@ -597,9 +605,7 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
     constexpr int kAhead = 2;
     const int quarter = warp & 3, piece = lane & 15;
     const bf16* plane = a.rope_plane + rank * 128 + piece * 8;
-    ClCursor c{item_lo, 0, 0, 0, 0, 0}, ld, pf;      // tiles computed, loaded, prefetched next
-    cl_settle(a.items, item_hi, c);
-    ld = pf = c;
+    ClCursor c = c0, ld = c0, pf = c0;               // tiles computed, loaded, prefetched next
     int row_q[kAhead + 1] = {};                      // cache rows of the tiles between ld and pf
     int n_q = 0;
     uint4 raw[8];
@@ -713,8 +719,8 @@ decode_cl_kernel(const __grid_constant__ CUtensorMap map_lat, const __grid_const
     float m_ref[4 * QW], l_sum[4 * QW];
     bool fresh = true;                               // the next tile is this stream's first of its item
     unsigned par = 0;
-    ClCursor c{item_lo, s, 0, 0, 0, 0};
-    cl_settle(a.items, item_hi, c);
+    ClCursor c = c0;
+    if (s) cl_advance(a.items, item_hi, c, 1);
     while (c.item < item_hi) {
       if (lane < QW) mbar_expect_tx(smem_u32(&bars->recv_full[s][q0 + lane]), (uint32_t)(C * 1024));
       if (fresh) {
@@ -960,7 +966,7 @@ int ekv_launch_decode_cl(const elitekv_layer* L, const elitekv_cache* cache, con
       rc = cl_make_map(&m_q, q_abs, (unsigned long long)B * L->n_h, L->kw, K::NH, 2 * a.ku);
     if (rc != ELITEKV_OK) return rc;
     a.items = ws.items;
-    a.worker_first = ws.worker_first;
+    a.worker_rec = ws.worker_rec;
     a.page_table = cv.page_table;
     a.part_acc = ws.part_acc;
     a.part_ml = ws.part_ml;

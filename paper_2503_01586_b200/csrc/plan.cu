@@ -13,10 +13,9 @@ namespace {
 
 template <class T>
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const PlanArgs a) {
-  ekv_pdl_wait();         // earlier kernels may still read the arrays written here
-  ekv_pdl_trigger();
+  ekv_pdl_trigger();      // (whoever comes next waits for this grid's completion itself)
   __shared__ PlanShared<T> sh;
-  plan_any(a, sh);
+  plan_behind_wait(a, sh);      // earlier kernels may still read the arrays written here
 }
 
 }  // namespace
@@ -34,7 +33,7 @@ extern "C" int elitekv_plan(const int32_t* seq_lens, int32_t B, int32_t tile_tok
     return ELITEKV_ERR_INVALID_ARG;
   if ((uintptr_t)items & 15) return ELITEKV_ERR_INVALID_ARG;
   return ekv_launch_plan(PlanArgs{seq_lens, B, tile_tokens, 0, max_items, items, seq_first_item, nullptr, nullptr, 0,
-                                  0x7fffffffLL, nullptr, 0}, (cudaStream_t)stream);
+                                  0x7fffffffLL, nullptr, 0, nullptr}, (cudaStream_t)stream);
 }
 
 extern "C" int elitekv_plan_workers(const int32_t* seq_lens, int32_t B, int32_t tile_tokens,
@@ -46,5 +45,5 @@ extern "C" int elitekv_plan_workers(const int32_t* seq_lens, int32_t B, int32_t 
     return ELITEKV_ERR_INVALID_ARG;
   if ((uintptr_t)items & 15) return ELITEKV_ERR_INVALID_ARG;
   return ekv_launch_plan(PlanArgs{seq_lens, B, tile_tokens, n_workers, max_items, items, seq_first_item, worker_first,
-                                  nullptr, 0, 0x7fffffffLL, nullptr, item_overhead_tiles}, (cudaStream_t)stream);
+                                  nullptr, 0, 0x7fffffffLL, nullptr, item_overhead_tiles, nullptr}, (cudaStream_t)stream);
 }

@@ -67,6 +67,8 @@ struct PlanArgs {
   long long max_len;           // tokens one sequence can hold: longer (or negative) lengths are recorded and clamped
   int32_t* status;
   int overhead;
+  int4* worker_rec;            // balanced plans, optional: [n_workers][2], what worker_first and items say of a worker's
+                               // first item in one place: first item, end of the items, sequence, first token | token count
 };
 // B lengths of up to max_len tokens make less than 2^31 tiles, and the tile that holds the last token ends below 2^31
 inline bool plan_narrow(int B, int tile, long long max_len, int overhead) {
@@ -81,6 +83,89 @@ __device__ __forceinline__ long long plan_div(long long x, long long y) {
 template <class T>
 __device__ __forceinline__ T plan_tiles(int n, int tile) {
   return sizeof(T) == 8 ? (T)plan_div((long long)n + tile - 1, tile) : ((T)n + tile - 1) / tile;
+}
+
+// One copy of the division for all its uses: see plan_quick
+static __device__ __noinline__ unsigned plan_udiv(unsigned x, unsigned y) { return x / y; }
+
+// Balanced plan of up to 32 sequences, a lane per sequence: every warp has the whole batch in its registers, so there
+// is no barrier and no shared memory.  A step's plan is run once, by one block, with instructions that are not in
+// the caches: 10 us where the uses of a search and of an item are unrolled and inlined one by one, 2 us when that
+// runs a second time at once.  So there is one copy of each, items and workers are chunks of one loop,
+// and a block that has to wait for the kernel before it makes the trip once without effect (dry): 2.5 to 3 us
+// behind the wait, 4 to 5 for plan_small.  (The even plan has hundreds of items, for which
+// a warp per 32 is the slower way: the smallest model's step 15.9 us, 14.6 with plan_small.)
+// False, with nothing but the counters and reports written, where a product does not fit 32 bits.
+// The arithmetic is that of plan_balanced below.
+__device__ __forceinline__ bool plan_quick_ok(const PlanArgs& a) { return a.n_workers > 0 && a.B <= 32; }
+__device__ __forceinline__ bool plan_quick(const PlanArgs& a, bool dry) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int t = threadIdx.x, lane = t & 31, B = a.B;
+  const unsigned overhead = a.overhead;
+  int n = 0;
+  if (dry) n = lane < B ? a.tile : 0;
+  else if (lane < B) n = checked_len(a.seq_lens, lane, a.max_len, a.status, t < 32);
+  if (!dry)
+    for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
+  const unsigned tiles = n > 0 ? plan_udiv((unsigned)n + a.tile - 1, (unsigned)a.tile) + overhead : 0;
+  // inclusive sums
+  unsigned g1 = 0, pieces = 0, w0 = 0, f1 = 0, total = 1, nw = 1;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    unsigned v = pass ? pieces : tiles;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned x = __shfl_up_sync(kAll, v, o);
+      if (lane >= o) v += x;
+    }
+    if (pass) {
+      f1 = v;
+      break;
+    }
+    g1 = v;
+    total = max(__shfl_sync(kAll, v, 31), 1u);
+    if (total >= plan_udiv(kAll, (unsigned)a.n_workers)) return false;
+    nw = min(total, (unsigned)a.n_workers);
+    w0 = plan_udiv((g1 - tiles + overhead + 1) * nw - 1, total);
+    const unsigned last = plan_udiv(g1 * nw - 1, total);
+    if (tiles > 0) pieces = last - w0 + 1;
+  }
+  const unsigned g0 = g1 - tiles, first = f1 - pieces;
+  const int n_items = (int)__shfl_sync(kAll, f1, 31);
+  if (!dry && t <= B) a.seq_first[t] = t < B ? (int)first : n_items;
+  // chunks of 32 items, then of 31 workers (and the one behind them, whose first item ends the last one's)
+  const int item_chunks = (a.max_items + 31) / 32, chunks = item_chunks + (a.n_workers + 31) / 31;
+#pragma unroll 1
+  for (int c = t >> 5; c < chunks; c += kPlanThreads / 32) {
+    const bool wk = c >= item_chunks;
+    const unsigned i = wk ? (c - item_chunks) * 31 + lane : c * 32 + lane;
+    // the sequence of item i, or of the first position of worker i's range: the last one whose first item (first
+    // position) is not past it; an empty sequence has that of the one behind it
+    const unsigned key = wk ? g0 : first, x = wk ? plan_udiv(min(i, nw) * total, nw) : i;
+    int s = 0;
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned k = __shfl_sync(kAll, key, s + o);      // (s + o <= 31)
+      if (s + o < B && k <= x) s += o;
+    }
+    const unsigned g = __shfl_sync(kAll, g0, s), tl = __shfl_sync(kAll, tiles, s), sw = __shfl_sync(kAll, w0, s);
+    const unsigned len = (unsigned)__shfl_sync(kAll, n, s), f = __shfl_sync(kAll, first, s);
+    const unsigned j = wk ? (i > sw ? i - sw : 0) : i - f, w = sw + j, base = g + overhead;
+    const unsigned ta = max(base, plan_udiv(w * total, nw)) - base, tb = min(g + tl, plan_udiv((w + 1) * total, nw)) - base;
+    const int tok0 = (int)(ta * a.tile), ntok = (int)min(tb * a.tile, len) - tok0;
+    const int lo = i < nw ? (int)(f + j) : n_items, hi = __shfl_down_sync(kAll, lo, 1);
+    if (dry) continue;
+    if (!wk) {
+      if (i < (unsigned)a.max_items) *(int4*)(a.items + 4 * i) = (int)i < n_items ? make_int4(s, tok0, ntok, (int)w) : make_int4(-1, 0, 0, 0);
+    } else if (lane < 31 && (int)i <= a.n_workers) {
+      a.worker_first[i] = lo;
+      if (a.worker_rec && (int)i < a.n_workers) {
+        a.worker_rec[2 * i] = make_int4(lo, hi, s, tok0);
+        a.worker_rec[2 * i + 1] = make_int4(ntok, 0, 0, 0);
+      }
+    }
+  }
+  return true;
 }
 
 // Batches of at most a sequence per thread: both plans in one trip for the lengths, two scans and one
@@ -164,18 +249,23 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh)
       if (s_wk[mid] < w) lo = mid + 1; else hi = mid;
     }
     a.worker_first[w] = lo;
+    if (a.worker_rec && w < a.n_workers) {
+      const bool any = lo < held && s_wk[lo] == w;
+      int end = lo;                          // (a worker has few items)
+      while (end < held && s_wk[end] == w) ++end;
+      const int4 x = any ? *(const int4*)(a.items + 4 * lo) : make_int4(0, 0, 0, 0);
+      a.worker_rec[2 * w] = make_int4(lo, end, x.x, x.y);
+      a.worker_rec[2 * w + 1] = make_int4(x.z, 0, 0, 0);
+    }
   }
 }
 
 template <class T>
 __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared<T>& sh) {
-  const int32_t* __restrict__ seq_lens = a.seq_lens;
   const int B = a.B, tile = a.tile, max_items = a.max_items, n_zero = a.n_zero;
   int32_t* __restrict__ items = a.items;
   int32_t* __restrict__ seq_first = a.seq_first;
   int32_t* __restrict__ zero_ints = a.zero_ints;
-  const long long max_len = a.max_len;
-  int32_t* status = a.status;
   T* const warp_tot = sh.warp_tot;
   long long& s_total = sh.total;
   const int t = threadIdx.x;
@@ -184,7 +274,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared<T>& sh) 
   __syncthreads();
   long long local = 0;
   for (int b = t; b < B; b += blockDim.x) {
-    int n = checked_len(seq_lens, b, max_len, status, true);
+    int n = checked_len(a.seq_lens, b, a.max_len, a.status, true);
     local += n > 0 ? plan_tiles<T>(n, tile) : 0;
   }
   if (local) atomicAdd((unsigned long long*)&s_total, (unsigned long long)local);
@@ -199,7 +289,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared<T>& sh) 
     const int b = b0 + t;
     int n = 0, tiles = 0, pieces = 0;
     if (b < B) {
-      n = checked_len(seq_lens, b, max_len, status, false);
+      n = checked_len(a.seq_lens, b, a.max_len, a.status, false);
       tiles = n > 0 ? (int)plan_tiles<T>(n, tile) : 0;
       pieces = (int)((tiles + target - 1) / target);
     }
@@ -234,14 +324,11 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared<T>& sh) 
 // sequence: they take room in a worker's quota and hold no tokens.
 template <class T>
 __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& sh) {
-  const int32_t* __restrict__ seq_lens = a.seq_lens;
   const int B = a.B, tile = a.tile, n_workers = a.n_workers, max_items = a.max_items, overhead = a.overhead, n_zero = a.n_zero;
   int32_t* __restrict__ items = a.items;
   int32_t* __restrict__ seq_first = a.seq_first;
   int32_t* __restrict__ worker_first = a.worker_first;
   int32_t* __restrict__ zero_ints = a.zero_ints;
-  const long long max_len = a.max_len;
-  int32_t* status = a.status;
   T* const warp_tot = sh.warp_tot;
   long long& s_total = sh.total;
   short* const s_wk = sh.wk;
@@ -251,7 +338,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& 
   __syncthreads();
   long long local = 0;
   for (int b = t; b < B; b += blockDim.x) {
-    int n = checked_len(seq_lens, b, max_len, status, true);
+    int n = checked_len(a.seq_lens, b, a.max_len, a.status, true);
     local += n > 0 ? plan_tiles<T>(n, tile) + overhead : 0;
   }
   if (local) atomicAdd((unsigned long long*)&s_total, (unsigned long long)local);
@@ -270,7 +357,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& 
       int n = 0;
       T tiles = 0;
       if (b < B) {
-        n = checked_len(seq_lens, b, max_len, status, false);
+        n = checked_len(a.seq_lens, b, a.max_len, a.status, false);
         tiles = n > 0 ? plan_tiles<T>(n, tile) + overhead : 0;     // with the empty tiles in front
       }
       T chunk_tiles;
@@ -331,8 +418,35 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& 
 }
 
 template <class T>
-__device__ __forceinline__ void plan_any(const PlanArgs& a, PlanShared<T>& sh) {
-  if (plan_small_ok(a)) plan_small(a, sh);
-  else if (a.n_workers > 0) plan_balanced(a, sh);
+__device__ __forceinline__ void plan_general(const PlanArgs& a, PlanShared<T>& sh) {
+  if (plan_small_ok(a)) {
+    plan_small(a, sh);
+    return;
+  }
+  if (a.n_workers > 0) plan_balanced(a, sh);
   else plan_even(a, sh);
+  if (a.worker_rec) {
+    __syncthreads();
+    for (int w = threadIdx.x; w < a.n_workers; w += kPlanThreads) {
+      const int lo = a.worker_first[w], hi = a.worker_first[w + 1];
+      const int4 x = lo < hi ? *(const int4*)(a.items + 4 * lo) : make_int4(0, 0, 0, 0);
+      a.worker_rec[2 * w] = make_int4(lo, hi, x.x, x.y);
+      a.worker_rec[2 * w + 1] = make_int4(x.z, 0, 0, 0);
+    }
+  }
+}
+// A whole plan, with the wait for the kernels before in front of the first trip to memory.
+template <class T>
+__device__ __forceinline__ void plan_behind_wait(const PlanArgs& a, PlanShared<T>& sh) {
+  bool done = false;
+  if (sizeof(T) == 4 && plan_quick_ok(a)) {
+#pragma unroll 1
+    for (int dry = 1; dry >= 0; --dry) {
+      if (!dry) ekv_pdl_wait();
+      done = plan_quick(a, dry);
+    }
+  } else {
+    ekv_pdl_wait();
+  }
+  if (!done) plan_general(a, sh);
 }

@@ -25,8 +25,7 @@ step_prep_kernel(const AbsorbArgs q, const AppendArgs t, const PlanArgs p, int n
   ekv_pdl_trigger();      // the attention kernel waits for this grid's completion itself
   int blk = blockIdx.x;
   if (blk == 0) {
-    ekv_pdl_wait();
-    plan_any(p, *(PlanShared<int>*)smem_b);
+    plan_behind_wait(p, *(PlanShared<int>*)smem_b);
     return;
   }
   blk -= 1;

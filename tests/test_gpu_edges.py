@@ -354,6 +354,17 @@ def test_plans_on_both_sides_of_a_sequence_per_thread(ek, B, n_workers):
     T.test_plan_partitions_every_sequence(ek, lens, B + 300)
 
 
+@pytest.mark.parametrize("B", [1, 32, 33, 257])
+def test_cluster_kernel_behind_every_form_of_the_plan(ek, B):
+    """The cluster kernel starts from the plan's record of each worker's first item, which a plan of a lane per
+    sequence (up to 32), of a thread per sequence (256) and of a loop writes in its own way; empty
+    sequences at the front, and workers without items."""
+    w = gen.shrink(gen.LLAMA7B_75, B=B, ctx=300)
+    st = H.setup(w, lens=[300] if B == 1 else [0 if b % 7 == 0 else 1 + (37 * b) % 150 for b in range(B)])
+    assert ek.elitekv_decode_plan_info(st.layer, st.cache, B)[0] == 4
+    H.check_parity(st, H.run_decode(st), H.sample_units(st, 24, seed=B))
+
+
 MOST = 2 ** 31 - 1
 
 
