@@ -478,8 +478,8 @@ def attend_rows_bench(ek, layer, cache, w, lens, device, flush, cache_bytes, rep
 def ropelite_bench(ek, device, reps: int = 3):
     """RoPElite search (Algorithm 1) on synthetic activations of one 7B-shaped layer: 32 heads,
     d_h = 128, a calibration sequence of 2048 tokens, r = 8 rounds.  ALU-bound: per causal pair and
-    chunk the kernel issues 9 FP32 lane instructions (two 2-term products, the rotated-minus-plain
-    term, the masked residual sum, the absolute difference into the candidate's running sum);
+    chunk the first round takes 7 FP32 lane operations (the chunk's term twice, summed and taken off),
+    a later one 4 (the term, taken off the kept sum, and the absolute difference into the candidate's distance);
     peak = SMs x 128 FP32 lanes x the maximum SM clock."""
     H, n, d_h, r = 32, 2048, 128, 8
     g = torch.Generator(device=device).manual_seed(31337)
@@ -497,7 +497,7 @@ def ropelite_bench(ek, device, reps: int = 3):
     torch.cuda.synchronize()
     ms = sum(a.elapsed_time(b) for a, b in evs) / reps
     pairs = H * n * (n + 1) // 2
-    lane_instr = 9.0 * (d_h // 2) * pairs * r
+    lane_instr = float(7 * (d_h // 2) + sum(4 * (d_h // 2 - k) for k in range(1, r))) * pairs
     props = torch.cuda.get_device_properties(device)
     peak = props.multi_processor_count * 128 * 1.965e9
     # the float64 oracle on a small sample of the same activations: one head, 256 tokens, one round

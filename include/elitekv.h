@@ -227,7 +227,8 @@ int elitekv_attend_rows(const elitekv_layer* layer, const elitekv_cache* cache, 
  *     chosen (the order elitekv_params.elite_idx wants).  dist_trace: optional fp32
  *     [r][n_heads][d_h/2], the distances of every round.
  * Sums are fp32 and added in a fixed order (results do not depend on scheduling).  workspace:
- * 256-byte aligned, elitekv_ropelite_workspace_size bytes. */
+ * 256-byte aligned, elitekv_ropelite_workspace_size bytes: beside small tables 11 MB a head at 2048 tokens of d_h 128
+ * (rotated rows, and the pairs' sums that a search keeps between rounds), for as many heads as fit 1 GiB at a time. */
 int elitekv_ropelite_workspace_size(int32_t n_heads, int32_t n, int32_t d_h, size_t* bytes);
 int elitekv_ropelite_distances(const void* Q, const void* K, int32_t n_heads, int32_t n, int32_t d_h,
                                float rope_base, const uint64_t* elite_mask, void* workspace,
