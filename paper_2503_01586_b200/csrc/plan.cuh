@@ -177,15 +177,18 @@ __device__ __forceinline__ bool plan_small_ok(const PlanArgs& a) {
   return a.B <= kPlanThreads && a.n_workers + a.B <= kPlanStage;
 }
 template <class T>
-__device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh) {
+__device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh, bool dry) {
   T *const warp_tot = sh.warp_tot, *const s_g0 = sh.g0, *const s_tiles = sh.tiles;
   int *const s_first = sh.first, *const s_len = sh.len;
   short *const s_w0 = sh.w0, *const s_wk = sh.wk;
   const int t = threadIdx.x, B = a.B;
   const bool balanced = a.n_workers > 0;
   const int overhead = balanced ? a.overhead : 0;      // empty tiles in front of every sequence
-  const int n = t < B ? checked_len(a.seq_lens, t, a.max_len, a.status, true) : 0;
-  for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
+  int n = 0;
+  if (dry) n = t < B ? a.tile : 0;
+  else if (t < B) n = checked_len(a.seq_lens, t, a.max_len, a.status, true);
+  if (!dry)
+    for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
   const T tiles = n > 0 ? (T)plan_div((long long)n + a.tile - 1, a.tile) + overhead : 0;
   T sum;
   const T g0 = block_exclusive_scan(tiles, warp_tot, &sum);
@@ -207,10 +210,10 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh)
   int n_items;
   const int first = block_exclusive_scan(pieces, warp_tot, &n_items);
   if (t < B) {
-    a.seq_first[t] = first;
+    if (!dry) a.seq_first[t] = first;
     s_first[t] = first; s_g0[t] = g0; s_len[t] = n; s_tiles[t] = tiles; s_w0[t] = (short)w0;
   }
-  if (t == 0) a.seq_first[B] = n_items;
+  if (t == 0 && !dry) a.seq_first[B] = n_items;
   __syncthreads();
   for (int it = t; it < a.max_items; it += kPlanThreads) {
     int4 item = make_int4(-1, 0, 0, 0);
@@ -237,7 +240,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh)
       const int tok0 = ta * a.tile;
       item = make_int4(lo, tok0, (int)min((T)tb * a.tile, (T)len) - tok0, w);
     }
-    *(int4*)(a.items + 4 * it) = item;
+    if (!dry) *(int4*)(a.items + 4 * it) = item;
   }
   if (!balanced) return;
   __syncthreads();
@@ -248,6 +251,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh)
       const int mid = (lo + hi) >> 1;
       if (s_wk[mid] < w) lo = mid + 1; else hi = mid;
     }
+    if (dry) continue;
     a.worker_first[w] = lo;
     if (a.worker_rec && w < a.n_workers) {
       const bool any = lo < held && s_wk[lo] == w;
@@ -418,11 +422,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& 
 }
 
 template <class T>
-__device__ __forceinline__ void plan_general(const PlanArgs& a, PlanShared<T>& sh) {
-  if (plan_small_ok(a)) {
-    plan_small(a, sh);
-    return;
-  }
+__device__ __forceinline__ void plan_large(const PlanArgs& a, PlanShared<T>& sh) {
   if (a.n_workers > 0) plan_balanced(a, sh);
   else plan_even(a, sh);
   if (a.worker_rec) {
@@ -435,18 +435,27 @@ __device__ __forceinline__ void plan_general(const PlanArgs& a, PlanShared<T>& s
     }
   }
 }
-// A whole plan, with the wait for the kernels before in front of the first trip to memory.
+// A whole plan, with the wait for the kernels before in front of the first trip to memory; the forms for up to
+// a sequence per thread make a first trip without effect before it (plan_quick).
 template <class T>
 __device__ __forceinline__ void plan_behind_wait(const PlanArgs& a, PlanShared<T>& sh) {
-  bool done = false;
   if (sizeof(T) == 4 && plan_quick_ok(a)) {
+    bool done = false;
 #pragma unroll 1
     for (int dry = 1; dry >= 0; --dry) {
       if (!dry) ekv_pdl_wait();
       done = plan_quick(a, dry);
     }
-  } else {
-    ekv_pdl_wait();
+    if (done) return;
   }
-  if (!done) plan_general(a, sh);
+  if (plan_small_ok(a)) {
+#pragma unroll 1
+    for (int dry = 1; dry >= 0; --dry) {
+      if (!dry) ekv_pdl_wait();
+      plan_small(a, sh, dry);
+    }
+    return;
+  }
+  ekv_pdl_wait();
+  plan_large(a, sh);
 }
