@@ -38,6 +38,11 @@
 // zero at negative relative positions, which is the causal mask.  Item results go to a
 // [head][item][chunk] array; the select kernel adds them in a fixed order (the result does not
 // depend on scheduling), masks the chunks already chosen and takes the first minimum.
+//
+// The kernels of a search are a chain of programmatic dependent launches: one is resident while the one before it
+// still writes.  What a kernel reads of its predecessors (tables, rotated rows, item results, masks, states) comes behind
+// ekv_pdl_wait, by the copy engine or with plain L2 loads: never ld.global.nc, which a compiler may make of a
+// `const __restrict__` pointer and move in front of the wait, and never from an L1 line that holds an older neighbour.
 #include "tc_ptx.cuh"
 
 namespace {
@@ -96,7 +101,7 @@ __global__ void ropelite_table_kernel(float2* __restrict__ cs, float* __restrict
 __device__ __forceinline__ void rl_rotate4(const bf16* row, const float2* cs, float2* out) {
   const uint4 raw = *(const uint4*)row;
   const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-  const float4 c01 = __ldg((const float4*)cs), c23 = __ldg((const float4*)cs + 1);
+  const float4 c01 = __ldcg((const float4*)cs), c23 = __ldcg((const float4*)cs + 1);
   const float2 c[4] = {{c01.x, c01.y}, {c01.z, c01.w}, {c23.x, c23.y}, {c23.z, c23.w}};
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -109,7 +114,7 @@ __device__ __forceinline__ void rl_rotate4(const bf16* row, const float2* cs, fl
 // copies them, per head Q [row tile][chunk][x, y][tile rows], K [tile of 128 keys][chunk][x, y][keys]; the first four of every
 // eight keys of a tile come before the others where a thread takes eight.  Every row tile, key tile and round reads them.
 // Grid (rows / 64, heads, Q or K), 256 threads.
-__global__ void ropelite_rotate_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, const float2* __restrict__ cs,
+__global__ void ropelite_rotate_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, const float2* cs,
                                        float* __restrict__ rot, int n, int n_pad, int half, int q_rows, int split) {
   ekv_pdl_wait();
   ekv_pdl_trigger();
@@ -248,11 +253,11 @@ __host__ __device__ inline long long rl_tiles_below(int mt) {
 
 template <int HALF, class F>
 __global__ void __launch_bounds__(F::THREADS, F::TR == 8 ? 3 : 2)
-ropelite_distance_kernel(const float* __restrict__ rot /* [heads]: Q, K (ropelite_rotate_kernel) */, int n, int n_pad,
-                         const float* __restrict__ sn, const unsigned long long* __restrict__ masks, int span,
+ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kernel) */, int n, int n_pad,
+                         const float* sn, const unsigned long long* masks, int span,
                          float* __restrict__ partial /* [heads][items][HALF] */,
-                         ulonglong2* __restrict__ kept /* [heads][tiles][VALUES][THREADS], null: R is not kept */,
-                         const RlState* __restrict__ state, int first_round, int last_round) {
+                         ulonglong2* kept /* [heads][tiles][VALUES][THREADS], null: R is not kept */,
+                         const RlState* state, int first_round, int last_round) {
   constexpr int TR = F::TR, TK = F::TK, NW = F::NW, THREADS = F::THREADS, ROWS = F::ROWS;
   extern __shared__ __align__(128) unsigned char smem_rl[];
   RlSmem<HALF, F>& sm = *(RlSmem<HALF, F>*)smem_rl;
@@ -268,20 +273,10 @@ ropelite_distance_kernel(const float* __restrict__ rot /* [heads]: Q, K (ropelit
   ekv_pdl_trigger();
   const int m0 = mt * ROWS;
   const int n_lo = kg * span * kRlKeys, n_hi = min(n_lo + span * kRlKeys, m0 + ROWS);
-  const unsigned long long mask = masks ? masks[head] : 0ull;
-  const int n_free = HALF - __popcll(HALF == 64 ? mask : mask & ((1ull << (HALF & 63)) - 1));
-  float* out = partial + ((size_t)head * gridDim.x + blockIdx.x) * HALF;
-  if (n_free <= 1) {                 // a single free chunk: R = D_j for every pair
-    for (int j = threadIdx.x; j < HALF; j += THREADS) out[j] = 0.f;
-    return;
-  }
-  const bool fresh = kept == nullptr || first_round || state[head].fresh;
-  // one that R has to lose, then the free ones
-  const int n_old = fresh ? 0 : 1, n_list = n_old + n_free, parts = (n_list + F::PART - 1) / F::PART;
-  if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
-    sm.list[n_old + threadIdx.x - __popcll(mask & ((1ull << threadIdx.x) - 1))] = threadIdx.x;
+  const unsigned long long mask = masks ? __ldcg(masks + head) : 0ull;
+  const int before = kept ? __ldcg(&state[head].last) : 0, again = kept ? __ldcg(&state[head].fresh) : 1;
+  // one trip to L2 for all three, and meanwhile:
   if (threadIdx.x == 0) {
-    if (!fresh) sm.list[0] = state[head].last;
     sm.failed = 0;
     for (int i = 0; i < F::STAGES; ++i) {
       mbar_init(smem_u32(&sm.full[i]), 1);
@@ -290,11 +285,23 @@ ropelite_distance_kernel(const float* __restrict__ rot /* [heads]: Q, K (ropelit
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_proxy_async();
   }
+  for (int e = threadIdx.x; e < HALF * NW * kRlAcc; e += THREADS) (&sm.acc[0][0])[e] = 0.f;
+  const int n_free = HALF - __popcll(HALF == 64 ? mask : mask & ((1ull << (HALF & 63)) - 1));
+  float* out = partial + ((size_t)head * gridDim.x + blockIdx.x) * HALF;
+  if (n_free <= 1) {                 // a single free chunk: R = D_j for every pair
+    for (int j = threadIdx.x; j < HALF; j += THREADS) out[j] = 0.f;
+    return;
+  }
+  const bool fresh = first_round || again;
+  // one that R has to lose, then the free ones
+  const int n_old = fresh ? 0 : 1, n_list = n_old + n_free, parts = (n_list + F::PART - 1) / F::PART;
+  if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
+    sm.list[n_old + threadIdx.x - __popcll(mask & ((1ull << threadIdx.x) - 1))] = threadIdx.x;
+  if (threadIdx.x == 0 && !fresh) sm.list[0] = before;
   if (kept)
     kept += (head * rl_tiles_below<F>((n + ROWS - 1) / ROWS) + rl_tiles_below<F>(mt)) * (F::VALUES * THREADS) + threadIdx.x;
   const float* rot_h = rot + (size_t)head * 4 * HALF * n_pad;
   const int sn_len = rl_sin_len(n);
-  for (int e = threadIdx.x; e < HALF * NW * kRlAcc; e += THREADS) (&sm.acc[0][0])[e] = 0.f;
   __syncthreads();
 
   // Steps of the block: for each key tile the parts of its list, twice where R is summed afresh.  The first
@@ -434,8 +441,7 @@ struct RsSmem {
 template <int HALF>
 __global__ void __launch_bounds__(32 * kRsWarps)
 ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, int n,
-                               const float2* __restrict__ cs, const float* __restrict__ sn,
-                               const unsigned long long* __restrict__ masks,
+                               const float2* cs, const float* sn, const unsigned long long* masks,
                                float* __restrict__ partial /* [heads][row tiles][HALF] */) {
   constexpr int d_h = 2 * HALF, THREADS = 32 * kRsWarps;
   extern __shared__ __align__(128) unsigned char smem_rl[];
@@ -444,7 +450,7 @@ ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restric
   ekv_pdl_wait();
   ekv_pdl_trigger();
   const int m0 = blockIdx.x * kRsRows, m_last = min(m0 + kRsRows, n) - 1;
-  const unsigned long long mask = masks ? masks[head] : 0ull;
+  const unsigned long long mask = masks ? __ldcg(masks + head) : 0ull;
   const bf16* Qh = Q + (size_t)head * n * d_h;
   const bf16* Kh = K + (size_t)head * n * d_h;
   for (int e = threadIdx.x; e < kRsRows * (HALF / 4); e += THREADS) {
@@ -510,20 +516,19 @@ ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restric
 // (+inf for chunks already chosen) and, when `elite_idx` is given, appends the first minimum to
 // the head's list and to its mask.
 constexpr int kRlSelect = 8;      // threads per chunk
-__global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_items, int half,
-                                       unsigned long long* __restrict__ masks, float* __restrict__ dist_out,
+__global__ void ropelite_select_kernel(const float* partial, int n_items, int half, unsigned long long* masks, float* __restrict__ dist_out,
                                        int32_t* __restrict__ elite_idx, int r, int round,
-                                       RlState* __restrict__ state) {
+                                       RlState* state) {
   __shared__ float s_d[kRlSelect][64];
   ekv_pdl_wait();
   ekv_pdl_trigger();
   const int head = blockIdx.x, j = threadIdx.x & 63, part = threadIdx.x >> 6;
-  const unsigned long long mask = masks ? masks[head] : 0ull;
+  const unsigned long long mask = masks ? __ldcg(masks + head) : 0ull;
   float v = 0.f;
   if (j < half) {
     const float* src = partial + (size_t)head * n_items * half + j;
 #pragma unroll 4
-    for (int t = part; t < n_items; t += kRlSelect) v += src[(size_t)t * half];
+    for (int t = part; t < n_items; t += kRlSelect) v += __ldcg(src + (size_t)t * half);
   }
   s_d[part][j] = v;
   __syncthreads();
@@ -548,8 +553,8 @@ __global__ void ropelite_select_kernel(const float* __restrict__ partial, int n_
       // The winner's distance is the L1 norm of the next round's R.  Taking chunks out of a kept R adds
       // rounding errors of the size of the R that was summed; below a quarter of it, or where anything
       // is not finite, R is summed afresh, so that the errors stay of the size of those of a sum.
-      float norm = state[head].norm;
-      if (round == 0 || state[head].fresh) {
+      float norm = __ldcg(&state[head].norm);
+      if (round == 0 || __ldcg(&state[head].fresh)) {
         norm = 0.f;
         for (int c = 0; c < half; ++c)
           if (!((mask >> c) & 1ull)) norm = fmaxf(norm, s_d[0][c]);
