@@ -226,7 +226,9 @@ int elitekv_attend_rows(const elitekv_layer* layer, const elitekv_cache* cache, 
  *   elitekv_ropelite_search: r rounds.  elite_idx: int32 [n_heads][r], chunks in the order
  *     chosen (the order elitekv_params.elite_idx wants).  dist_trace: optional fp32
  *     [r][n_heads][d_h/2], the distances of every round.
- * Sums are fp32 and added in a fixed order (results do not depend on scheduling).  workspace:
+ * Sums are fp32 and added in a fixed order (results do not depend on scheduling).  A wait inside a kernel that runs
+ * out, which nothing in a healthy run makes happen, ends the search of that head: its distances are NaN and
+ * its entries of elite_idx from that round on -1.  workspace:
  * 256-byte aligned, elitekv_ropelite_workspace_size bytes: beside small tables 11 MB a head at 2048 tokens of d_h 128
  * (rotated rows, and the pairs' sums that a search keeps between rounds), for as many heads as fit 1 GiB at a time. */
 int elitekv_ropelite_workspace_size(int32_t n_heads, int32_t n, int32_t d_h, size_t* bytes);
@@ -306,6 +308,13 @@ int elitekv_last_status_detail(const elitekv_layer* layer, int32_t detail[3]);
  * tensor memory, issues no copy and leaves the device usable.  poll_limit in [1, 2^20]. */
 int elitekv_selftest_bounded_wait(const elitekv_layer* layer, uint32_t poll_limit,
                                   elitekv_stream_t stream);
+
+/* Self-test of the search's bounded waits (the paper has no counterpart): two rounds over two heads of
+ * 130 tokens, d_h 64 (Q, K bf16 [2][130][64], elite_idx int32 [2][2], dist_trace fp32 [2][2][32], workspace as for
+ * elitekv_ropelite_search), by kernels that wait for copies which are not made, 1024 probes at a time.  Every entry of
+ * elite_idx must be -1 and every distance NaN; the blocks exit normally and leave the device usable. */
+int elitekv_selftest_search_timeout(const void* Q, const void* K, void* workspace, size_t workspace_bytes,
+                                    int32_t* elite_idx, float* dist_trace, elitekv_stream_t stream);
 
 /* Comparator: uncompressed RoPE multi-head attention decode (Sections 2.1 and 2.2) over a
  * contiguous cache of rotated keys and values.

@@ -81,6 +81,7 @@ def lib() -> C.CDLL:
         L.elitekv_check_status.argtypes = [vp, vp]
         L.elitekv_last_status_detail.argtypes = [vp, C.POINTER(i32 * 3)]
         L.elitekv_selftest_bounded_wait.argtypes = [vp, C.c_uint32, vp]
+        L.elitekv_selftest_search_timeout.argtypes = [vp, vp, vp, sz, vp, vp, vp]
         L.elitekv_mha_workspace_size.argtypes = [i32, i32, i32, C.POINTER(sz)]
         L.elitekv_mha_decode.argtypes = [vp, vp, vp, vp, i32, i32, i32, i64, C.c_float, vp, sz, vp, vp]
         L.elitekv_profile_enable.argtypes = [vp, i32]
@@ -92,7 +93,7 @@ def lib() -> C.CDLL:
                      "elitekv_plan", "elitekv_check_status", "elitekv_mha_workspace_size",
                      "elitekv_profile_enable", "elitekv_profile_collect", "elitekv_decode_static",
                      "elitekv_mha_decode", "elitekv_plan_workers", "elitekv_decode_plan_info",
-                     "elitekv_last_status_detail", "elitekv_selftest_bounded_wait",
+                     "elitekv_last_status_detail", "elitekv_selftest_bounded_wait", "elitekv_selftest_search_timeout",
                      "elitekv_project_append", "elitekv_decode_step", "elitekv_copy",
                      "elitekv_attend_rows_workspace_size", "elitekv_attend_rows",
                      "elitekv_ropelite_workspace_size", "elitekv_ropelite_distances", "elitekv_ropelite_search"):
@@ -309,6 +310,16 @@ def elitekv_ropelite_search(Q, K, r: int, rope_base: float = 10000.0, trace: boo
                                          rope_base, r, ws.data_ptr(), ws.numel(), _ptr(idx), _ptr(tr), _stream()),
            "elitekv_ropelite_search")
     return (idx, tr) if trace else idx
+
+
+def elitekv_selftest_search_timeout(Q, K):
+    """Q, K bf16 [2][130][64]: two rounds whose waits run out.  int32 [2][2] and fp32 [2][2][32]."""
+    ws = _ropelite_ws(Q)
+    idx = torch.empty((2, 2), dtype=torch.int32, device=Q.device)
+    tr = torch.empty((2, 2, 32), dtype=torch.float32, device=Q.device)
+    _check(lib().elitekv_selftest_search_timeout(_ptr(_dev(Q, torch.bfloat16)), _ptr(_dev(K, torch.bfloat16)), ws.data_ptr(),
+                                                 ws.numel(), _ptr(idx), _ptr(tr), _stream()), "elitekv_selftest_search_timeout")
+    return idx, tr
 
 
 def elitekv_copy(dst, src) -> None:

@@ -68,19 +68,29 @@ struct Rl {
 typedef Rl<8, 8> RlLarge;
 typedef Rl<4, 4> RlFew;
 
+// What a search keeps of a head from one round to the next, beside its sums R.
+struct __align__(16) RlState {
+  float norm;       // largest distance of the round that last summed R afresh
+  int last;         // chunk chosen in the round before
+  int fresh;        // the next round sums R afresh
+  int failed;       // a wait ran out: no more results for this head
+};
+
 // entries of a chunk's sine table: entry x holds 2 sin((x - kRlPad) theta / 2), zero up to kRlPad
 __host__ __device__ inline int rl_sin_len(int n) { return (n + 127) / 128 * 128 + kRlPad; }
 
 // (cos, sin)(pos theta_i / 2) laid out [pos][chunk], and the sine table [chunk][...];
 // double precision, rounded once
 __global__ void ropelite_table_kernel(float2* __restrict__ cs, float* __restrict__ sn, int n, int half, int d_h,
-                                      double base, unsigned long long* __restrict__ masks, int heads) {
+                                      double base, unsigned long long* __restrict__ masks, RlState* __restrict__ state, int heads) {
   ekv_pdl_wait();         // (here and below: the kernels of a search are a chain, each launched while the one before drains)
   ekv_pdl_trigger();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int len = rl_sin_len(n);
-  if (masks)                // a search begins with no chunk chosen
-    for (long long h = e; h < heads; h += (long long)gridDim.x * blockDim.x) masks[h] = 0;
+  for (long long h = e; h < heads; h += (long long)gridDim.x * blockDim.x) {
+    if (masks) masks[h] = 0;                 // a search begins with no chunk chosen
+    state[h] = RlState{0.f, 0, 1, 0};
+  }
   if (e >= (long long)len * half) return;
   const int i = (int)(e % half), x = (int)(e / half);
   const int pos = x - kRlPad;
@@ -145,7 +155,7 @@ struct RlSmem {
   float acc[HALF][F::NW * kRlAcc];     // running distances
   uint64_t full[F::STAGES], empty[F::STAGES];
   int list[HALF];                      // chunks in the order in which a tile needs them
-  int failed;
+  int n_hi;                            // end of the block's keys; 0: a wait ran out
 };
 
 // Two rows (r, r + 1) at a time: packed fp32 operations, each element rounded as by itself
@@ -230,18 +240,20 @@ __device__ __forceinline__ void rl_add(rl2 (&R)[F::TR / 2][F::TK], const RlChunk
       R[r][j] = rl_fma(rl_sin(o, r, j), t, R[r][j]);
     }
 }
+// Wait that parks between probes.  One that runs out sets the block's last key to 0, so that its warps leave with their next
+// tile, and the lane loads no more stages.  Lanes that differ meet again at the end of the step.  (The same with a vote
+// per wait, a flag that the loops test or a budget of probes for all waits of a thread: 1 to 3 % of a search.)
+__device__ __forceinline__ bool rl_wait(uint32_t bar, uint32_t parity, volatile int* n_hi, unsigned limit) {
+  unsigned tries = 0;
+  while (!mbar_try_wait(bar, parity))
+    if (++tries > limit) { *n_hi = 0; return false; }
+  return true;
+}
 __device__ __forceinline__ void rl_bulk(void* dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
                "l"((uint64_t)src), "r"(bytes), "r"(bar)
                : "memory");
 }
-
-// What a search keeps of a head from one round to the next, beside its sums R.
-struct RlState {
-  float norm;       // largest distance of the round that last summed R afresh
-  int last;         // chunk chosen in the round before
-  int fresh;        // the next round sums R afresh
-};
 
 // Tiles of 128 keys in a head's row tiles below mt (a row tile ends at the diagonal).
 template <class F>
@@ -251,13 +263,14 @@ __host__ __device__ inline long long rl_tiles_below(int mt) {
   return q * (a * (a + 1) / 2) + b * (a + 1);
 }
 
-template <int HALF, class F>
+// kSilent (self-test): stages are awaited that nobody fills, every wait with a short limit
+template <int HALF, class F, bool kSilent = false>
 __global__ void __launch_bounds__(F::THREADS, F::TR == 8 ? 3 : 2)
 ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kernel) */, int n, int n_pad,
                          const float* sn, const unsigned long long* masks, int span,
                          float* __restrict__ partial /* [heads][items][HALF] */,
                          ulonglong2* kept /* [heads][tiles][VALUES][THREADS], null: R is not kept */,
-                         const RlState* state, int first_round, int last_round) {
+                         RlState* state, int first_round, int last_round) {
   constexpr int TR = F::TR, TK = F::TK, NW = F::NW, THREADS = F::THREADS, ROWS = F::ROWS;
   extern __shared__ __align__(128) unsigned char smem_rl[];
   RlSmem<HALF, F>& sm = *(RlSmem<HALF, F>*)smem_rl;
@@ -274,10 +287,9 @@ ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kern
   const int m0 = mt * ROWS;
   const int n_lo = kg * span * kRlKeys, n_hi = min(n_lo + span * kRlKeys, m0 + ROWS);
   const unsigned long long mask = masks ? __ldcg(masks + head) : 0ull;
-  const int before = kept ? __ldcg(&state[head].last) : 0, again = kept ? __ldcg(&state[head].fresh) : 1;
-  // one trip to L2 for all three, and meanwhile:
+  const int4 kept_state = __ldcg((const int4*)&state[head]);      // RlState
+  // one trip to L2 for both, and meanwhile:
   if (threadIdx.x == 0) {
-    sm.failed = 0;
     for (int i = 0; i < F::STAGES; ++i) {
       mbar_init(smem_u32(&sm.full[i]), 1);
       mbar_init(smem_u32(&sm.empty[i]), NW);
@@ -288,16 +300,19 @@ ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kern
   for (int e = threadIdx.x; e < HALF * NW * kRlAcc; e += THREADS) (&sm.acc[0][0])[e] = 0.f;
   const int n_free = HALF - __popcll(HALF == 64 ? mask : mask & ((1ull << (HALF & 63)) - 1));
   float* out = partial + ((size_t)head * gridDim.x + blockIdx.x) * HALF;
-  if (n_free <= 1) {                 // a single free chunk: R = D_j for every pair
-    for (int j = threadIdx.x; j < HALF; j += THREADS) out[j] = 0.f;
+  if (n_free <= 1 || kept_state.w) {      // a single free chunk: R = D_j for every pair; or no result any more
+    for (int j = threadIdx.x; j < HALF; j += THREADS) out[j] = kept_state.w ? NAN : 0.f;
     return;
   }
-  const bool fresh = first_round || again;
+  const bool fresh = kept == nullptr || first_round || kept_state.z;
   // one that R has to lose, then the free ones
   const int n_old = fresh ? 0 : 1, n_list = n_old + n_free, parts = (n_list + F::PART - 1) / F::PART;
   if (threadIdx.x < HALF && !((mask >> threadIdx.x) & 1ull))
     sm.list[n_old + threadIdx.x - __popcll(mask & ((1ull << threadIdx.x) - 1))] = threadIdx.x;
-  if (threadIdx.x == 0 && !fresh) sm.list[0] = before;
+  if (threadIdx.x == 0) {
+    if (!fresh) sm.list[0] = kept_state.y;
+    sm.n_hi = n_hi;
+  }
   if (kept)
     kept += (head * rl_tiles_below<F>((n + ROWS - 1) / ROWS) + rl_tiles_below<F>(mt)) * (F::VALUES * THREADS) + threadIdx.x;
   const float* rot_h = rot + (size_t)head * 4 * HALF * n_pad;
@@ -307,21 +322,17 @@ ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kern
   // Steps of the block: for each key tile the parts of its list, twice where R is summed afresh.  The first
   // warp loads them.
   const int tile_steps = fresh ? 2 * parts : parts;
-  auto wait = [&](uint64_t* b, uint32_t parity) {
-    unsigned tries = 0;
-    while (!mbar_try_wait(smem_u32(b), parity))
-      if (++tries > kWaitLimit) { sm.failed = 1; break; }
-  };
+  constexpr unsigned kLimit = kSilent ? 1024 : kWaitLimit;
   int load_n0 = n_lo, load_step = 0, load_slot = 0;
   uint32_t load_parity = 1;
+  volatile int* const last_key = &sm.n_hi;
   auto load = [&] {
     if (load_n0 < n_hi) {
-      wait(&sm.empty[load_slot], load_parity);
+      if (!rl_wait(smem_u32(&sm.empty[load_slot]), load_parity, last_key, kLimit)) { load_n0 = n_hi; return; }
       const int c0 = load_step % parts * F::PART, cn = min(F::PART, n_list - c0);
       const uint32_t bar = smem_u32(&sm.full[load_slot]);
-      if (lane == 0) mbar_expect_tx(bar, (uint32_t)(cn * sizeof(RlChunk<F>)));
-      __syncwarp();
-      for (int e = lane; e < 3 * cn; e += 32) {
+      if (lane == 0) mbar_expect_tx(bar, (uint32_t)(cn * sizeof(RlChunk<F>)));      // (the phase waits for it, whatever lands before)
+      for (int e = kSilent ? 3 * cn : lane; e < 3 * cn; e += 32) {
         const int c = e / 3, what = e - 3 * c;
         const int i = sm.list[c0 + c];
         RlChunk<F>& ch = sm.ring[load_slot][c];
@@ -340,7 +351,7 @@ ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kern
   const int rg = warp * (32 / F::LANES) + lane / F::LANES, lk = lane % F::LANES;
   int slot = 0;
   uint32_t parity = 0;
-  for (int n0 = n_lo; n0 < n_hi; n0 += kRlKeys) {
+  for (int n0 = n_lo; n0 < __shfl_sync(0xffffffffu, *last_key, 0); n0 += kRlKeys) {
     // pairs of this warp that are not all above the diagonal, nor its rows past the last token
     const bool live = n0 < m0 + F::WROWS * (warp + 1) && m0 + F::WROWS * warp < n;
     rl2 R[TR / 2][TK];
@@ -359,7 +370,7 @@ ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kern
           R[u / (TK / 2)][u % (TK / 2) * 2 + 1] = v.y;
         }
       }
-      if (n0 + kRlKeys < n_hi && (threadIdx.x & 7) == 0) {      // the next tile's come into L2 meanwhile
+      if (n0 + kRlKeys < *last_key && (threadIdx.x & 7) == 0) {      // the next tile's come into L2 meanwhile
 #pragma unroll
         for (int u = 0; u < F::VALUES; ++u)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(keep_at + (F::VALUES + u) * THREADS));
@@ -368,7 +379,7 @@ ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kern
 #pragma unroll 1
     for (int step = 0; step < tile_steps; ++step) {
       if (warp == 0) load();
-      wait(&sm.full[slot], parity);
+      if (!rl_wait(smem_u32(&sm.full[slot]), parity, last_key, kLimit)) load_n0 = n_hi;
       if (live) {
         const bool sum = fresh && step < parts;
         int c = 0;
@@ -416,9 +427,18 @@ ropelite_distance_kernel(const float* rot /* [heads]: Q, K (ropelite_rotate_kern
     }
   }
   __syncthreads();
-  if (sm.failed) drain_after_abort();
+  if (sm.n_hi == 0) {
+    // the stages loaded and not yet used (fewer than there are) have time to land
+    if (warp == 0)
+      while (slot != load_slot) {
+        for (unsigned i = 0; i < 1024 && !mbar_try_wait(smem_u32(&sm.full[slot]), parity); ++i) {}
+        if (++slot == F::STAGES) { slot = 0; parity ^= 1; }
+      }
+    drain_after_abort();
+    if (threadIdx.x == 0) state[head].failed = 1;
+  }
   // block result: threads in a fixed order
-  const float bad = sm.failed ? NAN : 0.f;
+  const float bad = sm.n_hi == 0 ? NAN : 0.f;
   for (int c = n_old + warp; c < n_list; c += NW) {
     float v = 0.f;
 #pragma unroll
@@ -518,7 +538,7 @@ ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restric
 constexpr int kRlSelect = 8;      // threads per chunk
 __global__ void ropelite_select_kernel(const float* partial, int n_items, int half, unsigned long long* masks, float* __restrict__ dist_out,
                                        int32_t* __restrict__ elite_idx, int r, int round,
-                                       RlState* state) {
+                                       RlState* state /* null: the small form */, int keep) {
   __shared__ float s_d[kRlSelect][64];
   ekv_pdl_wait();
   ekv_pdl_trigger();
@@ -543,13 +563,15 @@ __global__ void ropelite_select_kernel(const float* partial, int n_items, int ha
     s_d[0][j] = v;
   }
   __syncthreads();
-  if (threadIdx.x == 0 && elite_idx) {
+  if (threadIdx.x == 0 && elite_idx && state && __ldcg(&state[head].failed)) {
+    elite_idx[(size_t)head * r + round] = -1;
+  } else if (threadIdx.x == 0 && elite_idx) {
     int best = 0;
     for (int c = 1; c < half; ++c)
       if (s_d[0][c] < s_d[0][best]) best = c;
     elite_idx[(size_t)head * r + round] = best;
     masks[head] = mask | (1ull << best);
-    if (state) {
+    if (keep) {
       // The winner's distance is the L1 norm of the next round's R.  Taking chunks out of a kept R adds
       // rounding errors of the size of the R that was summed; below a quarter of it, or where anything
       // is not finite, R is summed afresh, so that the errors stay of the size of those of a sum.
@@ -651,8 +673,10 @@ int rl_check(int heads, int n, int d_h) {
 struct RlRound {
   const bf16 *Q, *K;
   const unsigned long long* masks;
-  const RlState* state;         // null: R is not kept
+  RlState* state;
+  bool keep;                    // R is kept for the next round
   int first, last;              // round of the search
+  bool silent;                  // self-test (ropelite_distance_kernel)
 };
 template <int HALF>
 int rl_launch_half(const RlRound& d, int heads, int n, const RlCarve& c, unsigned char* base, cudaStream_t st) {
@@ -667,11 +691,12 @@ int rl_launch_half(const RlRound& d, int heads, int n, const RlCarve& c, unsigne
   } else {
     const auto launch = [&](auto form) -> int {
       using F = decltype(form);
-      const auto kern = ropelite_distance_kernel<HALF, F>;
+      const auto kern = HALF == 32 && F::TR == 4 && d.silent ? ropelite_distance_kernel<HALF, F, HALF == 32 && F::TR == 4>
+                                                             : ropelite_distance_kernel<HALF, F>;
       EKV_CUDA_OK(ekv_allow_smem(kern, sizeof(RlSmem<HALF, F>)));
       EKV_CUDA_OK(ekv_launch_pdl(kern, grid, dim3(F::THREADS), sizeof(RlSmem<HALF, F>), st, (const float*)(base + c.off_rot), n,
                                  rl_pad_n(n), sn, d.masks, c.span, partial,
-                                 d.state ? (ulonglong2*)(base + c.off_kept) : nullptr, d.state, d.first, d.last));
+                                 d.keep ? (ulonglong2*)(base + c.off_kept) : nullptr, d.state, d.first, d.last));
       return ELITEKV_OK;
     };
     const int rc = c.tr == 8 ? launch(RlLarge()) : launch(RlFew());
@@ -696,7 +721,8 @@ int rl_launch_table(const RlCarve& c, unsigned char* base_ptr, int n, int d_h, f
                     cudaStream_t st) {
   const long long total = (long long)rl_sin_len(n) * (d_h / 2);
   EKV_CUDA_OK(ekv_launch_pdl(ropelite_table_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st,
-                             (float2*)(base_ptr + c.off_cs), (float*)(base_ptr + c.off_sin), n, d_h / 2, d_h, (double)base, masks, heads));
+                             (float2*)(base_ptr + c.off_cs), (float*)(base_ptr + c.off_sin), n, d_h / 2, d_h, (double)base, masks,
+                             (RlState*)(base_ptr + c.off_state), heads));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }
@@ -724,56 +750,74 @@ extern "C" int elitekv_ropelite_distances(const void* Q, const void* K, int32_t 
   unsigned char* base = (unsigned char*)workspace;
   float* partial = (float*)(base + c.off_partial);
   cudaStream_t st = (cudaStream_t)stream;
-  rc = rl_launch_table(c, base, n, d_h, rope_base, nullptr, 0, st);
+  rc = rl_launch_table(c, base, n, d_h, rope_base, nullptr, n_heads, st);
   if (rc != ELITEKV_OK) return rc;
   unsigned long long* masks = (unsigned long long*)elite_mask;
+  RlState* state = (RlState*)(base + c.off_state);
   for (int h0 = 0; h0 < n_heads; h0 += c.group) {
     const int heads = n_heads - h0 < c.group ? n_heads - h0 : c.group;
     const size_t at = (size_t)h0 * n * d_h;
-    const RlRound d{(const bf16*)Q + at, (const bf16*)K + at, masks ? masks + h0 : nullptr, nullptr, 1, 1};
+    const RlRound d{(const bf16*)Q + at, (const bf16*)K + at, masks ? masks + h0 : nullptr, state + h0, false, 1, 1, false};
     rc = rl_launch_rotate(d.Q, d.K, heads, n, d_h, c, base, st);
     if (rc == ELITEKV_OK) rc = rl_launch_distance(d, heads, n, d_h, c, base, st);
     if (rc != ELITEKV_OK) return rc;
     EKV_CUDA_OK(ekv_launch_pdl(ropelite_select_kernel, dim3(heads), dim3(64 * kRlSelect), 0, st, partial, c.items, half,
-                               masks ? masks + h0 : nullptr, dist + (size_t)h0 * half, nullptr, 0, 0, nullptr));
+                               masks ? masks + h0 : nullptr, dist + (size_t)h0 * half, nullptr, 0, 0, nullptr, 0));
     EKV_CUDA_OK(cudaGetLastError());
   }
   return ELITEKV_OK;
 }
+
+namespace {
+
+int rl_search(const RlCarve& c, const void* Q, const void* K, int n_heads, int n, int d_h, float rope_base, int r, void* workspace,
+              size_t workspace_bytes, int32_t* elite_idx, float* dist_trace, cudaStream_t st, bool silent) {
+  const int half = d_h / 2;
+  if (((uintptr_t)workspace & 255) || workspace_bytes < c.total) return ELITEKV_ERR_WORKSPACE_TOO_SMALL;
+  unsigned char* base = (unsigned char*)workspace;
+  float* partial = (float*)(base + c.off_partial);
+  unsigned long long* masks = (unsigned long long*)(base + c.off_masks);
+  RlState* state = (RlState*)(base + c.off_state);
+  const bool keep = c.keep && r > 1;
+  int rc = rl_launch_table(c, base, n, d_h, rope_base, masks, n_heads, st);
+  if (rc != ELITEKV_OK) return rc;
+  for (int h0 = 0; h0 < n_heads; h0 += c.group) {
+    const int heads = n_heads - h0 < c.group ? n_heads - h0 : c.group;
+    const size_t at = (size_t)h0 * n * d_h;
+    rc = r > 0 ? rl_launch_rotate((const bf16*)Q + at, (const bf16*)K + at, heads, n, d_h, c, base, st) : ELITEKV_OK;
+    if (rc != ELITEKV_OK) return rc;
+    for (int round = 0; round < r; ++round) {
+      rc = rl_launch_distance(RlRound{(const bf16*)Q + at, (const bf16*)K + at, masks + h0, state + h0, keep, round == 0, round == r - 1, silent},
+                              heads, n, d_h, c, base, st);
+      if (rc != ELITEKV_OK) return rc;
+      EKV_CUDA_OK(ekv_launch_pdl(ropelite_select_kernel, dim3(heads), dim3(64 * kRlSelect), 0, st, partial, c.items, half, masks + h0,
+                                 dist_trace ? dist_trace + ((size_t)round * n_heads + h0) * half : nullptr,
+                                 elite_idx + (size_t)h0 * r, r, round, c.tr == 1 ? nullptr : state + h0, (int)keep));
+      EKV_CUDA_OK(cudaGetLastError());
+    }
+  }
+  return ELITEKV_OK;
+}
+
+}  // namespace
 
 extern "C" int elitekv_ropelite_search(const void* Q, const void* K, int32_t n_heads, int32_t n, int32_t d_h,
                                        float rope_base, int32_t r, void* workspace, size_t workspace_bytes,
                                        int32_t* elite_idx, float* dist_trace, elitekv_stream_t stream) {
   if (!Q || !K || !workspace || !elite_idx) return ELITEKV_ERR_INVALID_ARG;
   if (((uintptr_t)Q & 15) || ((uintptr_t)K & 15)) return ELITEKV_ERR_INVALID_ARG;
-  int rc = rl_check(n_heads, n, d_h);
+  const int rc = rl_check(n_heads, n, d_h);
   if (rc != ELITEKV_OK) return rc;
-  const int half = d_h / 2;
-  if (r < 0 || r > half) return ELITEKV_ERR_INVALID_ARG;
-  const RlCarve c = rl_carve(n_heads, n, half);
-  if (((uintptr_t)workspace & 255) || workspace_bytes < c.total) return ELITEKV_ERR_WORKSPACE_TOO_SMALL;
-  unsigned char* base = (unsigned char*)workspace;
-  float* partial = (float*)(base + c.off_partial);
-  unsigned long long* masks = (unsigned long long*)(base + c.off_masks);
-  RlState* state = (RlState*)(base + c.off_state);
-  cudaStream_t st = (cudaStream_t)stream;
-  rc = rl_launch_table(c, base, n, d_h, rope_base, masks, n_heads, st);
-  if (rc != ELITEKV_OK) return rc;
-  for (int h0 = 0; h0 < n_heads; h0 += c.group) {
-    const int heads = n_heads - h0 < c.group ? n_heads - h0 : c.group;
-    const size_t at = (size_t)h0 * n * d_h;
-    RlState* kept = c.keep && r > 1 ? state + h0 : nullptr;
-    rc = r > 0 ? rl_launch_rotate((const bf16*)Q + at, (const bf16*)K + at, heads, n, d_h, c, base, st) : ELITEKV_OK;
-    if (rc != ELITEKV_OK) return rc;
-    for (int round = 0; round < r; ++round) {
-      rc = rl_launch_distance(RlRound{(const bf16*)Q + at, (const bf16*)K + at, masks + h0, kept, round == 0, round == r - 1},
-                              heads, n, d_h, c, base, st);
-      if (rc != ELITEKV_OK) return rc;
-      EKV_CUDA_OK(ekv_launch_pdl(ropelite_select_kernel, dim3(heads), dim3(64 * kRlSelect), 0, st, partial, c.items, half, masks + h0,
-                                 dist_trace ? dist_trace + ((size_t)round * n_heads + h0) * half : nullptr,
-                                 elite_idx + (size_t)h0 * r, r, round, kept));
-      EKV_CUDA_OK(cudaGetLastError());
-    }
-  }
-  return ELITEKV_OK;
+  if (r < 0 || r > d_h / 2) return ELITEKV_ERR_INVALID_ARG;
+  return rl_search(rl_carve(n_heads, n, d_h / 2), Q, K, n_heads, n, d_h, rope_base, r, workspace, workspace_bytes, elite_idx,
+                   dist_trace, (cudaStream_t)stream, false);
+}
+
+// The distance kernel with stages that nobody fills, on two heads of 130 tokens and d_h 64, two rounds.
+extern "C" int elitekv_selftest_search_timeout(const void* Q, const void* K, void* workspace, size_t workspace_bytes,
+                                               int32_t* elite_idx, float* dist_trace, elitekv_stream_t stream) {
+  if (!Q || !K || !workspace || !elite_idx || !dist_trace || ((uintptr_t)Q & 15) || ((uintptr_t)K & 15)) return ELITEKV_ERR_INVALID_ARG;
+  const RlCarve c = rl_carve(2, 130, 32);
+  if (c.tr != 4) return ELITEKV_ERR_UNSUPPORTED_SHAPE;
+  return rl_search(c, Q, K, 2, 130, 64, 10000.f, 2, workspace, workspace_bytes, elite_idx, dist_trace, (cudaStream_t)stream, true);
 }

@@ -134,6 +134,17 @@ def test_search_in_groups_of_heads(ek):
         assert torch.allclose(t[:, 0], trace[:, h], rtol=1e-6) and torch.allclose(dist[h], trace[0, h], rtol=1e-6)
 
 
+def test_waits_that_run_out_are_reported(ek):
+    """Kernels that wait for copies which are never made: no index is made up, every round of both heads ends, and the
+    context stays usable."""
+    Q, K = (x.cuda() for x in _acts(2, 130, 64, 9))
+    good = ek.elitekv_ropelite_search(Q, K, 2, trace=True)
+    idx, trace = ek.elitekv_selftest_search_timeout(Q, K)
+    assert torch.all(idx == -1) and torch.all(torch.isnan(trace))
+    again = ek.elitekv_ropelite_search(Q, K, 2, trace=True)
+    assert all(torch.equal(a, b) for a, b in zip(good, again)) and torch.all(again[0] >= 0)
+
+
 def test_argument_checks(ek):
     Q, K = _acts(1, 8, 32, 1)
     with pytest.raises(ek.ElitekvError) as e:        # d_h = 32 is not covered
