@@ -40,9 +40,13 @@
 // depend on scheduling), masks the chunks already chosen and takes the first minimum.
 //
 // The kernels of a search are a chain of programmatic dependent launches: one is resident while the one before it
-// still writes.  What a kernel reads of its predecessors (tables, rotated rows, item results, masks, states) comes behind
-// ekv_pdl_wait, by the copy engine or with plain L2 loads: never ld.global.nc, which a compiler may make of a
-// `const __restrict__` pointer and move in front of the wait, and never from an L1 line that holds an older neighbour.
+// still writes.  What a kernel reads of its predecessors (tables, rotated rows, item results, masks, states) comes
+// behind ekv_pdl_wait, by the copy engine or with plain loads, from L2 where other blocks write the same line: never
+// ld.global.nc, which a compiler may make of a `const __restrict__` pointer and move in front of the wait.
+// Distance blocks that are placed while blocks of another kernel hold some of the SMs come to lie two on an SM beside
+// an empty one, half as fast in a call of one block an SM (16 heads x 150 tokens x d_h 128, one round, 53 us; now 45).  So the
+// kernels in front of them trigger at their end, the select kernel a launch latency before it, unless there are SMs
+// for the blocks of both (rl_apart).
 #include "tc_ptx.cuh"
 
 namespace {
@@ -82,9 +86,9 @@ __host__ __device__ inline int rl_sin_len(int n) { return (n + 127) / 128 * 128 
 // (cos, sin)(pos theta_i / 2) laid out [pos][chunk], and the sine table [chunk][...];
 // double precision, rounded once
 __global__ void ropelite_table_kernel(float2* __restrict__ cs, float* __restrict__ sn, int n, int half, int d_h,
-                                      double base, unsigned long long* __restrict__ masks, RlState* __restrict__ state, int heads) {
-  ekv_pdl_wait();         // (here and below: the kernels of a search are a chain, each launched while the one before drains)
-  ekv_pdl_trigger();
+                                      double base, unsigned long long* __restrict__ masks, RlState* __restrict__ state, int heads, int early) {
+  ekv_pdl_wait();
+  if (early) ekv_pdl_trigger();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int len = rl_sin_len(n);
   for (long long h = e; h < heads; h += (long long)gridDim.x * blockDim.x) {
@@ -111,7 +115,7 @@ __global__ void ropelite_table_kernel(float2* __restrict__ cs, float* __restrict
 __device__ __forceinline__ void rl_rotate4(const bf16* row, const float2* cs, float2* out) {
   const uint4 raw = *(const uint4*)row;
   const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-  const float4 c01 = __ldcg((const float4*)cs), c23 = __ldcg((const float4*)cs + 1);
+  const float4 c01 = *(const float4*)cs, c23 = *((const float4*)cs + 1);      // (a sector: the second half from L1)
   const float2 c[4] = {{c01.x, c01.y}, {c01.z, c01.w}, {c23.x, c23.y}, {c23.z, c23.w}};
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -127,7 +131,6 @@ __device__ __forceinline__ void rl_rotate4(const bf16* row, const float2* cs, fl
 __global__ void ropelite_rotate_kernel(const bf16* __restrict__ Q, const bf16* __restrict__ K, const float2* cs,
                                        float* __restrict__ rot, int n, int n_pad, int half, int q_rows, int split) {
   ekv_pdl_wait();
-  ekv_pdl_trigger();
   const int row = blockIdx.x * 64 + threadIdx.x % 64, head = blockIdx.y, k = blockIdx.z;
   const bf16* src = (k ? K : Q) + ((size_t)head * n + row) * 2 * half;
   const int tile = k ? kRlKeys : q_rows, in = row % tile;
@@ -538,10 +541,10 @@ ropelite_distance_small_kernel(const bf16* __restrict__ Q, const bf16* __restric
 constexpr int kRlSelect = 8;      // threads per chunk
 __global__ void ropelite_select_kernel(const float* partial, int n_items, int half, unsigned long long* masks, float* __restrict__ dist_out,
                                        int32_t* __restrict__ elite_idx, int r, int round,
-                                       RlState* state /* null: the small form */, int keep) {
+                                       RlState* state /* null: the small form */, int keep, int early) {
   __shared__ float s_d[kRlSelect][64];
   ekv_pdl_wait();
-  ekv_pdl_trigger();
+  if (early) ekv_pdl_trigger();
   const int head = blockIdx.x, j = threadIdx.x & 63, part = threadIdx.x >> 6;
   const unsigned long long mask = masks ? __ldcg(masks + head) : 0ull;
   float v = 0.f;
@@ -552,6 +555,7 @@ __global__ void ropelite_select_kernel(const float* partial, int n_items, int ha
   }
   s_d[part][j] = v;
   __syncthreads();
+  ekv_pdl_trigger();
   if (threadIdx.x < 64) {
     v = INFINITY;
     if (j < half && !((mask >> j) & 1ull)) {
@@ -717,12 +721,15 @@ int rl_launch_rotate(const bf16* Q, const bf16* K, int heads, int n, int d_h, co
   return ELITEKV_OK;
 }
 
+// one block per SM, whatever the other kernel's blocks hold
+int rl_apart(long long blocks) { return blocks <= 148; }
 int rl_launch_table(const RlCarve& c, unsigned char* base_ptr, int n, int d_h, float base, unsigned long long* masks, int heads,
                     cudaStream_t st) {
   const long long total = (long long)rl_sin_len(n) * (d_h / 2);
   EKV_CUDA_OK(ekv_launch_pdl(ropelite_table_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st,
                              (float2*)(base_ptr + c.off_cs), (float*)(base_ptr + c.off_sin), n, d_h / 2, d_h, (double)base, masks,
-                             (RlState*)(base_ptr + c.off_state), heads));
+                             (RlState*)(base_ptr + c.off_state), heads,
+                             c.tr == 1 && rl_apart((total + 255) / 256 + (long long)c.items * heads)));
   EKV_CUDA_OK(cudaGetLastError());
   return ELITEKV_OK;
 }
@@ -762,7 +769,7 @@ extern "C" int elitekv_ropelite_distances(const void* Q, const void* K, int32_t 
     if (rc == ELITEKV_OK) rc = rl_launch_distance(d, heads, n, d_h, c, base, st);
     if (rc != ELITEKV_OK) return rc;
     EKV_CUDA_OK(ekv_launch_pdl(ropelite_select_kernel, dim3(heads), dim3(64 * kRlSelect), 0, st, partial, c.items, half,
-                               masks ? masks + h0 : nullptr, dist + (size_t)h0 * half, nullptr, 0, 0, nullptr, 0));
+                               masks ? masks + h0 : nullptr, dist + (size_t)h0 * half, nullptr, 0, 0, nullptr, 0, 0));
     EKV_CUDA_OK(cudaGetLastError());
   }
   return ELITEKV_OK;
@@ -792,7 +799,7 @@ int rl_search(const RlCarve& c, const void* Q, const void* K, int n_heads, int n
       if (rc != ELITEKV_OK) return rc;
       EKV_CUDA_OK(ekv_launch_pdl(ropelite_select_kernel, dim3(heads), dim3(64 * kRlSelect), 0, st, partial, c.items, half, masks + h0,
                                  dist_trace ? dist_trace + ((size_t)round * n_heads + h0) * half : nullptr,
-                                 elite_idx + (size_t)h0 * r, r, round, c.tr == 1 ? nullptr : state + h0, (int)keep));
+                                 elite_idx + (size_t)h0 * r, r, round, c.tr == 1 ? nullptr : state + h0, (int)keep, rl_apart((long long)(c.items + 1) * heads)));
       EKV_CUDA_OK(cudaGetLastError());
     }
   }
