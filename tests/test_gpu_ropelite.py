@@ -110,6 +110,26 @@ def test_search_with_kept_sums(ek, H, n, d_h, r, graded):
         assert len(set(elite)) == r
 
 
+@pytest.mark.parametrize("H,n,d_h,r", [(24, 450, 128, 2), (32, 400, 128, 1), (5, 161, 128, 3), (160, 193, 64, 2), (20, 400, 64, 1),
+                                       (3, 130, 64, 2), (33, 300, 128, 1), (64, 521, 128, 4), (64, 300, 64, 5)])
+def test_search_by_every_form(ek, H, n, d_h, r):
+    """Few rounds run on resident operands (16, 8 and 4 rows per thread at both head dims) or staged ones that keep
+    nothing; the last two calls keep R over several key tiles of an item and rounds that are neither the first nor the last.
+    Distances against the float64 oracle on the GPU's own list so far, to the 1e-5 of the single rounds (fp32 sums of
+    up to n (n + 1) / 2 terms of relative rounding 2^-24 each, through chains of at most ~200 terms)."""
+    Q, K = _acts(H, n, d_h, 77 + n)
+    idx, trace = ek.elitekv_ropelite_search(Q.cuda(), K.cuda(), r, trace=True)
+    idx, trace = idx.cpu().numpy(), trace.cpu().double().numpy()
+    for h in {0, H - 1}:
+        q, k = Q[h].double().numpy(), K[h].double().numpy()
+        for rnd in range(r):
+            want = R.distances(q, k, idx[h, :rnd].tolist(), d_h)
+            fin = np.isfinite(want)
+            assert np.array_equal(np.isinf(trace[rnd, h]), ~fin)
+            assert np.allclose(trace[rnd, h][fin], want[fin], rtol=1e-5, atol=1e-6)
+            assert want[idx[h, rnd]] <= want[fin].min() * (1 + 1e-5)
+
+
 def test_search_energy_in_one_chunk(ek):
     """R is that chunk's D alone: it goes first, and what is left of R is nothing, not a rounding error."""
     Q, K = _acts(1, 200, 128, 5)
