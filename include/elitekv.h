@@ -229,9 +229,14 @@ int elitekv_attend_rows(const elitekv_layer* layer, const elitekv_cache* cache, 
  * Sums are fp32 and added in a fixed order (results do not depend on scheduling).  A wait inside a kernel that runs
  * out, which nothing in a healthy run makes happen, ends the search of that head: its distances are NaN and
  * its entries of elite_idx from that round on -1.  workspace:
- * 256-byte aligned, elitekv_ropelite_workspace_size bytes: beside small tables 11 MB a head at 2048 tokens of d_h 128
- * (rotated rows, and the pairs' sums that a search keeps between rounds), for as many heads as fit 1 GiB at a time. */
+ * 256-byte aligned.  elitekv_ropelite_workspace_size is enough for the fastest way of any call: beside small tables 11 MB a
+ * head at 2048 tokens of d_h 128 (rotated rows, and the pairs' sums that a search keeps between rounds), for as
+ * many heads as fit 1 GiB at a time.  elitekv_ropelite_workspace_size_rounds is what the fastest way of a search of so many
+ * rounds uses (1: of distances too, 2 MB for 32 heads of 2048 tokens where all rounds take 338); with rounds 0 it is
+ * the least that a call needs.  With anything between the two a call runs the fastest way that fits; with less than the
+ * least it is refused (ELITEKV_ERR_WORKSPACE_TOO_SMALL). */
 int elitekv_ropelite_workspace_size(int32_t n_heads, int32_t n, int32_t d_h, size_t* bytes);
+int elitekv_ropelite_workspace_size_rounds(int32_t n_heads, int32_t n, int32_t d_h, int32_t rounds, size_t* bytes);
 int elitekv_ropelite_distances(const void* Q, const void* K, int32_t n_heads, int32_t n, int32_t d_h,
                                float rope_base, const uint64_t* elite_mask, void* workspace,
                                size_t workspace_bytes, float* dist, elitekv_stream_t stream);

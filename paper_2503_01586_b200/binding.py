@@ -72,6 +72,7 @@ def lib() -> C.CDLL:
         L.elitekv_attend_rows_workspace_size.argtypes = [vp, i32, i32, C.POINTER(sz)]
         L.elitekv_attend_rows.argtypes = [vp, C.POINTER(CacheDesc), vp, vp, vp, i32, i32, vp, sz, vp, vp]
         L.elitekv_ropelite_workspace_size.argtypes = [i32, i32, i32, C.POINTER(sz)]
+        L.elitekv_ropelite_workspace_size_rounds.argtypes = [i32, i32, i32, i32, C.POINTER(sz)]
         L.elitekv_ropelite_distances.argtypes = [vp, vp, i32, i32, i32, C.c_float, vp, vp, sz, vp, vp]
         L.elitekv_ropelite_search.argtypes = [vp, vp, i32, i32, i32, C.c_float, i32, vp, sz, vp, vp, vp]
         L.elitekv_decode_static.argtypes = [vp, C.POINTER(CacheDesc), vp, vp, vp, i32, vp, vp]
@@ -96,7 +97,8 @@ def lib() -> C.CDLL:
                      "elitekv_last_status_detail", "elitekv_selftest_bounded_wait", "elitekv_selftest_search_timeout",
                      "elitekv_project_append", "elitekv_decode_step", "elitekv_copy",
                      "elitekv_attend_rows_workspace_size", "elitekv_attend_rows",
-                     "elitekv_ropelite_workspace_size", "elitekv_ropelite_distances", "elitekv_ropelite_search"):
+                     "elitekv_ropelite_workspace_size", "elitekv_ropelite_workspace_size_rounds",
+                     "elitekv_ropelite_distances", "elitekv_ropelite_search"):
             getattr(L, name).restype = C.c_int
         _lib = L
     return _lib
@@ -282,16 +284,25 @@ def elitekv_ropelite_workspace_size(n_heads: int, n: int, d_h: int) -> int:
     return b.value
 
 
-def _ropelite_ws(Q):
+def elitekv_ropelite_workspace_size_rounds(n_heads: int, n: int, d_h: int, rounds: int) -> int:
+    """What a search of so many rounds uses (1: distances); 0: the least that a call needs."""
+    b = C.c_size_t()
+    _check(lib().elitekv_ropelite_workspace_size_rounds(n_heads, n, d_h, rounds, C.byref(b)),
+           "elitekv_ropelite_workspace_size_rounds")
+    return b.value
+
+
+def _ropelite_ws(Q, rounds: int):
     H, n, d_h = Q.shape
-    return torch.empty(elitekv_ropelite_workspace_size(H, n, d_h), dtype=torch.uint8, device=Q.device)
+    rounds = max(1, min(rounds, d_h // 2))      # (what else there is to refuse, the call itself refuses)
+    return torch.empty(elitekv_ropelite_workspace_size_rounds(H, n, d_h, rounds), dtype=torch.uint8, device=Q.device)
 
 
 def elitekv_ropelite_distances(Q, K, rope_base: float = 10000.0, elite_mask=None, workspace=None):
     """Q, K bf16 [n_heads][n][d_h]; elite_mask optional int64 [n_heads] (bit i = chunk i chosen).
     Returns fp32 [n_heads][d_h/2]."""
     H, n, d_h = Q.shape
-    ws = _ropelite_ws(Q) if workspace is None else workspace
+    ws = _ropelite_ws(Q, 1) if workspace is None else workspace
     dist = torch.empty((H, d_h // 2), dtype=torch.float32, device=Q.device)
     _check(lib().elitekv_ropelite_distances(_ptr(_dev(Q, torch.bfloat16)), _ptr(_dev(K, torch.bfloat16)), H, n, d_h,
                                             rope_base, _ptr(_dev(elite_mask, torch.int64)) if elite_mask is not None else None,
@@ -303,7 +314,7 @@ def elitekv_ropelite_distances(Q, K, rope_base: float = 10000.0, elite_mask=None
 def elitekv_ropelite_search(Q, K, r: int, rope_base: float = 10000.0, trace: bool = False, workspace=None):
     """r greedy rounds for every head.  Returns int32 [n_heads][r] (and fp32 [r][n_heads][d_h/2])."""
     H, n, d_h = Q.shape
-    ws = _ropelite_ws(Q) if workspace is None else workspace
+    ws = _ropelite_ws(Q, r) if workspace is None else workspace
     idx = torch.empty((H, r), dtype=torch.int32, device=Q.device)
     tr = torch.empty((r, H, d_h // 2), dtype=torch.float32, device=Q.device) if trace else None
     _check(lib().elitekv_ropelite_search(_ptr(_dev(Q, torch.bfloat16)), _ptr(_dev(K, torch.bfloat16)), H, n, d_h,
@@ -314,7 +325,7 @@ def elitekv_ropelite_search(Q, K, r: int, rope_base: float = 10000.0, trace: boo
 
 def elitekv_selftest_search_timeout(Q, K):
     """Q, K bf16 [2][130][64]: two rounds whose waits run out.  int32 [2][2] and fp32 [2][2][32]."""
-    ws = _ropelite_ws(Q)
+    ws = torch.empty(elitekv_ropelite_workspace_size(2, 130, 64), dtype=torch.uint8, device=Q.device)
     idx = torch.empty((2, 2), dtype=torch.int32, device=Q.device)
     tr = torch.empty((2, 2, 32), dtype=torch.float32, device=Q.device)
     _check(lib().elitekv_selftest_search_timeout(_ptr(_dev(Q, torch.bfloat16)), _ptr(_dev(K, torch.bfloat16)), ws.data_ptr(),

@@ -841,20 +841,20 @@ double rl_time(const RlForm& f, const RlCarve& c, int heads, int n, int half, in
   return t;
 }
 
-// The layout of a call of `rounds` rounds that brings `room` bytes: the least one where nothing fits.
+// The layout of a call of `rounds` rounds that brings `room` bytes; the least one where that is too little for any.
 RlCarve rl_carve(int heads, int n, int half, int rounds, size_t room) {
   // Up to 64 tokens the small form is the fastest one while a few of its blocks share an SM, up to 128 tokens while each
   // has its own: a search of few tokens is a chain of small launches, its time that of one block.
   const long long small = (long long)heads * ((n + kRsRows - 1) / kRsRows);
   if (n <= 2 * kRsKeys && small <= (n > kRsKeys ? 1 : half == 64 ? 2 : 4) * kRlSms) return rl_layout(heads, n, half, kRlSmall, 1, false);
   const RlForm* forms = half == 64 ? kRlForms128 : kRlForms64;
-  RlCarve best = rl_layout(heads, n, half, kRlResident, 16, false);
-  double least = rl_time(forms[0], best, heads, n, half, rounds);
-  for (int i = 1; i < kRlForms; ++i) {
+  RlCarve best;
+  best.total = SIZE_MAX;
+  double least = INFINITY;
+  for (int i = 0; i < kRlForms; ++i) {
     const RlCarve c = rl_layout(heads, n, half, forms[i].kind, forms[i].tr, rounds > 1);
-    if (c.total > room) continue;
-    const double t = rl_time(forms[i], c, heads, n, half, rounds);
-    if (t < least) {
+    const double t = c.total <= room ? rl_time(forms[i], c, heads, n, half, rounds) : INFINITY;
+    if (t < least || (least == INFINITY && c.total < best.total)) {
       least = t;
       best = c;
     }
@@ -958,6 +958,15 @@ extern "C" int elitekv_ropelite_workspace_size(int32_t n_heads, int32_t n, int32
   return ELITEKV_OK;
 }
 
+extern "C" int elitekv_ropelite_workspace_size_rounds(int32_t n_heads, int32_t n, int32_t d_h, int32_t rounds, size_t* bytes) {
+  if (!bytes) return ELITEKV_ERR_INVALID_ARG;
+  const int rc = rl_check(n_heads, n, d_h);
+  if (rc != ELITEKV_OK) return rc;
+  if (rounds < 0 || rounds > d_h / 2) return ELITEKV_ERR_INVALID_ARG;
+  *bytes = rl_carve(n_heads, n, d_h / 2, rounds, rounds > 0 ? SIZE_MAX : 0).total;
+  return ELITEKV_OK;
+}
+
 extern "C" int elitekv_ropelite_distances(const void* Q, const void* K, int32_t n_heads, int32_t n, int32_t d_h,
                                           float rope_base, const uint64_t* elite_mask, void* workspace,
                                           size_t workspace_bytes, float* dist, elitekv_stream_t stream) {
@@ -966,7 +975,7 @@ extern "C" int elitekv_ropelite_distances(const void* Q, const void* K, int32_t 
   int rc = rl_check(n_heads, n, d_h);
   if (rc != ELITEKV_OK) return rc;
   const int half = d_h / 2;
-  const RlCarve c = rl_carve(n_heads, n, half, 1, SIZE_MAX);
+  const RlCarve c = rl_carve(n_heads, n, half, 1, workspace_bytes);
   if (((uintptr_t)workspace & 255) || workspace_bytes < c.total) return ELITEKV_ERR_WORKSPACE_TOO_SMALL;
   unsigned char* base = (unsigned char*)workspace;
   float* partial = (float*)(base + c.off_partial);
@@ -1030,7 +1039,7 @@ extern "C" int elitekv_ropelite_search(const void* Q, const void* K, int32_t n_h
   const int rc = rl_check(n_heads, n, d_h);
   if (rc != ELITEKV_OK) return rc;
   if (r < 0 || r > d_h / 2) return ELITEKV_ERR_INVALID_ARG;
-  return rl_search(rl_carve(n_heads, n, d_h / 2, r, SIZE_MAX), Q, K, n_heads, n, d_h, rope_base, r, workspace, workspace_bytes, elite_idx,
+  return rl_search(rl_carve(n_heads, n, d_h / 2, r, workspace_bytes), Q, K, n_heads, n, d_h, rope_base, r, workspace, workspace_bytes, elite_idx,
                    dist_trace, (cudaStream_t)stream, false);
 }
 

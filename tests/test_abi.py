@@ -41,6 +41,26 @@ def test_binding_exposes_the_same_names():
         assert hasattr(binding, name), name
 
 
+def test_search_workspace_is_what_the_call_uses():
+    """Single distances and one round bring no room for sums between rounds, whose size is a head's pairs; the least is tables
+    and item results, as for a search that never keeps anything."""
+    from paper_2503_01586_b200 import binding as ek
+    for H, n, d_h in ((32, 2048, 128), (4, 300, 64), (1, 1, 64), (1024, 2048, 128), (2, 1 << 20, 128)):
+        most = ek.elitekv_ropelite_workspace_size(H, n, d_h)
+        least = ek.elitekv_ropelite_workspace_size_rounds(H, n, d_h, 0)
+        for r in (1, 2, 8, d_h // 2):
+            assert least <= ek.elitekv_ropelite_workspace_size_rounds(H, n, d_h, r) <= most
+        # (cos, sin) and sines, items of a 128 x 128 tile at most, masks; four paddings to 256 bytes
+        half, tiles = d_h // 2, (n + 127) // 128
+        items = min(tiles * (tiles + 1) // 2, 16 * tiles) if n > 128 else max(tiles, -(-n // 16))
+        assert least <= half * (12 * n + 4 * (128 + 256) + 4 * H * items) + 8 * H + 1024
+    assert ek.elitekv_ropelite_workspace_size_rounds(32, 2048, 128, 1) < 3 << 20 < 300 << 20 < \
+        ek.elitekv_ropelite_workspace_size_rounds(32, 2048, 128, 8)
+    for bad in (-1, 65):
+        with pytest.raises(ek.ElitekvError):
+            ek.elitekv_ropelite_workspace_size_rounds(4, 300, 128, bad)
+
+
 def test_struct_layouts_match_the_header(tmp_path):
     """sizeof/offsetof as the C compiler sees the header vs. the ctypes mirror."""
     import subprocess

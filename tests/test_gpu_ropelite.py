@@ -130,6 +130,26 @@ def test_search_by_every_form(ek, H, n, d_h, r):
             assert want[idx[h, rnd]] <= want[fin].min() * (1 + 1e-5)
 
 
+@pytest.mark.parametrize("H,n,d_h,r", [(3, 300, 128, 5), (40, 260, 64, 4), (2, 90, 64, 3)])
+def test_search_in_any_workspace(ek, H, n, d_h, r):
+    """From the least workspace on a call runs the fastest way that fits, with the same distances (sums in another order:
+    fp32, 1e-6); less is refused."""
+    Q, K = (x.cuda() for x in _acts(H, n, d_h, 5 + n))
+    least = ek.elitekv_ropelite_workspace_size_rounds(H, n, d_h, 0)
+    sizes = [least] + [ek.elitekv_ropelite_workspace_size_rounds(H, n, d_h, k) for k in (1, r)] + [ek.elitekv_ropelite_workspace_size(H, n, d_h)]
+    idx, trace = ek.elitekv_ropelite_search(Q, K, r, trace=True)
+    dist = ek.elitekv_ropelite_distances(Q, K)
+    for size in sizes + [(sizes[0] + sizes[2]) // 2]:
+        ws = torch.full((size + 256,), 0x5a, dtype=torch.uint8, device="cuda")
+        i, t = ek.elitekv_ropelite_search(Q, K, r, trace=True, workspace=ws[:size])
+        assert torch.equal(i, idx) and torch.allclose(t, trace, rtol=1e-6, atol=1e-6)
+        assert torch.allclose(ek.elitekv_ropelite_distances(Q, K, workspace=ws[:size]), dist, rtol=1e-6, atol=1e-6)
+        assert torch.all(ws[size:] == 0x5a)
+    with pytest.raises(ek.ElitekvError) as e:
+        ek.elitekv_ropelite_search(Q, K, r, workspace=ws[:least - 1])
+    assert e.value.code == ek.ERR_WORKSPACE_TOO_SMALL
+
+
 def test_search_energy_in_one_chunk(ek):
     """R is that chunk's D alone: it goes first, and what is left of R is nothing, not a rounding error."""
     Q, K = _acts(1, 200, 128, 5)
