@@ -18,9 +18,22 @@ struct __align__(16) PlanShared {        // the block's shared memory
   short w0[kPlanThreads], wk[kPlanStage];    // wk: worker of each item (n_workers < 32768)
 };
 
-// exclusive scan over the block (warp shuffles + one shared array of warp totals)
+// The threads that make a plan.  A step's plan is run once, by one block, with instructions that are not in the caches:
+// most of its time.  So the last warp makes the same trip at once and without effect, with made-up lengths, one turn
+// of each loop, while the others still wait for the kernel before (or, where there is none, beside them).
+constexpr int kPlanWorkers = kPlanThreads - 32;
+struct PlanTeam {
+  int threads;      // of which thread t is one
+  bool dry;         // the last warp, by itself
+  __device__ __forceinline__ void sync() const {
+    if (dry) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+  }
+};
+
+// exclusive scan over the team (warp shuffles + one shared array of warp totals)
 template <class V, class T>
-__device__ __forceinline__ V block_exclusive_scan(V v, T* warp_tot, V* total) {
+__device__ __forceinline__ V block_exclusive_scan(const PlanTeam& team, V v, T* warp_tot, V* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   V incl = v;
 #pragma unroll
@@ -28,16 +41,16 @@ __device__ __forceinline__ V block_exclusive_scan(V v, T* warp_tot, V* total) {
     const V x = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += x;
   }
-  if (lane == 31) warp_tot[warp] = incl;
-  __syncthreads();
+  if (lane == 31 && !team.dry) warp_tot[warp] = incl;
+  team.sync();
   V before = 0, all = 0;
 #pragma unroll
   for (int w = 0; w < kPlanThreads / 32; ++w) {
-    const V t = (V)warp_tot[w];
+    const V t = w < team.threads / 32 ? (V)warp_tot[w] : 0;
     if (w < warp) before += t;
     all += t;
   }
-  __syncthreads();
+  team.sync();
   *total = all;
   return before + incl - v;
 }
@@ -89,11 +102,9 @@ __device__ __forceinline__ T plan_tiles(int n, int tile) {
 static __device__ __noinline__ unsigned plan_udiv(unsigned x, unsigned y) { return x / y; }
 
 // Balanced plan of up to 32 sequences, a lane per sequence: every warp has the whole batch in its registers, so there
-// is no barrier and no shared memory.  A step's plan is run once, by one block, with instructions that are not in
-// the caches: 10 us where the uses of a search and of an item are unrolled and inlined one by one, 2 us when that
-// runs a second time at once.  So there is one copy of each, items and workers are chunks of one loop,
-// and a block that has to wait for the kernel before it makes the trip once without effect (dry): 2.5 to 3 us
-// behind the wait, 4 to 5 for plan_small.  (The even plan has hundreds of items, for which
+// is no barrier and no shared memory.  Cold, it takes 10 us where the uses of a search and of an item are unrolled and inlined
+// one by one, 2 us when that runs a second time at once.  So there is one copy of each, items and workers are chunks
+// of one loop.  (The even plan has hundreds of items, for which
 // a warp per 32 is the slower way: the smallest model's step 15.9 us, 14.6 with plan_small.)
 // False, with nothing but the counters and reports written, where a product does not fit 32 bits.
 // The arithmetic is that of plan_balanced below.
@@ -106,7 +117,7 @@ __device__ __forceinline__ bool plan_quick(const PlanArgs& a, bool dry) {
   if (dry) n = lane < B ? a.tile : 0;
   else if (lane < B) n = checked_len(a.seq_lens, lane, a.max_len, a.status, t < 32);
   if (!dry)
-    for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
+    for (int i = t; i < a.n_zero; i += kPlanWorkers) a.zero_ints[i] = 0;
   const unsigned tiles = n > 0 ? plan_udiv((unsigned)n + a.tile - 1, (unsigned)a.tile) + overhead : 0;
   // inclusive sums
   unsigned g1 = 0, pieces = 0, w0 = 0, f1 = 0, total = 1, nw = 1;
@@ -136,7 +147,7 @@ __device__ __forceinline__ bool plan_quick(const PlanArgs& a, bool dry) {
   // chunks of 32 items, then of 31 workers (and the one behind them, whose first item ends the last one's)
   const int item_chunks = (a.max_items + 31) / 32, chunks = item_chunks + (a.n_workers + 31) / 31;
 #pragma unroll 1
-  for (int c = t >> 5; c < chunks; c += kPlanThreads / 32) {
+  for (int c = dry ? 0 : t >> 5; c < chunks; c += dry ? chunks : kPlanWorkers / 32) {
     const bool wk = c >= item_chunks;
     const unsigned i = wk ? (c - item_chunks) * 31 + lane : c * 32 + lane;
     // the sequence of item i, or of the first position of worker i's range: the last one whose first item (first
@@ -177,21 +188,22 @@ __device__ __forceinline__ bool plan_small_ok(const PlanArgs& a) {
   return a.B <= kPlanThreads && a.n_workers + a.B <= kPlanStage;
 }
 template <class T>
-__device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh, bool dry) {
+__device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh, const PlanTeam team) {
+  const bool dry = team.dry;      // nothing is written, shared memory neither: what a dry trip reads there is anybody's
   T *const warp_tot = sh.warp_tot, *const s_g0 = sh.g0, *const s_tiles = sh.tiles;
   int *const s_first = sh.first, *const s_len = sh.len;
   short *const s_w0 = sh.w0, *const s_wk = sh.wk;
-  const int t = threadIdx.x, B = a.B;
+  const int t = dry ? threadIdx.x % 32 : threadIdx.x, B = a.B;
   const bool balanced = a.n_workers > 0;
   const int overhead = balanced ? a.overhead : 0;      // empty tiles in front of every sequence
   int n = 0;
   if (dry) n = t < B ? a.tile : 0;
   else if (t < B) n = checked_len(a.seq_lens, t, a.max_len, a.status, true);
   if (!dry)
-    for (int i = t; i < a.n_zero; i += kPlanThreads) a.zero_ints[i] = 0;
+    for (int i = t; i < a.n_zero; i += team.threads) a.zero_ints[i] = 0;
   const T tiles = n > 0 ? (T)plan_div((long long)n + a.tile - 1, a.tile) + overhead : 0;
   T sum;
-  const T g0 = block_exclusive_scan(tiles, warp_tot, &sum);
+  const T g0 = block_exclusive_scan(team, tiles, warp_tot, &sum);
   const long long total = sum > 0 ? sum : 1;
   const long long nw = balanced ? (total < a.n_workers ? total : a.n_workers) : 1;
   auto bound = [&](long long w) -> long long { return plan_div(w * total, nw); };
@@ -208,14 +220,14 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh,
     }
   }
   int n_items;
-  const int first = block_exclusive_scan(pieces, warp_tot, &n_items);
-  if (t < B) {
-    if (!dry) a.seq_first[t] = first;
+  const int first = block_exclusive_scan(team, pieces, warp_tot, &n_items);
+  if (t < B && !dry) {
+    a.seq_first[t] = first;
     s_first[t] = first; s_g0[t] = g0; s_len[t] = n; s_tiles[t] = tiles; s_w0[t] = (short)w0;
   }
   if (t == 0 && !dry) a.seq_first[B] = n_items;
-  __syncthreads();
-  for (int it = t; it < a.max_items; it += kPlanThreads) {
+  team.sync();
+  for (int it = t; it < a.max_items; it += dry ? a.max_items : team.threads) {
     int4 item = make_int4(-1, 0, 0, 0);
     if (it < n_items) {
       int lo = 0, hi = B;                    // the last sequence whose first item is not past this one
@@ -231,7 +243,7 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh,
         w = s_w0[lo] + j;
         ta = (int)(max(base, bound(w)) - base);
         tb = (int)(min((long long)s_g0[lo] + tl, bound(w + 1)) - base);
-        s_wk[it] = (short)w;
+        if (!dry) s_wk[it] = (short)w;
       } else {
         const int np = (lo + 1 < B ? s_first[lo + 1] : n_items) - s_first[lo];
         ta = (int)plan_div((long long)tl * j, np);
@@ -243,9 +255,9 @@ __device__ __forceinline__ void plan_small(const PlanArgs& a, PlanShared<T>& sh,
     if (!dry) *(int4*)(a.items + 4 * it) = item;
   }
   if (!balanced) return;
-  __syncthreads();
-  const int held = min(n_items, a.max_items);
-  for (int w = t; w <= a.n_workers; w += kPlanThreads) {
+  team.sync();
+  const int held = dry ? 1 : min(n_items, a.max_items);
+  for (int w = t; w <= a.n_workers; w += dry ? a.n_workers + 1 : team.threads) {
     int lo = 0, hi = held;                   // first item whose worker is >= w
     while (lo < hi) {
       const int mid = (lo + hi) >> 1;
@@ -298,7 +310,7 @@ __device__ __forceinline__ void plan_even(const PlanArgs& a, PlanShared<T>& sh) 
       pieces = (int)((tiles + target - 1) / target);
     }
     int chunk_total;
-    const int first = carry + block_exclusive_scan(pieces, warp_tot, &chunk_total);
+    const int first = carry + block_exclusive_scan(PlanTeam{kPlanThreads, false}, pieces, warp_tot, &chunk_total);
     if (b < B) {
       seq_first[b] = first;
       for (int j = 0; j < pieces; ++j) {
@@ -365,7 +377,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& 
         tiles = n > 0 ? plan_tiles<T>(n, tile) + overhead : 0;     // with the empty tiles in front
       }
       T chunk_tiles;
-      const T g0 = carry_tiles + block_exclusive_scan(tiles, warp_tot, &chunk_tiles);
+      const T g0 = carry_tiles + block_exclusive_scan(PlanTeam{kPlanThreads, false}, tiles, warp_tot, &chunk_tiles);
       int pieces = 0, w0 = 0;
       if (tiles > 0) {
         w0 = owner(g0 + overhead);                                // workers that hold real tiles
@@ -373,7 +385,7 @@ __device__ __forceinline__ void plan_balanced(const PlanArgs& a, PlanShared<T>& 
         pieces = w1 - w0 + 1;
       }
       int chunk_items;
-      const int first = carry_items + block_exclusive_scan(pieces, warp_tot, &chunk_items);
+      const int first = carry_items + block_exclusive_scan(PlanTeam{kPlanThreads, false}, pieces, warp_tot, &chunk_items);
       if (b < B) {
         seq_first[b] = first;
         for (int j = 0; j < pieces; ++j) {
@@ -435,27 +447,21 @@ __device__ __forceinline__ void plan_large(const PlanArgs& a, PlanShared<T>& sh)
     }
   }
 }
-// A whole plan, with the wait for the kernels before in front of the first trip to memory; the forms for up to
-// a sequence per thread make a first trip without effect before it (plan_quick).
+// A whole plan, with the wait for the kernels before in front of the first trip to memory.  (Where every thread has a
+// sequence there is no warp to spare for the dry trip.  A dry trip of the whole block in front of the wait is as
+// good behind a running kernel, and 1.5 to 2 us more where there is none: an isolated step of the smallest model 21.7 us,
+// 20.3 so; 12 x 900 39.8 and 37.9.  With one 87.5 % 16 x 1500 takes 32.3 us a step back to back, 33.2 so.)
 template <class T>
 __device__ __forceinline__ void plan_behind_wait(const PlanArgs& a, PlanShared<T>& sh) {
-  if (sizeof(T) == 4 && plan_quick_ok(a)) {
-    bool done = false;
-#pragma unroll 1
-    for (int dry = 1; dry >= 0; --dry) {
-      if (!dry) ekv_pdl_wait();
-      done = plan_quick(a, dry);
-    }
-    if (done) return;
+  const bool spare = plan_small_ok(a) && a.B <= kPlanWorkers, dry = spare && threadIdx.x >= kPlanWorkers;
+  if (!dry) ekv_pdl_wait();
+  if (sizeof(T) == 4 && plan_quick_ok(a) && spare) {
+    const bool done = plan_quick(a, dry);
+    if (done || dry) return;
   }
   if (plan_small_ok(a)) {
-#pragma unroll 1
-    for (int dry = 1; dry >= 0; --dry) {
-      if (!dry) ekv_pdl_wait();
-      plan_small(a, sh, dry);
-    }
+    plan_small(a, sh, PlanTeam{dry ? 32 : spare ? kPlanWorkers : kPlanThreads, dry});
     return;
   }
-  ekv_pdl_wait();
   plan_large(a, sh);
 }

@@ -24,25 +24,25 @@ step_prep_kernel(const AbsorbArgs q, const AppendArgs t, const PlanArgs p, int n
   extern __shared__ __align__(16) unsigned char smem_b[];
   ekv_pdl_trigger();      // the attention kernel waits for this grid's completion itself
   int blk = blockIdx.x;
-  if (blk == 0) {
-    plan_behind_wait(p, *(PlanShared<int>*)smem_b);
+  if (blk != 0) {      // (the plan last in the code: 7B 75 % 8 x 1500 30.7 us a step, 31.3 with it first)
+    blk -= 1;
+    if (blk < n_append) {
+      ekv_pdl_wait();
+      if (vec) append_tokens<true>(t, blk, n_append);
+      else append_tokens<false>(t, blk, n_append);
+      return;
+    }
+    blk -= n_append;
+    if (blk < q.n_h) {
+      absorb_rope(q, blk);
+      return;
+    }
+    blk -= q.n_h;
+    const int h = blk % q.n_h, s = blk / q.n_h;
+    absorb_block<MT>(q, h, s % slices * kAbsorbCoords, s / slices * 16 * MT, smem_b);
     return;
   }
-  blk -= 1;
-  if (blk < n_append) {
-    ekv_pdl_wait();
-    if (vec) append_tokens<true>(t, blk, n_append);
-    else append_tokens<false>(t, blk, n_append);
-    return;
-  }
-  blk -= n_append;
-  if (blk < q.n_h) {
-    absorb_rope(q, blk);
-    return;
-  }
-  blk -= q.n_h;
-  const int h = blk % q.n_h, s = blk / q.n_h;
-  absorb_block<MT>(q, h, s % slices * kAbsorbCoords, s / slices * 16 * MT, smem_b);
+  plan_behind_wait(p, *(PlanShared<int>*)smem_b);
 }
 
 }  // namespace

@@ -365,6 +365,48 @@ def test_cluster_kernel_behind_every_form_of_the_plan(ek, B):
     H.check_parity(st, H.run_decode(st), H.sample_units(st, 24, seed=B))
 
 
+@pytest.mark.parametrize("ragged", [False, True])
+@pytest.mark.parametrize("B", [1, 2, 31, 32, 33, 224, 225, 256, 257])
+@pytest.mark.parametrize("kernel", [1, 2, 4])
+def test_plan_that_a_call_makes(ek, kernel, B, ragged):
+    """The exported plans take lengths of any size, in 64 bits; a decode call's own plan is another form of the code: 32-bit
+    sums, a lane per sequence (balanced plans, up to 32), a thread per sequence (224 beside the warp that makes the dry
+    trip, 256 without it), a loop beyond.  Read from the call's workspace (items and first items at its start, first items and
+    records of the workers at its end): the same plan, and each worker's record is its first item."""
+    w = gen.shrink(gen.LLAMA7B_75, B=B, ctx=200) if kernel > 1 else replace(gen.TINY, B=B, ctx=200)
+    lens = [0 if b % 5 in (0, 4) else 1 + (7919 * b) % 199 for b in range(B)] if ragged else [200] * B
+    st = H.setup(w, lens=[max(n, 1) for n in lens], fill=False, decode_kernel=kernel)
+    dev = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    size = ek.elitekv_decode_workspace_size(st.layer, B)
+    ws = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    q_rope = torch.zeros((B, w.n_h, 2 * w.r), dtype=torch.bfloat16, device="cuda")
+    q_abs = torch.zeros((B, w.n_h, st.layer.kw), dtype=torch.bfloat16, device="cuda")
+    ek.elitekv_decode(st.layer, st.cache, q_rope, q_abs, dev, ws)
+    got_kernel, tile, n_workers, max_items, overhead = ek.elitekv_decode_plan_info(st.layer, st.cache, B)
+    assert got_kernel == kernel and ek.elitekv_check_status(st.layer) == 0
+    up = lambda n: (n + 255) // 256 * 256
+    words = lambda at, n: ws[at:at + 4 * n].view(torch.int32).cpu()
+    if n_workers == 0:
+        items, first = ek.elitekv_plan(dev, tile, max_items)
+    else:
+        items, first, wfirst = ek.elitekv_plan_workers(dev, tile, n_workers, max_items, overhead)
+    assert torch.equal(words(0, 4 * max_items).view(-1, 4), items.cpu())
+    assert torch.equal(words(up(16 * max_items), B + 1), first.cpu())
+    if n_workers == 0:
+        return
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    at_rec = size - up(32 * sms)
+    at_first = at_rec - up(4 * (sms + 2))
+    assert torch.equal(words(at_first, n_workers + 1), wfirst.cpu())
+    if kernel == 4:
+        rec, items, wfirst = words(at_rec, 8 * n_workers).view(-1, 8), items.cpu(), wfirst.tolist()
+        for i in range(n_workers):
+            lo, hi = wfirst[i], wfirst[i + 1]
+            assert rec[i, :2].tolist() == [lo, hi]
+            if lo < hi:
+                assert rec[i, 2:5].tolist() == items[lo, :3].tolist()
+
+
 MOST = 2 ** 31 - 1
 
 
