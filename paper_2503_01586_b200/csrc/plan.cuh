@@ -50,6 +50,10 @@ __device__ __forceinline__ V block_exclusive_scan(const PlanTeam& team, V v, T* 
     if (w < warp) before += t;
     all += t;
   }
+  if (team.dry) {      // (its own warp's, so that the trip goes on as with lengths)
+    before = 0;
+    all = __shfl_sync(0xffffffffu, incl, 31);
+  }
   team.sync();
   *total = all;
   return before + incl - v;
