@@ -13,9 +13,8 @@ namespace {
 
 template <class T>
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const PlanArgs a) {
-  ekv_pdl_trigger();      // (whoever comes next waits for this grid's completion itself)
   __shared__ PlanShared<T> sh;
-  plan_behind_wait(a, sh);      // earlier kernels may still read the arrays written here
+  plan_behind_wait<true>(a, sh);      // earlier kernels may still read the arrays written here
 }
 
 }  // namespace

@@ -455,10 +455,15 @@ __device__ __forceinline__ void plan_large(const PlanArgs& a, PlanShared<T>& sh)
 // sequence there is no warp to spare for the dry trip.  A dry trip of the whole block in front of the wait is as
 // good behind a running kernel, and 1.5 to 2 us more where there is none: an isolated step of the smallest model 21.7 us,
 // 20.3 so; 12 x 900 39.8 and 37.9.  With one 87.5 % 16 x 1500 takes 32.3 us a step back to back, 33.2 so.)
-template <class T>
+// kAlone: the kernel is nothing but a plan, and triggers behind the wait.  In front of it, attention blocks came to wait on
+// SMs that blocks of the query preparation were yet to leave (87.5 % from hidden states, 32 x 8192: 127.2 us, 120.5 now).
+template <bool kAlone, class T>
 __device__ __forceinline__ void plan_behind_wait(const PlanArgs& a, PlanShared<T>& sh) {
   const bool spare = plan_small_ok(a) && a.B <= kPlanWorkers, dry = spare && threadIdx.x >= kPlanWorkers;
-  if (!dry) ekv_pdl_wait();
+  if (!dry) {
+    ekv_pdl_wait();
+    if (kAlone) ekv_pdl_trigger();
+  }
   if (sizeof(T) == 4 && plan_quick_ok(a) && spare) {
     const bool done = plan_quick(a, dry);
     if (done || dry) return;

@@ -42,7 +42,7 @@ step_prep_kernel(const AbsorbArgs q, const AppendArgs t, const PlanArgs p, int n
     absorb_block<MT>(q, h, s % slices * kAbsorbCoords, s / slices * 16 * MT, smem_b);
     return;
   }
-  plan_behind_wait(p, *(PlanShared<int>*)smem_b);
+  plan_behind_wait<false>(p, *(PlanShared<int>*)smem_b);
 }
 
 }  // namespace
