@@ -38,7 +38,10 @@ constexpr int kFK = 128;         // latent slice
 constexpr int kFD = 128;         // head dim
 constexpr int kFThreads = 256;
 constexpr int kFPitch = kFD + 8; // shared-memory row pitch in bf16: 16 bytes of padding keep ldmatrix free of bank conflicts
-constexpr int kFSum = 12;        // slice results in flight when they are added: 7B B16 2.4 us from the last arrival to the last store, 3.0 in fours
+// Slice results in flight when they are added.  Us a step with 4 / 6 / 8 / 12 / 24: 87.5 % 16 x 1500 (6 slices) 32.9 / 32.7 / 32.3 /
+// 33.3 / 34.6, 7B 75 % 1 x 1999 (12) 23.6 / 23.1 / 23.3 / 23.1 / 23.6, 32 x 1000 58.9 / 58.6 / 58.6 / 58.8 / 59.2, 13B 8 x 1000 (15)
+// 38.4 / 39.0 / 38.7 / 38.9 / 39.0, 50 % 8 x 1000 (24) 45.9 / 45.7 / 45.8 / 45.7 / 45.5.
+constexpr int kFSum = 6;
 constexpr int kFAhead = 4;       // partial results per row in flight beside the statistics
 
 // kMore: blocks start at group g0 of n_groups (calls of more rows than one grid holds).  kOne: one query row per sequence
