@@ -127,7 +127,42 @@ def test_search_by_every_form(ek, H, n, d_h, r):
             fin = np.isfinite(want)
             assert np.array_equal(np.isinf(trace[rnd, h]), ~fin)
             assert np.allclose(trace[rnd, h][fin], want[fin], rtol=1e-5, atol=1e-6)
+            # (2-norm of the errors: 5e-8 on every form, whether R is summed or kept)
+            assert np.linalg.norm(trace[rnd, h][fin] - want[fin]) <= 2e-7 * np.linalg.norm(want[fin])
             assert want[idx[h, rnd]] <= want[fin].min() * (1 + 1e-5)
+
+
+@pytest.mark.parametrize("d_h", [64, 128])
+def test_search_of_values_that_are_not_finite(ek, d_h):
+    """An infinity, a NaN and large finite values: a search that keeps R gives what one gives that sums it in every round (which
+    the least workspace makes it do), place by place."""
+    H, n, r = 4, 300, 9
+    Q, K = (x.cuda() for x in _acts(H, n, d_h, 21))
+    Q[0, 200, 5] = float("inf")
+    K[1, 17, 2] = float("nan")
+    Q[2] *= 1e30
+    big = ek.elitekv_ropelite_workspace_size(H, n, d_h)
+    least = ek.elitekv_ropelite_workspace_size_rounds(H, n, d_h, 0)
+    assert least < ek.elitekv_ropelite_workspace_size_rounds(H, n, d_h, r) <= big
+    (i, t), (i0, t0) = (ek.elitekv_ropelite_search(Q, K, r, trace=True, workspace=torch.empty(size, dtype=torch.uint8, device="cuda"))
+                        for size in (big, least))
+    assert torch.equal(i, i0) and torch.allclose(t, t0, rtol=1e-6, equal_nan=True)
+    assert torch.isnan(t[:, 1]).any() and torch.isfinite(t[0, 2:]).all()
+
+
+def test_search_of_a_head_too_long_to_keep(ek):
+    """A head of 23000 tokens needs more than the scratch for its sums: every round sums R, and is the single round for the
+    chunks chosen so far."""
+    n, d_h, r = 23000, 64, 3
+    g = torch.Generator(device="cuda").manual_seed(8)
+    Q, K = (torch.randn((1, n, d_h), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    assert ek.elitekv_ropelite_workspace_size(1, n, d_h) < 1 << 28
+    idx, trace = ek.elitekv_ropelite_search(Q, K, r, trace=True)
+    mask = 0
+    for rnd in range(r):
+        dist = ek.elitekv_ropelite_distances(Q, K, elite_mask=torch.tensor([mask], dtype=torch.int64, device="cuda"))
+        assert torch.allclose(trace[rnd], dist, rtol=1e-6)
+        mask |= 1 << int(idx[0, rnd])
 
 
 @pytest.mark.parametrize("H,n,d_h,r", [(3, 300, 128, 5), (40, 260, 64, 4), (2, 90, 64, 3)])
@@ -161,14 +196,18 @@ def test_search_energy_in_one_chunk(ek):
 
 
 def test_search_in_groups_of_heads(ek):
-    """More heads than the scratch holds at a time: the heads on both sides of the seam and the last one as in
-    calls of their own (sums in another order where the call's form differs: fp32, 1e-6)."""
+    """More heads than the scratch holds at a time (1 GiB; what one head more takes, from the sizes of small calls, counts
+    item results too, so that the seam lies within a head of it): the heads on both sides of the seam and the last one as
+    in calls of their own (sums in another order where the call's form differs: fp32, 1e-6)."""
     H, n, d_h, r = 100, 2048, 128, 2
+    size = lambda heads: ek.elitekv_ropelite_workspace_size_rounds(heads, n, d_h, r)
+    seam = (1 << 30) // (size(41) - size(40))
+    assert seam + 2 < H and size(H) < (1 << 30) + (1 << 25)
     g = torch.Generator(device="cuda").manual_seed(3)
     Q, K = (torch.randn((H, n, d_h), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
     idx, trace = ek.elitekv_ropelite_search(Q, K, r, trace=True)
     dist = ek.elitekv_ropelite_distances(Q, K)
-    for h in (0, 91, 92, 93, 94, 95, 96, 99):
+    for h in (0, seam - 2, seam - 1, seam, seam + 1, seam + 2, H - 1):
         one, t = ek.elitekv_ropelite_search(Q[h:h + 1].contiguous(), K[h:h + 1].contiguous(), r, trace=True)
         assert torch.equal(one[0], idx[h])
         assert torch.allclose(t[:, 0], trace[:, h], rtol=1e-6) and torch.allclose(dist[h], trace[0, h], rtol=1e-6)
