@@ -106,9 +106,9 @@ __device__ __forceinline__ T plan_tiles(int n, int tile) {
 static __device__ __noinline__ unsigned plan_udiv(unsigned x, unsigned y) { return x / y; }
 
 // Balanced plan of up to 32 sequences, a lane per sequence: every warp has the whole batch in its registers, so there
-// is no barrier and no shared memory.  Cold, it takes 10 us where the uses of a search and of an item are unrolled and inlined
-// one by one, 2 us when that runs a second time at once.  So there is one copy of each, items and workers are chunks
-// of one loop.  (The even plan has hundreds of items, for which
+// is no barrier and no shared memory.  A form with the uses of a search and of an item unrolled and inlined one by one
+// took 10 us cold, 2 us when it ran a second time at once.  So there is one copy of each here, items and workers are chunks
+// of one loop: 2.8 us behind the wait for one sequence, 3.0 for 16.  (The even plan has hundreds of items, for which
 // a warp per 32 is the slower way: the smallest model's step 15.9 us, 14.6 with plan_small.)
 // False, with nothing but the counters and reports written, where a product does not fit 32 bits.
 // The arithmetic is that of plan_balanced below.
@@ -185,8 +185,8 @@ __device__ __forceinline__ bool plan_quick(const PlanArgs& a, bool dry) {
 
 // Batches of at most a sequence per thread: both plans in one trip for the lengths, two scans and one
 // pass with a thread per ITEM.  (A thread per sequence that writes the sequence's items one after the
-// other, two 64-bit divisions each, took 9 us for one sequence in 33 items and 5 us for 16 sequences,
-// twice as long as the query preparation beside it; this form takes 2.3 and 3.6 us.)  The arithmetic is
+// other, two 64-bit divisions each, took twice as long as the query preparation beside it; this form, cold and without
+// the warming trip, 4.0 us for one sequence in 33 items and 5.0 for 16.)  The arithmetic is
 // that of plan_even and plan_balanced below.
 __device__ __forceinline__ bool plan_small_ok(const PlanArgs& a) {
   return a.B <= kPlanThreads && a.n_workers + a.B <= kPlanStage;

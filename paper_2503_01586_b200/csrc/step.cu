@@ -6,8 +6,9 @@
 // the chain of programmatic dependent launches.  Here they are blocks of one grid: block 0 the plan, then
 // the appended tokens, the query RoPE of a head each, and the (head, 128 coordinates, sequences)
 // blocks of the absorption, whose weight slabs are fetched before the dependency wait.
-// From the release of the grid by the previous step's combine to its end: one sequence 2.5 us, 7B 75 % B16
-// 3.7, ragged B64 7.0, 13B B32 5.3, 50 % B32 9.5 (11 to 12 us for the last three while a single warp fetched
+// From the release of the grid by the previous step's combine to its end: one sequence 2.8 us, 7B 75 % B16
+// 3.0 (the plan; the query preparation 2.6 and 2.9); while the plan was a thread per sequence at every size 4.0 and 5.0,
+// ragged B64 7.0, 13B B32 5.3, 50 % B32 9.5 (11 to 12 us for the last three while a single warp fetched
 // the weights and registers kept blocks waiting for a second wave; the 50 % shape's 833 blocks still do not
 // all fit).  As separate launches: 16 us at B16, 21 at ragged B64.
 #include "absorb.cuh"
